@@ -84,6 +84,46 @@ void release(ksc_split *s) {
     delete s;
 }
 
+// Plan of the tensor-core belt stage: the widest window and the most input rings of a
+// 16-ring tile, and the power of two that scales the kernel's largest value.
+int plan_belt_tc(ksc_split *s, const ksc::RingGeom &g, const std::vector<int2> &range,
+                 const std::vector<ksc::PairInfo> &pairs, const std::vector<int> &pair_base) {
+    if (s->path != 0 || s->n_items_belt == 0) return KSC_OK;
+    // Below about 3e8 belt pairs the FFMA kernel is the faster one: a tile spends 0.7 to
+    // 1.8 us on an input ring however short the window, and small maps have few tiles
+    // (FFMA / tensor stage, us: nside 64, 360': 58 / 72; 256, 160' (2.2e8 pairs): 91 / 99;
+    // 512, 60' (5e8): 123 / 115; 256, 640' (3.6e9): 542 / 371; 1024, 160': 3605 / 1177).
+    if (2.0 / 3.0 * ksc_cost_pairs(s->nside, s->theta_cut) < 3e8) return KSC_OK;
+    const int lo = s->plan.belt_lo, hi = s->plan.belt_hi, nb = ksc::belt_tc_rings();
+    int wpos = 0, nq = 0;
+    for (int r0 = lo; r0 <= hi; r0 += nb) {
+        int q0 = hi, q1 = lo;
+        for (int r = r0; r < std::min(r0 + nb, hi + 1); ++r) {
+            q0 = std::min(q0, std::max(range[r].x, lo));
+            q1 = std::max(q1, std::min(range[r].y, hi));
+            for (int q = std::max(range[r].x, lo); q <= std::min(range[r].y, hi); ++q) {
+                const int w = pairs[(size_t)pair_base[r] + (q - range[r].x)].w;
+                if (w >= 0) wpos = std::max(wpos, ksc::belt_tc_positions(w, g.len[r]));
+            }
+        }
+        nq = std::max(nq, q1 - q0 + 1);
+    }
+    std::vector<float4> tab(s->n_int);
+    const cudaError_t e = cudaMemcpy(tab.data(), s->d_tab, sizeof(float4) * tab.size(),
+                                     cudaMemcpyDeviceToHost);
+    if (e != cudaSuccess) return cuda_fail(e, "table download");
+    double top = 0.0;
+    for (const float4 &c : tab)
+        top = std::max({top, (double)std::fabs(c.x), std::fabs((double)c.x + c.y + c.z + c.w)});
+    if (top == 0.0) return KSC_OK;
+    const int ex = std::isfinite(top) ? 13 - std::ilogb(top) : 1000;
+    // scaled weights and sums stay normal FP32 numbers; otherwise the FFMA kernel
+    if (ex < -20 || ex > 40) return KSC_OK;
+    if (!ksc::belt_tc_plan(s->nside, wpos, nq, &s->btc)) s->btc.n_cols = 0;
+    s->btc.wscale = (float)std::ldexp(1.0, ex);
+    return KSC_OK;
+}
+
 // Geometry, work list and device table for the real-space part s->c_real.
 int finish_split(ksc_split *s, const ksc_split_opts &o) {
     const int nside = s->nside;
@@ -406,7 +446,7 @@ int finish_split(ksc_split *s, const ksc_split_opts &o) {
         p.belt_c1h = c1.h;
         p.belt_c1l = c1.l;
     }
-    return KSC_OK;
+    return plan_belt_tc(s, g, range, pairs, pair_base);
 }
 
 int check_common(int lmax, int nside, double theta_cut) {
@@ -441,6 +481,34 @@ int check_maps(const ksc_split *s, const void *a, const void *b) {
     if (((uintptr_t)a | (uintptr_t)b) & 15u)
         return fail(KSC_ERR_ARG, "maps must be 16-byte aligned");
     return KSC_OK;
+}
+
+// The belt stage (belt-belt ring pairs) of output rings [r0, r1]: the tensor-core kernel
+// where the split has a plan for it, then the FFMA kernel for the tiles it left (none of
+// them in an ordinary map: that launch reads the flags and ends); else the FFMA kernel.
+cudaError_t launch_belt(const ksc_split *s, const float *d_in, float *d_out, int n_maps,
+                        long long stride, int r0, int r1, cudaStream_t st) {
+    const int a = s->ring_first_belt[r0], b = s->ring_first_belt[r1 + 1];
+    if (a == b || s->n_items_belt == 0) return cudaSuccess;
+    if (s->btc.n_cols == 0)
+        return ksc::launch_conv_belt(s->plan, s->d_items_belt + a, b - a, s->seg_cap, d_in, d_out,
+                                     n_maps, stride, nullptr, nullptr, s->d_err, st);
+    const size_t bm_bytes = sizeof(unsigned) * (size_t)ksc::map_blocks(s->plan) * n_maps;
+    const size_t fl_bytes = (size_t)ksc::belt_tc_tiles(s->plan, s->btc) * n_maps;
+    unsigned char *ws = nullptr;  // block maxima, then the tiles' flags
+    cudaError_t e = cudaMallocAsync(&ws, bm_bytes + fl_bytes, st);
+    if (e != cudaSuccess) return e;
+    unsigned *bm = reinterpret_cast<unsigned *>(ws);
+    unsigned char *flags = ws + bm_bytes;
+    e = ksc::launch_block_max(s->plan, d_in, n_maps, stride, bm, st);
+    if (e == cudaSuccess)
+        e = ksc::launch_conv_belt_tc(s->plan, s->btc, d_in, d_out, n_maps, stride, r0, r1, bm,
+                                     flags, s->d_err, st);
+    if (e == cudaSuccess)
+        e = ksc::launch_conv_belt(s->plan, s->d_items_belt + a, b - a, s->seg_cap, d_in, d_out,
+                                  n_maps, stride, &s->btc, flags, s->d_err, st);
+    const cudaError_t f = cudaFreeAsync(ws, st);
+    return e != cudaSuccess ? e : f;
 }
 
 // Tensor-core belt stage for a stack of maps; grows the split's pre-tiled map
@@ -510,9 +578,7 @@ int launch_conv(const ksc_split *s, const float *d_in, float *d_out, int n_maps,
         int rc = launch_belt_tensor(s, d_in, d_out, n_maps, stride, st);
         if (rc) return rc;
     } else {
-        const int a = s->ring_first_belt[r0], b = s->ring_first_belt[r1 + 1];
-        e = ksc::launch_conv_belt(s->plan, s->d_items_belt + a, b - a, s->seg_cap, d_in, d_out,
-                                  n_maps, stride, s->d_err, st);
+        e = launch_belt(s, d_in, d_out, n_maps, stride, r0, r1, st);
         if (e != cudaSuccess) return cuda_fail(e, "belt kernel launch");
     }
     // northern rings r whose own or mirror ring (nr - 1 - r) lies in the band
@@ -926,8 +992,7 @@ int ksc_conv_real_multimap_stage(const ksc_split *s, const float *d_in, float *d
         if (n_maps >= 16 && s->tensor == 2 && s->n_items_mma > 0)
             return launch_belt_tensor(s, d_in, d_out, n_maps, stride, st);
         else
-            e = ksc::launch_conv_belt(s->plan, s->d_items_belt, s->n_items_belt, s->seg_cap,
-                                      d_in, d_out, n_maps, stride, s->d_err, st);
+            e = launch_belt(s, d_in, d_out, n_maps, stride, 0, s->plan.nrings - 1, st);
     } else if (stage == 2) {
         if (s->path == 1)
             e = ksc::launch_conv_general(s->plan, s->d_items, s->n_items, d_in, d_out, n_maps,
@@ -949,8 +1014,7 @@ int ksc_conv_real_stage(const ksc_split *s, const float *d_in, float *d_out, int
     cudaStream_t st = (cudaStream_t)stream;
     cudaError_t e;
     if (stage == 1) {
-        e = ksc::launch_conv_belt(s->plan, s->d_items_belt, s->n_items_belt, s->seg_cap, d_in,
-                                  d_out, 1, 0, s->d_err, st);
+        e = launch_belt(s, d_in, d_out, 1, 0, 0, s->plan.nrings - 1, st);
     } else if (stage == 2) {
         if (s->path == 1)
             e = ksc::launch_conv_general(s->plan, s->d_items, s->n_items, d_in, d_out, 1, 0, 0,

@@ -167,7 +167,9 @@ __device__ __forceinline__ bool belt_item(const ConvPlan &P, int r, int k0,
                                           const float *__restrict__ m, float *__restrict__ o,
                                           float *seg0, float *seg1, float *wbuf, uint64_t *bar,
                                           PairGeom *s_g, int *s_abort, uint32_t &phase0,
-                                          uint32_t &phase1, int seg_cap, int *__restrict__ err) {
+                                          uint32_t &phase1, int seg_cap, int *__restrict__ err,
+                                          const unsigned char *__restrict__ tf = nullptr,
+                                          int tile_shift = 0) {
     constexpr int kChunkT = kU * T;
     const int tid = threadIdx.x;
     const DevRing R = P.d_rings[r];
@@ -292,7 +294,7 @@ __device__ __forceinline__ bool belt_item(const ConvPlan &P, int r, int k0,
 #pragma unroll
     for (int u = 0; u < kU; ++u) {
         const int k = k0 + kb + u;
-        if (k < L) o[R.start + k] = sum[u] * P.domega;
+        if (k < L && (!tf || tf[k >> tile_shift])) o[R.start + k] = sum[u] * P.domega;
     }
     return true;
 }
@@ -316,18 +318,31 @@ __device__ __forceinline__ bool belt_item(const ConvPlan &P, int r, int k0,
     __syncthreads();                                                    \
     uint32_t phase0 = 0u, phase1 = 0u;
 
-// One split, items assigned round-robin; grid.y runs over maps.
+// One split, items assigned round-robin; grid.y runs over maps.  With flags (one byte
+// per tile of tile_rings belt rings x 2^tile_shift pixels, row_tiles tiles a row,
+// map_tiles a map) only the pixels of flagged tiles are computed and written.
 template <int T>
 __global__ void __launch_bounds__(T)
 conv_belt_kernel(const ConvPlan P, const int2 *__restrict__ items, int n_items,
                  const float *__restrict__ in, float *__restrict__ out, long long map_stride,
-                 int seg_cap, int *__restrict__ err) {
+                 int seg_cap, int *__restrict__ err, const unsigned char *__restrict__ flags,
+                 int tile_rings, int tile_shift, int row_tiles, int map_tiles) {
     KSC_BELT_SHARED_STATE
     const float *m = in + (long long)blockIdx.y * map_stride;
     float *o = out + (long long)blockIdx.y * map_stride;
     for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
-        if (!belt_item<T>(P, items[it].x, items[it].y, m, o, seg0, seg1, wbuf, bar, s_g,
-                          &s_abort, phase0, phase1, seg_cap, err))
+        const int r = items[it].x, k0 = items[it].y;
+        const unsigned char *tf = nullptr;
+        if (flags) {
+            tf = flags + (long long)blockIdx.y * map_tiles +
+                 (long long)((r - P.belt_lo) / tile_rings) * row_tiles;
+            const int t1 = (min(k0 + kU * T, 4 * P.nside) - 1) >> tile_shift;
+            int any = 0;
+            for (int t = k0 >> tile_shift; t <= t1; ++t) any |= tf[t];
+            if (!any) continue;
+        }
+        if (!belt_item<T>(P, r, k0, m, o, seg0, seg1, wbuf, bar, s_g, &s_abort, phase0, phase1,
+                          seg_cap, err, tf, tile_shift))
             return;
     }
 }
@@ -390,15 +405,23 @@ int belt_chunk() { return kChunk; }
 
 cudaError_t launch_conv_belt(const ConvPlan &p, const int2 *d_items, int n_items, int seg_cap,
                              const float *d_in, float *d_out, int n_maps, long long map_stride,
-                             int *d_err, cudaStream_t st) {
+                             const BeltTc *tc, const unsigned char *tile_flags, int *d_err,
+                             cudaStream_t st) {
     if (n_items <= 0 || n_maps <= 0) return cudaSuccess;
+    int shift = 0, row = 0, all = 0;
+    if (tile_flags) {
+        while ((1 << shift) < 8 * tc->n_cols) ++shift;
+        row = p.nside / (2 * tc->n_cols);
+        all = belt_tc_tiles(p, *tc);
+    }
     const size_t smem = sizeof(float) * 3 * (size_t)seg_cap;
     int blocks = 0;
     cudaError_t e = belt_grid(conv_belt_kernel<kThreads>, kThreads, smem, n_items, 0, &blocks);
     if (e != cudaSuccess) return e;
     dim3 grid(blocks, n_maps);
-    conv_belt_kernel<kThreads><<<grid, kThreads, smem, st>>>(p, d_items, n_items, d_in, d_out,
-                                                             map_stride, seg_cap, d_err);
+    conv_belt_kernel<kThreads><<<grid, kThreads, smem, st>>>(
+        p, d_items, n_items, d_in, d_out, map_stride, seg_cap, d_err, tile_flags,
+        belt_tc_rings(), shift, row, all);
     return cudaGetLastError();
 }
 

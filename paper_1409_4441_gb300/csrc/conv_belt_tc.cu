@@ -1,0 +1,708 @@
+// Real-space convolution, equatorial-belt ring pairs, on the tcgen05 tensor cores.
+//
+// For an output ring r and an input ring q of the belt the kernel weight depends on
+// Delta = k' - k only (conv_belt.cu), so the ring pair is a Toeplitz product.  A CTA
+// owns 16 consecutive output rings and 8 N consecutive pixels of each, and for every
+// input ring q in reach of one of them adds
+//
+//   D[(R, i), n] += sum_j A[(R, i), j] B[j, n],   A[(R, i), j] = w_R[d0 + j - i],
+//                                                 B[j, n] = m_q[k0 + d0 + j + 8 n],
+//
+// D[(R, i), n] being pixel k0 + 8 n + i of ring R: M = 128 rows are 16 rings x 8 offsets,
+// N columns are groups of eight pixels, K is the window.  Neither operand is copied out
+// to a full matrix.  B's core matrices (8 columns x 16 bytes) are read straight from the
+// input segment as it lies in shared memory: columns 8 elements (16 bytes) apart, so
+// K-adjacent core matrices overlap at a stride of 16 bytes.  A's eight rows of a ring are
+// the same weights shifted by one element each.  The padding of a window is 7 positions
+// plus the rounding to K = 16, against 13 to 25 of the FFMA form.
+//
+// Precision.  With the map scaled per tile and the weights per split so that their
+// largest magnitudes lie near 2^15 and 2^13, each value is the sum of two FP16 numbers,
+// v = h + l, l the rounding error of h: exactly v for |v| >= 2^-1 (24 bits in two parts
+// of 11 and a sign), within 2^-25 otherwise, i.e. within 2^-40 of the largest.  Three MMAs
+// per 16 positions sum w_h m_l, w_l m_h and w_h m_h in FP32; w_l m_l (below 2^-24 of the
+// product) is summed too where the weights are large, in the two steps of the closest
+// approach.  An MMA cuts every addend, the accumulator too, at 2^-25 of the largest one and
+// rounds the sum toward zero to 24 bits (found with known operands), so the order matters:
+// within 64 positions the small products first, the 64 positions that hold the closest
+// approach last, and its own two steps at the very end.  After each input ring the
+// accumulator is folded into FP32 totals with the rounding error of the sum (two-sum),
+// plus the 2^-24 of the partial that the cuts take from it on average, written back to
+// tensor memory as the start of a later partial.  The weights keep the rounding error of
+// their last addition in w_l.  Maps with an offset: where all of a tile's input is of one
+// size, a constant near its mean is taken off and put back through the sum of the weights,
+// so that the cuts, which are toward zero, do not add up.
+//
+// A tile where some block of 64 input pixels is more than 2^14 below the tile's largest
+// value (all-zero blocks aside), or that holds an infinity or NaN, is left to
+// conv_belt_kernel (belt_tc_flags): the scaled split would not carry its values to 26
+// bits of their neighbourhood, or would spread a NaN further than the window.
+//
+// Every mbarrier wait is bounded; a wait that runs out raises the device error flag.
+#include <algorithm>
+#include <cstdint>
+#include <cuda_fp16.h>
+
+#include "ksc_device.cuh"
+#include "ksc_internal.h"
+#include "ksc_tc.cuh"
+
+namespace ksc {
+namespace {
+
+constexpr int kT = 512;        // builder threads: warp R builds ring R's weights
+constexpr int kThreads = kT + 128;  // and a warpgroup whose first warp issues the MMAs
+constexpr int kRings = 16;     // output rings of a tile
+constexpr int kChunk = 128;    // window positions per A stage
+constexpr int kSteps = kChunk / 16;
+constexpr int kPartBytes = kRings * kChunk * 16;  // one FP16 part of an A stage (32 kB)
+constexpr int kStageBytes = 2 * kPartBytes;
+constexpr int kStages = 2;
+constexpr int kXExp = 14;      // a tile's largest |m| is scaled into [2^14, 2^15)
+constexpr uint32_t kRangeExp = 14;  // a block may lie this many powers of two below it
+
+// K-major, no swizzle: 8-row x 16-byte core matrices; lead = bytes between core matrices
+// adjacent in K, stride = bytes between groups of eight rows.
+__device__ __forceinline__ uint64_t tc_desc(uint32_t addr, uint32_t lead, uint32_t stride) {
+    return (uint64_t)((addr & 0x3FFFF) >> 4) | (uint64_t)((lead >> 4) & 0x3FFF) << 16 |
+           (uint64_t)((stride >> 4) & 0x3FFF) << 32 | (uint64_t)1 << 46;
+}
+
+// FP16 operands, FP32 accumulator, both K-major.
+__host__ __device__ constexpr uint32_t idesc_f16(int M, int N) {
+    return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+
+__device__ __forceinline__ void mma_f16(uint32_t tmem, uint64_t da, uint64_t db, uint32_t idesc,
+                                        uint32_t acc) {
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
+        "l"(da), "l"(db), "r"(idesc), "r"(acc));
+}
+
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t *v) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
+          "=r"(v[7])
+        : "r"(taddr));
+}
+
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t *v) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr),
+        "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+        : "memory");
+}
+
+// Two FP32 values in one register pair.
+__device__ __forceinline__ uint64_t pack2(uint32_t a, uint32_t b) {
+    return (uint64_t)b << 32 | a;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+// Bounded wait that also ends when another warp of the CTA has given up.
+__device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity,
+                                              volatile int *abort) {
+    for (int i = 0; i < 64; ++i) {
+        if (tc::mbar_wait(bar, parity, tc::kMaxWait / 64)) return true;
+        if (*abort) break;
+    }
+    *abort = 1;
+    return false;
+}
+
+// One input ring as seen by the tile: window [lo, hi] of Delta common to the tile's rings
+// (the widest one's), and the 16-position steps [s0, s1) of a grid of 128-position chunks
+// whose chunk `mid` is centred on the closest approach.  Position j stands for
+// Delta = d0 + j - i, i = 0..7.
+struct Window {
+    int d0, s0, s1, mid;
+};
+__host__ __device__ __forceinline__ Window tile_window(int w, int L) {
+    const bool whole = 2 * w + 1 >= L;  // the whole ring, each pixel once
+    const int lo = whole ? -(L / 2) : -w, hi = whole ? lo + L - 1 : w;
+    Window g;
+    // chunks left of the one with j = 64 in its middle (Delta = -4 .. 3 over i)
+    g.mid = (unsigned)(-lo + 3 - kChunk / 2 + kChunk - 1) / kChunk;
+    g.d0 = -(g.mid * kChunk + kChunk / 2) + 3;
+    g.s0 = (unsigned)(lo - g.d0) / 16;          // first j of any use: Delta = lo at i = 0
+    g.s1 = (unsigned)(hi - g.d0 + 7) / 16 + 1;  // last: Delta = hi at i = 7
+    return g;
+}
+// The chunks of a window in order of work: the closest approach's last.
+__device__ __forceinline__ int chunk_of(int cc, int c_hi, int mid) {
+    return cc == c_hi ? mid : (cc >= mid ? cc + 1 : cc);
+}
+
+// N columns: 8 N pixels per ring.  grid.x runs over tiles (16-ring block, pixel tile),
+// grid.y over maps.  Sixteen builder warps stage the map, evaluate the weights, lay out A
+// and fold the accumulators; a seventeenth issues the MMAs (the
+// rest of its warpgroup only gives its registers to the builders).  A builder warp hands a stage
+// over by arriving on a_full; that arrival also says that its part of the ring's input
+// segment is staged and that it has folded the accumulator the ring's MMAs will write
+// (each warp folds ring n - 2 before it arrives for ring n).
+template <int N>
+__global__ void __launch_bounds__(kThreads, 1)
+conv_belt_tc_kernel(const ConvPlan P, int block_lo, int n_tiles_k, int ring_lo, int ring_hi,
+                    const float *__restrict__ in, float *__restrict__ out, long long map_stride,
+                    const uint32_t *__restrict__ blockmax, long long block_stride,
+                    unsigned char *__restrict__ flags, int n_tiles, int wpos_cap, int nq_cap,
+                    float wscale, float wunscale, float domega_lo, int *__restrict__ err) {
+    constexpr int kCols = N / 4;  // columns per thread (four warps share a lane quarter)
+    constexpr int kStep = kCols < 16 ? 8 : 16;
+    constexpr uint32_t kTmem = 2 * N;
+    extern __shared__ __align__(1024) unsigned char smem[];
+    // A stages | two input segments (two FP16 parts each) | weights (h, l pairs) | windows
+    const int seg_cap = 8 * N + wpos_cap;  // elements
+    const int w_cap = wpos_cap + 16;
+    unsigned char *sA = smem;
+    __half *sB = reinterpret_cast<__half *>(smem + kStages * kStageBytes);
+    uint32_t *sW = reinterpret_cast<uint32_t *>(sB + 4 * seg_cap);
+    short *sQ = reinterpret_cast<short *>(sW + kRings * w_cap);
+    __shared__ __align__(8) uint64_t a_full[kStages], a_free[kStages], d_done[2];
+    __shared__ uint32_t tmem_base;
+    __shared__ uint32_t s_max, s_min;
+    __shared__ int s_abort, s_lo, s_hi, s_bad;
+    __shared__ float s_mean[kRings], s_wsum[kRings];
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rb = block_lo + blockIdx.x / n_tiles_k, ct = blockIdx.x % n_tiles_k;
+    const int r_first = P.belt_lo + rb * kRings;
+    const int n_rows = min(kRings, P.belt_hi - r_first + 1);
+    const int L = 4 * P.nside, k0 = ct * 8 * N;
+    const float *m = in + (long long)blockIdx.y * map_stride;
+    float *o = out + (long long)blockIdx.y * map_stride;
+    const uint32_t *bm = blockmax + (long long)blockIdx.y * block_stride;
+    const int start0 = P.d_rings[r_first].start;
+
+    // ---- the tile's input rings and windows, and the range of the values in them
+    if (tid == 0) {
+        s_max = 0u;
+        s_min = 0xffffffffu;
+        s_abort = s_bad = 0;
+        s_lo = P.belt_hi;
+        s_hi = P.belt_lo;
+        for (int b = 0; b < kStages; ++b) {
+            tc::mbar_init(&a_full[b], kRings);
+            tc::mbar_init(&a_free[b], 1);
+        }
+        for (int b = 0; b < 2; ++b) tc::mbar_init(&d_done[b], 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    if (warp == 0 && lane < n_rows) {
+        const int2 g = P.d_range[r_first + lane];
+        atomicMin(&s_lo, max(g.x, P.belt_lo));
+        atomicMax(&s_hi, min(g.y, P.belt_hi));
+    }
+    __syncthreads();
+    const int q_lo = s_lo, nq = s_hi - s_lo + 1;
+    uint32_t vmax = 0u, vmin = 0xffffffffu;
+    for (int q = q_lo + warp; q < q_lo + nq; q += kThreads / 32) {
+        int w = -1;
+        if (lane < n_rows) {
+            const int2 g = P.d_range[r_first + lane];
+            if (q >= g.x && q <= g.y) w = P.d_pairs[P.d_pair_base[r_first + lane] + q - g.x].w;
+        }
+        w = __reduce_max_sync(~0u, w);
+        w = min(w, L / 2);
+        if (w < 0) {
+            if (lane == 0 && q - q_lo < nq_cap) sQ[q - q_lo] = -1;
+            continue;
+        }
+        const Window g = tile_window(w, L);
+        if (lane == 0) {  // the host sized both for every tile: never expected
+            if (q - q_lo < nq_cap && 16 * (g.s1 - g.s0) <= wpos_cap) sQ[q - q_lo] = (short)w;
+            else s_bad = 1;
+        }
+        const int start = P.d_rings[q].start;
+        // pixels [a, a + len) of the ring, wrapped; every block of 64 map pixels in them
+        const int len = min(8 * N + 16 * (g.s1 - g.s0), L);
+        int a = (k0 + g.d0 + 16 * g.s0) % L;
+        a += a < 0 ? L : 0;
+        const int head = min(len, L - a);
+        for (int part = 0; part < 2; ++part) {
+            const int p0 = start + (part ? 0 : a), p1 = start + (part ? len - head : a + head);
+            if (p1 <= p0) continue;
+            for (int b = (p0 >> 6) + lane; b <= (p1 - 1) >> 6; b += 32) {
+                const uint32_t v = __ldg(bm + b);
+                vmax = max(vmax, v);
+                if (v) vmin = min(vmin, v);
+            }
+        }
+    }
+    vmax = __reduce_max_sync(~0u, vmax);
+    vmin = __reduce_min_sync(~0u, vmin);
+    if (warp < kRings) {  // mean of 512 of the tile's own pixels
+        float v = m[start0 + (warp < n_rows ? warp : 0) * L + k0 + lane * (N / 4)];
+#pragma unroll
+        for (int s = 16; s > 0; s >>= 1) v += __shfl_xor_sync(~0u, v, s);
+        if (lane == 0) s_mean[warp] = v * (1.0f / 32.0f);
+    }
+    if (lane == 0) {
+        atomicMax(&s_max, vmax);
+        atomicMin(&s_min, vmin);
+    }
+    if (warp == kRings) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                         tc::saddr(&tmem_base)),
+                     "r"(kTmem));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t tmem = tmem_base;
+    const uint32_t emax = s_max >> 23, emin = s_min >> 23;  // biased exponents
+    const bool zero = s_max == 0u;
+    // scales stay normal floats: exponents of 2^(14 - e) within [-126, 127]
+    const bool flag = !zero && (emax >= 255u || emax < 48u || emax > 206u || emin == 0u ||
+                                emax - emin > kRangeExp);
+    if (tid == 0) {
+        flags[(long long)blockIdx.y * n_tiles + rb * n_tiles_k + ct] = flag ? 1 : 0;
+        if (s_bad) atomicExch(err, KSC_ERR_DEVICE_BOUNDS);
+    }
+    // a constant taken off where every block is within a factor of four of the largest: a
+    // multiple of 2^-3 of the largest value's power of two (none for maps about zero)
+    float mean = 0.0f;
+    if (!zero && !flag && emax - emin <= 1u) {
+#pragma unroll
+        for (int i = 0; i < kRings; ++i) mean += s_mean[i];
+        const float quantum = __uint_as_float((emax - 3u) << 23);
+        mean = rintf(mean * (1.0f / kRings) / quantum) * quantum;
+    }
+    // |m - mean| may reach twice the largest |m|
+    const uint32_t ex = emax + (mean != 0.0f ? 1u : 0u);
+    const float xscale = zero || flag ? 1.0f : __uint_as_float((127u + kXExp + 127u - ex) << 23);
+    const float xunscale = zero || flag ? 1.0f : __uint_as_float((ex - kXExp) << 23);
+    bool drained = true;  // no MMA in flight can still write tensor memory
+
+    if (flag || s_bad) {
+        // left to the FFMA kernel (or never expected)
+    } else if (warp >= kRings) {
+        // ---- the issuing warp
+        if constexpr (N == 256) asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
+        if (warp == kRings && lane == 0) {
+            const uint32_t idesc = idesc_f16(128, N);
+            const uint32_t pa0 = tc::saddr(sA), pb0 = tc::saddr(sB);
+            const uint64_t a_hi = tc_desc(0, 128, kChunk * 16), b_hi = tc_desc(0, 16, 128);
+            const uint32_t a_l = kPartBytes >> 4, b_l = (uint32_t)(seg_cap * 2) >> 4;
+            uint32_t n_rings = 0, n_chunks = 0;
+            bool ok = true;
+            for (int qi = 0; qi < nq && ok; ++qi) {
+                const int w = sQ[qi];
+                if (w < 0) continue;
+                const Window g = tile_window(w, L);
+                const uint32_t b = n_rings & 1u;
+                const uint32_t d = tmem + b * N;
+                uint32_t acc = n_rings >= 2 ? 1u : 0u;
+                const int c_lo = g.s0 / kSteps, c_hi = (g.s1 - 1) / kSteps;
+                for (int cc = c_lo; cc <= c_hi; ++cc, ++n_chunks) {
+                    const int c = chunk_of(cc, c_hi, g.mid);
+                    const uint32_t st = n_chunks & 1u;
+                    if (!wait_or_abort(&a_full[st], (n_chunks >> 1) & 1u, &s_abort)) {
+                        ok = false;
+                        break;
+                    }
+                    tc::fence_after_sync();
+                    const int t0 = max(g.s0, kSteps * c), t1 = min(g.s1, kSteps * c + kSteps);
+                    // descriptors of step s: the stage's A at 256 s bytes, B at 32 s bytes
+                    const uint64_t da0 = a_hi + ((pa0 + st * kStageBytes) >> 4);
+                    const uint64_t db0 = b_hi + ((pb0 + b * 4 * seg_cap) >> 4);
+                    auto da = [&](int s) { return da0 + (uint32_t)((s - kSteps * c) * 16); };
+                    auto db = [&](int s) { return db0 + (uint32_t)((s - g.s0) * 2); };
+                    if (c == g.mid) {
+                        for (int s = kSteps * c + 3; s < kSteps * c + 5; ++s) {
+                            if (s < t0 || s >= t1) continue;
+                            mma_f16(d, da(s) + a_l, db(s) + b_l, idesc, acc);
+                            acc = 1u;
+                        }
+                    }
+                    for (int s = t0; s < t1; ++s) {
+                        mma_f16(d, da(s), db(s) + b_l, idesc, acc);
+                        mma_f16(d, da(s) + a_l, db(s), idesc, 1u);
+                        acc = 1u;
+                    }
+                    if (c == g.mid) {  // from the ends to the closest approach
+                        for (int e = 0; e < kSteps; ++e) {
+                            const int s = kSteps * c + ((e & 1) ? kSteps - 1 - (e >> 1) : e >> 1);
+                            if (s >= t0 && s < t1) mma_f16(d, da(s), db(s), idesc, 1u);
+                        }
+                    } else {
+                        for (int s = t0; s < t1; ++s) mma_f16(d, da(s), db(s), idesc, 1u);
+                    }
+                    tc::mma_commit(&a_free[st]);
+                }
+                if (!ok) break;
+                tc::mma_commit(&d_done[b]);
+                ++n_rings;
+            }
+            // every MMA has ended before the tensor memory goes (after an abort: bounded)
+            if (n_chunks > 0 && !ok)
+                drained = tc::mbar_wait(&a_free[(n_chunks - 1) & 1u], ((n_chunks - 1) >> 1) & 1u);
+        }
+        __syncwarp();
+    } else {
+        // ---- builder warps
+        // 640 x 96 registers at launch = 512 x 112 + 128 x 32
+        if constexpr (N == 256) asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
+        // this thread's accumulators: lane quarter warp & 3, columns (warp >> 2) kCols ..
+        const uint32_t td =
+            tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * kCols);
+        uint32_t *wr = sW + warp * w_cap;
+        const int my_r = r_first + warp;  // the ring this warp builds weights for
+        int2 rg = make_int2(P.belt_hi + 1, P.belt_lo - 1);
+        int base = 0, my_phase = 0;
+        if (warp < n_rows) {
+            rg = P.d_range[my_r];
+            base = P.d_pair_base[my_r] - rg.x;
+            my_phase = P.d_rings[my_r].phase;
+        }
+        const float moff = -mean * xscale;
+        uint64_t tot[kCols / 2];
+#pragma unroll
+        for (int c = 0; c < kCols / 2; ++c) tot[c] = 0ull;
+        float wsum = 0.0f, wcomp = 0.0f;
+        uint32_t n_rings = 0, n_chunks = 0;
+        bool ok = true;
+
+        // fold the accumulator of ring n into the totals, leaving in it the sums' rounding
+        // errors and the 2^-24 that the MMAs' cuts cost on average
+        auto drain = [&](uint32_t n) {
+            const uint32_t b = n & 1u;
+            if (!__all_sync(~0u, wait_or_abort(&d_done[b], (n >> 1) & 1u, &s_abort))) return false;
+            tc::fence_after_sync();
+            const uint64_t m1 = pack2(0xbf800000u, 0xbf800000u);  // -1
+            const uint64_t cut = pack2(0x33800000u, 0x33800000u);  // 2^-24
+            uint32_t v[kStep];
+#pragma unroll
+            for (int c = 0; c < kCols; c += kStep) {
+                const uint32_t t = td + b * N + c;
+                __syncwarp();
+                if constexpr (kStep == 16) tc::tmem_ld16(t, v); else tmem_ld8(t, v);
+                tc::tmem_wait_ld();
+#pragma unroll
+                for (int e = 0; e < kStep; e += 2) {
+                    const uint64_t y = pack2(v[e], v[e + 1]), t0 = tot[(c + e) / 2];
+                    const uint64_t s = add2(t0, y);
+                    const uint64_t r = fma2(y, cut, fma2(fma2(t0, m1, s), m1, y));
+                    tot[(c + e) / 2] = s;
+                    v[e] = (uint32_t)r;
+                    v[e + 1] = (uint32_t)(r >> 32);
+                }
+                if constexpr (kStep == 16) tc::tmem_st16(t, v); else tmem_st8(t, v);
+            }
+            tc::tmem_wait_st();
+            tc::fence_before_sync();
+            return true;
+        };
+
+        for (int qi = 0; qi < nq; ++qi) {
+            const int w = sQ[qi];
+            if (w < 0) continue;
+            const int q = q_lo + qi;
+            const uint32_t b = n_rings & 1u;
+            const Window g = tile_window(w, L);
+            const int n_pos = 16 * (g.s1 - g.s0);
+            const DevRing *Q = P.d_rings + q;
+            PairInfo pi;
+            pi.w = -1;
+            if (q >= rg.x && q <= rg.y) pi = P.d_pairs[base + q];
+            const int tdiff = my_phase - Q->phase;
+            // ---- the input segment, scaled and split into two FP16 parts
+            {
+                int a = (k0 + g.d0 + 16 * g.s0) % L;
+                a += a < 0 ? L : 0;
+                const float *ring = m + Q->start;
+                __half2 *bh = reinterpret_cast<__half2 *>(sB + b * 2 * seg_cap);
+                __half2 *bl = bh + seg_cap / 2;
+                const int n2 = (8 * N + n_pos) / 2;
+                auto load = [&](int e, float *x0, float *x1) {
+                    int i = a + 2 * e;
+                    while (i >= L) i -= L;
+                    *x0 = __ldg(ring + i);
+                    *x1 = __ldg(ring + (i + 1 == L ? 0 : i + 1));
+                };
+                auto put = [&](int e, float x0, float x1) {
+                    const float y0 = fmaf(x0, xscale, moff), y1 = fmaf(x1, xscale, moff);
+                    const __half2 h = __floats2half2_rn(y0, y1);
+                    const float2 f = __half22float2(h);
+                    bh[e] = h;
+                    bl[e] = __floats2half2_rn(y0 - f.x, y1 - f.y);
+                };
+                int e = tid;
+                for (; e + kT < n2; e += 2 * kT) {  // two pairs of loads in flight
+                    float x0, x1, y0, y1;
+                    load(e, &x0, &x1);
+                    load(e + kT, &y0, &y1);
+                    put(e, x0, x1);
+                    put(e + kT, y0, y1);
+                }
+                if (e < n2) {
+                    float x0, x1;
+                    load(e, &x0, &x1);
+                    put(e, x0, x1);
+                }
+            }
+            // ---- this warp's ring: its weights over the tile's window, Delta at element
+            // x = Delta + x_of; all of 0 .. n_x - 1 are written
+            {
+                const int x_of = 8 - g.d0 - 16 * g.s0;
+                const int n_x = n_pos + 16;
+                const bool whole = 2 * pi.w + 1 >= L;
+                const int lo = whole ? -(L / 2) : -pi.w, hi = whole ? lo + L - 1 : pi.w;
+                // w(Delta) = w(tdiff - Delta): both from one evaluation, but for whole rings
+                const int d_first = whole ? -x_of : (tdiff + 1) >> 1;
+                const int n_d =
+                    whole ? n_x : max(n_x - x_of - d_first, tdiff + x_of - d_first + 1);
+                const DF A{pi.Ah, pi.Al}, B{pi.Bh, pi.Bl};
+                // weight (scaled) and the scaled rounding error of its last addition
+                auto weight = [&](int d, float *we) {
+                    const float mf = (float)(tdiff - 2 * d);
+                    const float xh = mf * P.belt_c1h;
+                    const float xl = fmaf(mf, P.belt_c1h, -xh) + mf * P.belt_c1l;
+                    int ti;
+                    float f;
+                    const bool in = chord_to_table_sel(A, B, sin_df(xh, xl), P.nint2, &ti, &f) &&
+                                    d >= lo && d <= hi;  // (no ring in reach: hi < lo)
+                    const float4 c = __ldg(&P.d_tab[min(ti, P.n_int - 1)]);
+                    const float t = f * fmaf(f, fmaf(f, c.w, c.z), c.y);
+                    const float v = c.x + t, bb = v - c.x;
+                    *we = in ? ((c.x - (v - bb)) + (t - bb)) * wscale : 0.0f;
+                    return in ? v * wscale : 0.0f;
+                };
+                auto put = [&](int i, float v, float ve) {
+                    const int x = d_first + i + x_of, y = tdiff - d_first - i + x_of;
+                    const __half h = __float2half_rn(v);
+                    const __half l = __float2half_rn((v - __half2float(h)) + ve);
+                    const uint32_t hl = (uint32_t)__half_as_ushort(l) << 16 | __half_as_ushort(h);
+                    if (x < n_x) wr[x] = hl;
+                    if (!whole && y >= 0) wr[y] = hl;
+                    if (mean != 0.0f) {  // sum of the ring's weights (Kahan)
+                        const float z = (!whole && y != x ? 2.0f : 1.0f) * v - wcomp, t = wsum + z;
+                        wcomp = (t - wsum) - z;
+                        wsum = t;
+                    }
+                };
+                __syncwarp();
+                int i = lane;
+                if (pi.w < 0) {
+                    for (; i < n_x; i += 32) wr[i] = 0u;
+                } else {
+                    for (; i + 32 < n_d; i += 64) {  // two evaluations in flight
+                        float e0, e1;
+                        const float v0 = weight(d_first + i, &e0), v1 = weight(d_first + i + 32, &e1);
+                        put(i, v0, e0);
+                        put(i + 32, v1, e1);
+                    }
+                    if (i < n_d) {
+                        float e0;
+                        const float v0 = weight(d_first + i, &e0);
+                        put(i, v0, e0);
+                    }
+                }
+                __syncwarp();
+            }
+            // ---- A, chunk by chunk
+            const int c_lo = g.s0 / kSteps, c_hi = (g.s1 - 1) / kSteps;
+            for (int cc = c_lo; cc <= c_hi; ++cc, ++n_chunks) {
+                const int c = chunk_of(cc, c_hi, g.mid);
+                const uint32_t st = n_chunks & 1u;
+                if (n_chunks >= kStages &&
+                    !__all_sync(~0u,
+                                wait_or_abort(&a_free[st], ((n_chunks >> 1) - 1u) & 1u, &s_abort))) {
+                    ok = false;
+                    break;
+                }
+                const int t0 = max(g.s0, kSteps * c), t1 = min(g.s1, kSteps * c + kSteps);
+                unsigned char *sa = sA + st * kStageBytes + warp * (kChunk * 16) +
+                                    (t0 - kSteps * c) * 256;
+                const uint32_t *src = wr + 8 + 16 * (t0 - g.s0);
+                // core matrix e / 8, row e % 8: eight weights from element 8 (e / 8) - e % 8
+                for (int e = lane; e < 16 * (t1 - t0); e += 32) {
+                    const uint32_t *p = src + 8 * (e >> 3) - (e & 7);
+                    uint32_t v[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) v[j] = p[j];
+                    *reinterpret_cast<uint4 *>(sa + 16 * e) =
+                        make_uint4(__byte_perm(v[0], v[1], 0x5410), __byte_perm(v[2], v[3], 0x5410),
+                                   __byte_perm(v[4], v[5], 0x5410), __byte_perm(v[6], v[7], 0x5410));
+                    *reinterpret_cast<uint4 *>(sa + kPartBytes + 16 * e) =
+                        make_uint4(__byte_perm(v[0], v[1], 0x7632), __byte_perm(v[2], v[3], 0x7632),
+                                   __byte_perm(v[4], v[5], 0x7632), __byte_perm(v[6], v[7], 0x7632));
+                }
+                tc::fence_async_smem();
+                tc::fence_before_sync();
+                __syncwarp();
+                if (lane == 0)
+                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(
+                                     tc::saddr(&a_full[st]))
+                                 : "memory");
+            }
+            if (!ok) break;
+            ++n_rings;
+            // the previous ring's accumulator while this ring's MMAs run
+            if (n_rings >= 2 && !(ok = drain(n_rings - 2))) break;
+        }
+        if (ok && n_rings >= 1) ok = drain(n_rings - 1);
+        if (ok) {
+            if (mean != 0.0f) {
+                wsum -= wcomp;
+#pragma unroll
+                for (int s = 16; s > 0; s >>= 1) wsum += __shfl_xor_sync(~0u, wsum, s);
+                if (lane == 0) s_wsum[warp] = wsum * wunscale * mean;
+                asm volatile("bar.sync 1, %0;" ::"r"(kT) : "memory");  // the builder warps
+            }
+            // out = domega (unscale (total + what its folds still owe) + mean sum of weights)
+            const int row = (warp & 3) * 32 + lane, rr = r_first + (row >> 3);
+            const bool live = (row >> 3) < n_rows && rr >= ring_lo && rr <= ring_hi;
+            float *dst = o + start0 + (row >> 3) * L + k0 + (row & 7) + (warp >> 2) * kCols * 8;
+            const float unscale = xunscale * wunscale;
+            const float base_v = mean != 0.0f ? s_wsum[row >> 3] : 0.0f;
+#pragma unroll
+            for (int c = 0; c < kCols; c += 8) {
+                uint32_t v0[8], v1[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) v0[e] = v1[e] = 0u;
+                if (n_rings >= 1) tmem_ld8(td + c, v0);
+                if (n_rings >= 2) tmem_ld8(td + N + c, v1);
+                tc::tmem_wait_ld();
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const uint64_t tt = tot[(c + e) / 2];
+                    const float r = (__uint_as_float(v0[e]) + __uint_as_float(v1[e])) * unscale;
+                    const float t = __uint_as_float((e & 1) ? (uint32_t)(tt >> 32) : (uint32_t)tt) * unscale;
+                    const float hi = t + base_v;  // two-sum
+                    const float bb = hi - t;
+                    const float lo = ((t - (hi - bb)) + (base_v - bb)) + r;
+                    if (live) dst[8 * (c + e)] = fmaf(hi, P.domega, fmaf(hi, domega_lo, lo * P.domega));
+                }
+            }
+        }
+    }
+    tc::fence_before_sync();
+    const bool all_drained = __syncthreads_and(drained);
+    if (s_abort && tid == 0) atomicExch(err, all_drained ? KSC_ERR_TIMEOUT : KSC_ERR_TIMEOUT_UNDRAINED);
+    // tensor memory that an MMA may still write is not freed
+    if (warp == kRings && all_drained)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                     "r"(kTmem));
+}
+
+// blockmax[map][b] = the bits of the largest |m| over map pixels [64 b, 64 b + 64)
+// (infinities and NaNs compare above every number).  One read of the map.
+__global__ void __launch_bounds__(256)
+block_max_kernel(const float *__restrict__ in, long long map_stride, int n_blocks,
+                 uint32_t *__restrict__ blockmax, long long block_stride) {
+    const float4 *m = reinterpret_cast<const float4 *>(in + (long long)blockIdx.y * map_stride);
+    uint32_t *bm = blockmax + (long long)blockIdx.y * block_stride;
+    const int half = (blockIdx.x * 256 + threadIdx.x) >> 4, l16 = threadIdx.x & 15;
+    const int n_half = gridDim.x * 16;
+    for (int b = half; b < n_blocks; b += n_half) {
+        const float4 v = __ldg(m + (long long)b * 16 + l16);
+        uint32_t x = max(max(__float_as_uint(v.x) & 0x7fffffffu, __float_as_uint(v.y) & 0x7fffffffu),
+                         max(__float_as_uint(v.z) & 0x7fffffffu, __float_as_uint(v.w) & 0x7fffffffu));
+        const uint32_t mask = 0xffffu << (threadIdx.x & 16);
+        x = __reduce_max_sync(mask, x);
+        if (l16 == 0) bm[b] = x;
+    }
+}
+
+template <int N>
+size_t tc_smem(int wpos, int nq) {
+    return (size_t)kStages * kStageBytes + 2 * 4 * (size_t)(8 * N + wpos) +
+           4 * (size_t)kRings * (wpos + 16) + 2 * (size_t)((nq + 1) & ~1);
+}
+
+template <int N>
+cudaError_t launch_tc(const ConvPlan &p, const BeltTc &t, const float *d_in, float *d_out,
+                      int n_maps, long long map_stride, int r0, int r1, const uint32_t *bm,
+                      long long bm_stride, unsigned char *flags, int *d_err, cudaStream_t st) {
+    const int lo = std::max(r0, p.belt_lo), hi = std::min(r1, p.belt_hi);
+    const int b0 = (lo - p.belt_lo) / kRings, b1 = (hi - p.belt_lo) / kRings;
+    const int tk = p.nside / (2 * N);
+    const size_t smem = tc_smem<N>(t.wpos, t.nq);
+    cudaError_t e = cudaFuncSetAttribute(conv_belt_tc_kernel<N>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    dim3 grid((b1 - b0 + 1) * tk, n_maps);
+    conv_belt_tc_kernel<N><<<grid, kThreads, smem, st>>>(
+        p, b0, tk, r0, r1, d_in, d_out, map_stride, bm, bm_stride, flags, belt_tc_tiles(p, t),
+        t.wpos, t.nq, t.wscale, 1.0f / t.wscale,
+        (float)(4.0 * 3.14159265358979323846 / p.npix - (double)p.domega), d_err);
+    return cudaGetLastError();
+}
+
+} // namespace
+
+int belt_tc_rings() { return kRings; }
+
+int belt_tc_tiles(const ConvPlan &p, const BeltTc &t) {
+    return ((p.belt_hi - p.belt_lo) / kRings + 1) * (p.nside / (2 * t.n_cols));
+}
+
+int belt_tc_positions(int w, int L) {
+    const Window g = tile_window(std::min(w, L / 2), L);
+    return 16 * (g.s1 - g.s0);
+}
+
+bool belt_tc_plan(int nside, int wpos, int nq, BeltTc *t) {
+    t->n_cols = 0;
+    if (nside < 64 || wpos <= 0) return false;
+    t->wpos = wpos;
+    t->nq = nq;
+    const int n_blocks = (2 * nside + kRings) / kRings;
+    double best = 0.0;
+    for (int n = 32; n <= 256 && 2 * n <= nside; n *= 2) {
+        const size_t smem = n == 256 ? tc_smem<256>(wpos, nq) : n == 128 ? tc_smem<128>(wpos, nq)
+                            : n == 64 ? tc_smem<64>(wpos, nq) : tc_smem<32>(wpos, nq);
+        if (smem > 226u * 1024) continue;
+        // waves of one CTA per SM x the larger of the MMAs' and the builders' cycles
+        const double waves = std::ceil(n_blocks * (nside / (2.0 * n)) / 152.0);
+        const double mma = wpos / 16.0 * 3.0 * std::max(n / 2.0, 48.0);
+        const double build = 500.0 + wpos * 12.0 + n * 6.0;
+        const double cost = waves * std::max(mma, build);
+        if (t->n_cols == 0 || cost < best) {
+            best = cost;
+            t->n_cols = n;
+        }
+    }
+    return t->n_cols > 0;
+}
+
+long long map_blocks(const ConvPlan &p) { return p.npix / 64; }
+
+cudaError_t launch_block_max(const ConvPlan &p, const float *d_in, int n_maps,
+                             long long map_stride, uint32_t *bm, cudaStream_t st) {
+    const int n = (int)map_blocks(p);
+    dim3 grid(std::min((n + 15) / 16, 152 * 8), n_maps);
+    block_max_kernel<<<grid, 256, 0, st>>>(d_in, map_stride, n, bm, n);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_conv_belt_tc(const ConvPlan &p, const BeltTc &t, const float *d_in,
+                                float *d_out, int n_maps, long long map_stride, int r0, int r1,
+                                const uint32_t *bm, unsigned char *flags, int *d_err,
+                                cudaStream_t st) {
+    if (r0 > p.belt_hi || r1 < p.belt_lo) return cudaSuccess;
+    const long long bs = map_blocks(p);
+    switch (t.n_cols) {
+    case 256: return launch_tc<256>(p, t, d_in, d_out, n_maps, map_stride, r0, r1, bm, bs, flags, d_err, st);
+    case 128: return launch_tc<128>(p, t, d_in, d_out, n_maps, map_stride, r0, r1, bm, bs, flags, d_err, st);
+    case 64: return launch_tc<64>(p, t, d_in, d_out, n_maps, map_stride, r0, r1, bm, bs, flags, d_err, st);
+    default: return launch_tc<32>(p, t, d_in, d_out, n_maps, map_stride, r0, r1, bm, bs, flags, d_err, st);
+    }
+}
+
+} // namespace ksc

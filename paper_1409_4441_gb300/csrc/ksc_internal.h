@@ -186,9 +186,36 @@ cudaError_t launch_conv_general(const ConvPlan &p, const WorkItem *d_items,
 // Circulant belt-belt kernel; items are (belt ring, first pixel) chunks of
 // belt_chunk() pixels; seg_cap floats per shared-memory buffer.
 int belt_chunk();
+// With tile_flags (of launch_conv_belt_tc, [map][tile]) only the pixels of flagged tiles
+// are computed and written.
+struct BeltTc;
 cudaError_t launch_conv_belt(const ConvPlan &p, const int2 *d_items, int n_items,
                              int seg_cap, const float *d_in, float *d_out, int n_maps,
-                             long long map_stride, int *d_err, cudaStream_t st);
+                             long long map_stride, const BeltTc *tc,
+                             const unsigned char *tile_flags, int *d_err, cudaStream_t st);
+
+// Belt-belt ring pairs on the tensor cores (conv_belt_tc.cu): tiles of 16 belt rings x
+// 8 n_cols pixels; n_cols = 0 where the plan does not fit (belt_tc_plan returns false).
+struct BeltTc {
+    int n_cols = 0;      // MMA columns, 8 pixels each: 32, 64, 128 or 256
+    int wpos = 0;        // most window positions of a tile and an input ring
+    int nq = 0;          // most input rings of a tile
+    float wscale = 1.0f; // power of two that takes the largest weight to [2^13, 2^15)
+};
+int belt_tc_rings();                      // output rings of a tile
+int belt_tc_positions(int w, int L);      // window positions for a half window w
+bool belt_tc_plan(int nside, int wpos, int nq, BeltTc *t);
+int belt_tc_tiles(const ConvPlan &p, const BeltTc &t);
+long long map_blocks(const ConvPlan &p);  // blocks of 64 pixels in a map
+// bm[map][block] = bits of the block's largest |m|; map_blocks() words per map
+cudaError_t launch_block_max(const ConvPlan &p, const float *d_in, int n_maps,
+                             long long map_stride, unsigned *bm, cudaStream_t st);
+// Writes output rings [r0, r1] of the belt but for the tiles it flags (tiles whose values
+// span too wide a range, or are not finite), which launch_conv_belt then computes.
+cudaError_t launch_conv_belt_tc(const ConvPlan &p, const BeltTc &t, const float *d_in,
+                                float *d_out, int n_maps, long long map_stride, int r0, int r1,
+                                const unsigned *bm, unsigned char *flags, int *d_err,
+                                cudaStream_t st);
 
 // tcgen05 multi-map kernel for belt ring pairs: items are (belt ring, first
 // pixel) blocks of belt_mma_block() outputs; maps in groups of belt_mma_maps().
@@ -327,6 +354,7 @@ struct ksc_split {
     float *d_ws = nullptr;                 // pre-tiled map stack (tensor path workspace)
     size_t ws_floats = 0;
     int *d_err = nullptr;                  // device error flag (bounded waits)
+    ksc::BeltTc btc;                       // tensor-core belt stage (n_cols 0: not used)
     ksc::ConvPlan plan{};
 
     // end-to-end host path (one call at a time per split: host_mu)
