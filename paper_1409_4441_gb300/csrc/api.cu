@@ -78,6 +78,14 @@ void release(ksc_split *s) {
     cudaFree(s->d_items_mma);
     cudaFree(s->d_ws);
     cudaFree(s->d_items_belt);
+    cudaFree(s->d_cap_tiles);
+    cudaFree(s->d_cap_tiles_lpt);
+    cudaFree(s->d_ncut);
+    cudaFree(s->d_coef_off);
+    cudaFree(s->d_coef);
+    cudaFree(s->d_irr_items);
+    cudaFree(s->d_irr_first);
+    cudaFree(s->d_irr);
     cudaFree(s->d_err);
     cudaFree(s->d_io);
     if (s->own_stream) cudaStreamDestroy(s->own_stream);
@@ -85,10 +93,30 @@ void release(ksc_split *s) {
 }
 
 // Plan of the tensor-core belt stage: the widest window and the most input rings of a
-// 16-ring tile, and the power of two that scales the kernel's largest value.
+// 16-ring tile, and the power of two that scales the kernel's largest value (for the cap
+// stage too).
 int plan_belt_tc(ksc_split *s, const ksc::RingGeom &g, const std::vector<int2> &range,
                  const std::vector<ksc::PairInfo> &pairs, const std::vector<int> &pair_base) {
     if (s->path != 0 || s->n_items_belt == 0) return KSC_OK;
+    std::vector<float4> tab(s->n_int);
+    const cudaError_t e = cudaMemcpy(tab.data(), s->d_tab, sizeof(float4) * tab.size(),
+                                     cudaMemcpyDeviceToHost);
+    if (e != cudaSuccess) return cuda_fail(e, "table download");
+    double top = 0.0;
+    for (const float4 &c : tab)
+        top = std::max({top, (double)std::fabs(c.x), std::fabs((double)c.x + c.y + c.z + c.w)});
+    // scaled weights and sums stay normal FP32 numbers; otherwise the FFMA kernels
+    const int ex = std::isfinite(top) && top > 0.0 ? 13 - std::ilogb(top) : 1000;
+    if (ex < -20 || ex > 40) {
+        s->ctc.ring_end = s->ctc.ring_first - 1;
+        return KSC_OK;
+    }
+    s->btc.wscale = s->ctc.wscale = (float)std::ldexp(1.0, ex);
+    s->ctc.wunscale = 1.0f / s->ctc.wscale;
+    s->ctc.domega_lo = (float)(4.0 * kPi / s->plan.npix - (double)s->plan.domega);
+    s->ctc.d_ncut = s->d_ncut;
+    s->ctc.d_coef_off = s->d_coef_off;
+    s->ctc.d_coef = s->d_coef;
     // Below about 3e8 belt pairs the FFMA kernel is the faster one: a tile spends 0.7 to
     // 1.8 us on an input ring however short the window, and small maps have few tiles
     // (FFMA / tensor stage, us: nside 64, 360': 58 / 72; 256, 160' (2.2e8 pairs): 91 / 99;
@@ -108,20 +136,178 @@ int plan_belt_tc(ksc_split *s, const ksc::RingGeom &g, const std::vector<int2> &
         }
         nq = std::max(nq, q1 - q0 + 1);
     }
-    std::vector<float4> tab(s->n_int);
-    const cudaError_t e = cudaMemcpy(tab.data(), s->d_tab, sizeof(float4) * tab.size(),
-                                     cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(e, "table download");
-    double top = 0.0;
-    for (const float4 &c : tab)
-        top = std::max({top, (double)std::fabs(c.x), std::fabs((double)c.x + c.y + c.z + c.w)});
-    if (top == 0.0) return KSC_OK;
-    const int ex = std::isfinite(top) ? 13 - std::ilogb(top) : 1000;
-    // scaled weights and sums stay normal FP32 numbers; otherwise the FFMA kernel
-    if (ex < -20 || ex > 40) return KSC_OK;
     if (!ksc::belt_tc_plan(s->nside, wpos, nq, &s->btc)) s->btc.n_cols = 0;
-    s->btc.wscale = (float)std::ldexp(1.0, ex);
     return KSC_OK;
+}
+
+// Plan of the tensor-core cap stage (host): the tiles of the northern rings that have a cap
+// input, the sizes of the kernel's buffers, and the ring pairs that go the direct way:
+// windows that are whole rings or wider than any farther from the poles, input rings of
+// fewer than 32 pixels.
+struct CapPlan {
+    std::vector<int2> tiles;         // {rings - 1 << 16 | first ring, sectors << 16 | sector}
+    std::vector<double> cost;        // of each tile
+    std::vector<int> ncut;           // per ring pair: the largest |N| within the cut, -1: none
+    std::vector<unsigned> coef_off;  // per ring pair, in units of four words; then their end
+    std::vector<int> irr, irr_first; // input rings that go the direct way, per output ring
+    std::vector<int2> irr_items;
+    int n_ext = 0;                   // intervals of the K_r table run past the cut
+};
+void plan_cap_tc(ksc_split *s, const ksc_split_opts &o, const ksc::RingGeom &g,
+                 const std::vector<int2> &range, const std::vector<ksc::PairInfo> &pairs,
+                 const std::vector<int> &pair_base, CapPlan *plan) {
+    const int nside = s->nside, nr = 4 * nside - 1, eq = (nr - 1) / 2;
+    const int belt_lo = nside - 1, belt_hi = 3 * nside - 1;
+    if (s->path != 0 || o.exact_weights || o.cap_kernel != 0 || nside < 64 || nside > 4096 ||
+        s->theta_cut >= kPi || s->n_items_belt == 0)
+        return;
+    // Below about 8e9 pairs with a cap ring the gather is the faster one: a tile spends about
+    // 5 us on an input ring, with few tiles on small maps (gather / tensor stage, ms: nside
+    // 256, 640' (1.8e9 pairs): 0.85 / 1.09; 512, 160': 0.84 / 1.00; 256, 30 deg (1.4e10): 8.7 /
+    // 7.4; 512, 640' (2.9e10): 9.0 / 7.1; 1024, 160': 7.5 / 6.6; 2048, 240' (1.0e12): 150 / 108).
+    if (ksc_cost_pairs(nside, s->theta_cut) / 3.0 < 8e9) return;
+    // the cells' polynomials: Chebyshev interpolation of degree n leaves, of a term l of the
+    // kernel, at most about 4 J_{n+1}(l h / 2) ~ 4 (l h / 4)^{n+1} / (n+1)!, h the largest
+    // pixel step (1.2826 / nside at the poles)
+    {
+        const int n = ksc::cap_tc_degree();
+        double err = 0.0, all = 0.0, fact = 1.0;
+        for (int i = 2; i <= n + 1; ++i) fact *= i;
+        for (int l = 0; l <= s->lmax; ++l) {
+            const double a = (2.0 * l + 1.0) * std::fabs(s->c_real[l]);
+            err += a * 4.0 * std::pow(l * 1.2826 / nside / 4.0, n + 1) / fact;
+            all += a;
+        }
+        if (!(err <= 5e-8 * all)) return;
+    }
+    const double dc = s->chord_cut, n_int = s->n_int;
+    const double scale2 = (n_int / dc) * (n_int / dc), nint2 = n_int * n_int;
+    // room for the table past the cut (chords up to 2)
+    const double h = dc / n_int;
+    const int n_ext = s->n_int + (int)std::ceil(1.7 * 1.2826 / nside / h) + 4;
+    if (n_ext * h >= 2.0) return;
+    int last = -1;  // the last northern ring with a cap input
+    for (int r = 0; r <= eq; ++r)
+        if (r < belt_lo || range[r].x < belt_lo || range[r].y > belt_hi) last = r;
+    auto considered = [&](int r, int q) {
+        return !(r >= belt_lo && q >= belt_lo && q <= belt_hi);
+    };
+    // edge cell of a regular pair from its cut
+    auto cell = [&](int nc, int L) { return nc >= L ? (nc - L) / (2 * L) + 1 : 0; };
+    constexpr int kDirect = -2;
+    plan->ncut.assign(pairs.size(), -1);
+    std::vector<int> widest(last + 1, 0);  // widest regular window of a ring; -1: it has others
+#pragma omp parallel for schedule(dynamic, 16)
+    for (int r = 0; r <= last; ++r) {
+        for (int q = range[r].x; q <= range[r].y; ++q) {
+            const size_t ip = (size_t)pair_base[r] + (q - range[r].x);
+            if (!considered(r, q) || pairs[ip].hw < 0.0f) continue;
+            const double dz = g.z[r] - g.z[q];
+            const double ds = (g.z[q] - g.z[r]) * (g.z[q] + g.z[r]) / (g.s[r] + g.s[q]);
+            const double A2 = (dz * dz + ds * ds) * scale2, B2 = 4.0 * g.s[r] * g.s[q] * scale2;
+            if (A2 >= nint2) continue;
+            const double sx2 = (nint2 - A2) / B2, c = kPi / (2.0 * (double)g.len[r] * (double)g.len[q]);
+            int nc = kDirect;
+            if (sx2 < 1.0 && g.len[q] >= 32) {
+                nc = (int)std::floor(std::asin(std::sqrt(sx2)) / c);
+                if (2 * cell(nc, g.len[r]) + 1 > g.len[q]) nc = kDirect;
+            }
+            plan->ncut[ip] = nc;
+            if (nc == kDirect && g.len[q] >= 32) widest[r] = -1;
+            else if (widest[r] >= 0 && nc >= 0) widest[r] = std::max(widest[r], cell(nc, g.len[r]));
+        }
+    }
+    // near the poles windows widen to whole rings: past the widest of the other rings, direct
+    const int j_max = *std::max_element(widest.begin(), widest.end());
+    plan->irr_first.assign(nr + 1, 0);
+    long long widest_n = 0;
+    for (int r = 0; r <= last; ++r) {
+        plan->irr_first[r] = (int)plan->irr.size();
+        for (int q = range[r].x; q <= range[r].y; ++q) {
+            int &nc = plan->ncut[(size_t)pair_base[r] + (q - range[r].x)];
+            if (nc >= 0 && cell(nc, g.len[r]) > j_max) nc = kDirect;
+            if (nc != kDirect) continue;
+            nc = -1;
+            plan->irr.push_back(q);
+            widest_n = std::max(widest_n, 2LL * g.len[r] * g.len[q]);
+        }
+        if ((int)plan->irr.size() > plan->irr_first[r])
+            for (int k0 = 0; k0 < g.len[r] / 4; k0 += 32) plan->irr_items.push_back(make_int2(r, k0));
+    }
+    for (int r = last + 1; r <= nr; ++r) plan->irr_first[r] = (int)plan->irr.size();
+    if (widest_n >= 1LL << 24) {  // (their integers are exact in FP32)
+        plan->tiles.clear();
+        return;
+    }
+    // blocks of two rings: input rings, windows, sectors
+    // (cap rings or belt rings, not both; an odd ring out alone)
+    ksc::CapTc c;
+    for (int r0 = 0, r1; r0 <= last; r0 = r1 + 1) {
+        r1 = r0 < belt_lo && ((belt_lo - r0) & 1) ? r0 : std::min(r0 + 1, r0 < belt_lo ? belt_lo - 1 : last);
+        const int q0 = std::min(range[r0].x, range[r1].x), q1 = std::max(range[r0].y, range[r1].y);
+        const int L0 = g.len[r0], L1 = g.len[r1];
+        int lq_max = 0, jm = 0;
+        double work = 0.0;
+        bool one = true;  // the whole ring as one sector
+        int span_one = 0;
+        for (int q = q0; q <= q1; ++q) {
+            int w = -1;
+            for (int r = r0; r <= r1; ++r) {
+                if (q < range[r].x || q > range[r].y) continue;
+                const int nc = plan->ncut[(size_t)pair_base[r] + (q - range[r].x)];
+                if (nc >= 0) w = std::max(w, cell(nc, g.len[r]));
+            }
+            if (w < 0) continue;
+            const int Lq = g.len[q], tq = g.phase[q];
+            auto pos = [&](int k, int t, int L) {
+                return (int)(((long long)(2 * k + t) * Lq + (long long)(1 - tq) * L) / (2 * L));
+            };
+            const int lo = std::min(pos(0, g.phase[r0], L0), pos(0, g.phase[r1], L1));
+            const int hi = std::max(pos(L0 - 1, g.phase[r0], L0), pos(L1 - 1, g.phase[r1], L1));
+            span_one = std::max(span_one, hi - lo + 1);
+            one = span_one <= ksc::cap_tc_span();
+            lq_max = std::max(lq_max, Lq);
+            jm = std::max(jm, w);
+            const int np = ksc::cap_tc_positions(w, Lq);
+            c.wpos = std::max(c.wpos, np);
+            work += np + 60.0;
+        }
+        // (cap rings without a regular pair have a tile too: it writes what the direct ones add to)
+        if (lq_max == 0 && r0 >= belt_lo) continue;
+        // a sector's positions: L' / n, the rings' different first outputs, rounding
+        int n_sec = 1;
+        if (!one) {
+            const int slack = (lq_max + L0 - 1) / L0 + 4;
+            n_sec = (lq_max + ksc::cap_tc_span() - slack - 1) / (ksc::cap_tc_span() - slack);
+            n_sec = std::max(n_sec, 2);
+        }
+        c.nq = std::max(c.nq, q1 - q0 + 1);
+        c.jcap = std::max(c.jcap, jm + 1);
+        c.tcap = std::max(c.tcap, (std::max(L0, L1) + n_sec - 1) / n_sec + 1);
+        c.span = std::max(c.span, one ? span_one : (lq_max + n_sec - 1) / n_sec + (lq_max + L0 - 1) / L0 + 4);
+        for (int t = 0; t < n_sec; ++t) {
+            plan->tiles.push_back(make_int2((r1 - r0) << 16 | r0, n_sec << 16 | t));
+            plan->cost.push_back(work);
+        }
+    }
+    c.span = std::min((c.span + 15) & ~15, ksc::cap_tc_span());
+    // the coefficients: up to 8 GB (2.4 GB at nside 2048 with a 240' cut); beyond it the
+    // gather, which keeps none
+    unsigned long long n4 = 0;
+    plan->coef_off.assign(pairs.size() + 1, 0u);
+    for (int r = 0; r <= last; ++r)
+        for (int q = range[r].x; q <= range[r].y; ++q) {
+            const size_t ip = (size_t)pair_base[r] + (q - range[r].x);
+            plan->coef_off[ip] = (unsigned)n4;
+            if (plan->ncut[ip] >= 0) n4 += ksc::cap_tc_words(cell(plan->ncut[ip], g.len[r])) / 4;
+        }
+    if (!ksc::cap_tc_fits(c) || n4 * 16 > 8ull << 30) plan->tiles.clear();
+    if (plan->tiles.empty()) return;
+    plan->coef_off.back() = (unsigned)n4;
+    c.ring_first = 0;
+    c.ring_end = last;
+    plan->n_ext = n_ext;
+    s->ctc = c;
 }
 
 // Geometry, work list and device table for the real-space part s->c_real.
@@ -327,6 +513,10 @@ int finish_split(ksc_split *s, const ksc_split_opts &o) {
         s->frac_tabulated = all > 0.0 ? tab / all : 0.0;
     }
 
+    CapPlan cap;
+    plan_cap_tc(s, o, g, range, pairs, pair_base, &cap);
+    const int n_ext = cap.n_ext;
+
     // The symmetric items longest first, for whole-map launches: CTAs claim items
     // in list order, so the long items start first and the short ones fill the tail.
     // The tensor cap kernel has items of its own size.
@@ -360,6 +550,32 @@ int finish_split(ksc_split *s, const ksc_split_opts &o) {
         s->ring_first_smma[nr] = (int)items_smma.size();
     }
     std::vector<ksc::WorkItem> items_smma_lpt = lpt(items_smma, ksc::sym_mma_chunk());
+    std::vector<int2> cap_tiles_lpt;
+    {
+        std::vector<int> order(cap.tiles.size());
+        for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
+        std::stable_sort(order.begin(), order.end(),
+                         [&](int a, int b) { return cap.cost[a] > cap.cost[b]; });
+        for (int i : order) cap_tiles_lpt.push_back(cap.tiles[i]);
+        s->n_cap_tiles = (int)cap.tiles.size();
+        s->cap_tile_first.assign(nr + 1, 0);
+        size_t i = 0;
+        for (int r = 0; r <= nr; ++r) {
+            while (i < cap.tiles.size() && (cap.tiles[i].x & 0xffff) < r) ++i;
+            s->cap_tile_first[r] = (int)i;
+        }
+        s->irr_item_first.assign(nr + 1, 0);
+        i = 0;
+        for (int r = 0; r <= nr; ++r) {
+            while (i < cap.irr_items.size() && cap.irr_items[i].x < r) ++i;
+            s->irr_item_first[r] = (int)i;
+        }
+    }
+    std::vector<float2> ringc(s->n_cap_tiles ? nr : 0);
+    for (size_t r = 0; r < ringc.size(); ++r) {
+        const ksc::DF c = ksc::df_from_double(kPi / (double)g.len[r]);
+        ringc[r] = make_float2(c.h, c.l);
+    }
     s->n_items_smma = (int)items_smma.size();
     s->cap_kernel = o.cap_kernel;
 
@@ -392,28 +608,67 @@ int finish_split(ksc_split *s, const ksc_split_opts &o) {
         return cuda_fail(e, "upload work list");
     if ((e = dev_upload(&s->d_items_mma, items_mma.data(), items_mma.size())) != cudaSuccess)
         return cuda_fail(e, "upload work list");
+    if (s->n_cap_tiles) {
+        if ((e = dev_upload(&s->d_cap_tiles, cap.tiles.data(), cap.tiles.size())) != cudaSuccess ||
+            (e = dev_upload(&s->d_cap_tiles_lpt, cap_tiles_lpt.data(), cap_tiles_lpt.size())) !=
+                cudaSuccess ||
+            (e = dev_upload(&s->d_ncut, cap.ncut.data(), cap.ncut.size())) != cudaSuccess ||
+            (e = dev_upload(&s->d_coef_off, cap.coef_off.data(), cap.coef_off.size())) != cudaSuccess ||
+            (e = dev_upload(&s->d_irr_items, cap.irr_items.data(), cap.irr_items.size())) != cudaSuccess ||
+            (e = dev_upload(&s->d_irr_first, cap.irr_first.data(), cap.irr_first.size())) != cudaSuccess ||
+            (e = dev_upload(&s->d_irr, cap.irr.data(), cap.irr.size())) != cudaSuccess ||
+            (e = dev_malloc((void **)&s->d_coef, 16ull * cap.coef_off.back())) != cudaSuccess)
+            return cuda_fail(e, "cap tiles and coefficients");
+    }
     if ((e = dev_malloc((void **)&s->d_err, sizeof(int))) != cudaSuccess)
         return cuda_fail(e, "error flag");
     if ((e = cudaMemset(s->d_err, 0, sizeof(int))) != cudaSuccess)
         return cuda_fail(e, "error flag");
 
     // Table build on the GPU: FP64 Legendre recurrence per node (csrc/table.cu).
-    double *d_c = nullptr, *d_nodes = nullptr;
+    double *d_c = nullptr;
     if ((e = dev_upload(&d_c, s->c_real.data(), s->c_real.size())) != cudaSuccess)
         return cuda_fail(e, "upload coefficients");
-    if ((e = dev_malloc((void **)&d_nodes, sizeof(double) * 2 * (n_int + 1))) != cudaSuccess) {
+    // With a tensor-core cap stage the table runs past the cut; its intervals up to the
+    // cut, and the entry at the cut with its higher terms dropped, are the table proper.
+    const int n_build = s->n_cap_tiles ? n_ext : n_int;
+    // nodes | the table run past the cut, its rounding errors, pi / L per ring
+    const size_t b_nodes = sizeof(double) * 2 * (size_t)(n_build + 1);
+    const size_t b_ext = s->n_cap_tiles ? sizeof(float4) * (size_t)(n_build + 1) : 0;
+    const size_t b_lo = s->n_cap_tiles ? (sizeof(float) * (size_t)n_build + 15) / 16 * 16 : 0;
+    unsigned char *d_scratch = nullptr;
+    if ((e = dev_malloc((void **)&d_scratch,
+                        (b_nodes + 15) / 16 * 16 + b_ext + b_lo + sizeof(float2) * ringc.size())) !=
+        cudaSuccess) {
         cudaFree(d_c);
         return cuda_fail(e, "allocate table nodes");
     }
     if ((e = dev_malloc((void **)&s->d_tab, sizeof(float4) * (n_int + 1))) != cudaSuccess) {
-        cudaFree(d_c); cudaFree(d_nodes);
+        cudaFree(d_c); cudaFree(d_scratch);
         return cuda_fail(e, "allocate table");
     }
-    ksc::TableBuild tb{d_c, s->lmax, n_int, s->chord_cut / n_int, s->d_tab, d_nodes, 1};
+    double *d_nodes = reinterpret_cast<double *>(d_scratch);
+    float4 *d_ext = reinterpret_cast<float4 *>(d_scratch + (b_nodes + 15) / 16 * 16);
+    float *d_lo = reinterpret_cast<float *>(d_ext + b_ext / sizeof(float4));
+    float2 *d_ringc = reinterpret_cast<float2 *>(reinterpret_cast<unsigned char *>(d_lo) + b_lo);
+    float4 *built = s->n_cap_tiles ? d_ext : s->d_tab;
+    ksc::TableBuild tb{d_c, s->lmax, n_build, s->chord_cut / n_int, built, d_nodes, 1};
+    if (s->n_cap_tiles) tb.d_lo = d_lo;
     e = ksc::launch_table_build(tb, 0);
+    if (e == cudaSuccess && s->n_cap_tiles) {
+        e = cudaMemcpyAsync(s->d_tab, built, sizeof(float4) * (n_int + 1),
+                            cudaMemcpyDeviceToDevice, 0);
+        if (e == cudaSuccess) e = cudaMemsetAsync(&s->d_tab[n_int].z, 0, 2 * sizeof(float), 0);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(d_ringc, ringc.data(), sizeof(float2) * ringc.size(),
+                                cudaMemcpyHostToDevice, 0);
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(0);
     cudaFree(d_c);
-    cudaFree(d_nodes);
+    struct Scratch {  // freed when the construction ends, whichever way
+        void *p;
+        ~Scratch() { cudaFree(p); }
+    } scratch_owner{d_scratch};
     if (e != cudaSuccess) return cuda_fail(e, "table build");
 
     ksc::ConvPlan &p = s->plan;
@@ -446,7 +701,13 @@ int finish_split(ksc_split *s, const ksc_split_opts &o) {
         p.belt_c1h = c1.h;
         p.belt_c1l = c1.l;
     }
-    return plan_belt_tc(s, g, range, pairs, pair_base);
+    const int rc = plan_belt_tc(s, g, range, pairs, pair_base);
+    if (rc || s->ctc.ring_end < s->ctc.ring_first) return rc;
+    ksc::CapCoef cc{d_ext, d_lo, d_ringc, s->d_coef, n_ext, (float)((double)n_ext * n_ext), {}, {}};
+    e = ksc::launch_cap_coef(s->plan, s->ctc, cc, 0);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(0);
+    if (e != cudaSuccess) return cuda_fail(e, "cap coefficients");
+    return KSC_OK;
 }
 
 int check_common(int lmax, int nside, double theta_cut) {
@@ -483,32 +744,70 @@ int check_maps(const ksc_split *s, const void *a, const void *b) {
     return KSC_OK;
 }
 
+// Scratch of one convolution call, from the stream-ordered allocator: the map's block
+// maxima, the belt tiles' flags, the rings' ranges and the cap rings' flags.
+struct CallScratch {
+    unsigned char *mem = nullptr;
+    unsigned *bm = nullptr;
+    uint2 *ranges = nullptr;
+    int *cap_flags = nullptr;
+    unsigned char *belt_flags = nullptr;
+    cudaStream_t st = nullptr;
+    CallScratch() = default;
+    CallScratch(const CallScratch &) = delete;
+    CallScratch &operator=(const CallScratch &) = delete;
+    ~CallScratch() {
+        if (mem) cudaFreeAsync(mem, st);
+    }
+};
+
+bool has_cap_tc(const ksc_split *s) { return s->ctc.ring_end >= s->ctc.ring_first; }
+
+// Takes the scratch the split's tensor-core stages need (none: no-op) and starts the
+// launches that fill it.
+cudaError_t start_scratch(const ksc_split *s, const float *d_in, int n_maps, long long stride,
+                          cudaStream_t st, CallScratch *w) {
+    const bool cap = has_cap_tc(s), belt = s->btc.n_cols > 0;
+    if (!cap && !belt) return cudaSuccess;
+    const int nr = s->plan.nrings;
+    const size_t b_rr = cap ? sizeof(uint2) * (size_t)nr * n_maps : 0;
+    const size_t b_bm = sizeof(unsigned) * (size_t)ksc::map_blocks(s->plan) * n_maps;
+    const size_t b_cf = cap ? sizeof(int) * (size_t)(nr + 1) * n_maps : 0;
+    const size_t b_bf = belt ? (size_t)ksc::belt_tc_tiles(s->plan, s->btc) * n_maps : 0;
+    w->st = st;
+    cudaError_t e = cudaMallocAsync(&w->mem, b_rr + b_bm + b_cf + b_bf, st);
+    if (e != cudaSuccess) {
+        w->mem = nullptr;
+        return e;
+    }
+    w->ranges = reinterpret_cast<uint2 *>(w->mem);
+    w->bm = reinterpret_cast<unsigned *>(w->mem + b_rr);
+    w->cap_flags = reinterpret_cast<int *>(w->mem + b_rr + b_bm);
+    w->belt_flags = w->mem + b_rr + b_bm + b_cf;
+    e = ksc::launch_block_max(s->plan, d_in, n_maps, stride, w->bm, st);
+    if (e == cudaSuccess && cap) {
+        e = cudaMemsetAsync(w->cap_flags, 0, b_cf, st);
+        if (e == cudaSuccess)
+            e = ksc::launch_ring_range(s->plan, w->bm, n_maps, w->ranges, st);
+    }
+    return e;
+}
+
 // The belt stage (belt-belt ring pairs) of output rings [r0, r1]: the tensor-core kernel
 // where the split has a plan for it, then the FFMA kernel for the tiles it left (none of
 // them in an ordinary map: that launch reads the flags and ends); else the FFMA kernel.
 cudaError_t launch_belt(const ksc_split *s, const float *d_in, float *d_out, int n_maps,
-                        long long stride, int r0, int r1, cudaStream_t st) {
+                        long long stride, int r0, int r1, const CallScratch &w, cudaStream_t st) {
     const int a = s->ring_first_belt[r0], b = s->ring_first_belt[r1 + 1];
     if (a == b || s->n_items_belt == 0) return cudaSuccess;
     if (s->btc.n_cols == 0)
         return ksc::launch_conv_belt(s->plan, s->d_items_belt + a, b - a, s->seg_cap, d_in, d_out,
                                      n_maps, stride, nullptr, nullptr, s->d_err, st);
-    const size_t bm_bytes = sizeof(unsigned) * (size_t)ksc::map_blocks(s->plan) * n_maps;
-    const size_t fl_bytes = (size_t)ksc::belt_tc_tiles(s->plan, s->btc) * n_maps;
-    unsigned char *ws = nullptr;  // block maxima, then the tiles' flags
-    cudaError_t e = cudaMallocAsync(&ws, bm_bytes + fl_bytes, st);
+    const cudaError_t e = ksc::launch_conv_belt_tc(s->plan, s->btc, d_in, d_out, n_maps, stride,
+                                                   r0, r1, w.bm, w.belt_flags, s->d_err, st);
     if (e != cudaSuccess) return e;
-    unsigned *bm = reinterpret_cast<unsigned *>(ws);
-    unsigned char *flags = ws + bm_bytes;
-    e = ksc::launch_block_max(s->plan, d_in, n_maps, stride, bm, st);
-    if (e == cudaSuccess)
-        e = ksc::launch_conv_belt_tc(s->plan, s->btc, d_in, d_out, n_maps, stride, r0, r1, bm,
-                                     flags, s->d_err, st);
-    if (e == cudaSuccess)
-        e = ksc::launch_conv_belt(s->plan, s->d_items_belt + a, b - a, s->seg_cap, d_in, d_out,
-                                  n_maps, stride, &s->btc, flags, s->d_err, st);
-    const cudaError_t f = cudaFreeAsync(ws, st);
-    return e != cudaSuccess ? e : f;
+    return ksc::launch_conv_belt(s->plan, s->d_items_belt + a, b - a, s->seg_cap, d_in, d_out,
+                                 n_maps, stride, &s->btc, w.belt_flags, s->d_err, st);
 }
 
 // Tensor-core belt stage for a stack of maps; grows the split's pre-tiled map
@@ -539,7 +838,7 @@ int launch_belt_tensor(const ksc_split *cs, const float *d_in, float *d_out, int
 // the items longest first, bands their rings' items in ring order.
 cudaError_t launch_caps(const ksc_split *s, const float *d_in, float *d_out, int n_maps,
                         long long stride, int lo, int hi, int r0, int r1, bool stack,
-                        cudaStream_t st) {
+                        const CallScratch &w, cudaStream_t st) {
     const bool whole = r0 == 0 && r1 == s->plan.nrings - 1;
     const int belt_split = s->n_items_belt > 0 ? 1 : 0;
     if (stack && s->tensor >= 1)
@@ -553,8 +852,24 @@ cudaError_t launch_caps(const ksc_split *s, const float *d_in, float *d_out, int
     }
     const int c = s->ring_first_sym[lo], d = s->ring_first_sym[hi + 1];
     const ksc::WorkItem *its = whole ? s->d_items_sym_lpt : s->d_items_sym + c;
-    return ksc::launch_conv_sym(s->plan, its, d - c, d_in, d_out, n_maps, stride, belt_split,
-                                r0, r1, s->d_err, st);
+    if (!has_cap_tc(s))
+        return ksc::launch_conv_sym(s->plan, its, d - c, d_in, d_out, n_maps, stride, belt_split,
+                                    r0, r1, d - c, nullptr, s->d_err, st);
+    // the tensor-core stage, the irregular ring pairs, then the gather for the rings that
+    // the first flagged (none in an ordinary map: that launch reads a flag and ends)
+    // (a tile holds rings r and r + 1: from the one that may start just before lo)
+    const int t0 = whole ? 0 : s->cap_tile_first[std::max(lo - 1, 0)];
+    const int t1 = whole ? s->n_cap_tiles : s->cap_tile_first[hi + 1];
+    cudaError_t e = ksc::launch_conv_cap_tc(
+        s->plan, s->ctc, whole ? s->d_cap_tiles_lpt : s->d_cap_tiles + t0, t1 - t0, d_in, d_out,
+        n_maps, stride, belt_split, r0, r1, w.ranges, w.cap_flags, s->d_err, st);
+    if (e != cudaSuccess) return e;
+    const int i0 = s->irr_item_first[lo], i1 = s->irr_item_first[hi + 1];
+    e = ksc::launch_cap_direct(s->plan, s->d_irr_items + i0, i1 - i0, s->d_irr_first, s->d_irr,
+                               d_in, d_out, n_maps, stride, r0, r1, w.cap_flags, st);
+    if (e != cudaSuccess) return e;
+    return ksc::launch_conv_sym(s->plan, its, d - c, d_in, d_out, n_maps, stride, belt_split, r0,
+                                r1, 0, w.cap_flags, s->d_err, st);
 }
 
 // The real-space convolution of output rings [r0, r1] (0-based, inclusive).
@@ -572,13 +887,16 @@ int launch_conv(const ksc_split *s, const float *d_in, float *d_out, int n_maps,
         if (e != cudaSuccess) return cuda_fail(e, "gather kernel launch");
         return KSC_OK;
     }
+    CallScratch w;
+    e = start_scratch(s, d_in, n_maps, stride, st, &w);
+    if (e != cudaSuccess) return cuda_fail(e, "call scratch");
     const bool whole = r0 == 0 && r1 == s->plan.nrings - 1;
     const bool stack = whole && n_maps >= 16;
     if (stack && s->tensor == 2 && s->n_items_mma > 0) {
         int rc = launch_belt_tensor(s, d_in, d_out, n_maps, stride, st);
         if (rc) return rc;
     } else {
-        e = launch_belt(s, d_in, d_out, n_maps, stride, r0, r1, st);
+        e = launch_belt(s, d_in, d_out, n_maps, stride, r0, r1, w, st);
         if (e != cudaSuccess) return cuda_fail(e, "belt kernel launch");
     }
     // northern rings r whose own or mirror ring (nr - 1 - r) lies in the band
@@ -588,7 +906,7 @@ int launch_conv(const ksc_split *s, const float *d_in, float *d_out, int n_maps,
     const int m0 = std::max(0, nr - 1 - r1), m1 = std::min(nr - 1 - r0, eq);
     if (m0 <= m1) { lo = std::min(lo, m0); hi = std::max(hi, m1); }  // mirror in band
     if (lo <= hi) {
-        e = launch_caps(s, d_in, d_out, n_maps, stride, lo, hi, r0, r1, stack, st);
+        e = launch_caps(s, d_in, d_out, n_maps, stride, lo, hi, r0, r1, stack, w, st);
         if (e != cudaSuccess) return cuda_fail(e, "symmetric kernel launch");
     }
     return KSC_OK;
@@ -986,22 +1304,23 @@ int ksc_conv_real_multimap_stage(const ksc_split *s, const float *d_in, float *d
     if (n_maps < 1 || n_maps > 65535) return fail(KSC_ERR_ARG, "n_maps outside 1..65535");
     cudaStream_t st = (cudaStream_t)stream;
     const long long stride = s->plan.npix;
-    cudaError_t e;
+    if (stage != 1 && stage != 2) return fail(KSC_ERR_ARG, "stage must be 1 or 2");
+    CallScratch w;
+    cudaError_t e = s->path == 1 ? cudaSuccess : start_scratch(s, d_in, n_maps, stride, st, &w);
+    if (e != cudaSuccess) return cuda_fail(e, "call scratch");
     if (stage == 1) {
         if (s->path == 1) return KSC_OK;
         if (n_maps >= 16 && s->tensor == 2 && s->n_items_mma > 0)
             return launch_belt_tensor(s, d_in, d_out, n_maps, stride, st);
         else
-            e = launch_belt(s, d_in, d_out, n_maps, stride, 0, s->plan.nrings - 1, st);
-    } else if (stage == 2) {
+            e = launch_belt(s, d_in, d_out, n_maps, stride, 0, s->plan.nrings - 1, w, st);
+    } else {
         if (s->path == 1)
             e = ksc::launch_conv_general(s->plan, s->d_items, s->n_items, d_in, d_out, n_maps,
                                          stride, 0, nullptr, st);
         else
             e = launch_caps(s, d_in, d_out, n_maps, stride, 0, (s->plan.nrings - 1) / 2, 0,
-                            s->plan.nrings - 1, n_maps >= 16, st);
-    } else {
-        return fail(KSC_ERR_ARG, "stage must be 1 or 2");
+                            s->plan.nrings - 1, n_maps >= 16, w, st);
     }
     if (e != cudaSuccess) return cuda_fail(e, "stage launch");
     return KSC_OK;
@@ -1012,18 +1331,19 @@ int ksc_conv_real_stage(const ksc_split *s, const float *d_in, float *d_out, int
     int rc = check_maps(s, d_in, d_out);
     if (rc) return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    cudaError_t e;
+    if (stage != 1 && stage != 2) return fail(KSC_ERR_ARG, "stage must be 1 or 2");
+    CallScratch w;
+    cudaError_t e = s->path == 1 ? cudaSuccess : start_scratch(s, d_in, 1, 0, st, &w);
+    if (e != cudaSuccess) return cuda_fail(e, "call scratch");
     if (stage == 1) {
-        e = launch_belt(s, d_in, d_out, 1, 0, 0, s->plan.nrings - 1, st);
-    } else if (stage == 2) {
+        e = launch_belt(s, d_in, d_out, 1, 0, 0, s->plan.nrings - 1, w, st);
+    } else {
         if (s->path == 1)
             e = ksc::launch_conv_general(s->plan, s->d_items, s->n_items, d_in, d_out, 1, 0, 0,
                                          nullptr, st);
         else
             e = launch_caps(s, d_in, d_out, 1, 0, 0, (s->plan.nrings - 1) / 2, 0,
-                            s->plan.nrings - 1, false, st);
-    } else {
-        return fail(KSC_ERR_ARG, "stage must be 1 or 2");
+                            s->plan.nrings - 1, false, w, st);
     }
     if (e != cudaSuccess) return cuda_fail(e, "stage launch");
     return KSC_OK;

@@ -21,11 +21,11 @@
 // v = h + l, l the rounding error of h: exactly v for |v| >= 2^-1 (24 bits in two parts
 // of 11 and a sign), within 2^-25 otherwise, i.e. within 2^-40 of the largest.  Three MMAs
 // per 16 positions sum w_h m_l, w_l m_h and w_h m_h in FP32; w_l m_l (below 2^-24 of the
-// product) is summed too where the weights are large, in the two steps of the closest
+// product) is summed too where the weights are large, in the step of the closest
 // approach.  An MMA cuts every addend, the accumulator too, at 2^-25 of the largest one and
 // rounds the sum toward zero to 24 bits (found with known operands), so the order matters:
-// within 64 positions the small products first, the 64 positions that hold the closest
-// approach last, and its own two steps at the very end.  After each input ring the
+// within 128 positions the small products first, the 128 positions that hold the closest
+// approach last, and its own step at the very end.  After each input ring the
 // accumulator is folded into FP32 totals with the rounding error of the sum (two-sum),
 // plus the 2^-24 of the partial that the cuts take from it on average, written back to
 // tensor memory as the start of a later partial.  The weights keep the rounding error of
@@ -41,11 +41,10 @@
 // Every mbarrier wait is bounded; a wait that runs out raises the device error flag.
 #include <algorithm>
 #include <cstdint>
-#include <cuda_fp16.h>
 
 #include "ksc_device.cuh"
 #include "ksc_internal.h"
-#include "ksc_tc.cuh"
+#include "ksc_tc_split.cuh"
 
 namespace ksc {
 namespace {
@@ -58,43 +57,6 @@ constexpr int kSteps = kChunk / 16;
 constexpr int kPartBytes = kRings * kChunk * 16;  // one FP16 part of an A stage (32 kB)
 constexpr int kStageBytes = 2 * kPartBytes;
 constexpr int kStages = 2;
-constexpr int kXExp = 14;      // a tile's largest |m| is scaled into [2^14, 2^15)
-constexpr uint32_t kRangeExp = 14;  // a block may lie this many powers of two below it
-
-// K-major, no swizzle: 8-row x 16-byte core matrices; lead = bytes between core matrices
-// adjacent in K, stride = bytes between groups of eight rows.
-__device__ __forceinline__ uint64_t tc_desc(uint32_t addr, uint32_t lead, uint32_t stride) {
-    return (uint64_t)((addr & 0x3FFFF) >> 4) | (uint64_t)((lead >> 4) & 0x3FFF) << 16 |
-           (uint64_t)((stride >> 4) & 0x3FFF) << 32 | (uint64_t)1 << 46;
-}
-
-// FP16 operands, FP32 accumulator, both K-major.
-__host__ __device__ constexpr uint32_t idesc_f16(int M, int N) {
-    return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-__device__ __forceinline__ void mma_f16(uint32_t tmem, uint64_t da, uint64_t db, uint32_t idesc,
-                                        uint32_t acc) {
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-        "l"(da), "l"(db), "r"(idesc), "r"(acc));
-}
-
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t *v) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-          "=r"(v[7])
-        : "r"(taddr));
-}
-
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t *v) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr),
-        "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
-        : "memory");
-}
 
 // Two FP32 values in one register pair.
 __device__ __forceinline__ uint64_t pack2(uint32_t a, uint32_t b) {
@@ -111,38 +73,18 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
     return d;
 }
 
-// Bounded wait that also ends when another warp of the CTA has given up.
-__device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity,
-                                              volatile int *abort) {
-    for (int i = 0; i < 64; ++i) {
-        if (tc::mbar_wait(bar, parity, tc::kMaxWait / 64)) return true;
-        if (*abort) break;
-    }
-    *abort = 1;
-    return false;
-}
+using tc::Window;
+using tc::chunk_of;
+using tc::idesc_f16;
+using tc::kRangeExp;
+using tc::kXExp;
+using tc::mma_f16;
+using tc::tmem_ld8;
+using tc::tmem_st8;
+using tc::wait_or_abort;
 
-// One input ring as seen by the tile: window [lo, hi] of Delta common to the tile's rings
-// (the widest one's), and the 16-position steps [s0, s1) of a grid of 128-position chunks
-// whose chunk `mid` is centred on the closest approach.  Position j stands for
-// Delta = d0 + j - i, i = 0..7.
-struct Window {
-    int d0, s0, s1, mid;
-};
 __host__ __device__ __forceinline__ Window tile_window(int w, int L) {
-    const bool whole = 2 * w + 1 >= L;  // the whole ring, each pixel once
-    const int lo = whole ? -(L / 2) : -w, hi = whole ? lo + L - 1 : w;
-    Window g;
-    // chunks left of the one with j = 64 in its middle (Delta = -4 .. 3 over i)
-    g.mid = (unsigned)(-lo + 3 - kChunk / 2 + kChunk - 1) / kChunk;
-    g.d0 = -(g.mid * kChunk + kChunk / 2) + 3;
-    g.s0 = (unsigned)(lo - g.d0) / 16;          // first j of any use: Delta = lo at i = 0
-    g.s1 = (unsigned)(hi - g.d0 + 7) / 16 + 1;  // last: Delta = hi at i = 7
-    return g;
-}
-// The chunks of a window in order of work: the closest approach's last.
-__device__ __forceinline__ int chunk_of(int cc, int c_hi, int mid) {
-    return cc == c_hi ? mid : (cc >= mid ? cc + 1 : cc);
+    return tc::tile_window<kChunk>(w, L);
 }
 
 // N columns: 8 N pixels per ring.  grid.x runs over tiles (16-ring block, pixel tile),
@@ -296,7 +238,7 @@ conv_belt_tc_kernel(const ConvPlan P, int block_lo, int n_tiles_k, int ring_lo, 
         if (warp == kRings && lane == 0) {
             const uint32_t idesc = idesc_f16(128, N);
             const uint32_t pa0 = tc::saddr(sA), pb0 = tc::saddr(sB);
-            const uint64_t a_hi = tc_desc(0, 128, kChunk * 16), b_hi = tc_desc(0, 16, 128);
+            const uint64_t a_hi = tc::desc(0, 128, kChunk * 16), b_hi = tc::desc(0, 16, 128);
             const uint32_t a_l = kPartBytes >> 4, b_l = (uint32_t)(seg_cap * 2) >> 4;
             uint32_t n_rings = 0, n_chunks = 0;
             bool ok = true;
@@ -322,12 +264,10 @@ conv_belt_tc_kernel(const ConvPlan P, int block_lo, int n_tiles_k, int ring_lo, 
                     const uint64_t db0 = b_hi + ((pb0 + b * 4 * seg_cap) >> 4);
                     auto da = [&](int s) { return da0 + (uint32_t)((s - kSteps * c) * 16); };
                     auto db = [&](int s) { return db0 + (uint32_t)((s - g.s0) * 2); };
-                    if (c == g.mid) {
-                        for (int s = kSteps * c + 3; s < kSteps * c + 5; ++s) {
-                            if (s < t0 || s >= t1) continue;
-                            mma_f16(d, da(s) + a_l, db(s) + b_l, idesc, acc);
-                            acc = 1u;
-                        }
+                    const int s_c = kSteps * c + kSteps / 2;  // the closest approach's step
+                    if (c == g.mid && s_c >= t0 && s_c < t1) {
+                        mma_f16(d, da(s_c) + a_l, db(s_c) + b_l, idesc, acc);
+                        acc = 1u;
                     }
                     for (int s = t0; s < t1; ++s) {
                         mma_f16(d, da(s), db(s) + b_l, idesc, acc);
@@ -545,10 +485,7 @@ conv_belt_tc_kernel(const ConvPlan P, int block_lo, int n_tiles_k, int ring_lo, 
                 tc::fence_async_smem();
                 tc::fence_before_sync();
                 __syncwarp();
-                if (lane == 0)
-                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(
-                                     tc::saddr(&a_full[st]))
-                                 : "memory");
+                if (lane == 0) tc::mbar_arrive(&a_full[st]);
             }
             if (!ok) break;
             ++n_rings;
@@ -556,14 +493,14 @@ conv_belt_tc_kernel(const ConvPlan P, int block_lo, int n_tiles_k, int ring_lo, 
             if (n_rings >= 2 && !(ok = drain(n_rings - 2))) break;
         }
         if (ok && n_rings >= 1) ok = drain(n_rings - 1);
-        if (ok) {
-            if (mean != 0.0f) {
-                wsum -= wcomp;
+        if (mean != 0.0f) {  // every builder warp comes here, after an abort too
+            wsum -= wcomp;
 #pragma unroll
-                for (int s = 16; s > 0; s >>= 1) wsum += __shfl_xor_sync(~0u, wsum, s);
-                if (lane == 0) s_wsum[warp] = wsum * wunscale * mean;
-                asm volatile("bar.sync 1, %0;" ::"r"(kT) : "memory");  // the builder warps
-            }
+            for (int s = 16; s > 0; s >>= 1) wsum += __shfl_xor_sync(~0u, wsum, s);
+            if (lane == 0) s_wsum[warp] = wsum * wunscale * mean;
+            asm volatile("bar.sync 1, %0;" ::"r"(kT) : "memory");
+        }
+        if (ok) {
             // out = domega (unscale (total + what its folds still owe) + mean sum of weights)
             const int row = (warp & 3) * 32 + lane, rr = r_first + (row >> 3);
             const bool live = (row >> 3) < n_rows && rr >= ring_lo && rr <= ring_hi;

@@ -1,0 +1,991 @@
+// Real-space convolution, ring pairs with a polar-cap ring, on the tcgen05 tensor cores.
+//
+// For output ring r (L pixels) and input ring q (L' pixels), output pixel k lies at
+// s_k = n_k + f_k in units of q's pixels, n_k whole, f_k = rem_k / (2 L) in [-1/2, 1/2),
+// and the weight of input pixel n_k - j is W(f_k + j), W smooth in its argument as far as
+// the cut.  On each unit cell W is a polynomial of degree 8,
+//
+//   W(f + j) = sum_p c_p[j] f^p,      so      out_k += sum_p f_k^p y_p[n_k],
+//   y_p[n] = sum_j c_p[j] m_q[n - j]:
+//
+// nine Toeplitz products on the input ring's own grid, whose weights no longer depend on
+// the output pixel, and one short polynomial per output pixel and input ring, where the
+// gather (conv_sym.cu) evaluates a weight per class and input pixel.  With l_max = 2 nside
+// the degree-8 interpolant is within 2e-9 of the kernel's peak (4e-9 at l_max = 3 nside;
+// the host checks); c_p falls off as the derivatives do: c_8 / 2^8 is about 1e-6.
+//
+// A CTA owns two adjacent rings and their southern mirrors (which share every weight) over
+// one sector of longitude.  Per input ring:
+//
+//   D_h[m, (R, p, i)] = sum_x A_h[m, x] B[(R, p, i), x],   A_h[m, x] = m_q[n0 + d0 + x + 8 m],
+//   D_h[m, (R, p, i)] = y_p[n0 + 8 m + i] of ring R on hemisphere h:
+//
+// M = 128 rows are groups of eight input positions, N = 2 rings x 9 powers x 8 offsets.
+// As in the belt kernel neither operand is a full matrix: A's rows are 16 bytes apart in
+// the staged ring segment, B's eight rows of one (R, p) are one sequence shifted by i.
+//
+// Precision as in conv_belt_tc.cu: two FP16 parts of map and weights, w_h m_h in one FP32
+// accumulator, w_h m_l + w_l m_h (and w_l m_l in the step of the closest approach) in a
+// second one; for p = 6, 7, 8 (coefficients below 2^-12 of the peak) w_h m_h alone; far
+// chunks first.  The polynomial and the pixels of the two cells that the cut divides (at
+// most one pixel a side, tested with the exact integers) are in FP32, the sum over input
+// rings compensated.
+//
+// The coefficients c_p[j] depend on the ring pair alone and are laid out once per split
+// (cap_coef_kernel: about 7 ms and 2.4 GB at nside 2048 with a 240' cut); evaluated inside
+// this kernel they took half of its instructions, for every sector again.
+//
+// Ring pairs near the poles whose window is the whole ring or close to it, and input rings of
+// fewer than 32 pixels, go through cap_direct_kernel: every weight from the chord, each for
+// the four quarter turns and the two hemispheres.
+//
+// A pair of rings whose input rings span more than 2^14 in largest magnitudes (all-zero
+// blocks aside) or hold an infinity or NaN is flagged and left to conv_sym_kernel.
+#include <algorithm>
+#include <cmath>
+#include <cstdint>
+
+#include "ksc_device.cuh"
+#include "ksc_internal.h"
+#include "ksc_tc_split.cuh"
+
+namespace ksc {
+namespace {
+
+constexpr int kEpi = 256;          // threads that sum up: a warp per ring and 256 positions
+constexpr int kBuild = 256;        // threads that stage and lay out the operands
+constexpr int kT = kEpi + kBuild;
+constexpr int kThreads = kT + 128; // and four warps that issue the MMAs
+constexpr int kP = 9;              // polynomial coefficients
+constexpr int kP3 = 6;             // of which three-product ones
+constexpr int kG = 2 * kP;         // (ring, power) groups of eight B rows
+constexpr int kG3 = 2 * kP3;
+constexpr int kN = 8 * kG;         // columns of an accumulator (144)
+constexpr int kN3 = 8 * kG3;       // columns of the three-product groups (96)
+constexpr int kHemi = kN + kN3;    // columns of a hemisphere: leading and small products
+constexpr int kChunk = 32;         // window positions per B stage
+constexpr int kSteps = kChunk / 16;
+// K-adjacent core matrices of B lie 144 bytes apart, so that eight lanes that each write a
+// row of their own core matrix reach all banks (at 128 bytes they share four)
+constexpr int kLead = 144;
+constexpr int kGroupBytes = kChunk / 8 * kLead;
+constexpr int kStageBytes = (kG + kG3) * kGroupBytes;  // high parts, then low parts
+constexpr int kStages = 3;
+constexpr int kSpan = 1024;        // positions of a tile (128 rows of eight)
+constexpr int kOut = 9;            // outputs a lane carries at a time
+constexpr int kTurn = 32 * 10;     // float2 of a warp's turning buffer (10 per 8 positions)
+constexpr int kXr = 7;             // staged elements of a builder thread and hemisphere
+
+using tc::Window;
+__host__ __device__ __forceinline__ Window window_of(int w, int L) {
+    return tc::tile_window<kChunk>(w, L);
+}
+
+// Interpolation nodes: 0 and the other Chebyshev nodes of [-1/2, 1/2] at nine points, to 2^-10 (so
+// that j + g is exact in FP32).
+__host__ __device__ constexpr float node(int s) {
+    return s == 0 ? 0.0f : s == 1 ? 175.0f / 1024 : s == 2 ? 329.0f / 1024
+           : s == 3 ? 443.0f / 1024 : 504.0f / 1024;
+}
+
+// Two FP32 values in one register pair.
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+    return (uint64_t)__float_as_uint(b) << 32 | __float_as_uint(a);
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+// Group of (ring R, power p): three-product groups first.
+__device__ __forceinline__ int group_of(int R, int p) {
+    return p < kP3 ? R * kP3 + p : kG3 + R * (kP - kP3) + p - kP3;
+}
+
+// Wait that gives up at once when the CTA has (builder warps meet at barriers: none of
+// them may leave the loop).
+__device__ __forceinline__ void wait_all(uint64_t *bar, uint32_t parity, volatile int *abort) {
+    if (!*abort) tc::wait_or_abort(bar, parity, abort);
+    __syncwarp();
+}
+
+__device__ __forceinline__ void copy16(void *dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tc::saddr(dst)), "l"(src) : "memory");
+}
+
+struct QInfo {      // an input ring as the tile sees it
+    int n0;         // first position (input pixel) of row 0
+    int eR[2];      // rem <= eR: the right edge cell's pixel lies within the cut
+    uint32_t off[2];  // first coefficient word of each ring, in units of four
+    int start[2];   // first pixel of the ring and of its mirror
+    int a;          // ring pixel of element 0 of the staged segments
+    short len, phase;  // of the input ring
+    short n_e;      // elements staged
+    short base;     // d0 + 16 s0: Delta of element 0 at offset i = 0
+    short jE[2];    // edge cell of each ring (-1: no pixel within the cut)
+    short s0, s1, mid, pad;  // window steps and the chunk of the closest approach
+};
+
+// Words of a ring pair's coefficients, [cell][power], rounded up to 16 bytes.
+__host__ __device__ __forceinline__ int coef_words(int jE) { return (kP * (jE + 1) + 3) & ~3; }
+
+// grid.x runs over tiles {rings - 1 << 16 | first ring, sectors << 16 | sector}, grid.y over
+// maps.  Eight builder warps
+// stage ring n + 1 while the tensor cores work on ring n and eight summing warps on ring
+// n - 1 (their accumulators are the same: a summing warp reads them power by power and
+// gives them back with d_free before it adds up).
+//
+// A summing warp owns ring R and 256 positions.  Its lanes take consecutive outputs; the
+// accumulators come in rows of eight positions a lane, so each power of both hemispheres
+// is turned in shared memory (as (north, south) pairs, which the polynomial, the edge
+// pixels and the sums keep as FP32 pairs).
+__global__ void __launch_bounds__(kThreads, 1)
+conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ tiles,
+                   const float *__restrict__ in, float *__restrict__ out, long long map_stride,
+                   int belt_split, int band_lo, int band_hi, const uint2 *__restrict__ ring_range,
+                   int *__restrict__ flags, int *__restrict__ err) {
+    extern __shared__ __align__(1024) unsigned char smem[];
+    // B stages | map segments [h][buffer][part] | turning buffers | totals (north, south:
+    // sums, compensations) [ring] | the segments as they are, (north, south) [buffer] |
+    // coefficients as stored [buffer] | coefficient sequences | input rings
+    const int xc = C.span + C.wpos;
+    // words of one coefficient sequence, two FP16 elements each; 16-byte rows, and 20 words
+    // more than a multiple of 32 so that the groups start in different banks
+    const int w_cap = ((C.wpos / 2 + 8 + 11) & ~31) + 20;
+    const int k_cap = 2 * coef_words(C.jcap - 1);
+    unsigned char *sB = smem;
+    __half *sX = reinterpret_cast<__half *>(smem + kStages * kStageBytes);
+    float2 *sY = reinterpret_cast<float2 *>(sX + 8 * xc);
+    float4 *sT = reinterpret_cast<float4 *>(sY + kEpi / 32 * kTurn);
+    float2 *sF = reinterpret_cast<float2 *>(sT + 2 * C.tcap);
+    uint32_t *sK = reinterpret_cast<uint32_t *>(sF + 2 * xc);
+    uint32_t *sC = sK + 2 * k_cap;
+    QInfo *sQ = reinterpret_cast<QInfo *>(sC + 2 * (kG + kG3) * w_cap);
+    __shared__ __align__(8) uint64_t b_full[kStages], b_free[kStages], d_done, d_free[2], e_ready[2],
+        s_drain[4];
+    __shared__ uint32_t tmem_base, s_max, s_min;
+    __shared__ int s_abort, s_lo, s_hi, s_bad;
+    __shared__ float s_mean[kT / 32], s_edge[2][2][kP + 3], s_sum[2][2][kP];
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int2 tile = tiles[blockIdx.x];
+    const int r0 = tile.x & 0xffff, n_r = (tile.x >> 16) + 1;
+    const int sector = tile.y & 0xffff, n_sec = tile.y >> 16;
+    const bool add = belt_split && r0 >= P.belt_lo;
+    const float *m = in + (long long)blockIdx.y * map_stride;
+    float *o = out + (long long)blockIdx.y * map_stride;
+    const uint2 *rr = ring_range + (long long)blockIdx.y * P.nrings;
+    const DevRing Ra = P.d_rings[r0], Rb = P.d_rings[r0 + n_r - 1];
+    const int L0 = Ra.len, L1 = Rb.len;
+    auto sec_lo = [&](int L, int s) { return (int)(((long long)s * L + n_sec - 1) / n_sec); };
+    const int k_lo0 = sec_lo(L0, sector), k_hi0 = sec_lo(L0, sector + 1) - 1;
+    const int k_lo1 = sec_lo(L1, sector), k_hi1 = n_r == 2 ? sec_lo(L1, sector + 1) - 1 : k_lo1 - 1;
+
+    if (tid == 0) {
+        s_max = 0u;
+        s_min = 0xffffffffu;
+        s_abort = s_bad = 0;
+        s_lo = min(P.d_range[r0].x, P.d_range[r0 + n_r - 1].x);
+        s_hi = max(P.d_range[r0].y, P.d_range[r0 + n_r - 1].y);
+        for (int b = 0; b < kStages; ++b) {
+            tc::mbar_init(&b_full[b], kBuild / 32);
+            tc::mbar_init(&b_free[b], 4);
+        }
+        tc::mbar_init(&d_done, 4);
+        for (int b = 0; b < 4; ++b) tc::mbar_init(&s_drain[b], 1);
+        for (int b = 0; b < 2; ++b) {  // ring n uses the one of its parity
+            tc::mbar_init(&d_free[b], kEpi / 32);
+            tc::mbar_init(&e_ready[b], kBuild / 32);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    const int q_lo = s_lo, nq = s_hi - s_lo + 1;
+    // ---- the input rings as the tile sees them, and the range of their values
+    uint32_t vmax = 0u, vmin = 0xffffffffu;
+    for (int qi = tid; qi < nq; qi += kThreads) {
+        const int q = q_lo + qi;
+        const DevRing Q = P.d_rings[q];
+        QInfo g;
+        g.jE[0] = g.jE[1] = -1;
+        g.eR[0] = g.eR[1] = 0;
+        g.off[0] = g.off[1] = 0u;
+        const bool skip = add && q >= P.belt_lo && q <= P.belt_hi;
+        for (int R = 0; R < n_r && !skip; ++R) {
+            const int2 rg = P.d_range[r0 + R];
+            if (q < rg.x || q > rg.y) continue;
+            const int ip = P.d_pair_base[r0 + R] + q - rg.x;
+            const int ncut = C.d_ncut[ip], L = R ? L1 : L0;
+            if (ncut < 0) continue;
+            g.jE[R] = ncut >= L ? (short)((ncut - L) / (2 * L) + 1) : 0;
+            g.eR[R] = ncut - 2 * L * g.jE[R];
+            g.off[R] = C.d_coef_off[ip];
+        }
+        const int w = max((int)g.jE[0], (int)g.jE[1]);
+        // positions of the sector's first and last outputs
+        auto pos = [&](int k, int t, int L) {
+            return (int)((unsigned)((2 * k + t) * Q.len + (1 - Q.phase) * L) / (unsigned)(2 * L));
+        };
+        int lo = 0x7fffffff, hi = -1;
+        if (k_hi0 >= k_lo0) {
+            lo = pos(k_lo0, Ra.phase, L0);
+            hi = pos(k_hi0, Ra.phase, L0);
+        }
+        if (k_hi1 >= k_lo1) {
+            lo = min(lo, pos(k_lo1, Rb.phase, L1));
+            hi = max(hi, pos(k_hi1, Rb.phase, L1));
+        }
+        g.n0 = lo;
+        g.len = (short)Q.len;
+        g.phase = (short)Q.phase;
+        g.start[0] = Q.start;
+        g.start[1] = P.d_rings[P.nrings - 1 - q].start;
+        if (w >= 0) {
+            const Window v = window_of(w, Q.len);
+            g.s0 = (short)v.s0;
+            g.s1 = (short)v.s1;
+            g.mid = (short)v.mid;
+            g.base = (short)(v.d0 + 16 * v.s0);
+            g.n_e = (short)(((hi - lo + 8) & ~7) + 16 * (v.s1 - v.s0));
+            g.a = (lo + g.base) % Q.len;
+            g.a += g.a < 0 ? Q.len : 0;
+            // sized by the host for every tile: never expected
+            if (16 * (v.s1 - v.s0) > C.wpos || w + 1 > C.jcap || hi - lo + 1 > C.span ||
+                g.n_e > kXr * kBuild || hi < lo || 2 * w + 1 > Q.len)
+                s_bad = 1;
+            for (int h = 0; h < 2; ++h) {
+                const uint2 e = rr[h ? P.nrings - 1 - q : q];
+                vmax = max(vmax, e.x);
+                vmin = min(vmin, e.y);
+            }
+        }
+        if (qi < C.nq) sQ[qi] = g;
+        else s_bad = 1;
+    }
+    vmax = __reduce_max_sync(~0u, vmax);
+    vmin = __reduce_min_sync(~0u, vmin);
+    if (warp < kT / 32) {  // mean of 512 pixels of the tile's first ring
+        float v = m[Ra.start + (int)((long long)tid * L0 / kT)];
+#pragma unroll
+        for (int s = 16; s > 0; s >>= 1) v += __shfl_xor_sync(~0u, v, s);
+        if (lane == 0) s_mean[warp] = v * (1.0f / 32.0f);
+    }
+    if (lane == 0) {
+        atomicMax(&s_max, vmax);
+        atomicMin(&s_min, vmin);
+    }
+    if (tid == 0 && max(k_hi0 - k_lo0, k_hi1 - k_lo1) + 1 > C.tcap) s_bad = 1;
+    for (int e = tid; e < 2 * C.tcap; e += kThreads) sT[e] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (warp == kT / 32) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                         tc::saddr(&tmem_base)),
+                     "r"(512));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t tmem = tmem_base;
+    const uint32_t emax = s_max >> 23, emin = s_min >> 23;  // biased exponents
+    const bool zero = s_max == 0u;
+    const bool flag = !zero && (emax >= 255u || emax < 48u || emax > 206u || emin == 0u ||
+                                emax - emin > tc::kRangeExp);
+    if (tid == 0) {
+        if (flag) {
+            int *f = flags + (long long)blockIdx.y * (P.nrings + 1);
+            f[r0] = 1;
+            f[r0 + n_r - 1] = 1;
+            f[P.nrings] = 1;
+        }
+        if (s_bad) atomicExch(err, KSC_ERR_DEVICE_BOUNDS);
+    }
+    // a constant taken off where every block is within a factor of four of the largest: a
+    // multiple of 2^-3 of the largest value's power of two (none for maps about zero)
+    float mean = 0.0f;
+    if (!zero && !flag && emax - emin <= 1u) {
+#pragma unroll
+        for (int i = 0; i < kT / 32; ++i) mean += s_mean[i];
+        const float quantum = __uint_as_float((emax - 3u) << 23);
+        mean = rintf(mean * (1.0f / (kT / 32)) / quantum) * quantum;
+    }
+    const uint32_t ex = emax + (mean != 0.0f ? 1u : 0u);
+    const float xscale = zero || flag ? 1.0f : __uint_as_float((127u + tc::kXExp + 127u - ex) << 23);
+    const float xunscale = zero || flag ? 1.0f : __uint_as_float((ex - tc::kXExp) << 23);
+    const float ms = mean * xscale;
+    bool drained = true;
+
+    if (flag || s_bad) {
+        // left to the gather (or never expected)
+    } else if (warp >= kT / 32) {
+        // ---- the issuing warps: one per hemisphere and accumulator (an MMA takes its
+        // thread about as long to issue as 80 columns take to compute)
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
+        if (lane == 0) {
+            const int h = warp & 1;
+            const bool small = warp & 2;  // the small products' accumulator, else the leading ones'
+            const uint32_t idesc = small ? tc::idesc_f16(128, kN3) : tc::idesc_f16(128, kN);
+            const uint32_t d = tmem + h * kHemi + (small ? kN : 0);
+            const uint64_t b_base = tc::desc(tc::saddr(sB), kLead, kGroupBytes);
+            const uint64_t a_base = tc::desc(tc::saddr(sX) + h * 8 * xc, 16, 128);
+            const uint32_t a_l = (uint32_t)(2 * xc) >> 4, b_l = (kG * kGroupBytes) >> 4;
+            uint32_t n = 0, n_chunks = 0, st = 0, ph = 0;
+            bool ok = true;
+            for (int qi = 0; qi < nq && ok; ++qi) {
+                const QInfo &g = sQ[qi];
+                if (max((int)g.jE[0], (int)g.jE[1]) < 0) continue;
+                const int s0 = g.s0, s1 = g.s1, mid = g.mid;
+                const int c_lo = s0 / kSteps, c_hi = (s1 - 1) / kSteps;
+                const uint64_t da0 = a_base + (n & 1u) * ((4 * xc) >> 4);
+                if (n > 0 && !tc::wait_or_abort(&d_free[(n - 1u) & 1u], ((n - 1u) >> 1) & 1u, &s_abort))
+                    break;
+                uint32_t acc = 0u;
+                for (int cc = c_lo; cc <= c_hi; ++cc, ++n_chunks) {
+                    const int c = tc::chunk_of(cc, c_hi, mid);
+                    if (!tc::wait_or_abort(&b_full[st], ph, &s_abort)) {
+                        ok = false;
+                        break;
+                    }
+                    tc::fence_after_sync();
+                    const int t0 = max(s0, kSteps * c), t1 = min(s1, kSteps * c + kSteps);
+                    // descriptors of step t0; a step is 32 bytes of the segment, two core
+                    // matrices of B
+                    uint64_t da = da0 + (uint32_t)((t0 - s0) * 2);
+                    uint64_t db = b_base + (uint32_t)((st * kStageBytes) >> 4) +
+                                  (uint32_t)((t0 - kSteps * c) * (2 * kLead / 16));
+                    if (small) {
+                        const int s_c = kSteps * c + kSteps / 2 - t0;  // the closest approach's step
+                        if (c == mid && s_c >= 0 && s_c < t1 - t0) {
+                            tc::mma_f16(d, da + (uint32_t)(2 * s_c) + a_l,
+                                        db + (uint32_t)(s_c * (2 * kLead / 16)) + b_l, idesc, acc);
+                            acc = 1u;
+                        }
+#pragma unroll
+                        for (int s = 0; s < kSteps; ++s) {
+                            if (s >= t1 - t0) break;
+                            tc::mma_f16(d, da + (uint32_t)(2 * s), db + (uint32_t)(s * (2 * kLead / 16)) + b_l,
+                                        idesc, acc);
+                            tc::mma_f16(d, da + (uint32_t)(2 * s) + a_l,
+                                        db + (uint32_t)(s * (2 * kLead / 16)), idesc, 1u);
+                            acc = 1u;
+                        }
+                    } else {
+#pragma unroll
+                        for (int s = 0; s < kSteps; ++s) {  // (the closest approach's is the last)
+                            if (s >= t1 - t0) break;
+                            tc::mma_f16(d, da + (uint32_t)(2 * s), db + (uint32_t)(s * (2 * kLead / 16)),
+                                        idesc, acc);
+                            acc = 1u;
+                        }
+                    }
+                    tc::mma_commit(&b_free[st]);
+                    if (++st == kStages) {
+                        st = 0;
+                        ph ^= 1u;
+                    }
+                }
+                if (!ok) break;
+                tc::mma_commit(&d_done);
+                ++n;
+            }
+            // (after an abort: nothing of this thread is in flight when its last commit is done)
+            if (n_chunks > 0 && s_abort) {
+                tc::mma_commit(&s_drain[warp & 3]);
+                drained = tc::mbar_wait(&s_drain[warp & 3], 0u);
+            }
+        }
+        __syncwarp();
+    } else {
+        // 640 x 96 registers at launch = 512 x 112 + 128 x 32
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
+        if (warp < kEpi / 32) {
+            // ---- summing warps
+            const int R = warp >> 2, quarter = warp & 3;
+            const int L = R ? L1 : L0, t = R ? Rb.phase : Ra.phase;
+            const int k_lo = R ? k_lo1 : k_lo0, k_hi = R ? k_hi1 : k_hi0;
+            const int two_l = 2 * L;
+            const float inv2L = 1.0f / (float)two_l;
+            float4 *tot = sT + R * C.tcap;
+            float2 *turn = sY + warp * kTurn;
+            const uint32_t td = tmem + ((uint32_t)(quarter * 32) << 16);
+            const uint64_t m1 = pack2(-1.0f, -1.0f), cut = pack2(-0x1p-24f, -0x1p-24f);
+            uint32_t n = 0;
+            for (int qi = 0; qi < nq; ++qi) {
+                const QInfo g = sQ[qi];
+                if (max((int)g.jE[0], (int)g.jE[1]) < 0) continue;
+                const uint32_t buf = n & 1u;
+                wait_all(&e_ready[buf], (n >> 1) & 1u, &s_abort);
+                // the ring's other warps have added ring n - 1: outputs change hands
+                asm volatile("bar.sync %0, 128;" ::"r"(2 + R) : "memory");
+                const int jE = g.jE[R], Lq = g.len, step = 2 * Lq;
+                // outputs at positions n0 + 256 quarter .. + 255: k in [kA, kB]
+                auto first = [&](int pos) {  // ceil(num / step)
+                    const int num = (2 * pos + g.phase - 1) * L - t * Lq;
+                    int k = (int)((float)num / (float)step);
+                    k += k * step < num ? 1 : 0;
+                    k -= (k - 1) * step >= num ? 1 : 0;
+                    return k;
+                };
+                const int p0 = g.n0 + 256 * quarter;
+                const int kA = max(first(p0), k_lo);
+                const int kB = jE < 0 ? kA - 1 : min(first(p0 + 256) - 1, k_hi);
+                bool waited = false;
+                for (int kb = kA; kb <= kB; kb += 32 * kOut) {
+                    float f[kOut];
+                    uint64_t e2[kOut], v[kOut];
+                    int at[kOut];
+                    float ec[kP];  // the edge cell's polynomial, for the map as stored
+#pragma unroll
+                    for (int p = 0; p < kP; ++p) ec[p] = s_edge[buf][R][p] * xscale;
+                    const int eR = g.eR[R];
+                    const float2 *x = sF + buf * xc;
+#pragma unroll
+                    for (int o = 0; o < kOut; ++o) {
+                        // position and offset of output k (clamped: the last ones are not kept)
+                        const int k = min(kb + 32 * o + lane, kB);
+                        const int u = (2 * k + t) * Lq + (1 - g.phase) * L - two_l * p0;
+                        int i = (int)((float)u * inv2L);
+                        int rem = u - i * two_l;
+                        if (rem < 0) {
+                            --i;
+                            rem += two_l;
+                        } else if (rem >= two_l) {
+                            ++i;
+                            rem -= two_l;
+                        }
+                        rem -= L;
+                        f[o] = (float)rem * inv2L;
+                        at[o] = i + (i >> 3) * 2;
+                        const float fo = f[o], f2 = fo * fo;
+                        // the edge cells' weights: even and odd parts
+                        const float we = fmaf(f2, fmaf(f2, fmaf(f2, fmaf(f2, ec[8], ec[6]), ec[4]), ec[2]), ec[0]);
+                        const float wo = fo * fmaf(f2, fmaf(f2, fmaf(f2, ec[7], ec[5]), ec[3]), ec[1]);
+                        const bool in_r = rem <= eR, in_l = rem >= -eR;
+                        const float wr = jE > 0 ? (in_r ? we + wo : 0.0f) : (in_r && in_l ? we : 0.0f);
+                        const float wl = jE > 0 && in_l ? we - wo : 0.0f;
+                        // elements of positions n - jE and n + jE
+                        const int er = 256 * quarter + i - jE - g.base;
+                        const float2 xr = x[er], xl = x[er + 2 * jE];
+                        e2[o] = fma2(pack2(wl, wl), pack2(xl.x, xl.y),
+                                     fma2(pack2(wr, wr), pack2(xr.x, xr.y), 0ull));
+                        v[o] = 0ull;
+                    }
+                    if (!waited) {  // the accumulators (the edge pixels came from the map)
+                        wait_all(&d_done, n & 1u, &s_abort);
+                        tc::fence_after_sync();
+                        waited = true;
+                    }
+#pragma unroll 1
+                    for (int p = kP - 1; p >= 0; --p) {
+                        const uint32_t c = td + (uint32_t)(8 * group_of(R, p));
+                        uint32_t a[8], b[8];
+                        tc::tmem_ld8(c, a);
+                        tc::tmem_ld8(c + kHemi, b);
+                        float off = 0.0f;
+                        if (mean != 0.0f && !(p & 1)) off = ms * s_sum[buf][R][p];
+                        uint64_t w[8];
+                        if (p < kP3) {
+                            uint32_t xa[8], xb[8];
+                            tc::tmem_ld8(c + kN, xa);
+                            tc::tmem_ld8(c + kN + kHemi, xb);
+                            tc::tmem_wait_ld();
+#pragma unroll
+                            for (int i = 0; i < 8; ++i)
+                                w[i] = add2((uint64_t)b[i] << 32 | a[i], (uint64_t)xb[i] << 32 | xa[i]);
+                        } else {
+                            tc::tmem_wait_ld();
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) w[i] = (uint64_t)b[i] << 32 | a[i];
+                        }
+                        if (mean != 0.0f)
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) w[i] = add2(w[i], pack2(off, off));
+                        __syncwarp();
+                        ulonglong2 *dst = reinterpret_cast<ulonglong2 *>(turn + 10 * lane);
+#pragma unroll
+                        for (int i = 0; i < 8; i += 2) dst[i / 2] = make_ulonglong2(w[i], w[i + 1]);
+                        __syncwarp();
+#pragma unroll
+                        for (int o = 0; o < kOut; ++o)
+                            v[o] = fma2(v[o], pack2(f[o], f[o]),
+                                        *reinterpret_cast<const uint64_t *>(turn + at[o]));
+                    }
+                    if (kb + 32 * kOut > kB) {  // the accumulators are no longer needed
+                        tc::fence_before_sync();
+                        __syncwarp();
+                        if (lane == 0) tc::mbar_arrive(&d_free[buf]);
+                    }
+#pragma unroll
+                    for (int o = 0; o < kOut; ++o) {
+                        const int k = kb + 32 * o + lane;
+                        if (k > kB) break;
+                        // Kahan, with the 2^-24 that the MMAs' cuts cost on average
+                        const uint64_t z = add2(v[o], e2[o]);
+                        ulonglong2 *q = reinterpret_cast<ulonglong2 *>(tot + k - k_lo);
+                        ulonglong2 s = *q;
+                        const uint64_t d = fma2(s.y, m1, z), w = add2(s.x, d);
+                        s.y = fma2(z, cut, fma2(d, m1, fma2(s.x, m1, w)));
+                        s.x = w;
+                        *q = s;
+                    }
+                }
+                if (!waited) {  // no outputs here: keep step
+                    wait_all(&d_done, n & 1u, &s_abort);
+                    if (lane == 0) tc::mbar_arrive(&d_free[buf]);
+                }
+                ++n;
+            }
+            asm volatile("bar.sync 4, %0;" ::"r"(kEpi) : "memory");
+            // ---- outputs: four warps per (ring, hemisphere) in turn
+            for (int h = 0; h < 2; ++h) {
+                const int ring = h ? P.nrings - 1 - (r0 + R) : r0 + R;
+                if (R >= n_r || ring < band_lo || ring > band_hi || (h && ring == r0 + R) || s_abort)
+                    continue;
+                float *dst = o + P.d_rings[ring].start;
+                const float unscale = xunscale * C.wunscale;
+                for (int k = k_lo + quarter * 32 + lane; k <= k_hi; k += 128) {
+                    const float4 s = tot[k - k_lo];
+                    const float hi = (h ? s.y : s.x) * unscale, lo = -(h ? s.w : s.z) * unscale;
+                    const float v = fmaf(hi, P.domega, fmaf(hi, C.domega_lo, lo * P.domega));
+                    if (add) dst[k] += v;
+                    else dst[k] = v;
+                }
+            }
+        } else {
+            // ---- builder warps
+            const int bt = tid - kEpi, bw = warp - kEpi / 32;
+            uint32_t n = 0, n_chunks = 0;
+            float xn[kXr], xs[kXr];
+            // loads of an input ring: segments into registers, coefficients by async copies
+            auto fetch = [&](int qi, uint32_t m_) {
+                const QInfo g = sQ[qi];
+                const float *rn = m + g.start[0], *rs = m + g.start[1];
+#pragma unroll
+                for (int e = 0; e < kXr; ++e) {
+                    if (bt + e * kBuild >= g.n_e) break;
+                    int i = g.a + bt + e * kBuild;
+                    while (i >= g.len) i -= g.len;
+                    xn[e] = __ldg(rn + i);
+                    xs[e] = __ldg(rs + i);
+                }
+                uint32_t *dst = sK + (m_ & 1u) * k_cap;
+                const int w0 = g.jE[0] >= 0 ? coef_words(g.jE[0]) / 4 : 0;
+                const int w1 = g.jE[1] >= 0 ? coef_words(g.jE[1]) / 4 : 0;
+                for (int e = bt; e < w0 + w1; e += kBuild)
+                    copy16(dst + 4 * e, C.d_coef + 4ull * (e < w0 ? g.off[0] + e : g.off[1] + (e - w0)));
+                asm volatile("cp.async.commit_group;" ::: "memory");
+            };
+            auto next = [&](int qi) {  // the next input ring with pixels within the cut
+                while (qi < nq && max(sQ[qi].jE[0], sQ[qi].jE[1]) < 0) ++qi;
+                return qi;
+            };
+            int qi = next(0);
+            if (qi < nq) fetch(qi, 0u);
+            while (qi < nq) {
+                const QInfo g = sQ[qi];
+                const uint32_t buf = n & 1u;
+                const int n_pos = 16 * (g.s1 - g.s0);
+                // ring n - 2 has left these buffers
+                if (n >= 2) wait_all(&d_free[buf], ((n >> 1) - 1u) & 1u, &s_abort);
+                // ---- the segments, as they are and scaled and split
+#pragma unroll
+                for (int e = 0; e < kXr; ++e) {
+                    const int i = bt + e * kBuild;
+                    if (i >= g.n_e) break;
+                    sF[buf * xc + i] = make_float2(xn[e], xs[e]);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        __half *xh = sX + (h * 2 + buf) * 2 * xc;
+                        const float y = fmaf(h ? xs[e] : xn[e], xscale, -ms);
+                        const __half hh = __float2half_rn(y);
+                        xh[i] = hh;
+                        xh[xc + i] = __float2half_rn(y - __half2float(hh));
+                    }
+                }
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+                asm volatile("bar.sync 1, %0;" ::"r"(kBuild) : "memory");
+                // ---- the coefficient sequences of each group (R, p): element x is
+                // c_p[-Delta] at Delta = x + base - 8, c_p[-j] = (-1)^p c_p[j], zero beyond
+                // the interior cells.  Word k of the even sequence holds elements 2k and
+                // 2k + 1, of the odd one 2k - 1 and 2k; high parts of all groups, then low
+                // parts of the first kG3.
+                const uint32_t *raw = sK + buf * k_cap;
+                const int raw1 = g.jE[0] >= 0 ? coef_words(g.jE[0]) : 0;
+                {
+                    const int n_w = n_pos / 2 + 8, n_blk = (n_w + 31) / 32;
+                    for (int task = bw; task < kG * n_blk; task += kBuild / 32) {
+                        const int grp = task % kG, k = task / kG * 32 + lane;
+                        // (ring, power) of the group
+                        const int R = grp < kG3 ? grp / kP3 : (grp - kG3) / (kP - kP3);
+                        const int p = grp < kG3 ? grp - R * kP3 : grp - kG3 - R * (kP - kP3) + kP3;
+                        const int jE = g.jE[R];
+                        if (k >= n_w) continue;
+                        const uint32_t flip = p & 1 ? 0x80008000u : 0u;
+                        const uint32_t *src = raw + (R ? raw1 : 0) + p;
+                        uint32_t c[3];
+#pragma unroll
+                        for (int i = 0; i < 3; ++i) {
+                            const int dl = 2 * k - 9 + i + g.base, j = dl < 0 ? -dl : dl;
+                            c[i] = j < jE ? src[j * kP] ^ (dl > 0 ? flip : 0u) : 0u;
+                        }
+                        uint32_t *d = sC + 2 * grp * w_cap + k;
+                        d[0] = __byte_perm(c[1], c[2], 0x5410);
+                        d[w_cap] = __byte_perm(c[0], c[1], 0x5410);
+                        if (p < kP3) {
+                            d += 2 * kG * w_cap;
+                            d[0] = __byte_perm(c[1], c[2], 0x7632);
+                            d[w_cap] = __byte_perm(c[0], c[1], 0x7632);
+                        }
+                    }
+                    // the edge cells: in FP32, not in the products
+                    if (bt < 2 * kP) {
+                        const int R = bt >= kP, p = bt - R * kP, jE = g.jE[R];
+                        if (jE >= 0) {
+                            const uint32_t hl = raw[(R ? raw1 : 0) + jE * kP + p];
+                            s_edge[buf][R][p] = __half2float(__ushort_as_half((unsigned short)hl)) +
+                                                __half2float(__ushort_as_half((unsigned short)(hl >> 16)));
+                        }
+                    }
+                    if (mean != 0.0f) {  // sums of the even coefficients over a window
+                        for (int task = bw; task < 10; task += kBuild / 32) {
+                            const int R = task / 5, p = 2 * (task % 5);
+                            const uint32_t *src = raw + (R ? raw1 : 0) + p;
+                            float s = 0.0f, comp = 0.0f;
+                            for (int j = lane; j < g.jE[R]; j += 32) {
+                                const uint32_t hl = src[j * kP];
+                                const float c = __half2float(__ushort_as_half((unsigned short)hl)) +
+                                                __half2float(__ushort_as_half((unsigned short)(hl >> 16)));
+                                const float z = (j ? 2.0f : 1.0f) * c - comp;
+                                const float w = s + z;
+                                comp = (w - s) - z;
+                                s = w;
+                            }
+                            s -= comp;
+#pragma unroll
+                            for (int k = 16; k > 0; k >>= 1) s += __shfl_xor_sync(~0u, s, k);
+                            if (lane == 0) s_sum[buf][R][p] = s;
+                        }
+                    }
+                }
+                const int qn = next(qi + 1);
+                if (qn < nq) fetch(qn, n + 1u);
+                asm volatile("bar.sync 1, %0;" ::"r"(kBuild) : "memory");
+                if (lane == 0) tc::mbar_arrive(&e_ready[buf]);
+                // ---- B, chunk by chunk
+                const int c_lo = g.s0 / kSteps, c_hi = (g.s1 - 1) / kSteps;
+                for (int cc = c_lo; cc <= c_hi; ++cc, ++n_chunks) {
+                    const int c = tc::chunk_of(cc, c_hi, g.mid);
+                    const uint32_t st = n_chunks % kStages;
+                    if (n_chunks >= kStages)
+                        wait_all(&b_free[st], (n_chunks / kStages - 1u) & 1u, &s_abort);
+                    const int t0 = max((int)g.s0, kSteps * c), t1 = min((int)g.s1, kSteps * c + kSteps);
+                    unsigned char *sb = sB + st * kStageBytes + (t0 - kSteps * c) * 2 * kLead;
+                    // a thread lays out one core matrix (eight rows) of one group: rows of even
+                    // i from the words of the even sequence, of odd i from the odd one, four
+                    // words a row, row i two elements before row i - 2
+                    const int cols = 2 * (t1 - t0);  // core matrices of a group: 2 or 4
+                    const int w0 = 4 + 8 * (t0 - g.s0);  // word of the step's first element
+                    for (int e = bt; e < (kG + kG3) * cols; e += kBuild) {
+                        const int grp = cols == 4 ? e >> 2 : e >> 1, kg = e - grp * cols;
+                        const uint32_t *p = sC + 2 * grp * w_cap + w0 + 4 * kg;
+                        unsigned char *dst = sb + grp * kGroupBytes + kg * kLead;
+#pragma unroll
+                        for (int odd = 0; odd < 2; ++odd) {
+                            const uint4 lo = *reinterpret_cast<const uint4 *>(p + odd * w_cap - 4);
+                            const uint4 hi = *reinterpret_cast<const uint4 *>(p + odd * w_cap);
+                            uint4 *d = reinterpret_cast<uint4 *>(dst) + odd;
+                            d[0] = hi;
+                            d[2] = make_uint4(lo.w, hi.x, hi.y, hi.z);
+                            d[4] = make_uint4(lo.z, lo.w, hi.x, hi.y);
+                            d[6] = make_uint4(lo.y, lo.z, lo.w, hi.x);
+                        }
+                    }
+                    tc::fence_async_smem();
+                    __syncwarp();
+                    if (lane == 0) tc::mbar_arrive(&b_full[st]);
+                }
+                qi = qn;
+                ++n;
+            }
+        }
+    }
+    tc::fence_before_sync();
+    const bool all_drained = __syncthreads_and(drained);
+    if (s_abort && tid == 0) atomicExch(err, all_drained ? KSC_ERR_TIMEOUT : KSC_ERR_TIMEOUT_UNDRAINED);
+    // tensor memory that an MMA may still write is not freed
+    if (warp == kT / 32 && all_drained)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+}
+
+// Coefficients of the regular ring pairs of output ring r, one warp per pair, one
+// lane per cell: the kernel at nine nodes of the cell, its value at a table node as an FP32
+// pair, then the interpolating polynomial in FP64 (even and odd parts apart), each
+// coefficient scaled and split into two FP16 parts.
+__global__ void __launch_bounds__(256)
+cap_coef_kernel(const ConvPlan P, const CapTc C, const CapCoef K, int ring_lo, int ring_hi) {
+    const int r = ring_lo + blockIdx.x;
+    if (r > ring_hi) return;
+    const int2 rg = P.d_range[r];
+    const int L = P.d_rings[r].len, lane = threadIdx.x & 31;
+    for (int q = rg.x + (threadIdx.x >> 5); q <= rg.y; q += 8) {
+        const int ip = P.d_pair_base[r] + q - rg.x;
+        const int ncut = C.d_ncut[ip];
+        if (ncut < 0) continue;
+        const int jE = ncut >= L ? (ncut - L) / (2 * L) + 1 : 0;
+        const PairInfo pi = P.d_pairs[ip];
+        const DF A{pi.Ah, pi.Al}, B{pi.Bh, pi.Bl};
+        const float2 cq = K.d_ringc[q];  // pi / L' as a double-float pair
+        uint32_t *dst = K.d_coef + 4ull * C.d_coef_off[ip];
+        for (int j = lane; j <= jE; j += 32) {
+            auto value = [&](float x) {
+                const float xh = x * cq.x;
+                const float xl = fmaf(x, cq.x, -xh) + x * cq.y;
+                int ti;
+                float f;
+                chord_to_table_sel(A, B, sin_df(xh, xl), K.next2, &ti, &f);
+                ti = min(ti, K.n_ext - 1);
+                const float4 c = __ldg(&K.d_tab[ti]);
+                return (double)c.x + ((double)__ldg(&K.d_tab_lo[ti]) +
+                                      (double)(f * fmaf(f, fmaf(f, c.w, c.z), c.y)));
+            };
+            const double w0 = value((float)j);
+            double e4[4], o4[4], c[kP];
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                const float gs = s == 0 ? node(1) : s == 1 ? node(2) : s == 2 ? node(3) : node(4);
+                const double a = value((float)j + gs), b = value((float)j - gs);
+                e4[s] = 0.5 * (a + b) - w0;
+                o4[s] = 0.5 * (a - b);
+            }
+            c[0] = w0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                double e = 0.0, d = 0.0;
+#pragma unroll
+                for (int s = 0; s < 4; ++s) {
+                    e = fma(K.me[4 * k + s], e4[s], e);
+                    d = fma(K.mo[4 * k + s], o4[s], d);
+                }
+                c[2 * k + 2] = e;
+                c[2 * k + 1] = j == 0 ? 0.0 : d;  // even about cell 0
+            }
+#pragma unroll
+            for (int p = 0; p < kP; ++p) {
+                const double v = c[p] * (double)C.wscale;
+                const __half h = __float2half_rn((float)v);
+                const __half l = __float2half_rn((float)(v - (double)__half2float(h)));
+                dst[j * kP + p] = (uint32_t)__half_as_ushort(l) << 16 | __half_as_ushort(h);
+            }
+        }
+    }
+}
+
+// The irregular ring pairs of output ring r (and its mirror), added to the output.  A block
+// takes 32 first-quarter positions of r, a lane each; its eight warps share the ring's list
+// of input rings.  For one input pixel all lanes read the same values, eight (four quarter
+// turns, two hemispheres) per weight.
+__global__ void __launch_bounds__(256)
+cap_direct_kernel(const ConvPlan P, const int2 *__restrict__ items,
+                  const int *__restrict__ list_first, const int *__restrict__ list,
+                  const float *__restrict__ in, float *__restrict__ out, long long map_stride,
+                  int band_lo, int band_hi, const int *__restrict__ flags) {
+    __shared__ float part[8][8][32];
+    const int2 it = items[blockIdx.x];
+    const int r = it.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (flags[(long long)blockIdx.y * (P.nrings + 1) + r]) return;
+    const float *m = in + (long long)blockIdx.y * map_stride;
+    float *o = out + (long long)blockIdx.y * map_stride;
+    const DevRing R = P.d_rings[r];
+    const int L = R.len, Q = L / 4, k = min(it.y + lane, Q - 1);
+    const int base = P.d_pair_base[r] - P.d_range[r].x;
+    float sum[8], comp[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) sum[i] = comp[i] = 0.0f;
+    for (int e = list_first[r] + warp; e < list_first[r + 1]; e += 8) {
+        const int q = list[e];
+        const DevRing G = P.d_rings[q];
+        const int Lq = G.len, Qq = Lq / 4;
+        const PairInfo pi = P.d_pairs[base + q];
+        const DF A{pi.Ah, pi.Al}, B{pi.Bh, pi.Bl};
+        const float *xn = m + G.start, *xs = m + P.d_rings[P.nrings - 1 - q].start;
+        const int full = 2 * L * Lq;
+        int n0 = (2 * k + R.phase) * Lq - G.phase * L;  // N of input pixel 0
+        for (int j0 = 0; j0 < Lq; j0 += 64) {
+            float acc[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) acc[i] = 0.0f;
+            const int j1 = min(j0 + 64, Lq);
+#pragma unroll 4
+            for (int j = j0; j < j1; ++j) {
+                int n = n0 - 2 * j * L;  // folded to half a turn
+                n += n < -(full / 2) ? full : 0;
+                n -= n > full / 2 ? full : 0;
+                const float nf = (float)n;
+                const float xh = nf * pi.ch, xl = fmaf(nf, pi.ch, -xh) + nf * pi.cl;
+                int ti;
+                float f;
+                const bool in_cut = chord_to_table_sel(A, B, sin_df(xh, xl), P.nint2, &ti, &f);
+                const float w = in_cut ? hermite(__ldg(&P.d_tab[min(ti, P.n_int)]), f) : 0.0f;
+#pragma unroll
+                for (int a = 0; a < 4; ++a) {
+                    int i = j + a * Qq;
+                    i -= i >= Lq ? Lq : 0;
+                    acc[a] = fmaf(w, __ldg(xn + i), acc[a]);
+                    acc[4 + a] = fmaf(w, __ldg(xs + i), acc[4 + a]);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const float y = acc[i] - comp[i], t = sum[i] + y;
+                comp[i] = (t - sum[i]) - y;
+                sum[i] = t;
+            }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) part[warp][i][lane] = sum[i] - comp[i];
+    __syncthreads();
+    // image `warp` of every position: the warps' sums in order
+    const int a = warp & 3, south = warp >> 2;
+    const int rs = P.nrings - 1 - r, ring = south ? rs : r;
+    if (it.y + lane < Q && ring >= band_lo && ring <= band_hi && !(south && rs == r)) {
+        float s = 0.0f, c = 0.0f;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float y = part[i][warp][lane] - c, t = s + y;
+            c = (t - s) - y;
+            s = t;
+        }
+        float *dst = o + P.d_rings[ring].start + it.y + lane + a * Q;
+        *dst = fmaf(s, P.domega, *dst);
+    }
+}
+
+// ring_range[map][ring] = the largest and the smallest nonzero block maximum (bits) over
+// the 64-pixel blocks that the ring touches; one warp per ring.
+__global__ void __launch_bounds__(256)
+ring_range_kernel(const ConvPlan P, const uint32_t *__restrict__ blockmax, long long block_stride,
+                  uint2 *__restrict__ ring_range) {
+    const uint32_t *bm = blockmax + (long long)blockIdx.y * block_stride;
+    const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (r >= P.nrings) return;
+    const DevRing R = P.d_rings[r];
+    uint32_t mx = 0u, mn = 0xffffffffu;
+    for (int b = (R.start >> 6) + lane; b <= (R.start + R.len - 1) >> 6; b += 32) {
+        const uint32_t v = __ldg(bm + b);
+        mx = max(mx, v);
+        if (v) mn = min(mn, v);
+    }
+    mx = __reduce_max_sync(~0u, mx);
+    mn = __reduce_min_sync(~0u, mn);
+    if (lane == 0) ring_range[(long long)blockIdx.y * P.nrings + r] = make_uint2(mx, mn);
+}
+
+size_t cap_smem(const CapTc &c) {
+    const size_t xc = c.span + c.wpos, w_cap = ((c.wpos / 2 + 8 + 11) & ~31) + 20;
+    const size_t body = 2 * 8 * xc + 8 * (size_t)(kEpi / 32) * kTurn + 16 * 2 * (size_t)c.tcap +
+                        8 * 2 * xc + 4 * 4 * (size_t)coef_words(c.jcap - 1) +
+                        4 * 2 * (kG + kG3) * w_cap + sizeof(QInfo) * (size_t)c.nq;
+    // (the rows past a tile's last position read up to 1024 + wpos elements of a segment)
+    return (size_t)kStages * kStageBytes + std::max(body, (size_t)2 * (6 * xc + kSpan + c.wpos + xc));
+}
+
+// Inverse of a 4 x 4 matrix (Gauss-Jordan with row pivots).
+void invert4(double a[4][4], double inv[4][4]) {
+    for (int i = 0; i < 4; ++i)
+        for (int j = 0; j < 4; ++j) inv[i][j] = i == j;
+    for (int c = 0; c < 4; ++c) {
+        int p = c;
+        for (int i = c + 1; i < 4; ++i)
+            if (std::fabs(a[i][c]) > std::fabs(a[p][c])) p = i;
+        for (int j = 0; j < 4; ++j) {
+            std::swap(a[c][j], a[p][j]);
+            std::swap(inv[c][j], inv[p][j]);
+        }
+        const double d = a[c][c];
+        for (int j = 0; j < 4; ++j) {
+            a[c][j] /= d;
+            inv[c][j] /= d;
+        }
+        for (int i = 0; i < 4; ++i) {
+            if (i == c) continue;
+            const double f = a[i][c];
+            for (int j = 0; j < 4; ++j) {
+                a[i][j] -= f * a[c][j];
+                inv[i][j] -= f * inv[c][j];
+            }
+        }
+    }
+}
+
+} // namespace
+
+int cap_tc_span() { return kSpan; }
+int cap_tc_degree() { return kP - 1; }
+int cap_tc_positions(int w, int L) {
+    const Window v = window_of(w, L);
+    return 16 * (v.s1 - v.s0);
+}
+
+bool cap_tc_fits(const CapTc &c) {
+    return cap_smem(c) <= 226u * 1024 && c.span + c.wpos <= kXr * kBuild;
+}
+
+int cap_tc_words(int jE) { return coef_words(jE); }
+
+cudaError_t launch_cap_coef(const ConvPlan &p, const CapTc &c, const CapCoef &k, cudaStream_t st) {
+    CapCoef kk = k;
+    double a[4][4], inv[4][4];
+    for (int s = 0; s < 4; ++s)
+        for (int i = 0; i < 4; ++i) a[s][i] = std::pow((double)node(s + 1), 2 * (i + 1));
+    invert4(a, inv);
+    for (int i = 0; i < 4; ++i)
+        for (int s = 0; s < 4; ++s) kk.me[4 * i + s] = inv[i][s];
+    for (int s = 0; s < 4; ++s)
+        for (int i = 0; i < 4; ++i) a[s][i] = std::pow((double)node(s + 1), 2 * i + 1);
+    invert4(a, inv);
+    for (int i = 0; i < 4; ++i)
+        for (int s = 0; s < 4; ++s) kk.mo[4 * i + s] = inv[i][s];
+    cap_coef_kernel<<<c.ring_end - c.ring_first + 1, 256, 0, st>>>(p, c, kk, c.ring_first, c.ring_end);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_ring_range(const ConvPlan &p, const unsigned *bm, int n_maps, uint2 *rr,
+                              cudaStream_t st) {
+    dim3 grid((p.nrings + 7) / 8, n_maps);
+    ring_range_kernel<<<grid, 256, 0, st>>>(p, bm, map_blocks(p), rr);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_cap_direct(const ConvPlan &p, const int2 *d_items, int n_items,
+                              const int *d_first, const int *d_list, const float *d_in,
+                              float *d_out, int n_maps, long long map_stride, int band_lo,
+                              int band_hi, const int *flags, cudaStream_t st) {
+    if (n_items <= 0) return cudaSuccess;
+    dim3 grid(n_items, n_maps);
+    cap_direct_kernel<<<grid, 256, 0, st>>>(p, d_items, d_first, d_list, d_in, d_out, map_stride,
+                                            band_lo, band_hi, flags);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_conv_cap_tc(const ConvPlan &p, const CapTc &c, const int2 *d_tiles, int n_tiles,
+                               const float *d_in, float *d_out, int n_maps, long long map_stride,
+                               int belt_split, int band_lo, int band_hi, const uint2 *rr,
+                               int *flags, int *d_err, cudaStream_t st) {
+    if (n_tiles <= 0) return cudaSuccess;
+    const size_t smem = cap_smem(c);
+    cudaError_t e = cudaFuncSetAttribute(conv_cap_tc_kernel,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    dim3 grid(n_tiles, n_maps);
+    conv_cap_tc_kernel<<<grid, kThreads, smem, st>>>(p, c, d_tiles, d_in, d_out, map_stride,
+                                                     belt_split, band_lo, band_hi, rr, flags, d_err);
+    return cudaGetLastError();
+}
+
+} // namespace ksc

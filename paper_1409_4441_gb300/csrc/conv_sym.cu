@@ -618,18 +618,22 @@ __device__ __forceinline__ void sym_dispatch(const ConvPlan &P, int ring, int k0
 // One split; grid.y runs over maps.  CTAs claim items in list order through a
 // counter per map (zero at launch), so the long items of a longest-first list
 // start first and the short ones fill the tail.  (One code path for whole maps
-// and latitude bands keeps their outputs bitwise equal.)
+// and latitude bands keeps their outputs bitwise equal.)  Items from n_first on are
+// taken only where the tensor-core cap kernel has flagged their ring (ring_flags, one
+// word per ring and one for any of them, per map).
 template <class S>
 __global__ void __launch_bounds__(S::T, S::MINB)
 conv_sym_kernel(const ConvPlan P, const WorkItem *__restrict__ items, int n_items,
                 const float *__restrict__ in, float *__restrict__ out, long long map_stride,
-                int belt_split, int band_lo, int band_hi, int *__restrict__ counters,
+                int belt_split, int band_lo, int band_hi, int n_first,
+                const int *__restrict__ ring_flags, int *__restrict__ counters,
                 int *__restrict__ err) {
     __shared__ SymRing sR[kRingChunk];
     __shared__ int sW[4 * (S::T / 32)];  // per-warp walk extents (lockstep path)
     __shared__ __align__(16) float st[kImg * S::kStride];
     __shared__ int s_next;
     extern __shared__ float4 xt[];  // S::kXCap cells
+    const int *rf = ring_flags + (long long)blockIdx.y * (P.nrings + 1);
     const float *m = in + (long long)blockIdx.y * map_stride;
     float *o = out + (long long)blockIdx.y * map_stride;
     for (;;) {
@@ -639,6 +643,10 @@ conv_sym_kernel(const ConvPlan P, const WorkItem *__restrict__ items, int n_item
         const int it = s_next;
         if (it >= n_items) break;
         const WorkItem w = items[it];
+        if (it >= n_first) {
+            if (!rf[P.nrings]) break;
+            if (!rf[w.ring]) continue;
+        }
         sym_dispatch<S>(P, w.ring, w.k0, belt_split, band_lo, band_hi, m, o, sR, st, xt, sW, err);
     }
 }
@@ -702,7 +710,8 @@ cudaError_t sym_grid(K kernel, int threads, size_t dyn_smem, int n_items, int pe
 template <class S>
 cudaError_t sym_launch(const ConvPlan &p, const WorkItem *d_items, int n_items,
                        const float *d_in, float *d_out, int n_maps, long long map_stride,
-                       int belt_split, int band_lo, int band_hi, int *d_err, cudaStream_t st) {
+                       int belt_split, int band_lo, int band_hi, int n_first,
+                       const int *ring_flags, int *d_err, cudaStream_t st) {
     int blocks = 0;
     cudaError_t e = sym_grid(conv_sym_kernel<S>, S::T, S::kDynSmem, n_items, 0, &blocks);
     if (e != cudaSuccess) return e;
@@ -715,7 +724,8 @@ cudaError_t sym_launch(const ConvPlan &p, const WorkItem *d_items, int n_items,
         dim3 grid(blocks, n_maps);
         conv_sym_kernel<S><<<grid, S::T, S::kDynSmem, st>>>(p, d_items, n_items, d_in, d_out,
                                                            map_stride, belt_split, band_lo,
-                                                           band_hi, ctr, d_err);
+                                                           band_hi, n_first, ring_flags, ctr,
+                                                           d_err);
         e = cudaGetLastError();
     }
     const cudaError_t f = cudaFreeAsync(ctr, st);
@@ -735,14 +745,14 @@ int sym_chunk(int nside) { return nside >= 2048 ? ShapeC3::kClasses : ShapeWide:
 
 cudaError_t launch_conv_sym(const ConvPlan &p, const WorkItem *d_items, int n_items,
                             const float *d_in, float *d_out, int n_maps, long long map_stride,
-                            int belt_split, int band_lo, int band_hi, int *d_err,
-                            cudaStream_t st) {
+                            int belt_split, int band_lo, int band_hi, int n_first,
+                            const int *ring_flags, int *d_err, cudaStream_t st) {
     if (n_items <= 0 || n_maps <= 0) return cudaSuccess;
     if (sym_chunk(p.nside) == ShapeC3::kClasses)
         return sym_launch<ShapeC3>(p, d_items, n_items, d_in, d_out, n_maps, map_stride,
-                                   belt_split, band_lo, band_hi, d_err, st);
+                                   belt_split, band_lo, band_hi, n_first, ring_flags, d_err, st);
     return sym_launch<ShapeWide>(p, d_items, n_items, d_in, d_out, n_maps, map_stride,
-                                 belt_split, band_lo, band_hi, d_err, st);
+                                 belt_split, band_lo, band_hi, n_first, ring_flags, d_err, st);
 }
 
 int sym_variants() { return 3; }

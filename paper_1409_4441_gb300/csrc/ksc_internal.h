@@ -145,6 +145,7 @@ struct TableBuild {
     double *d_nodes;    // 2*(n_int+1) scratch: node values, node slopes
     int pad = 0;        // also write entry n_int: the constant-slope extension past d_cut,
                         // so that table position u = n_int needs no index clamp
+    float *d_lo = nullptr;  // n_int values: node value - its FP32 rounding (NULL: not wanted)
 };
 cudaError_t launch_table_build(const TableBuild &tb, cudaStream_t st);
 
@@ -217,6 +218,48 @@ cudaError_t launch_conv_belt_tc(const ConvPlan &p, const BeltTc &t, const float 
                                 const unsigned *bm, unsigned char *flags, int *d_err,
                                 cudaStream_t st);
 
+// Ring pairs with a cap ring on the tensor cores (conv_cap_tc.cu): tiles {rings - 1 << 16 |
+// first ring, sectors << 16 | sector} of rings ring_first .. ring_end and their mirrors.
+struct CapTc {
+    int ring_first = 0, ring_end = -1;  // covered northern rings (none: end < first)
+    int wpos = 0, nq = 0, jcap = 0, tcap = 0;  // most window positions, input rings, cells, outputs
+    int span = 0;                              // most positions of a tile (a multiple of 16)
+    float wscale = 1.0f, wunscale = 1.0f, domega_lo = 0.0f;
+    const int *d_ncut = nullptr;        // per ring pair: largest |N| within the cut, or -1
+    const unsigned *d_coef_off = nullptr;  // per ring pair: its coefficients (units of 4 words)
+    const unsigned *d_coef = nullptr;   // (FP16 h, l) words, [cell][power]
+};
+struct CapCoef {                        // what building the coefficients needs
+    const float4 *d_tab;                // the K_r table run past the cut ...
+    const float *d_tab_lo;              // ... and the rounding errors of its node values
+    const float2 *d_ringc;              // per ring: pi / L as a double-float pair
+    unsigned *d_coef;
+    int n_ext;                          // intervals of d_tab
+    float next2;                        // n_ext^2
+    double me[16], mo[16];              // node values -> even, odd coefficients
+};
+int cap_tc_words(int jE);               // words of a ring pair with edge cell jE
+cudaError_t launch_cap_coef(const ConvPlan &p, const CapTc &c, const CapCoef &k, cudaStream_t st);
+// Adds the irregular ring pairs (list[list_first[r]] .. of output ring r) of rings that are
+// not flagged; items {ring, first of 32 first-quarter positions}.
+cudaError_t launch_cap_direct(const ConvPlan &p, const int2 *d_items, int n_items,
+                              const int *d_first, const int *d_list, const float *d_in,
+                              float *d_out, int n_maps, long long map_stride, int band_lo,
+                              int band_hi, const int *flags, cudaStream_t st);
+int cap_tc_span();                       // input positions of a tile
+int cap_tc_degree();                     // of the cells' polynomials
+int cap_tc_positions(int w, int L);
+bool cap_tc_fits(const CapTc &c);
+cudaError_t launch_ring_range(const ConvPlan &p, const unsigned *bm, int n_maps, uint2 *rr,
+                              cudaStream_t st);
+// Writes (adds, for belt rings with belt_split) the tiles' outputs in rings [band_lo,
+// band_hi] but for the ring pairs it flags (flags[map][ring], flags[map][nrings]: any),
+// which conv_sym_kernel then computes; flags must be zero at launch.
+cudaError_t launch_conv_cap_tc(const ConvPlan &p, const CapTc &c, const int2 *d_tiles, int n_tiles,
+                               const float *d_in, float *d_out, int n_maps, long long map_stride,
+                               int belt_split, int band_lo, int band_hi, const uint2 *rr,
+                               int *flags, int *d_err, cudaStream_t st);
+
 // tcgen05 multi-map kernel for belt ring pairs: items are (belt ring, first
 // pixel) blocks of belt_mma_block() outputs; maps in groups of belt_mma_maps().
 int belt_mma_block();
@@ -235,11 +278,13 @@ cudaError_t launch_conv_belt_mma(const ConvPlan &p, const int2 *d_items, int n_i
 int sym_chunk(int nside);
 int sym_classes(int len, int phase);  // reflection classes of a ring's first quarter
 // CTAs claim items in list order through per-call counters taken from the
-// stream-ordered allocator.
+// stream-ordered allocator.  Items from n_first on are taken only where ring_flags
+// ([map][nrings + 1], the last word: any) says so (n_first = n_items: no flags).
 cudaError_t launch_conv_sym(const ConvPlan &p, const WorkItem *d_items, int n_items,
                             const float *d_in, float *d_out, int n_maps,
                             long long map_stride, int belt_split, int band_lo,
-                            int band_hi, int *d_err, cudaStream_t st);
+                            int band_hi, int n_first, const int *ring_flags, int *d_err,
+                            cudaStream_t st);
 
 // ---------------------------------------------------------------------------
 // Batched persistent launches (csrc/batch.cpp).  An entry is one map convolved
@@ -355,6 +400,16 @@ struct ksc_split {
     size_t ws_floats = 0;
     int *d_err = nullptr;                  // device error flag (bounded waits)
     ksc::BeltTc btc;                       // tensor-core belt stage (n_cols 0: not used)
+    ksc::CapTc ctc;                        // tensor-core cap stage (ring_end < ring_first: not used)
+    int2 *d_cap_tiles = nullptr;           // its tiles in ring order ...
+    int2 *d_cap_tiles_lpt = nullptr;       // ... and longest first (whole map)
+    int n_cap_tiles = 0;
+    std::vector<int> cap_tile_first;       // per ring: first tile of rings >= it (nrings + 1)
+    int *d_ncut = nullptr;
+    unsigned *d_coef_off = nullptr, *d_coef = nullptr;
+    int2 *d_irr_items = nullptr;           // irregular ring pairs: items in ring order,
+    std::vector<int> irr_item_first;       // per ring: first item of rings >= it (nrings + 1),
+    int *d_irr_first = nullptr, *d_irr = nullptr;  // per-ring lists of input rings
     ksc::ConvPlan plan{};
 
     // end-to-end host path (one call at a time per split: host_mu)

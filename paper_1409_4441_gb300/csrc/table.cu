@@ -44,7 +44,7 @@ __global__ void node_values_kernel(const double *__restrict__ c, int lmax, int n
 
 __global__ void hermite_coeff_kernel(const double *__restrict__ nodeK,
                                      const double *__restrict__ nodeD, int n_int, double h,
-                                     int pad, float4 *__restrict__ tab) {
+                                     int pad, float4 *__restrict__ tab, float *__restrict__ lo) {
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (pad && k == n_int) {
         tab[k] = make_float4((float)nodeK[k], (float)(h * nodeD[k]), 0.0f, 0.0f);
@@ -59,6 +59,7 @@ __global__ void hermite_coeff_kernel(const double *__restrict__ nodeK,
     c.z = (float)(3.0 * (y1 - y0) - 2.0 * m0 - m1);
     c.w = (float)(2.0 * (y0 - y1) + m0 + m1);
     tab[k] = c;
+    if (lo) lo[k] = (float)(y0 - (double)c.x);
 }
 
 } // namespace
@@ -69,7 +70,8 @@ cudaError_t launch_table_build(const TableBuild &tb, cudaStream_t st) {
     node_values_kernel<<<(n_nodes + 127) / 128, 128, 0, st>>>(tb.d_c, tb.lmax, n_nodes, tb.h,
                                                              nodeK, nodeD);
     hermite_coeff_kernel<<<(tb.n_int + 1 + 255) / 256, 256, 0, st>>>(nodeK, nodeD, tb.n_int,
-                                                                   tb.h, tb.pad, tb.d_tab);
+                                                                   tb.h, tb.pad, tb.d_tab,
+                                                                   tb.d_lo);
     return cudaGetLastError();
 }
 
