@@ -11,19 +11,24 @@
 // Condon-Shortley phase, from their three-term recurrence in l at fixed m
 // (lambda_mm = sqrt((2m+1)/4pi prod_{k<=m} (2k-1)/2k) sin^m theta; lambda_{m+1,m}
 // = sqrt(2m+3) z lambda_mm; lambda_lm = A_l (z lambda_{l-1,m} - lambda_{l-2,m} /
-// A_{l-1}), A_l = sqrt((4l^2-1)/(l^2-m^2))), in FP64 with a scale exponent:
-// near the poles sin^m theta underflows any floating format, so values are
-// carried as v 2^(600 e) and summed only once e reaches 0 (while e < 0 the true
-// value is below 2^-300).  North and south rings share |z| (lambda_lm(-z) =
-// (-1)^(l+m) lambda_lm(z)), so each recurrence serves a ring pair through its
-// even and odd partial sums.
+// A_{l-1}), A_l = sqrt((4l^2-1)/(l^2-m^2))).  The recurrence and the sums over l and over
+// rings run on FP32 pairs (hi + lo, 48 bits): the FP64 units of a GB300 do 1/64 of its FP32
+// operations, and FP64 recurrences took 100 of the 154 ms of both transforms at nside 2048,
+// l_cut 1024.  After a few thousand steps a pair is still within 1e-10, far inside the FP32
+// that the ring sums keep.  Near the poles sin^m theta underflows any floating format, so
+// values are carried as v 2^(120 e) and summed only once e reaches 0 (while e < 0 the
+// true value is below 2^-60).  North and south rings share |z| (lambda_lm(-z) = (-1)^(l+m)
+// lambda_lm(z)), so each recurrence serves a ring pair through its even and odd partial
+// sums.  Orders beyond l sin theta + 16 + 9 l^(1/3) stay below 2^-60 for every l <= l_max (the
+// functions decay exponentially past their turning point): a ring leaves them out.
 //
-// The ring sums over m (synthesis) and over pixels (analysis) are direct sums in
-// FP32 restricted to m <= l_max: pixel k of a ring of L pixels with phase flag t
-// sits at phi_k = pi (2k + t) / L, so m phi_k = pi J / L with the exact integer
-// J = m (2k + t) mod 2L; the twiddles advance by one complex product per step
-// and are re-anchored from the exact J every 8 steps (the products' rounding
-// drifts by about one FP32 ulp per step in between).
+// Ring sums: pixel k of a ring of L pixels with phase flag t sits at phi_k = pi (2k + t) / L.
+// Belt rings (L = 4 nside, a power of two) go through an FP32 FFT in shared memory, north
+// and mirror ring as one complex sequence.  Cap rings (L = 4i) are summed directly over a
+// quarter: the quarter turns of pixel k1 enter order m through m mod 4 alone.  m phi_k =
+// pi J / L with the exact integer J = m (2k + t) mod 2L; the twiddles advance by one complex
+// product per step and are re-anchored from the exact J every 8 steps (the products'
+// rounding drifts by about one FP32 ulp per step in between).
 #include <cstdint>
 
 #include "ksc_internal.h"
@@ -33,7 +38,7 @@ namespace {
 
 constexpr double kPi = 3.14159265358979323846;
 constexpr int kAnchor = 8;        // twiddle steps between exact re-anchors
-constexpr double kScale = 600.0;  // log2 of one scale step of the recurrence
+constexpr double kScale = 120.0;  // log2 of one scale step of the recurrence
 
 __host__ __device__ inline long long n_alm(int lmax) {
     return (long long)(lmax + 1) * (lmax + 2) / 2;
@@ -80,289 +85,649 @@ __device__ inline ShtRing sht_ring(int n, int r) {
     return g;
 }
 
-// Start of the recurrence at l = m: lambda_mm = v 2^(600 e), v in [2^-300, 2^300).
-__device__ inline void lambda_mm(int m, double s, double *v, int *e) {
-    // log2 lambda_mm = 1/2 log2((2m+1)/4pi) + 1/2 log2((2m)! / (4^m m!^2)) + m log2 s
-    const double lg = 0.5 * log2((2.0 * m + 1.0) / (4.0 * kPi)) +
-                      0.5 * (lgamma(2.0 * m + 1.0) - 2.0 * lgamma(m + 1.0)) / log(2.0) - m +
-                      (m > 0 ? m * log2(s) : 0.0);
-    int ee = (int)floor((lg + 300.0) / kScale);
-    if (ee > 0) ee = 0;
-    *e = ee;
-    *v = exp2(lg - kScale * ee);
+// ---- FP32 pairs (hi + lo) -----------------------------------------------------
+struct F2 {
+    float h, l;
+};
+__device__ __forceinline__ F2 f2_of(double v) {
+    F2 r;
+    r.h = (float)v;
+    r.l = (float)(v - (double)r.h);
+    return r;
+}
+__device__ __forceinline__ F2 f2_norm(float h, float l) {
+    F2 r;
+    r.h = h + l;
+    r.l = l - (r.h - h);
+    return r;
+}
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {  // not normalised: |l| a few ulps of h
+    F2 r;
+    r.h = a.h * b.h;
+    r.l = fmaf(a.l, b.h, fmaf(a.h, b.l, fmaf(a.h, b.h, -r.h)));
+    return r;
+}
+__device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
+    const float s = a.h + b.h, t = s - a.h;
+    return f2_norm(s, ((a.h - (s - t)) + (b.h - t)) + (a.l + b.l));
 }
 
-// The recurrence coefficients of order m in shared memory: A[l] (l = m+1..lmax)
-// and B[l] = 1 / A[l-1] (l = m+2..lmax).
-__device__ inline void build_coeffs(int m, int lmax, double *A, double *B) {
-    for (int l = m + 1 + threadIdx.x; l <= lmax; l += blockDim.x) {
-        const double ll = (double)l, mm = (double)m;
-        A[l] = sqrt((4.0 * ll * ll - 1.0) / ((ll - mm) * (ll + mm)));
-        if (l >= m + 2) {
-            const double l1 = ll - 1.0;
-            B[l] = sqrt((l1 - mm) * (l1 + mm) / (4.0 * l1 * l1 - 1.0));
-        }
-    }
+// Orders above this do not reach 2^-60 on a ring (see the top of the file).
+__device__ __forceinline__ int order_limit(int lmax, double s) {
+    const float lim = (float)lmax * (float)s + 16.0f + 9.0f * cbrtf((float)lmax);
+    return min(lmax, (int)lim);
 }
 
-// Synthesis, Legendre part: G[ring][m] = sum_l a_lm lambda_lm(z_ring) for every
-// northern ring (and its southern mirror) of the block's range and order m =
-// blockIdx.y.  One thread per northern ring.
-__global__ void __launch_bounds__(128)
-sht_leg_synth(int nside, int lmax, const double2 *__restrict__ alm, float2 *__restrict__ G) {
-    extern __shared__ double coef[];
-    const int m = blockIdx.y;
-    double *A = coef, *B = coef + (lmax + 1);
-    build_coeffs(m, lmax, A, B);
-    __syncthreads();
-    const int nnorth = 2 * nside, nr = 4 * nside - 1;
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= nnorth) return;
-    const ShtRing g = sht_ring(nside, r);
-    const double2 *a = alm + alm_base(lmax, m);
-    double v2 = 0.0, v1;
+// log2 lambda_mm - m log2 sin(theta)
+__device__ inline double log2_norm(int m) {
+    return 0.5 * log2((2.0 * m + 1.0) / (4.0 * kPi)) +
+           0.5 * (lgamma(2.0 * m + 1.0) - 2.0 * lgamma(m + 1.0)) / log(2.0) - m;
+}
+
+// The recurrence of one (ring, order): v1 = lambda_{l}, v2 = lambda_{l-1}, both 2^(120 e)
+// times the true values.
+struct Rec {
+    F2 z, v1, v2;
     int e;
-    lambda_mm(m, g.s, &v1, &e);
-    double er = 0.0, ei = 0.0, orr = 0.0, oi = 0.0;  // even / odd (l - m) sums
-    if (e == 0) {
-        const double2 c = __ldg(a + m);
-        er = v1 * c.x;
-        ei = v1 * c.y;
+    __device__ __forceinline__ void start(int m, double lg0, const ShtRing &g) {
+        z = f2_of(g.z);
+        const double lg = lg0 + (m > 0 ? m * log2(g.s) : 0.0);
+        e = min(0, (int)floor((lg + 60.0) / kScale));
+        v1 = f2_of(exp2(lg - kScale * e));
+        v2 = F2{0.0f, 0.0f};
     }
-    const double z = g.z;
-    for (int l = m + 1; l <= lmax; ++l) {
-        const double v = A[l] * (z * v1 - (l >= m + 2 ? B[l] * v2 : 0.0));
+    // lambda_{l+1} = A (z lambda_l - B lambda_{l-1}), c = A as a pair, B as a pair
+    __device__ __forceinline__ void step(float4 c) {
+        const F2 x = f2_mul(z, v1), y = f2_mul(F2{c.z, c.w}, v2);
+        const float d = x.h - y.h, t = d - x.h;
+        const F2 w = f2_norm(d, ((x.h - (d - t)) - (y.h + t)) + (x.l - y.l));
+        const F2 r = f2_mul(F2{c.x, c.y}, w);
         v2 = v1;
-        v1 = v;
-        if (e < 0) {
-            if (fabs(v1) >= 0x1p300) {  // one scale step up
-                v1 *= 0x1p-600;
-                v2 *= 0x1p-600;
-                ++e;
-            }
-            if (e < 0) continue;
+        v1 = f2_norm(r.h, r.l);
+        if (e < 0 && fabsf(v1.h) >= 0x1p60f) {
+            const float q = 0x1p-120f;
+            v1.h *= q; v1.l *= q; v2.h *= q; v2.l *= q;
+            ++e;
         }
-        const double2 c = __ldg(a + l);
-        if ((l - m) & 1) {
-            orr = fma(v1, c.x, orr);
-            oi = fma(v1, c.y, oi);
-        } else {
-            er = fma(v1, c.x, er);
-            ei = fma(v1, c.y, ei);
+    }
+};
+
+constexpr int kTile = 128;  // degrees whose coefficients a block stages at a time
+
+// Coefficients of the step to degree l (l > m): A_l and B_l = 1 / A_{l-1} (0 at l = m + 1).
+__device__ inline float4 step_coeffs(int l, int m) {
+    const double ll = (double)l, mm = (double)m, l1 = ll - 1.0;
+    const F2 a = f2_of(sqrt((4.0 * ll * ll - 1.0) / ((ll - mm) * (ll + mm))));
+    const F2 b = l > m + 1 ? f2_of(sqrt((l1 - mm) * (l1 + mm) / (4.0 * l1 * l1 - 1.0))) : F2{0.0f, 0.0f};
+    return make_float4(a.h, a.l, b.h, b.l);
+}
+
+// Synthesis, Legendre part: G[ring][m] = sum_l a_lm lambda_lm(z_ring) for the northern rings
+// (and their southern mirrors) of the block's range and order m = blockIdx.y, R rings a
+// thread.  Orders past a ring's limit are not written (nor read).
+template <int R>
+__global__ void __launch_bounds__(256)
+sht_leg_synth(int nside, int lmax, const double2 *__restrict__ alm, float2 *__restrict__ G) {
+    __shared__ float4 co[kTile], al[kTile];
+    __shared__ double s_lg;
+    const int m = blockIdx.y, nnorth = 2 * nside, nr = 4 * nside - 1;
+    const int r0 = blockIdx.x * 256 * R + threadIdx.x;
+    if (threadIdx.x == 0) s_lg = log2_norm(m);
+    __syncthreads();
+    Rec rec[R];
+    F2 er[R], ei[R], od[R], oi[R];  // even / odd (l - m) sums
+    bool live[R], any = false;
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+        const int r = r0 + 256 * j;
+        er[j] = ei[j] = od[j] = oi[j] = F2{0.0f, 0.0f};
+        live[j] = false;
+        if (r < nnorth) {
+            const ShtRing g = sht_ring(nside, r);
+            live[j] = m <= order_limit(lmax, g.s);
+            if (live[j]) rec[j].start(m, s_lg, g);
+        }
+        any |= live[j];
+    }
+    if (!__syncthreads_or(any)) return;
+    const bool warp_any = __any_sync(~0u, any);
+    const double2 *a = alm + alm_base(lmax, m);
+    for (int l0 = m; l0 <= lmax; l0 += kTile) {
+        const int n = min(kTile, lmax + 1 - l0);
+        __syncthreads();
+        for (int i = threadIdx.x; i < n; i += 256) {
+            if (l0 + i > m) co[i] = step_coeffs(l0 + i, m);
+            const double2 c = __ldg(a + l0 + i);
+            const F2 x = f2_of(c.x), y = f2_of(c.y);
+            al[i] = make_float4(x.h, x.l, y.h, y.l);
+        }
+        __syncthreads();
+        if (!warp_any) continue;
+        for (int i = 0; i < n; ++i) {
+            const float4 c = co[i], x = al[i];
+            const bool odd = (l0 + i - m) & 1;
+#pragma unroll
+            for (int j = 0; j < R; ++j) {
+                if (!live[j]) continue;
+                if (l0 + i > m) rec[j].step(c);
+                if (rec[j].e < 0) continue;
+                const F2 pr = f2_mul(rec[j].v1, F2{x.x, x.y}), pi = f2_mul(rec[j].v1, F2{x.z, x.w});
+                if (odd) {
+                    od[j] = f2_add(od[j], pr);
+                    oi[j] = f2_add(oi[j], pi);
+                } else {
+                    er[j] = f2_add(er[j], pr);
+                    ei[j] = f2_add(ei[j], pi);
+                }
+            }
         }
     }
     const long long stride = lmax + 1;
-    G[(long long)r * stride + m] = make_float2((float)(er + orr), (float)(ei + oi));
-    const int rs = nr - 1 - r;
-    if (rs != r) G[(long long)rs * stride + m] = make_float2((float)(er - orr), (float)(ei - oi));
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+        const int r = r0 + 256 * j, rs = nr - 1 - r;
+        if (!live[j]) continue;
+        const F2 a0 = f2_add(er[j], od[j]), a1 = f2_add(ei[j], oi[j]);
+        G[(long long)r * stride + m] = make_float2(a0.h, a1.h);
+        if (rs == r) continue;
+        od[j].h = -od[j].h; od[j].l = -od[j].l;
+        oi[j].h = -oi[j].h; oi[j].l = -oi[j].l;
+        const F2 b0 = f2_add(er[j], od[j]), b1 = f2_add(ei[j], oi[j]);
+        G[(long long)rs * stride + m] = make_float2(b0.h, b1.h);
+    }
 }
 
-// e^{i pi J / L} for the exact integer J = a b mod 2L (a, b >= 0), to about one
-// FP32 ulp: J / L = hi + lo with hi the rounded quotient and lo = (J - hi L) / L
-// (the remainder exact by the fused multiply-add), J folded into [-L, L); the
-// rounding of hi is undone to first order, e^{i pi lo} = 1 + i pi lo.
-__device__ inline float2 twiddle(long long a, long long b, int L) {
-    long long J = (a % (2LL * L)) * (b % (2LL * L)) % (2LL * L);
-    if (J >= L) J -= 2LL * L;
-    const float fj = (float)J, fl = (float)L;  // exact: |J|, L <= 2^15
-    const float hi = fj / fl;
-    const float lo = fmaf(-hi, fl, fj) / fl;
+// Analysis, Legendre part: alm[l, m] = c K_l sum_rings lambda_lm(z) F_m over all northern
+// rings and their mirrors for order m = lmax - blockIdx.x; c = 4 pi / Npix, K_l = kl[l] (kl
+// NULL: 1).  One block per order, R rings a thread, in passes over the rings.  The
+// threads' terms of eight degrees go through shared memory: within a warp 32 -> 4 partial
+// sums a degree, then over the warps, in a fixed order and on FP32 pairs throughout.  The
+// F_m enter divided by the power of two that covers the number of rings (exact; c carries it
+// back), so that a sum over all rings stays in range wherever the F_m do.
+template <int R>
+__global__ void __launch_bounds__(256)
+sht_leg_anal(int nside, int lmax, const float2 *__restrict__ F, const double *__restrict__ kl,
+             double scale, double c, double2 *__restrict__ alm) {
+    extern __shared__ float4 acc[];  // [lmax + 1 - m]: re, im pairs
+    __shared__ float4 co[kTile], term[8][8][33], part[8][8];
+    __shared__ double s_lg;
+    const int m = lmax - blockIdx.x, nnorth = 2 * nside, nr = 4 * nside - 1;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const long long stride = lmax + 1;
+    for (int i = threadIdx.x; i <= lmax - m; i += 256) acc[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (threadIdx.x == 0) s_lg = log2_norm(m);
+    __syncthreads();
+    for (int base = 0; base < nnorth; base += 256 * R) {
+        Rec rec[R];
+        F2 sr[R], si[R], dr[R], di[R];  // F north + south (even l - m), north - south (odd)
+        bool live[R], any = false;
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+            const int r = base + 256 * j + threadIdx.x;
+            live[j] = false;
+            if (r < nnorth) {
+                const ShtRing g = sht_ring(nside, r);
+                live[j] = m <= order_limit(lmax, g.s);
+                if (live[j]) {
+                    rec[j].start(m, s_lg, g);
+                    const int rs = nr - 1 - r;
+                    const float2 fn = F[(long long)r * stride + m];
+                    const float2 fs = rs != r ? F[(long long)rs * stride + m] : make_float2(0.0f, 0.0f);
+                    sr[j] = f2_of(scale * ((double)fn.x + (double)fs.x));
+                    si[j] = f2_of(scale * ((double)fn.y + (double)fs.y));
+                    dr[j] = f2_of(scale * ((double)fn.x - (double)fs.x));
+                    di[j] = f2_of(scale * ((double)fn.y - (double)fs.y));
+                }
+            }
+            any |= live[j];
+        }
+        if (!__syncthreads_or(any)) continue;
+        const bool warp_any = __any_sync(~0u, any);
+        for (int l0 = m; l0 <= lmax; l0 += kTile) {
+            const int n = min(kTile, lmax + 1 - l0);
+            __syncthreads();
+            for (int i = threadIdx.x; i < n; i += 256)
+                if (l0 + i > m) co[i] = step_coeffs(l0 + i, m);
+            __syncthreads();
+            for (int i0 = 0; i0 < n; i0 += 8) {
+                if (warp_any) {
+#pragma unroll 2
+                    for (int i = 0; i < 8; ++i) {
+                        F2 tr{0.0f, 0.0f}, ti{0.0f, 0.0f};
+                        if (i0 + i < n) {
+                            const float4 cc = co[i0 + i];
+                            const bool odd = (l0 + i0 + i - m) & 1;
+#pragma unroll
+                            for (int j = 0; j < R; ++j) {
+                                if (!live[j]) continue;
+                                if (l0 + i0 + i > m) rec[j].step(cc);
+                                if (rec[j].e < 0) continue;
+                                tr = f2_add(tr, f2_mul(rec[j].v1, odd ? dr[j] : sr[j]));
+                                ti = f2_add(ti, f2_mul(rec[j].v1, odd ? di[j] : si[j]));
+                            }
+                        }
+                        term[warp][i][lane] = make_float4(tr.h, tr.l, ti.h, ti.l);
+                    }
+                    __syncwarp();
+                    // lane: degree lane / 4, the eight terms from 8 (lane % 4)
+                    F2 tr{0.0f, 0.0f}, ti{0.0f, 0.0f};
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const float4 t = term[warp][lane >> 2][8 * (lane & 3) + k];
+                        tr = f2_add(tr, F2{t.x, t.y});
+                        ti = f2_add(ti, F2{t.z, t.w});
+                    }
+#pragma unroll
+                    for (int o = 1; o < 4; o <<= 1) {
+                        F2 x, y;
+                        x.h = __shfl_xor_sync(~0u, tr.h, o);
+                        x.l = __shfl_xor_sync(~0u, tr.l, o);
+                        y.h = __shfl_xor_sync(~0u, ti.h, o);
+                        y.l = __shfl_xor_sync(~0u, ti.l, o);
+                        tr = f2_add(tr, x);
+                        ti = f2_add(ti, y);
+                    }
+                    if ((lane & 3) == 0) part[warp][lane >> 2] = make_float4(tr.h, tr.l, ti.h, ti.l);
+                } else if (lane < 8) {
+                    part[warp][lane] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                }
+                __syncthreads();
+                if (threadIdx.x < 8 && i0 + (int)threadIdx.x < n) {
+                    const float4 o = acc[l0 - m + i0 + threadIdx.x];
+                    F2 tr{o.x, o.y}, ti{o.z, o.w};
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const float4 t = part[k][threadIdx.x];
+                        tr = f2_add(tr, F2{t.x, t.y});
+                        ti = f2_add(ti, F2{t.z, t.w});
+                    }
+                    acc[l0 - m + i0 + threadIdx.x] = make_float4(tr.h, tr.l, ti.h, ti.l);
+                }
+                __syncthreads();
+            }
+        }
+    }
+    __syncthreads();
+    double2 *a = alm + alm_base(lmax, m);
+    for (int l = m + threadIdx.x; l <= lmax; l += 256) {
+        const float4 t = acc[l - m];
+        const double w = c * (kl ? kl[l] : 1.0);
+        a[l] = make_double2(w * ((double)t.x + (double)t.y), w * ((double)t.z + (double)t.w));
+    }
+}
+
+// ---- ring sums ----------------------------------------------------------------
+__device__ __forceinline__ float2 cmul(float2 a, float2 b) {
+    return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
+}
+
+// e^{i pi J / L} for an exact integer 0 <= J < 2L, to about one FP32 ulp: J / L = hi + lo with
+// hi the rounded quotient and lo = (J - hi L) / L (the remainder exact by the fused
+// multiply-add), J folded into [-L, L); the rounding of hi is undone to first order,
+// e^{i pi lo} = 1 + i pi lo.
+__device__ __forceinline__ float2 twiddle(int J, float L, float inv_l) {
+    const float fj = (float)(J >= (int)L ? J - 2 * (int)L : J);  // exact: |J|, L <= 2^15
+    const float hi = fj * inv_l;
+    const float lo = fmaf(-hi, L, fj) * inv_l;
     float sn, cs;
     sincospif(hi, &sn, &cs);
     const float d = 3.14159265f * lo;
     return make_float2(fmaf(-sn, d, cs), fmaf(cs, d, sn));
 }
 
-__device__ inline float2 cmul(float2 a, float2 b) {
-    return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
+__device__ __forceinline__ void fold(float &sum, float &comp, float v) {  // Kahan
+    const float y = v - comp, t = sum + y;
+    comp = (t - sum) - y;
+    sum = t;
 }
 
-// Synthesis, ring part: for northern ring r = blockIdx.x and its mirror, pixel k
-// gets sum_m w_m Re(G_m e^{i m phi_k}) (w_0 = 1, else 2); add != 0 adds it to
-// the map.  G of both rings staged in shared memory (pre-weighted).
+// Synthesis, ring part, any ring length 4 Q: for northern ring r and its mirror,
+// pixel k1 + a Q (a = 0..3) gets sum_m w_m Re(G_m e^{i m phi}) = Re sum_c i^{a c} S_c(k1), S_c
+// the sum over the orders m = c mod 4 at pixel k1 (w_0 = 1, else 2).  add != 0 adds it to the
+// map.  The orders are staged in shared memory 1024 at a time.
+constexpr int kOrders = 1024;
 __global__ void __launch_bounds__(256)
-sht_dft_synth(int nside, int lmax, const float2 *__restrict__ G, float *__restrict__ map,
-              int add) {
-    extern __shared__ float2 gs[];  // [2][lmax + 1]
-    const int r = blockIdx.x, nr = 4 * nside - 1, rs = nr - 1 - r;
+sht_ring_synth(int nside, int lmax, int r_first, const float2 *__restrict__ G,
+               float *__restrict__ map, int add) {
+    __shared__ float4 gs[kOrders];  // north, south
+    // the longest rings first
+    const int r = r_first + gridDim.x - 1 - blockIdx.x, nr = 4 * nside - 1, rs = nr - 1 - r;
     const bool mirror = rs != r;
     const long long stride = lmax + 1;
-    for (int m = threadIdx.x; m <= lmax; m += blockDim.x) {
-        const float w = m == 0 ? 1.0f : 2.0f;
-        const float2 a = G[(long long)r * stride + m];
-        gs[m] = make_float2(w * a.x, w * a.y);
-        const float2 b = mirror ? G[(long long)rs * stride + m] : make_float2(0.0f, 0.0f);
-        gs[stride + m] = make_float2(w * b.x, w * b.y);
-    }
-    __syncthreads();
-    const ShtRing g = sht_ring(nside, r);
-    const int L = g.len;
-    const ShtRing h = sht_ring(nside, rs);
-    for (int k = threadIdx.x; k < L; k += blockDim.x) {
-        const long long q = 2LL * k + g.t;  // m phi_k = pi m q / L
-        const float2 step = twiddle(1, q, L);
-        float sn = 0.0f, cn = 0.0f, ss = 0.0f, cc = 0.0f;  // sums and compensations
-        for (int m0 = 0; m0 <= lmax; m0 += kAnchor) {
-            float2 w = twiddle(m0, q, L);
-            float pn = 0.0f, ps = 0.0f;
-            const int m1 = min(m0 + kAnchor, lmax + 1);
-            for (int m = m0; m < m1; ++m) {
-                const float2 a = gs[m], b = gs[stride + m];
-                pn = fmaf(a.x, w.x, fmaf(-a.y, w.y, pn));
-                ps = fmaf(b.x, w.x, fmaf(-b.y, w.y, ps));
-                w = cmul(w, step);
+    const ShtRing g = sht_ring(nside, r), h = sht_ring(nside, rs);
+    const int L = g.len, Q = L / 4, lim = order_limit(lmax, g.s);
+    const float fl = (float)L, inv_l = 1.0f / fl;
+    for (int k0 = blockIdx.y * 256; k0 < Q; k0 += gridDim.y * 256) {
+        const int k = k0 + threadIdx.x;
+        const int q = 2 * min(k, Q - 1) + g.t;  // m phi = pi m q / L
+        const float2 step = twiddle(q, fl, inv_l);
+        const int j8 = (kAnchor * q) % (2 * L);
+        float sum[4][4], comp[4][4];  // [class][north re, im, south re, im]
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) sum[c][i] = comp[c][i] = 0.0f;
+        int J = 0;
+        for (int m0 = 0; m0 <= lim; m0 += kOrders) {
+            const int n = min(kOrders, lim + 1 - m0), n8 = (n + 7) & ~7;
+            __syncthreads();
+            for (int i = threadIdx.x; i < n8; i += 256) {
+                const float w = m0 + i == 0 ? 1.0f : 2.0f;
+                const float2 zero = make_float2(0.0f, 0.0f);
+                const float2 a = i < n ? G[(long long)r * stride + m0 + i] : zero;
+                const float2 b = i < n && mirror ? G[(long long)rs * stride + m0 + i] : zero;
+                gs[i] = make_float4(w * a.x, w * a.y, w * b.x, w * b.y);
             }
-            // compensated accumulation of the chunk partials
-            float y = pn - cn, t2 = sn + y;
-            cn = (t2 - sn) - y;
-            sn = t2;
-            y = ps - cc;
-            t2 = ss + y;
-            cc = (t2 - ss) - y;
-            ss = t2;
-        }
-        float *on = map + g.start + k;
-        if (add) *on += sn; else *on = sn;
-        if (mirror) {
-            float *os = map + h.start + k;
-            if (add) *os += ss; else *os = ss;
-        }
-    }
-}
-
-constexpr int kAnalChunk = 4096;  // pixels of each ring staged per pass
-
-// Analysis, ring part: F[ring][m] = sum_k m_k e^{-i m phi_k} for northern ring r =
-// blockIdx.x and its mirror, every m <= lmax (threads over m).  Pixels staged in
-// shared memory in chunks; FP32 partials over 64 pixels summed in FP64.
-__global__ void __launch_bounds__(256)
-sht_dft_anal(int nside, int lmax, const float *__restrict__ map, float2 *__restrict__ F) {
-    __shared__ float2 px[kAnalChunk];  // (north, south) pixel values
-    const int r = blockIdx.x, nr = 4 * nside - 1, rs = nr - 1 - r;
-    const bool mirror = rs != r;
-    const ShtRing g = sht_ring(nside, r);
-    const ShtRing h = sht_ring(nside, rs);
-    const int L = g.len;
-    const long long stride = lmax + 1;
-    const int per = (lmax + blockDim.x) / blockDim.x;  // orders per thread
-    for (int j = 0; j < per; ++j) {
-        const int m = threadIdx.x + j * blockDim.x;
-        const bool live = m <= lmax;
-        // step e^{-i m 2 pi / L}; the pixels of the chunk are k0 .. k0 + n - 1
-        const float2 st = live ? twiddle(m, 2, L) : make_float2(1.0f, 0.0f);
-        const float2 step = make_float2(st.x, -st.y);
-        double fnr = 0.0, fni = 0.0, fsr = 0.0, fsi = 0.0;
-        for (int k0 = 0; k0 < L; k0 += kAnalChunk) {
-            const int n = min(kAnalChunk, L - k0);
             __syncthreads();
-            for (int k = threadIdx.x; k < n; k += blockDim.x)
-                px[k] = make_float2(map[g.start + k0 + k], mirror ? map[h.start + k0 + k] : 0.0f);
-            __syncthreads();
-            if (!live) continue;
-            for (int b0 = 0; b0 < n; b0 += 64) {
-                float pnr = 0.0f, pni = 0.0f, psr = 0.0f, psi = 0.0f;
-                const int b1 = min(b0 + 64, n);
-                for (int a0 = b0; a0 < b1; a0 += kAnchor) {
-                    const float2 c = twiddle(m, 2LL * (k0 + a0) + g.t, L);
-                    float2 w = make_float2(c.x, -c.y);  // e^{-i m phi_k}
-                    const int a1 = min(a0 + kAnchor, b1);
-                    for (int k = a0; k < a1; ++k) {
-                        const float2 v = px[k];
-                        pnr = fmaf(v.x, w.x, pnr);
-                        pni = fmaf(v.x, w.y, pni);
-                        psr = fmaf(v.y, w.x, psr);
-                        psi = fmaf(v.y, w.y, psi);
+            for (int i = 0; i < n8; i += 2 * kAnchor) {
+                float p[4][4];
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) p[c][e] = 0.0f;
+#pragma unroll
+                for (int half = 0; half < 2; ++half) {
+                    if (i + half * kAnchor >= n8) break;
+                    float2 w = twiddle(J, fl, inv_l);
+                    J += j8;
+                    J -= J >= 2 * L ? 2 * L : 0;
+#pragma unroll
+                    for (int e = 0; e < kAnchor; ++e) {
+                        const float4 a = gs[i + half * kAnchor + e];
+                        float (&c)[4] = p[e & 3];
+                        c[0] = fmaf(a.x, w.x, fmaf(-a.y, w.y, c[0]));
+                        c[1] = fmaf(a.x, w.y, fmaf(a.y, w.x, c[1]));
+                        c[2] = fmaf(a.z, w.x, fmaf(-a.w, w.y, c[2]));
+                        c[3] = fmaf(a.z, w.y, fmaf(a.w, w.x, c[3]));
                         w = cmul(w, step);
                     }
                 }
-                fnr += pnr;
-                fni += pni;
-                fsr += psr;
-                fsi += psi;
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) fold(sum[c][e], comp[c][e], p[c][e]);
             }
         }
-        if (live) {
-            F[(long long)r * stride + m] = make_float2((float)fnr, (float)fni);
-            if (mirror) F[(long long)rs * stride + m] = make_float2((float)fsr, (float)fsi);
+        if (k >= Q) continue;
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            if (s && !mirror) break;
+            const float r0 = sum[0][2 * s], r1 = sum[1][2 * s], i1 = sum[1][2 * s + 1];
+            const float r2 = sum[2][2 * s], r3 = sum[3][2 * s], i3 = sum[3][2 * s + 1];
+            // Re sum_c i^{a c} S_c
+            const float v[4] = {(r0 + r2) + (r1 + r3), (r0 - r2) + (i3 - i1), (r0 + r2) - (r1 + r3),
+                                (r0 - r2) - (i3 - i1)};
+            float *o = map + (s ? h.start : g.start) + k;
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                if (add) o[a * Q] += v[a];
+                else o[a * Q] = v[a];
+            }
         }
     }
 }
 
-// Analysis, Legendre part: alm[l, m] += c K_l sum_rings lambda_lm(z) F_m for the
-// northern rings of the block's range (one per thread, with their mirrors) and
-// order m = blockIdx.y; c = 4 pi / Npix, K_l = kl[l] (kl NULL: 1).  Each warp
-// sums its 32 rings by shuffles, lane 0 adds to alm (zeroed by the caller).
-__global__ void __launch_bounds__(128)
-sht_leg_anal(int nside, int lmax, const float2 *__restrict__ F, const double *__restrict__ kl,
-             double c, double2 *__restrict__ alm) {
-    extern __shared__ double coef[];
-    const int m = blockIdx.y;
-    double *A = coef, *B = coef + (lmax + 1);
-    build_coeffs(m, lmax, A, B);
-    __syncthreads();
-    const int nnorth = 2 * nside, nr = 4 * nside - 1;
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool live = r < nnorth;
-    const int lane = threadIdx.x & 31;
+// Analysis, ring part, any ring length 4 Q: F[ring][m] = sum_k m_k e^{-i m phi_k} for
+// northern ring r and its mirror, threads over m <= the ring's limit.  The quarter turns of
+// pixel k1 enter order m as Y_c(k1) = sum_a (-i)^{a c} m_{k1 + a Q}, c = m mod 4; staged in
+// shared memory 512 pixels at a time (classes 0 and 2 are real, 3 is conjugate to 1).
+constexpr int kPix = 512;
+__global__ void __launch_bounds__(256)
+sht_ring_anal(int nside, int lmax, int r_first, const float *__restrict__ map,
+              float2 *__restrict__ F) {
+    __shared__ float4 y[4][kPix + 1];  // [class]: north re, im, south re, im
+    // the longest rings first
+    const int r = r_first + gridDim.x - 1 - blockIdx.x, nr = 4 * nside - 1, rs = nr - 1 - r;
+    const bool mirror = rs != r;
     const long long stride = lmax + 1;
-    double sr = 0.0, si = 0.0, dr = 0.0, di = 0.0, z = 0.0, v1 = 0.0, v2 = 0.0;
-    int e = -1;
-    if (live) {
-        const ShtRing g = sht_ring(nside, r);
-        z = g.z;
-        const int rs = nr - 1 - r;
-        const float2 fn = F[(long long)r * stride + m];
-        const float2 fs = rs != r ? F[(long long)rs * stride + m] : make_float2(0.0f, 0.0f);
-        sr = (double)fn.x + fs.x;  // even l - m: lambda(z) = lambda(-z)
-        si = (double)fn.y + fs.y;
-        dr = (double)fn.x - fs.x;  // odd l - m
-        di = (double)fn.y - fs.y;
-        lambda_mm(m, g.s, &v1, &e);
-    }
-    double2 *a = alm + alm_base(lmax, m);
-    for (int l = m; l <= lmax; ++l) {
-        if (l > m) {
-            const double v = A[l] * (z * v1 - (l >= m + 2 ? B[l] * v2 : 0.0));
-            v2 = v1;
-            v1 = v;
-            if (e < 0 && fabs(v1) >= 0x1p300) {
-                v1 *= 0x1p-600;
-                v2 *= 0x1p-600;
-                ++e;
+    const ShtRing g = sht_ring(nside, r), h = sht_ring(nside, rs);
+    const int L = g.len, Q = L / 4, lim = order_limit(lmax, g.s);
+    const float fl = (float)L, inv_l = 1.0f / fl;
+    for (int m0 = blockIdx.y * 256; m0 <= lim; m0 += gridDim.y * 256) {
+        const int m = m0 + threadIdx.x, c = m & 3, mr = m % (2 * L);
+        // e^{-i m phi_k}: J = -m (2k + t) mod 2L
+        const int j1 = (2 * L - 2 * mr % (2 * L)) % (2 * L);
+        const float2 step = twiddle(j1, fl, inv_l);
+        const int j8 = (int)((8LL * j1) % (2 * L));
+        int J = g.t ? (2 * L - mr) % (2 * L) : 0;
+        float sum[4] = {0.0f, 0.0f, 0.0f, 0.0f}, comp[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        for (int k0 = 0; k0 < Q; k0 += kPix) {
+            const int n = min(kPix, Q - k0), n8 = (n + 7) & ~7;
+            __syncthreads();
+            for (int i = threadIdx.x; i < n8; i += 256) {
+                float v[2][4];
+#pragma unroll
+                for (int s = 0; s < 2; ++s)
+#pragma unroll
+                    for (int a = 0; a < 4; ++a)
+                        v[s][a] = i < n && (!s || mirror)
+                                      ? __ldg(map + (s ? h.start : g.start) + k0 + i + a * Q)
+                                      : 0.0f;
+                float e[2], o[2], x[2], z[2];
+#pragma unroll
+                for (int s = 0; s < 2; ++s) {
+                    e[s] = (v[s][0] + v[s][2]) + (v[s][1] + v[s][3]);
+                    o[s] = (v[s][0] + v[s][2]) - (v[s][1] + v[s][3]);
+                    x[s] = v[s][0] - v[s][2];
+                    z[s] = v[s][3] - v[s][1];  // (-i)(v1 - v3): imaginary part -(v1 - v3)
+                }
+                y[0][i] = make_float4(e[0], 0.0f, e[1], 0.0f);
+                y[1][i] = make_float4(x[0], z[0], x[1], z[1]);
+                y[2][i] = make_float4(o[0], 0.0f, o[1], 0.0f);
+                y[3][i] = make_float4(x[0], -z[0], x[1], -z[1]);
+            }
+            __syncthreads();
+            for (int i = 0; i < n8; i += kAnchor) {
+                float2 w = twiddle(J, fl, inv_l);
+                J += j8;
+                J -= J >= 2 * L ? 2 * L : 0;
+                float p[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+                for (int e = 0; e < kAnchor; ++e) {
+                    const float4 a = y[c][i + e];
+                    p[0] = fmaf(a.x, w.x, fmaf(-a.y, w.y, p[0]));
+                    p[1] = fmaf(a.x, w.y, fmaf(a.y, w.x, p[1]));
+                    p[2] = fmaf(a.z, w.x, fmaf(-a.w, w.y, p[2]));
+                    p[3] = fmaf(a.z, w.y, fmaf(a.w, w.x, p[3]));
+                    w = cmul(w, step);
+                }
+#pragma unroll
+                for (int e = 0; e < 4; ++e) fold(sum[e], comp[e], p[e]);
             }
         }
-        const bool on = live && e == 0;
-        if (!__any_sync(0xffffffffu, on)) continue;
-        const bool odd = (l - m) & 1;
-        double xr = on ? v1 * (odd ? dr : sr) : 0.0;
-        double xi = on ? v1 * (odd ? di : si) : 0.0;
-        for (int o = 16; o > 0; o >>= 1) {
-            xr += __shfl_down_sync(0xffffffffu, xr, o);
-            xi += __shfl_down_sync(0xffffffffu, xi, o);
+        if (m > lim) continue;
+        F[(long long)r * stride + m] = make_float2(sum[0], sum[1]);
+        if (mirror) F[(long long)rs * stride + m] = make_float2(sum[2], sum[3]);
+    }
+}
+
+// In-place FFT of 2^lg complex values in shared memory, sign -1 forward, +1 inverse
+// (unnormalised): Stockham radix 4 with one radix-2 pass when lg is odd; a thread holds the
+// values of its four butterflies between the two barriers of a pass.  tw[k] = e^{-2 pi i k /
+// n} for k < n / 4; the other quadrants by exact rotations.
+__device__ __forceinline__ float2 fft_twiddle(const float2 *tw, int k, int lgq, float sgn) {
+    const float2 w = tw[k & ((1 << lgq) - 1)];
+    const int quad = k >> lgq;  // times (-i)^quad
+    float2 v = quad & 1 ? make_float2(w.y, -w.x) : w;
+    if (quad & 2) v = make_float2(-v.x, -v.y);
+    return make_float2(v.x, -sgn * v.y);
+}
+__device__ __forceinline__ void fft_shared(float2 *x, const float2 *tw, int lg, float sgn) {
+    const int n = 1 << lg, q = n >> 2, T = blockDim.x;
+    int ls = 0;  // log2 of the stride s
+    for (; ls + 2 <= lg; ls += 2) {
+        float2 y[4][4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            const int t = threadIdx.x + b * T;
+            if (t >= q) break;
+            const float2 a0 = x[t], a1 = x[t + q], a2 = x[t + 2 * q], a3 = x[t + 3 * q];
+            const int k = (t >> ls) << ls;  // p s
+            const float2 s02 = make_float2(a0.x + a2.x, a0.y + a2.y), d02 = make_float2(a0.x - a2.x, a0.y - a2.y);
+            const float2 s13 = make_float2(a1.x + a3.x, a1.y + a3.y), d13 = make_float2(a1.x - a3.x, a1.y - a3.y);
+            const float2 jd = make_float2(-sgn * d13.y, sgn * d13.x);  // sgn i d13
+            y[b][0] = make_float2(s02.x + s13.x, s02.y + s13.y);
+            y[b][1] = cmul(make_float2(d02.x + jd.x, d02.y + jd.y), fft_twiddle(tw, k, lg - 2, sgn));
+            y[b][2] = cmul(make_float2(s02.x - s13.x, s02.y - s13.y), fft_twiddle(tw, 2 * k, lg - 2, sgn));
+            y[b][3] = cmul(make_float2(d02.x - jd.x, d02.y - jd.y), fft_twiddle(tw, 3 * k, lg - 2, sgn));
         }
-        if (lane == 0) {
-            const double w = c * (kl ? kl[l] : 1.0);
-            atomicAdd(&a[l].x, w * xr);
-            atomicAdd(&a[l].y, w * xi);
+        __syncthreads();
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            const int t = threadIdx.x + b * T;
+            if (t >= q) break;
+            const int lo = t & ((1 << ls) - 1), o = ((t >> ls) << (ls + 2)) + lo;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) x[o + (j << ls)] = y[b][j];
+        }
+        __syncthreads();
+    }
+    if (ls < lg) {  // one radix-2 pass, stride n / 2
+        const int hN = n >> 1;
+        for (int t = threadIdx.x; t < hN; t += T) {
+            const float2 a = x[t], b = x[t + hN];
+            x[t] = make_float2(a.x + b.x, a.y + b.y);
+            x[t + hN] = make_float2(a.x - b.x, a.y - b.y);
+        }
+        __syncthreads();
+    }
+}
+__device__ __forceinline__ void fft_table(float2 *tw, int lg) {
+    const float inv = 2.0f / (float)(1 << lg);
+    for (int k = threadIdx.x; k < (1 << (lg - 2)); k += blockDim.x) {
+        float sn, cs;
+        sincospif(-(float)k * inv, &sn, &cs);  // the argument is exact
+        tw[k] = make_float2(cs, sn);
+    }
+}
+
+// Analysis of belt ring r = r_first + blockIdx.x and its mirror by one FFT of north + i south.
+__global__ void __launch_bounds__(1024)
+sht_fft_anal(int nside, int lmax, int lg, int r_first, const float *__restrict__ map,
+             float2 *__restrict__ F) {
+    extern __shared__ float2 fx[];
+    const int n = 1 << lg;
+    float2 *tw = fx + n;
+    const int r = r_first + blockIdx.x, rs = 4 * nside - 2 - r;
+    const bool mirror = rs != r;
+    const ShtRing g = sht_ring(nside, r), h = sht_ring(nside, rs);
+    fft_table(tw, lg);
+    for (int k = threadIdx.x; k < n; k += blockDim.x)
+        fx[k] = make_float2(__ldg(map + g.start + k), mirror ? __ldg(map + h.start + k) : 0.0f);
+    __syncthreads();
+    fft_shared(fx, tw, lg, -1.0f);
+    const long long stride = lmax + 1;
+    const int lim = order_limit(lmax, g.s);
+    const float inv = 1.0f / (float)n;
+    for (int m = threadIdx.x; m <= lim; m += blockDim.x) {
+        const float2 a = fx[m & (n - 1)], b = fx[(n - m) & (n - 1)];
+        float2 fn = make_float2(0.5f * (a.x + b.x), 0.5f * (a.y - b.y));
+        float2 fs = make_float2(0.5f * (a.y + b.y), 0.5f * (b.x - a.x));
+        if (g.t) {  // e^{-i pi m / n}, the argument exact
+            float sn, cs;
+            sincospif(-(float)m * inv, &sn, &cs);
+            fn = cmul(fn, make_float2(cs, sn));
+            fs = cmul(fs, make_float2(cs, sn));
+        }
+        F[(long long)r * stride + m] = fn;
+        if (mirror) F[(long long)rs * stride + m] = fs;
+    }
+}
+
+// Synthesis of belt ring r and its mirror: bin b of the Hermitian spectra collects the orders
+// m = b and, conjugate, m = -b mod n (each w_m / 2 G_m e^{i pi m t / n}); north + i south.
+__global__ void __launch_bounds__(1024)
+sht_fft_synth(int nside, int lmax, int lg, int r_first, const float2 *__restrict__ G,
+              float *__restrict__ map, int add) {
+    extern __shared__ float2 fx[];
+    const int n = 1 << lg;
+    float2 *tw = fx + n;
+    const int r = r_first + blockIdx.x, rs = 4 * nside - 2 - r;
+    const bool mirror = rs != r;
+    const ShtRing g = sht_ring(nside, r), h = sht_ring(nside, rs);
+    const long long stride = lmax + 1;
+    const int lim = order_limit(lmax, g.s);
+    const float inv = 1.0f / (float)n;
+    fft_table(tw, lg);
+    for (int b = threadIdx.x; b < n; b += blockDim.x) {
+        float2 zn = make_float2(0.0f, 0.0f), zs = zn;
+        auto take = [&](int m, float conj) {
+            if (m > lim) return;
+            float2 a = G[(long long)r * stride + m];
+            float2 c = mirror ? G[(long long)rs * stride + m] : make_float2(0.0f, 0.0f);
+            if (g.t) {
+                float sn, cs;
+                sincospif((float)m * inv, &sn, &cs);
+                a = cmul(a, make_float2(cs, sn));
+                c = cmul(c, make_float2(cs, sn));
+            }
+            const float w = m == 0 ? 0.5f : 1.0f;
+            zn.x = fmaf(w, a.x, zn.x);
+            zn.y = fmaf(conj * w, a.y, zn.y);
+            zs.x = fmaf(w, c.x, zs.x);
+            zs.y = fmaf(conj * w, c.y, zs.y);
+        };
+        const int nb = (n - b) & (n - 1);
+        take(b, 1.0f);
+        take(b + n, 1.0f);
+        take(nb, -1.0f);
+        take(nb + n, -1.0f);
+        fx[b] = make_float2(zn.x - zs.y, zn.y + zs.x);
+    }
+    __syncthreads();
+    fft_shared(fx, tw, lg, 1.0f);
+    for (int k = threadIdx.x; k < n; k += blockDim.x) {
+        const float2 v = fx[k];
+        float *on = map + g.start + k, *os = map + h.start + k;
+        if (add) *on += v.x;
+        else *on = v.x;
+        if (mirror) {
+            if (add) *os += v.y;
+            else *os = v.y;
         }
     }
 }
 
-// Dynamic shared memory of the Legendre kernels (A and B tables) and of the
-// synthesis ring kernel (two rings' G): the same size; above 48 kB the kernels
-// are opted in for it.
-cudaError_t leg_smem(int lmax, size_t *bytes) {
-    *bytes = sizeof(double) * 2 * (size_t)(lmax + 1);
-    if (*bytes <= 48 * 1024) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(sht_leg_synth,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*bytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(sht_leg_anal, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)*bytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(sht_dft_synth, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)*bytes);
-    return e;
+// log2 of the belt rings' length where they go through the FFT (16 <= L <= 16384), else 0.
+int belt_fft(int nside) {
+    int lg = 2;
+    while ((1 << (lg - 2)) < nside) ++lg;
+    return lg >= 4 && lg <= 14 ? lg : 0;
+}
+
+// Rings first .. last (northern half) by direct quarter sums; the rest of [0, 2 nside) by FFT.
+cudaError_t ring_synth(int nside, int lmax, const float2 *G, float *map, int add, cudaStream_t st) {
+    const int lg = belt_fft(nside), n_cap = lg ? nside - 1 : 2 * nside;
+    if (n_cap > 0) {
+        dim3 grid(n_cap, nside > 512 ? 2 : 1);
+        sht_ring_synth<<<grid, 256, 0, st>>>(nside, lmax, 0, G, map, add);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess || !lg) return e;
+    }
+    const size_t smem = sizeof(float2) * (5u << (lg - 2));
+    cudaError_t e = cudaFuncSetAttribute(sht_fft_synth, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
+    if (e != cudaSuccess) return e;
+    sht_fft_synth<<<nside + 1, 1 << (lg - 4 > 5 ? lg - 4 : 5), smem, st>>>(nside, lmax, lg, nside - 1,
+                                                                          G, map, add);
+    return cudaGetLastError();
+}
+
+cudaError_t ring_anal(int nside, int lmax, const float *map, float2 *F, cudaStream_t st) {
+    const int lg = belt_fft(nside), n_cap = lg ? nside - 1 : 2 * nside;
+    if (n_cap > 0) {
+        dim3 grid(n_cap, (lmax + 256) / 256);
+        sht_ring_anal<<<grid, 256, 0, st>>>(nside, lmax, 0, map, F);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess || !lg) return e;
+    }
+    const size_t smem = sizeof(float2) * (5u << (lg - 2));
+    cudaError_t e = cudaFuncSetAttribute(sht_fft_anal, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
+    if (e != cudaSuccess) return e;
+    sht_fft_anal<<<nside + 1, 1 << (lg - 4 > 5 ? lg - 4 : 5), smem, st>>>(nside, lmax, lg, nside - 1,
+                                                                         map, F);
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -370,21 +735,20 @@ cudaError_t leg_smem(int lmax, size_t *bytes) {
 // alm (device, n_alm(lmax) complex) -> map (device FP32); add != 0 adds.
 cudaError_t sht_synthesis(int nside, int lmax, const double2 *d_alm, float *d_map, int add,
                           cudaStream_t st) {
-    size_t cs = 0;
-    cudaError_t e = leg_smem(lmax, &cs);
-    if (e != cudaSuccess) return e;
     const int nr = 4 * nside - 1, nnorth = 2 * nside;
     float2 *G = nullptr;
-    if ((e = cudaMallocAsync(&G, sizeof(float2) * (size_t)nr * (lmax + 1), st)) != cudaSuccess)
-        return e;
-    dim3 grid((nnorth + 127) / 128, lmax + 1);
-    sht_leg_synth<<<grid, 128, cs, st>>>(nside, lmax, d_alm, G);
-    e = cudaGetLastError();
-    if (e == cudaSuccess) {
-        sht_dft_synth<<<nnorth, 256, cs, st>>>(
-            nside, lmax, G, d_map, add);
-        e = cudaGetLastError();
+    cudaError_t e = cudaMallocAsync(&G, sizeof(float2) * (size_t)nr * (lmax + 1), st);
+    if (e != cudaSuccess) return e;
+    // two rings a thread share the staged coefficients; one where rings are few
+    if (nnorth > 512) {
+        dim3 grid((nnorth + 511) / 512, lmax + 1);
+        sht_leg_synth<2><<<grid, 256, 0, st>>>(nside, lmax, d_alm, G);
+    } else {
+        dim3 grid((nnorth + 255) / 256, lmax + 1);
+        sht_leg_synth<1><<<grid, 256, 0, st>>>(nside, lmax, d_alm, G);
     }
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = ring_synth(nside, lmax, G, d_map, add, st);
     const cudaError_t f = cudaFreeAsync(G, st);
     return e != cudaSuccess ? e : f;
 }
@@ -393,22 +757,19 @@ cudaError_t sht_synthesis(int nside, int lmax, const double2 *d_alm, float *d_ma
 // when kl (device, lmax + 1 doubles) is given.
 cudaError_t sht_analysis(int nside, int lmax, const float *d_map, const double *d_kl,
                          double2 *d_alm, cudaStream_t st) {
-    size_t cs = 0;
-    cudaError_t e = leg_smem(lmax, &cs);
-    if (e != cudaSuccess) return e;
     const int nr = 4 * nside - 1, nnorth = 2 * nside;
+    const size_t smem = sizeof(float4) * (size_t)(lmax + 1);
+    auto kernel = nnorth > 512 ? sht_leg_anal<4> : sht_leg_anal<1>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
     float2 *F = nullptr;
     if ((e = cudaMallocAsync(&F, sizeof(float2) * (size_t)nr * (lmax + 1), st)) != cudaSuccess)
         return e;
-    e = cudaMemsetAsync(d_alm, 0, sizeof(double2) * (size_t)n_alm(lmax), st);
+    e = ring_anal(nside, lmax, d_map, F, st);
     if (e == cudaSuccess) {
-        sht_dft_anal<<<nnorth, 256, 0, st>>>(nside, lmax, d_map, F);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) {
-        const double c = 4.0 * kPi / (12.0 * (double)nside * (double)nside);
-        dim3 grid((nnorth + 127) / 128, lmax + 1);
-        sht_leg_anal<<<grid, 128, cs, st>>>(nside, lmax, F, d_kl, c, d_alm);
+        const double up = 4.0 * (double)nside;
+        const double c = 4.0 * kPi / (12.0 * (double)nside * (double)nside) * up;
+        kernel<<<lmax + 1, 256, smem, st>>>(nside, lmax, F, d_kl, 1.0 / up, c, d_alm);
         e = cudaGetLastError();
     }
     const cudaError_t f = cudaFreeAsync(F, st);
