@@ -117,11 +117,12 @@ int plan_belt_tc(ksc_split *s, const ksc::RingGeom &g, const std::vector<int2> &
     s->ctc.d_ncut = s->d_ncut;
     s->ctc.d_coef_off = s->d_coef_off;
     s->ctc.d_coef = s->d_coef;
-    // Below about 3e8 belt pairs the FFMA kernel is the faster one: a tile spends 0.7 to
-    // 1.8 us on an input ring however short the window, and small maps have few tiles
-    // (FFMA / tensor stage, us: nside 64, 360': 58 / 72; 256, 160' (2.2e8 pairs): 91 / 99;
-    // 512, 60' (5e8): 123 / 115; 256, 640' (3.6e9): 542 / 371; 1024, 160': 3605 / 1177).
-    if (2.0 / 3.0 * ksc_cost_pairs(s->nside, s->theta_cut) < 3e8) return KSC_OK;
+    // Below about 8e8 belt pairs the FFMA kernel is the faster one: a tile spends 0.7 to
+    // 1.8 us on an input ring however short the window, small maps have few tiles, and the
+    // block maxima (5 us) and their scratch come on top (FFMA / tensor stage, us: nside 64,
+    // 360': 58 / 72; 256, 160' (2.2e8 pairs): 91 / 99; 512, 60' (5e8): 123 / 122, the call's
+    // first pass 483 / 580; 256, 640' (3.6e9): 542 / 371; 1024, 160': 3605 / 1177).
+    if (2.0 / 3.0 * ksc_cost_pairs(s->nside, s->theta_cut) < 8e8) return KSC_OK;
     const int lo = s->plan.belt_lo, hi = s->plan.belt_hi, nb = ksc::belt_tc_rings();
     int wpos = 0, nq = 0;
     for (int r0 = lo; r0 <= hi; r0 += nb) {
@@ -744,14 +745,9 @@ int check_maps(const ksc_split *s, const void *a, const void *b) {
     return KSC_OK;
 }
 
-// Scratch of one convolution call, from the stream-ordered allocator: the map's block
-// maxima, the belt tiles' flags, the rings' ranges and the cap rings' flags.
-struct CallScratch {
-    unsigned char *mem = nullptr;
-    unsigned *bm = nullptr;
-    uint2 *ranges = nullptr;
-    int *cap_flags = nullptr;
-    unsigned char *belt_flags = nullptr;
+// One convolution call's scratch, from the stream-ordered allocator.
+struct CallScratch : ksc::ConvScratch {
+    void *mem = nullptr;
     cudaStream_t st = nullptr;
     CallScratch() = default;
     CallScratch(const CallScratch &) = delete;
@@ -761,53 +757,18 @@ struct CallScratch {
     }
 };
 
-bool has_cap_tc(const ksc_split *s) { return s->ctc.ring_end >= s->ctc.ring_first; }
-
-// Takes the scratch the split's tensor-core stages need (none: no-op) and starts the
-// launches that fill it.
-cudaError_t start_scratch(const ksc_split *s, const float *d_in, int n_maps, long long stride,
+// Takes the scratch and starts the launches that fill it.
+cudaError_t start_scratch(const ksc_split *s, const ksc::MapSet &maps, int n_maps,
                           cudaStream_t st, CallScratch *w) {
-    const bool cap = has_cap_tc(s), belt = s->btc.n_cols > 0;
-    if (!cap && !belt) return cudaSuccess;
-    const int nr = s->plan.nrings;
-    const size_t b_rr = cap ? sizeof(uint2) * (size_t)nr * n_maps : 0;
-    const size_t b_bm = sizeof(unsigned) * (size_t)ksc::map_blocks(s->plan) * n_maps;
-    const size_t b_cf = cap ? sizeof(int) * (size_t)(nr + 1) * n_maps : 0;
-    const size_t b_bf = belt ? (size_t)ksc::belt_tc_tiles(s->plan, s->btc) * n_maps : 0;
+    const size_t bytes = ksc::conv_scratch_bytes(s, n_maps);
+    if (bytes == 0) return cudaSuccess;
     w->st = st;
-    cudaError_t e = cudaMallocAsync(&w->mem, b_rr + b_bm + b_cf + b_bf, st);
+    const cudaError_t e = cudaMallocAsync(&w->mem, bytes, st);
     if (e != cudaSuccess) {
         w->mem = nullptr;
         return e;
     }
-    w->ranges = reinterpret_cast<uint2 *>(w->mem);
-    w->bm = reinterpret_cast<unsigned *>(w->mem + b_rr);
-    w->cap_flags = reinterpret_cast<int *>(w->mem + b_rr + b_bm);
-    w->belt_flags = w->mem + b_rr + b_bm + b_cf;
-    e = ksc::launch_block_max(s->plan, d_in, n_maps, stride, w->bm, st);
-    if (e == cudaSuccess && cap) {
-        e = cudaMemsetAsync(w->cap_flags, 0, b_cf, st);
-        if (e == cudaSuccess)
-            e = ksc::launch_ring_range(s->plan, w->bm, n_maps, w->ranges, st);
-    }
-    return e;
-}
-
-// The belt stage (belt-belt ring pairs) of output rings [r0, r1]: the tensor-core kernel
-// where the split has a plan for it, then the FFMA kernel for the tiles it left (none of
-// them in an ordinary map: that launch reads the flags and ends); else the FFMA kernel.
-cudaError_t launch_belt(const ksc_split *s, const float *d_in, float *d_out, int n_maps,
-                        long long stride, int r0, int r1, const CallScratch &w, cudaStream_t st) {
-    const int a = s->ring_first_belt[r0], b = s->ring_first_belt[r1 + 1];
-    if (a == b || s->n_items_belt == 0) return cudaSuccess;
-    if (s->btc.n_cols == 0)
-        return ksc::launch_conv_belt(s->plan, s->d_items_belt + a, b - a, s->seg_cap, d_in, d_out,
-                                     n_maps, stride, nullptr, nullptr, s->d_err, st);
-    const cudaError_t e = ksc::launch_conv_belt_tc(s->plan, s->btc, d_in, d_out, n_maps, stride,
-                                                   r0, r1, w.bm, w.belt_flags, s->d_err, st);
-    if (e != cudaSuccess) return e;
-    return ksc::launch_conv_belt(s->plan, s->d_items_belt + a, b - a, s->seg_cap, d_in, d_out,
-                                 n_maps, stride, &s->btc, w.belt_flags, s->d_err, st);
+    return ksc::start_conv_scratch(s, maps, n_maps, w->mem, w, st);
 }
 
 // Tensor-core belt stage for a stack of maps; grows the split's pre-tiled map
@@ -832,46 +793,6 @@ int launch_belt_tensor(const ksc_split *cs, const float *d_in, float *d_out, int
     return KSC_OK;
 }
 
-// The cap stage for the items of northern rings [lo, hi], writing output rings
-// [r0, r1]: the map-stack tensor kernel for whole-map stacks, else the FFMA gather
-// or the single-map tensor kernel (ksc_split_opts.cap_kernel).  Whole maps take
-// the items longest first, bands their rings' items in ring order.
-cudaError_t launch_caps(const ksc_split *s, const float *d_in, float *d_out, int n_maps,
-                        long long stride, int lo, int hi, int r0, int r1, bool stack,
-                        const CallScratch &w, cudaStream_t st) {
-    const bool whole = r0 == 0 && r1 == s->plan.nrings - 1;
-    const int belt_split = s->n_items_belt > 0 ? 1 : 0;
-    if (stack && s->tensor >= 1)
-        return ksc::launch_conv_sym_mma(s->plan, s->d_items_smma_lpt, s->n_items_smma, d_in,
-                                        d_out, n_maps, stride, belt_split, s->d_err, st);
-    if (s->cap_kernel == 1) {
-        const int c = s->ring_first_smma[lo], d = s->ring_first_smma[hi + 1];
-        const ksc::WorkItem *its = whole ? s->d_items_smma_lpt : s->d_items_smma + c;
-        return ksc::launch_conv_sym_tc(s->plan, its, d - c, d_in, d_out, n_maps, stride,
-                                       belt_split, r0, r1, s->d_err, st);
-    }
-    const int c = s->ring_first_sym[lo], d = s->ring_first_sym[hi + 1];
-    const ksc::WorkItem *its = whole ? s->d_items_sym_lpt : s->d_items_sym + c;
-    if (!has_cap_tc(s))
-        return ksc::launch_conv_sym(s->plan, its, d - c, d_in, d_out, n_maps, stride, belt_split,
-                                    r0, r1, d - c, nullptr, s->d_err, st);
-    // the tensor-core stage, the irregular ring pairs, then the gather for the rings that
-    // the first flagged (none in an ordinary map: that launch reads a flag and ends)
-    // (a tile holds rings r and r + 1: from the one that may start just before lo)
-    const int t0 = whole ? 0 : s->cap_tile_first[std::max(lo - 1, 0)];
-    const int t1 = whole ? s->n_cap_tiles : s->cap_tile_first[hi + 1];
-    cudaError_t e = ksc::launch_conv_cap_tc(
-        s->plan, s->ctc, whole ? s->d_cap_tiles_lpt : s->d_cap_tiles + t0, t1 - t0, d_in, d_out,
-        n_maps, stride, belt_split, r0, r1, w.ranges, w.cap_flags, s->d_err, st);
-    if (e != cudaSuccess) return e;
-    const int i0 = s->irr_item_first[lo], i1 = s->irr_item_first[hi + 1];
-    e = ksc::launch_cap_direct(s->plan, s->d_irr_items + i0, i1 - i0, s->d_irr_first, s->d_irr,
-                               d_in, d_out, n_maps, stride, r0, r1, w.cap_flags, st);
-    if (e != cudaSuccess) return e;
-    return ksc::launch_conv_sym(s->plan, its, d - c, d_in, d_out, n_maps, stride, belt_split, r0,
-                                r1, 0, w.cap_flags, s->d_err, st);
-}
-
 // The real-space convolution of output rings [r0, r1] (0-based, inclusive).
 // Default path: circulant belt kernel first (writes belt outputs), then the
 // symmetric gather (writes cap outputs, adds cap inputs to belt outputs).
@@ -887,8 +808,9 @@ int launch_conv(const ksc_split *s, const float *d_in, float *d_out, int n_maps,
         if (e != cudaSuccess) return cuda_fail(e, "gather kernel launch");
         return KSC_OK;
     }
+    const ksc::MapSet maps{d_in, d_out, stride};
     CallScratch w;
-    e = start_scratch(s, d_in, n_maps, stride, st, &w);
+    e = start_scratch(s, maps, n_maps, st, &w);
     if (e != cudaSuccess) return cuda_fail(e, "call scratch");
     const bool whole = r0 == 0 && r1 == s->plan.nrings - 1;
     const bool stack = whole && n_maps >= 16;
@@ -896,7 +818,7 @@ int launch_conv(const ksc_split *s, const float *d_in, float *d_out, int n_maps,
         int rc = launch_belt_tensor(s, d_in, d_out, n_maps, stride, st);
         if (rc) return rc;
     } else {
-        e = launch_belt(s, d_in, d_out, n_maps, stride, r0, r1, w, st);
+        e = ksc::launch_belt(s, maps, n_maps, r0, r1, w, s->d_err, st);
         if (e != cudaSuccess) return cuda_fail(e, "belt kernel launch");
     }
     // northern rings r whose own or mirror ring (nr - 1 - r) lies in the band
@@ -906,7 +828,7 @@ int launch_conv(const ksc_split *s, const float *d_in, float *d_out, int n_maps,
     const int m0 = std::max(0, nr - 1 - r1), m1 = std::min(nr - 1 - r0, eq);
     if (m0 <= m1) { lo = std::min(lo, m0); hi = std::max(hi, m1); }  // mirror in band
     if (lo <= hi) {
-        e = launch_caps(s, d_in, d_out, n_maps, stride, lo, hi, r0, r1, stack, w, st);
+        e = ksc::launch_caps(s, maps, n_maps, lo, hi, r0, r1, stack, w, s->d_err, st);
         if (e != cudaSuccess) return cuda_fail(e, "symmetric kernel launch");
     }
     return KSC_OK;
@@ -915,6 +837,101 @@ int launch_conv(const ksc_split *s, const float *d_in, float *d_out, int n_maps,
 } // namespace
 
 namespace ksc {
+
+bool has_cap_tc(const ksc_split *s) { return s->ctc.ring_end >= s->ctc.ring_first; }
+
+size_t conv_scratch_bytes(const ksc_split *s, int n_maps) {
+    const bool cap = has_cap_tc(s), belt = s->btc.n_cols > 0;
+    const size_t nr = (size_t)s->plan.nrings;
+    if (!cap && !belt) return 0;
+    size_t b = sizeof(int);  // the gather's claim counter
+    b += sizeof(unsigned) * (size_t)map_blocks(s->plan);
+    if (cap) b += sizeof(uint2) * nr + sizeof(int) * (nr + 1);
+    if (belt) b += (size_t)belt_tc_tiles(s->plan, s->btc);
+    return b * (size_t)n_maps;
+}
+
+cudaError_t start_conv_scratch(const ksc_split *s, const MapSet &maps, int n_maps, void *mem,
+                               ConvScratch *w, cudaStream_t st) {
+    const bool cap = has_cap_tc(s), belt = s->btc.n_cols > 0;
+    if (!cap && !belt) return cudaSuccess;
+    const size_t nr = (size_t)s->plan.nrings, n = (size_t)n_maps;
+    unsigned char *at = static_cast<unsigned char *>(mem);
+    const auto take = [&](size_t bytes) {
+        unsigned char *p = at;
+        at += bytes * n;
+        return p;
+    };
+    if (cap) w->ranges = reinterpret_cast<uint2 *>(take(sizeof(uint2) * nr));
+    w->counters = reinterpret_cast<int *>(take(sizeof(int)));
+    if (cap) w->cap_flags = reinterpret_cast<int *>(take(sizeof(int) * (nr + 1)));
+    unsigned char *const zero_end = at;
+    w->bm = reinterpret_cast<unsigned *>(take(sizeof(unsigned) * (size_t)map_blocks(s->plan)));
+    if (belt) w->belt_flags = at;
+    const size_t n_zero = (size_t)(zero_end - (unsigned char *)w->counters);
+    cudaError_t e = launch_block_max(s->plan, maps, n_maps, w->bm, w->counters,
+                                     (long long)(n_zero / sizeof(int)), st);
+    if (e == cudaSuccess && cap) e = launch_ring_range(s->plan, w->bm, n_maps, w->ranges, st);
+    return e;
+}
+
+// The belt stage (belt-belt ring pairs) of output rings [r0, r1]: the tensor-core kernel
+// where the split has a plan for it, then the FFMA kernel for the tiles it left (none of
+// them in an ordinary map: that launch reads the flags and ends); else the FFMA kernel.
+cudaError_t launch_belt(const ksc_split *s, const MapSet &maps, int n_maps, int r0, int r1,
+                        const ConvScratch &w, int *d_err, cudaStream_t st) {
+    const int a = s->ring_first_belt[r0], b = s->ring_first_belt[r1 + 1];
+    if (a == b || s->n_items_belt == 0) return cudaSuccess;
+    if (s->btc.n_cols == 0)
+        return launch_conv_belt(s->plan, s->d_items_belt + a, b - a, s->seg_cap, maps, n_maps,
+                                nullptr, nullptr, d_err, st);
+    const cudaError_t e = launch_conv_belt_tc(s->plan, s->btc, maps, n_maps, r0, r1, w.bm,
+                                              w.belt_flags, d_err, st);
+    if (e != cudaSuccess) return e;
+    return launch_conv_belt(s->plan, s->d_items_belt + a, b - a, s->seg_cap, maps, n_maps,
+                            &s->btc, w.belt_flags, d_err, st);
+}
+
+// The cap stage for the items of northern rings [lo, hi], writing output rings
+// [r0, r1]: the map-stack tensor kernel for whole-map stacks, else the FFMA gather
+// or the single-map tensor kernel (ksc_split_opts.cap_kernel).  Whole maps take
+// the items longest first, bands their rings' items in ring order.
+cudaError_t launch_caps(const ksc_split *s, const MapSet &maps, int n_maps, int lo, int hi,
+                        int r0, int r1, bool stack, const ConvScratch &w, int *d_err,
+                        cudaStream_t st) {
+    const bool whole = r0 == 0 && r1 == s->plan.nrings - 1;
+    const int belt_split = s->n_items_belt > 0 ? 1 : 0;
+    if (stack && s->tensor >= 1)
+        return launch_conv_sym_mma(s->plan, s->d_items_smma_lpt, s->n_items_smma, maps.in,
+                                        maps.out, n_maps, maps.stride, belt_split, d_err, st);
+    if (s->cap_kernel == 1) {
+        const int c = s->ring_first_smma[lo], d = s->ring_first_smma[hi + 1];
+        const WorkItem *its = whole ? s->d_items_smma_lpt : s->d_items_smma + c;
+        return launch_conv_sym_tc(s->plan, its, d - c, maps.in, maps.out, n_maps, maps.stride,
+                                       belt_split, r0, r1, d_err, st);
+    }
+    const int c = s->ring_first_sym[lo], d = s->ring_first_sym[hi + 1];
+    const WorkItem *its = whole ? s->d_items_sym_lpt : s->d_items_sym + c;
+    if (!has_cap_tc(s))
+        return launch_conv_sym(s->plan, its, d - c, maps, n_maps, belt_split, r0, r1, d - c,
+                                    nullptr, w.counters, d_err, st);
+    // the tensor-core stage, the irregular ring pairs, then the gather for the rings that
+    // the first flagged (none in an ordinary map: that launch reads a flag and ends)
+    // (a tile holds rings r and r + 1: from the one that may start just before lo)
+    const int t0 = whole ? 0 : s->cap_tile_first[std::max(lo - 1, 0)];
+    const int t1 = whole ? s->n_cap_tiles : s->cap_tile_first[hi + 1];
+    cudaError_t e = launch_conv_cap_tc(
+        s->plan, s->ctc, whole ? s->d_cap_tiles_lpt : s->d_cap_tiles + t0, t1 - t0, maps,
+        n_maps, belt_split, r0, r1, w.ranges, w.cap_flags, d_err, st);
+    if (e != cudaSuccess) return e;
+    const int i0 = s->irr_item_first[lo], i1 = s->irr_item_first[hi + 1];
+    e = launch_cap_direct(s->plan, s->d_irr_items + i0, i1 - i0, s->d_irr_first, s->d_irr,
+                               maps, n_maps, r0, r1, w.cap_flags, st);
+    if (e != cudaSuccess) return e;
+    return launch_conv_sym(s->plan, its, d - c, maps, n_maps, belt_split, r0, r1, 0,
+                                w.cap_flags, w.counters, d_err, st);
+}
+
 void set_last_error(const std::string &msg) { g_last_error = msg; }
 
 bool inject_alloc_fault(int n) {
@@ -1305,22 +1322,23 @@ int ksc_conv_real_multimap_stage(const ksc_split *s, const float *d_in, float *d
     cudaStream_t st = (cudaStream_t)stream;
     const long long stride = s->plan.npix;
     if (stage != 1 && stage != 2) return fail(KSC_ERR_ARG, "stage must be 1 or 2");
+    const ksc::MapSet maps{d_in, d_out, stride};
     CallScratch w;
-    cudaError_t e = s->path == 1 ? cudaSuccess : start_scratch(s, d_in, n_maps, stride, st, &w);
+    cudaError_t e = s->path == 1 ? cudaSuccess : start_scratch(s, maps, n_maps, st, &w);
     if (e != cudaSuccess) return cuda_fail(e, "call scratch");
     if (stage == 1) {
         if (s->path == 1) return KSC_OK;
         if (n_maps >= 16 && s->tensor == 2 && s->n_items_mma > 0)
             return launch_belt_tensor(s, d_in, d_out, n_maps, stride, st);
         else
-            e = launch_belt(s, d_in, d_out, n_maps, stride, 0, s->plan.nrings - 1, w, st);
+            e = ksc::launch_belt(s, maps, n_maps, 0, s->plan.nrings - 1, w, s->d_err, st);
     } else {
         if (s->path == 1)
             e = ksc::launch_conv_general(s->plan, s->d_items, s->n_items, d_in, d_out, n_maps,
                                          stride, 0, nullptr, st);
         else
-            e = launch_caps(s, d_in, d_out, n_maps, stride, 0, (s->plan.nrings - 1) / 2, 0,
-                            s->plan.nrings - 1, n_maps >= 16, w, st);
+            e = ksc::launch_caps(s, maps, n_maps, 0, (s->plan.nrings - 1) / 2, 0,
+                                 s->plan.nrings - 1, n_maps >= 16, w, s->d_err, st);
     }
     if (e != cudaSuccess) return cuda_fail(e, "stage launch");
     return KSC_OK;
@@ -1332,18 +1350,19 @@ int ksc_conv_real_stage(const ksc_split *s, const float *d_in, float *d_out, int
     if (rc) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     if (stage != 1 && stage != 2) return fail(KSC_ERR_ARG, "stage must be 1 or 2");
+    const ksc::MapSet maps{d_in, d_out, 0};
     CallScratch w;
-    cudaError_t e = s->path == 1 ? cudaSuccess : start_scratch(s, d_in, 1, 0, st, &w);
+    cudaError_t e = s->path == 1 ? cudaSuccess : start_scratch(s, maps, 1, st, &w);
     if (e != cudaSuccess) return cuda_fail(e, "call scratch");
     if (stage == 1) {
-        e = launch_belt(s, d_in, d_out, 1, 0, 0, s->plan.nrings - 1, w, st);
+        e = ksc::launch_belt(s, maps, 1, 0, s->plan.nrings - 1, w, s->d_err, st);
     } else {
         if (s->path == 1)
             e = ksc::launch_conv_general(s->plan, s->d_items, s->n_items, d_in, d_out, 1, 0, 0,
                                          nullptr, st);
         else
-            e = launch_caps(s, d_in, d_out, 1, 0, 0, (s->plan.nrings - 1) / 2, 0,
-                            s->plan.nrings - 1, false, w, st);
+            e = ksc::launch_caps(s, maps, 1, 0, (s->plan.nrings - 1) / 2, 0, s->plan.nrings - 1,
+                                 false, w, s->d_err, st);
     }
     if (e != cudaSuccess) return cuda_fail(e, "stage launch");
     return KSC_OK;

@@ -12,6 +12,13 @@
 // and replayed; the map pointers live in a device entry table that a run
 // refreshes only when they change.
 //
+// Entries whose split has a tensor-core plan (large enough for it, see the rules where the
+// plans are made) leave those lists: the entries of one split run as one stack through the
+// single-map kernels' tensor-core stages, which read their maps through the same entry
+// table.  The belt stage or both stages go that way.  (8 maps of nside 256, 4 of 512 and 1 of
+// 1024, cuts of 16 beams: belt lists 10.8 ms, as stacks 5.0 ms; the nside-1024 caps 7.3 and
+// 6.6 ms; the run 33.2 and 26.7 ms.)
+//
 // The tile variants are the full and half block size of the belt kernel
 // (2080 or 1040 outputs per item) and three gather tiles: 256 reflection
 // classes per item with 4096-cell weight tables (two CTAs per SM), 128 classes
@@ -69,6 +76,14 @@ struct Launch {
     int seg_cap;  // belt only
 };
 
+// Entries of one split on the tensor-core stages: count entries from table row first on.
+struct TcGroup {
+    const ksc_split *split;
+    int first, count;
+    size_t at;  // its scratch
+};
+constexpr int kMaxStack = 32768;  // entries of one launch (gridDim.y)
+
 } // namespace
 
 struct ksc_batch {
@@ -84,7 +99,10 @@ struct ksc_batch {
     long long n_pairs = 0;                   // in-disc pairs per run, when every split counted them
 
     ksc::ConvPlan *d_plans = nullptr;
-    ksc::BatchEntry *d_entries = nullptr;
+    ksc::BatchEntry *d_entries = nullptr;    // n in the caller's order, then those of tc_order
+    std::vector<int> tc_order;               // entries on the tensor-core stages, by split
+    std::vector<TcGroup> tc;
+    void *d_scratch = nullptr;               // the groups' scratch
     int4 *d_items = nullptr;
     int *d_counters = nullptr;  // one per launch
     int *d_err = nullptr;
@@ -122,8 +140,9 @@ int sym_classes_of(const ksc_split *s, int r) {
 }
 
 // Item lists of the entries `sel` under per-group variants; appends launches
-// (belt launches first).  Entries on the general path are skipped.
-void build_items(const ksc_batch *b, const std::vector<int> &sel,
+// (belt launches first).  Entries on the general path are skipped, and those of the
+// tensor-core stages unless every is set (the autotuner times the tiles on them too).
+void build_items(const ksc_batch *b, const std::vector<int> &sel, bool every,
                  const std::vector<std::pair<int, int>> &vars, std::vector<int4> *items,
                  std::vector<Launch> *launches, int *n_belt, int *n_sym) {
     struct Costed {
@@ -139,6 +158,9 @@ void build_items(const ksc_batch *b, const std::vector<int> &sel,
             for (int e : sel) {
                 const ksc_split *s = b->splits[e];
                 if (s->path != 0) continue;
+                if (!every && !b->tc.empty() && s->btc.n_cols > 0 &&
+                    (kind == 0 || ksc::has_cap_tc(s)))
+                    continue;
                 const std::pair<int, int> var = vars[b->group_of[e]];
                 const int nr = s->plan.nrings, eq = (nr - 1) / 2;
                 std::vector<Costed> list;
@@ -215,14 +237,63 @@ int rebuild(ksc_batch *b) {
     for (int i = 0; i < b->n; ++i) all[i] = i;
     std::vector<int4> items;
     std::vector<Launch> launches;
-    build_items(b, all, b->variants, &items, &launches, &b->n_items_belt, &b->n_items_sym);
+    build_items(b, all, false, b->variants, &items, &launches, &b->n_items_belt, &b->n_items_sym);
     return upload_items(b, items, launches);
 }
 
-// Enqueue counter reset + launches (+ general-path entries) on st.
+// Groups the entries on the tensor-core stages by split and takes their scratch.
+cudaError_t plan_tc(ksc_batch *b) {
+    size_t bytes = 0;
+    for (size_t p = 0; p < b->uniq.size(); ++p) {
+        const ksc_split *s = b->uniq[p];
+        if (s->path != 0 || s->btc.n_cols == 0) continue;
+        for (int i = 0; i < b->n; ++i) {
+            if (b->plan_of[i] != (int)p) continue;
+            if (b->tc.empty() || b->tc.back().split != s || b->tc.back().count == kMaxStack)
+                b->tc.push_back({s, b->n + (int)b->tc_order.size(), 0, 0});
+            ++b->tc.back().count;
+            b->tc_order.push_back(i);
+        }
+    }
+    for (TcGroup &g : b->tc) {
+        g.at = bytes;
+        bytes += (ksc::conv_scratch_bytes(g.split, g.count) + 255) & ~(size_t)255;
+    }
+    return bytes ? cudaMalloc(&b->d_scratch, bytes) : cudaSuccess;
+}
+
+int enqueue_tc(const ksc_batch *b, cudaStream_t st) {
+    for (const TcGroup &g : b->tc) {
+        const ksc_split *s = g.split;
+        ksc::MapSet maps;
+        maps.table = b->d_entries + g.first;
+        ksc::ConvScratch w;
+        const int last = s->plan.nrings - 1;
+        cudaError_t e = ksc::start_conv_scratch(s, maps, g.count,
+                                                static_cast<char *>(b->d_scratch) + g.at, &w, st);
+        if (e == cudaSuccess) e = ksc::launch_belt(s, maps, g.count, 0, last, w, b->d_err, st);
+        if (e == cudaSuccess && ksc::has_cap_tc(s))
+            e = ksc::launch_caps(s, maps, g.count, 0, last / 2, 0, last, false, w, b->d_err, st);
+        if (e != cudaSuccess) return bcuda(e, "batch tensor-core stage");
+    }
+    return KSC_OK;
+}
+
+// Kernel launches of a group per run: block maxima, the belt stage and its fallback; ring
+// ranges, the cap stage, its irregular pairs and its fallback.
+int tc_launches(const TcGroup &g) {
+    return ksc::has_cap_tc(g.split) ? 7 : 3;
+}
+
+// Enqueue counter reset + launches on st; with general, the tensor-core groups before them
+// and the general-path entries after them.
 int enqueue(ksc_batch *b, const std::vector<Launch> &launches, const int4 *d_items,
             const std::vector<int> *general, cudaStream_t st) {
     cudaError_t e;
+    if (general) {
+        const int rc = enqueue_tc(b, st);
+        if (rc) return rc;
+    }
     if (!launches.empty() &&
         (e = cudaMemsetAsync(b->d_counters, 0, sizeof(int) * launches.size(), st)) != cudaSuccess)
         return bcuda(e, "batch counter reset");
@@ -273,7 +344,9 @@ int set_entries(ksc_batch *b, const float *const *d_in, float *const *d_out, cud
     if (b->uploaded && (e = cudaEventSynchronize(b->upload_done)) != cudaSuccess)
         return bcuda(e, "batch entry staging");
     std::memcpy(b->h_entries, cur.data(), sizeof(ksc::BatchEntry) * b->n);
-    if ((e = cudaMemcpyAsync(b->d_entries, b->h_entries, sizeof(ksc::BatchEntry) * b->n,
+    for (size_t i = 0; i < b->tc_order.size(); ++i) b->h_entries[b->n + i] = cur[b->tc_order[i]];
+    if ((e = cudaMemcpyAsync(b->d_entries, b->h_entries,
+                             sizeof(ksc::BatchEntry) * (b->n + b->tc_order.size()),
                              cudaMemcpyHostToDevice, st)) != cudaSuccess)
         return bcuda(e, "batch entry upload");
     if ((e = cudaEventRecord(b->upload_done, st)) != cudaSuccess)
@@ -314,6 +387,7 @@ void batch_free(ksc_batch *b) {
     batch_release_items(b);
     cudaFree(b->d_plans);
     cudaFree(b->d_entries);
+    cudaFree(b->d_scratch);
     cudaFree(b->d_err);
     if (b->h_entries) cudaFreeHost(b->h_entries);
     if (b->upload_done) cudaEventDestroy(b->upload_done);
@@ -375,14 +449,21 @@ int ksc_batch_create(const ksc_split *const *splits, int n, const ksc_batch_opts
     if (!counted) b->n_pairs = -1;
     std::vector<ksc::ConvPlan> plans;
     for (const ksc_split *s : b->uniq) plans.push_back(s->plan);
-    cudaError_t e;
+    cudaError_t e = plan_tc(b);
+    if (e != cudaSuccess) {  // without scratch the lists take every entry
+        cudaGetLastError();
+        b->d_scratch = nullptr;
+        b->tc.clear();
+        b->tc_order.clear();
+    }
+    const size_t n_table = (size_t)n + b->tc_order.size();
     if ((e = cudaMalloc(&b->d_plans, sizeof(ksc::ConvPlan) * plans.size())) != cudaSuccess ||
         (e = cudaMemcpy(b->d_plans, plans.data(), sizeof(ksc::ConvPlan) * plans.size(),
                         cudaMemcpyHostToDevice)) != cudaSuccess ||
-        (e = cudaMalloc(&b->d_entries, sizeof(ksc::BatchEntry) * n)) != cudaSuccess ||
+        (e = cudaMalloc(&b->d_entries, sizeof(ksc::BatchEntry) * n_table)) != cudaSuccess ||
         (e = cudaMalloc(&b->d_err, sizeof(int))) != cudaSuccess ||
         (e = cudaMemset(b->d_err, 0, sizeof(int))) != cudaSuccess ||
-        (e = cudaMallocHost(&b->h_entries, sizeof(ksc::BatchEntry) * n)) != cudaSuccess ||
+        (e = cudaMallocHost(&b->h_entries, sizeof(ksc::BatchEntry) * n_table)) != cudaSuccess ||
         (e = cudaEventCreateWithFlags(&b->upload_done, cudaEventDisableTiming)) != cudaSuccess) {
         batch_free(b);
         return bcuda(e, "batch device state");
@@ -432,7 +513,7 @@ int ksc_batch_autotune(ksc_batch *b, const float *const *d_in, float *const *d_o
             std::vector<int4> items;
             std::vector<Launch> launches;
             int nb = 0, ns = 0;
-            build_items(b, sel, vars, &items, &launches, &nb, &ns);
+            build_items(b, sel, true, vars, &items, &launches, &nb, &ns);
             // temporary item list and counters, timed per launch (median of 3 after a warm-up)
             int4 *d_items = nullptr;
             int *saved_ctr = b->d_counters;
@@ -503,6 +584,7 @@ int ksc_batch_info(const ksc_batch *b, ksc_batch_desc *d) {
     d->n_items_belt = b->n_items_belt;
     d->n_items_sym = b->n_items_sym;
     d->n_launches = (int)b->launches.size() + (int)b->general.size();
+    for (const TcGroup &g : b->tc) d->n_launches += tc_launches(g);
     d->use_graph = b->opts.use_graph;
     d->n_pairs = b->n_pairs;
     d->n_groups = (int)b->nsides.size();

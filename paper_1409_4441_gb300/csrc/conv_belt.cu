@@ -324,12 +324,12 @@ __device__ __forceinline__ bool belt_item(const ConvPlan &P, int r, int k0,
 template <int T>
 __global__ void __launch_bounds__(T)
 conv_belt_kernel(const ConvPlan P, const int2 *__restrict__ items, int n_items,
-                 const float *__restrict__ in, float *__restrict__ out, long long map_stride,
+                 const MapSet maps,
                  int seg_cap, int *__restrict__ err, const unsigned char *__restrict__ flags,
                  int tile_rings, int tile_shift, int row_tiles, int map_tiles) {
     KSC_BELT_SHARED_STATE
-    const float *m = in + (long long)blockIdx.y * map_stride;
-    float *o = out + (long long)blockIdx.y * map_stride;
+    const float *__restrict__ m = maps.input(blockIdx.y);
+    float *__restrict__ o = maps.output(blockIdx.y);
     for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
         const int r = items[it].x, k0 = items[it].y;
         const unsigned char *tf = nullptr;
@@ -404,9 +404,8 @@ cudaError_t belt_grid(K kernel, int threads, size_t smem, int n_items, int per_s
 int belt_chunk() { return kChunk; }
 
 cudaError_t launch_conv_belt(const ConvPlan &p, const int2 *d_items, int n_items, int seg_cap,
-                             const float *d_in, float *d_out, int n_maps, long long map_stride,
-                             const BeltTc *tc, const unsigned char *tile_flags, int *d_err,
-                             cudaStream_t st) {
+                             const MapSet &maps, int n_maps, const BeltTc *tc,
+                             const unsigned char *tile_flags, int *d_err, cudaStream_t st) {
     if (n_items <= 0 || n_maps <= 0) return cudaSuccess;
     int shift = 0, row = 0, all = 0;
     if (tile_flags) {
@@ -420,7 +419,7 @@ cudaError_t launch_conv_belt(const ConvPlan &p, const int2 *d_items, int n_items
     if (e != cudaSuccess) return e;
     dim3 grid(blocks, n_maps);
     conv_belt_kernel<kThreads><<<grid, kThreads, smem, st>>>(
-        p, d_items, n_items, d_in, d_out, map_stride, seg_cap, d_err, tile_flags,
+        p, d_items, n_items, maps, seg_cap, d_err, tile_flags,
         belt_tc_rings(), shift, row, all);
     return cudaGetLastError();
 }

@@ -97,7 +97,7 @@ __host__ __device__ __forceinline__ Window tile_window(int w, int L) {
 template <int N>
 __global__ void __launch_bounds__(kThreads, 1)
 conv_belt_tc_kernel(const ConvPlan P, int block_lo, int n_tiles_k, int ring_lo, int ring_hi,
-                    const float *__restrict__ in, float *__restrict__ out, long long map_stride,
+                    const MapSet maps,
                     const uint32_t *__restrict__ blockmax, long long block_stride,
                     unsigned char *__restrict__ flags, int n_tiles, int wpos_cap, int nq_cap,
                     float wscale, float wunscale, float domega_lo, int *__restrict__ err) {
@@ -123,8 +123,8 @@ conv_belt_tc_kernel(const ConvPlan P, int block_lo, int n_tiles_k, int ring_lo, 
     const int r_first = P.belt_lo + rb * kRings;
     const int n_rows = min(kRings, P.belt_hi - r_first + 1);
     const int L = 4 * P.nside, k0 = ct * 8 * N;
-    const float *m = in + (long long)blockIdx.y * map_stride;
-    float *o = out + (long long)blockIdx.y * map_stride;
+    const float *__restrict__ m = maps.input(blockIdx.y);
+    float *__restrict__ o = maps.output(blockIdx.y);
     const uint32_t *bm = blockmax + (long long)blockIdx.y * block_stride;
     const int start0 = P.d_rings[r_first].start;
 
@@ -538,11 +538,15 @@ conv_belt_tc_kernel(const ConvPlan P, int block_lo, int n_tiles_k, int ring_lo, 
 }
 
 // blockmax[map][b] = the bits of the largest |m| over map pixels [64 b, 64 b + 64)
-// (infinities and NaNs compare above every number).  One read of the map.
+// (infinities and NaNs compare above every number).  One read of the map.  Clears the
+// n_zero words that the call's later kernels count and flag in.
 __global__ void __launch_bounds__(256)
-block_max_kernel(const float *__restrict__ in, long long map_stride, int n_blocks,
-                 uint32_t *__restrict__ blockmax, long long block_stride) {
-    const float4 *m = reinterpret_cast<const float4 *>(in + (long long)blockIdx.y * map_stride);
+block_max_kernel(const MapSet maps, int n_blocks, uint32_t *__restrict__ blockmax,
+                 long long block_stride, int *__restrict__ zero, long long n_zero) {
+    for (long long i = (blockIdx.y * (long long)gridDim.x + blockIdx.x) * 256 + threadIdx.x;
+         i < n_zero; i += (long long)gridDim.x * gridDim.y * 256)
+        zero[i] = 0;
+    const float4 *m = reinterpret_cast<const float4 *>(maps.input(blockIdx.y));
     uint32_t *bm = blockmax + (long long)blockIdx.y * block_stride;
     const int half = (blockIdx.x * 256 + threadIdx.x) >> 4, l16 = threadIdx.x & 15;
     const int n_half = gridDim.x * 16;
@@ -563,8 +567,8 @@ size_t tc_smem(int wpos, int nq) {
 }
 
 template <int N>
-cudaError_t launch_tc(const ConvPlan &p, const BeltTc &t, const float *d_in, float *d_out,
-                      int n_maps, long long map_stride, int r0, int r1, const uint32_t *bm,
+cudaError_t launch_tc(const ConvPlan &p, const BeltTc &t, const MapSet &maps, int n_maps,
+                      int r0, int r1, const uint32_t *bm,
                       long long bm_stride, unsigned char *flags, int *d_err, cudaStream_t st) {
     const int lo = std::max(r0, p.belt_lo), hi = std::min(r1, p.belt_hi);
     const int b0 = (lo - p.belt_lo) / kRings, b1 = (hi - p.belt_lo) / kRings;
@@ -575,7 +579,7 @@ cudaError_t launch_tc(const ConvPlan &p, const BeltTc &t, const float *d_in, flo
     if (e != cudaSuccess) return e;
     dim3 grid((b1 - b0 + 1) * tk, n_maps);
     conv_belt_tc_kernel<N><<<grid, kThreads, smem, st>>>(
-        p, b0, tk, r0, r1, d_in, d_out, map_stride, bm, bm_stride, flags, belt_tc_tiles(p, t),
+        p, b0, tk, r0, r1, maps, bm, bm_stride, flags, belt_tc_tiles(p, t),
         t.wpos, t.nq, t.wscale, 1.0f / t.wscale,
         (float)(4.0 * 3.14159265358979323846 / p.npix - (double)p.domega), d_err);
     return cudaGetLastError();
@@ -620,25 +624,24 @@ bool belt_tc_plan(int nside, int wpos, int nq, BeltTc *t) {
 
 long long map_blocks(const ConvPlan &p) { return p.npix / 64; }
 
-cudaError_t launch_block_max(const ConvPlan &p, const float *d_in, int n_maps,
-                             long long map_stride, uint32_t *bm, cudaStream_t st) {
+cudaError_t launch_block_max(const ConvPlan &p, const MapSet &maps, int n_maps, uint32_t *bm,
+                             int *zero, long long n_zero, cudaStream_t st) {
     const int n = (int)map_blocks(p);
     dim3 grid(std::min((n + 15) / 16, 152 * 8), n_maps);
-    block_max_kernel<<<grid, 256, 0, st>>>(d_in, map_stride, n, bm, n);
+    block_max_kernel<<<grid, 256, 0, st>>>(maps, n, bm, n, zero, n_zero);
     return cudaGetLastError();
 }
 
-cudaError_t launch_conv_belt_tc(const ConvPlan &p, const BeltTc &t, const float *d_in,
-                                float *d_out, int n_maps, long long map_stride, int r0, int r1,
-                                const uint32_t *bm, unsigned char *flags, int *d_err,
-                                cudaStream_t st) {
+cudaError_t launch_conv_belt_tc(const ConvPlan &p, const BeltTc &t, const MapSet &maps,
+                                int n_maps, int r0, int r1, const uint32_t *bm, unsigned char *flags,
+                                int *d_err, cudaStream_t st) {
     if (r0 > p.belt_hi || r1 < p.belt_lo) return cudaSuccess;
     const long long bs = map_blocks(p);
     switch (t.n_cols) {
-    case 256: return launch_tc<256>(p, t, d_in, d_out, n_maps, map_stride, r0, r1, bm, bs, flags, d_err, st);
-    case 128: return launch_tc<128>(p, t, d_in, d_out, n_maps, map_stride, r0, r1, bm, bs, flags, d_err, st);
-    case 64: return launch_tc<64>(p, t, d_in, d_out, n_maps, map_stride, r0, r1, bm, bs, flags, d_err, st);
-    default: return launch_tc<32>(p, t, d_in, d_out, n_maps, map_stride, r0, r1, bm, bs, flags, d_err, st);
+    case 256: return launch_tc<256>(p, t, maps, n_maps, r0, r1, bm, bs, flags, d_err, st);
+    case 128: return launch_tc<128>(p, t, maps, n_maps, r0, r1, bm, bs, flags, d_err, st);
+    case 64: return launch_tc<64>(p, t, maps, n_maps, r0, r1, bm, bs, flags, d_err, st);
+    default: return launch_tc<32>(p, t, maps, n_maps, r0, r1, bm, bs, flags, d_err, st);
     }
 }
 

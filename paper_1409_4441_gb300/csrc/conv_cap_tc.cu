@@ -147,7 +147,7 @@ __host__ __device__ __forceinline__ int coef_words(int jE) { return (kP * (jE + 
 // pixels and the sums keep as FP32 pairs).
 __global__ void __launch_bounds__(kThreads, 1)
 conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ tiles,
-                   const float *__restrict__ in, float *__restrict__ out, long long map_stride,
+                   const MapSet maps,
                    int belt_split, int band_lo, int band_hi, const uint2 *__restrict__ ring_range,
                    int *__restrict__ flags, int *__restrict__ err) {
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -178,8 +178,8 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
     const int r0 = tile.x & 0xffff, n_r = (tile.x >> 16) + 1;
     const int sector = tile.y & 0xffff, n_sec = tile.y >> 16;
     const bool add = belt_split && r0 >= P.belt_lo;
-    const float *m = in + (long long)blockIdx.y * map_stride;
-    float *o = out + (long long)blockIdx.y * map_stride;
+    const float *__restrict__ m = maps.input(blockIdx.y);
+    float *__restrict__ o = maps.output(blockIdx.y);
     const uint2 *rr = ring_range + (long long)blockIdx.y * P.nrings;
     const DevRing Ra = P.d_rings[r0], Rb = P.d_rings[r0 + n_r - 1];
     const int L0 = Ra.len, L1 = Rb.len;
@@ -792,14 +792,14 @@ cap_coef_kernel(const ConvPlan P, const CapTc C, const CapCoef K, int ring_lo, i
 __global__ void __launch_bounds__(256)
 cap_direct_kernel(const ConvPlan P, const int2 *__restrict__ items,
                   const int *__restrict__ list_first, const int *__restrict__ list,
-                  const float *__restrict__ in, float *__restrict__ out, long long map_stride,
+                  const MapSet maps,
                   int band_lo, int band_hi, const int *__restrict__ flags) {
     __shared__ float part[8][8][32];
     const int2 it = items[blockIdx.x];
     const int r = it.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (flags[(long long)blockIdx.y * (P.nrings + 1) + r]) return;
-    const float *m = in + (long long)blockIdx.y * map_stride;
-    float *o = out + (long long)blockIdx.y * map_stride;
+    const float *__restrict__ m = maps.input(blockIdx.y);
+    float *__restrict__ o = maps.output(blockIdx.y);
     const DevRing R = P.d_rings[r];
     const int L = R.len, Q = L / 4, k = min(it.y + lane, Q - 1);
     const int base = P.d_pair_base[r] - P.d_range[r].x;
@@ -963,28 +963,27 @@ cudaError_t launch_ring_range(const ConvPlan &p, const unsigned *bm, int n_maps,
 }
 
 cudaError_t launch_cap_direct(const ConvPlan &p, const int2 *d_items, int n_items,
-                              const int *d_first, const int *d_list, const float *d_in,
-                              float *d_out, int n_maps, long long map_stride, int band_lo,
-                              int band_hi, const int *flags, cudaStream_t st) {
+                              const int *d_first, const int *d_list, const MapSet &maps,
+                              int n_maps, int band_lo, int band_hi, const int *flags,
+                              cudaStream_t st) {
     if (n_items <= 0) return cudaSuccess;
     dim3 grid(n_items, n_maps);
-    cap_direct_kernel<<<grid, 256, 0, st>>>(p, d_items, d_first, d_list, d_in, d_out, map_stride,
-                                            band_lo, band_hi, flags);
+    cap_direct_kernel<<<grid, 256, 0, st>>>(p, d_items, d_first, d_list, maps, band_lo, band_hi,
+                                            flags);
     return cudaGetLastError();
 }
 
 cudaError_t launch_conv_cap_tc(const ConvPlan &p, const CapTc &c, const int2 *d_tiles, int n_tiles,
-                               const float *d_in, float *d_out, int n_maps, long long map_stride,
-                               int belt_split, int band_lo, int band_hi, const uint2 *rr,
-                               int *flags, int *d_err, cudaStream_t st) {
+                               const MapSet &maps, int n_maps, int belt_split, int band_lo,
+                               int band_hi, const uint2 *rr, int *flags, int *d_err, cudaStream_t st) {
     if (n_tiles <= 0) return cudaSuccess;
     const size_t smem = cap_smem(c);
     cudaError_t e = cudaFuncSetAttribute(conv_cap_tc_kernel,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     dim3 grid(n_tiles, n_maps);
-    conv_cap_tc_kernel<<<grid, kThreads, smem, st>>>(p, c, d_tiles, d_in, d_out, map_stride,
-                                                     belt_split, band_lo, band_hi, rr, flags, d_err);
+    conv_cap_tc_kernel<<<grid, kThreads, smem, st>>>(p, c, d_tiles, maps, belt_split, band_lo,
+                                                     band_hi, rr, flags, d_err);
     return cudaGetLastError();
 }
 

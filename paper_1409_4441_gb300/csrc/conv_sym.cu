@@ -624,7 +624,7 @@ __device__ __forceinline__ void sym_dispatch(const ConvPlan &P, int ring, int k0
 template <class S>
 __global__ void __launch_bounds__(S::T, S::MINB)
 conv_sym_kernel(const ConvPlan P, const WorkItem *__restrict__ items, int n_items,
-                const float *__restrict__ in, float *__restrict__ out, long long map_stride,
+                const MapSet maps,
                 int belt_split, int band_lo, int band_hi, int n_first,
                 const int *__restrict__ ring_flags, int *__restrict__ counters,
                 int *__restrict__ err) {
@@ -634,8 +634,8 @@ conv_sym_kernel(const ConvPlan P, const WorkItem *__restrict__ items, int n_item
     __shared__ int s_next;
     extern __shared__ float4 xt[];  // S::kXCap cells
     const int *rf = ring_flags + (long long)blockIdx.y * (P.nrings + 1);
-    const float *m = in + (long long)blockIdx.y * map_stride;
-    float *o = out + (long long)blockIdx.y * map_stride;
+    const float *__restrict__ m = maps.input(blockIdx.y);
+    float *__restrict__ o = maps.output(blockIdx.y);
     for (;;) {
         __syncthreads();  // every thread has read the previous claim
         if (threadIdx.x == 0) s_next = atomicAdd(&counters[blockIdx.y], 1);
@@ -709,26 +709,29 @@ cudaError_t sym_grid(K kernel, int threads, size_t dyn_smem, int n_items, int pe
 
 template <class S>
 cudaError_t sym_launch(const ConvPlan &p, const WorkItem *d_items, int n_items,
-                       const float *d_in, float *d_out, int n_maps, long long map_stride,
-                       int belt_split, int band_lo, int band_hi, int n_first,
-                       const int *ring_flags, int *d_err, cudaStream_t st) {
+                       const MapSet &maps, int n_maps, int belt_split, int band_lo, int band_hi,
+                       int n_first, const int *ring_flags, int *d_counters, int *d_err,
+                       cudaStream_t st) {
     int blocks = 0;
     cudaError_t e = sym_grid(conv_sym_kernel<S>, S::T, S::kDynSmem, n_items, 0, &blocks);
     if (e != cudaSuccess) return e;
-    // per-call claim counters, stream-ordered so that calls on several streams
-    // may overlap
-    int *ctr = nullptr;
+    // without the caller's counters, per-call ones, stream-ordered so that calls on several
+    // streams may overlap (taken here, behind the belt stage: in front of it the allocation
+    // of a first call, some 60 us, has nothing to hide behind)
+    int *ctr = d_counters;
     const size_t bytes = sizeof(int) * (size_t)n_maps;
-    if ((e = cudaMallocAsync(&ctr, bytes, st)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(ctr, 0, bytes, st)) == cudaSuccess) {
+    if (!ctr) {
+        if ((e = cudaMallocAsync(&ctr, bytes, st)) != cudaSuccess) return e;
+        e = cudaMemsetAsync(ctr, 0, bytes, st);
+    }
+    if (e == cudaSuccess) {
         dim3 grid(blocks, n_maps);
-        conv_sym_kernel<S><<<grid, S::T, S::kDynSmem, st>>>(p, d_items, n_items, d_in, d_out,
-                                                           map_stride, belt_split, band_lo,
-                                                           band_hi, n_first, ring_flags, ctr,
-                                                           d_err);
+        conv_sym_kernel<S><<<grid, S::T, S::kDynSmem, st>>>(p, d_items, n_items, maps, belt_split,
+                                                           band_lo, band_hi, n_first, ring_flags,
+                                                           ctr, d_err);
         e = cudaGetLastError();
     }
-    const cudaError_t f = cudaFreeAsync(ctr, st);
+    const cudaError_t f = d_counters ? cudaSuccess : cudaFreeAsync(ctr, st);
     return e != cudaSuccess ? e : f;
 }
 
@@ -744,15 +747,14 @@ int sym_classes(int len, int phase) {
 int sym_chunk(int nside) { return nside >= 2048 ? ShapeC3::kClasses : ShapeWide::kClasses; }
 
 cudaError_t launch_conv_sym(const ConvPlan &p, const WorkItem *d_items, int n_items,
-                            const float *d_in, float *d_out, int n_maps, long long map_stride,
-                            int belt_split, int band_lo, int band_hi, int n_first,
-                            const int *ring_flags, int *d_err, cudaStream_t st) {
+                            const MapSet &maps, int n_maps, int belt_split, int band_lo,
+                            int band_hi, int n_first, const int *ring_flags, int *d_counters,
+                            int *d_err, cudaStream_t st) {
     if (n_items <= 0 || n_maps <= 0) return cudaSuccess;
-    if (sym_chunk(p.nside) == ShapeC3::kClasses)
-        return sym_launch<ShapeC3>(p, d_items, n_items, d_in, d_out, n_maps, map_stride,
-                                   belt_split, band_lo, band_hi, n_first, ring_flags, d_err, st);
-    return sym_launch<ShapeWide>(p, d_items, n_items, d_in, d_out, n_maps, map_stride,
-                                 belt_split, band_lo, band_hi, n_first, ring_flags, d_err, st);
+    const auto launch = sym_chunk(p.nside) == ShapeC3::kClasses ? sym_launch<ShapeC3>
+                                                                : sym_launch<ShapeWide>;
+    return launch(p, d_items, n_items, maps, n_maps, belt_split, band_lo, band_hi, n_first,
+                  ring_flags, d_counters, d_err, st);
 }
 
 int sym_variants() { return 3; }

@@ -184,6 +184,30 @@ cudaError_t launch_conv_general(const ConvPlan &p, const WorkItem *d_items,
                                 int n_maps, long long map_stride, int belt_split,
                                 unsigned long long *d_count, cudaStream_t st);
 
+struct BatchEntry {
+    const float *in;
+    float *out;
+    int plan;        // index into the batch's ConvPlan array
+    int belt_split;  // 1: the belt kernel wrote this entry's belt-belt part
+};
+
+// The maps of a launch (blockIdx.y): a stack at a fixed stride, or a device table's entries
+// (a batch, whose captured launches outlive the maps of one run).
+struct MapSet {
+    const float *in = nullptr;
+    float *out = nullptr;
+    long long stride = 0;
+    const BatchEntry *table = nullptr;
+#ifdef __CUDACC__
+    __device__ __forceinline__ const float *input(int i) const {
+        return table ? table[i].in : in + i * stride;
+    }
+    __device__ __forceinline__ float *output(int i) const {
+        return table ? table[i].out : out + i * stride;
+    }
+#endif
+};
+
 // Circulant belt-belt kernel; items are (belt ring, first pixel) chunks of
 // belt_chunk() pixels; seg_cap floats per shared-memory buffer.
 int belt_chunk();
@@ -191,8 +215,7 @@ int belt_chunk();
 // are computed and written.
 struct BeltTc;
 cudaError_t launch_conv_belt(const ConvPlan &p, const int2 *d_items, int n_items,
-                             int seg_cap, const float *d_in, float *d_out, int n_maps,
-                             long long map_stride, const BeltTc *tc,
+                             int seg_cap, const MapSet &maps, int n_maps, const BeltTc *tc,
                              const unsigned char *tile_flags, int *d_err, cudaStream_t st);
 
 // Belt-belt ring pairs on the tensor cores (conv_belt_tc.cu): tiles of 16 belt rings x
@@ -208,15 +231,15 @@ int belt_tc_positions(int w, int L);      // window positions for a half window 
 bool belt_tc_plan(int nside, int wpos, int nq, BeltTc *t);
 int belt_tc_tiles(const ConvPlan &p, const BeltTc &t);
 long long map_blocks(const ConvPlan &p);  // blocks of 64 pixels in a map
-// bm[map][block] = bits of the block's largest |m|; map_blocks() words per map
-cudaError_t launch_block_max(const ConvPlan &p, const float *d_in, int n_maps,
-                             long long map_stride, unsigned *bm, cudaStream_t st);
+// bm[map][block] = bits of the block's largest |m|; map_blocks() words per map; clears
+// zero[0 .. n_zero)
+cudaError_t launch_block_max(const ConvPlan &p, const MapSet &maps, int n_maps, unsigned *bm,
+                             int *zero, long long n_zero, cudaStream_t st);
 // Writes output rings [r0, r1] of the belt but for the tiles it flags (tiles whose values
 // span too wide a range, or are not finite), which launch_conv_belt then computes.
-cudaError_t launch_conv_belt_tc(const ConvPlan &p, const BeltTc &t, const float *d_in,
-                                float *d_out, int n_maps, long long map_stride, int r0, int r1,
-                                const unsigned *bm, unsigned char *flags, int *d_err,
-                                cudaStream_t st);
+cudaError_t launch_conv_belt_tc(const ConvPlan &p, const BeltTc &t, const MapSet &maps,
+                                int n_maps, int r0, int r1, const unsigned *bm,
+                                unsigned char *flags, int *d_err, cudaStream_t st);
 
 // Ring pairs with a cap ring on the tensor cores (conv_cap_tc.cu): tiles {rings - 1 << 16 |
 // first ring, sectors << 16 | sector} of rings ring_first .. ring_end and their mirrors.
@@ -243,9 +266,9 @@ cudaError_t launch_cap_coef(const ConvPlan &p, const CapTc &c, const CapCoef &k,
 // Adds the irregular ring pairs (list[list_first[r]] .. of output ring r) of rings that are
 // not flagged; items {ring, first of 32 first-quarter positions}.
 cudaError_t launch_cap_direct(const ConvPlan &p, const int2 *d_items, int n_items,
-                              const int *d_first, const int *d_list, const float *d_in,
-                              float *d_out, int n_maps, long long map_stride, int band_lo,
-                              int band_hi, const int *flags, cudaStream_t st);
+                              const int *d_first, const int *d_list, const MapSet &maps,
+                              int n_maps, int band_lo, int band_hi, const int *flags,
+                              cudaStream_t st);
 int cap_tc_span();                       // input positions of a tile
 int cap_tc_degree();                     // of the cells' polynomials
 int cap_tc_positions(int w, int L);
@@ -256,9 +279,9 @@ cudaError_t launch_ring_range(const ConvPlan &p, const unsigned *bm, int n_maps,
 // band_hi] but for the ring pairs it flags (flags[map][ring], flags[map][nrings]: any),
 // which conv_sym_kernel then computes; flags must be zero at launch.
 cudaError_t launch_conv_cap_tc(const ConvPlan &p, const CapTc &c, const int2 *d_tiles, int n_tiles,
-                               const float *d_in, float *d_out, int n_maps, long long map_stride,
-                               int belt_split, int band_lo, int band_hi, const uint2 *rr,
-                               int *flags, int *d_err, cudaStream_t st);
+                               const MapSet &maps, int n_maps, int belt_split, int band_lo,
+                               int band_hi, const uint2 *rr, int *flags, int *d_err,
+                               cudaStream_t st);
 
 // tcgen05 multi-map kernel for belt ring pairs: items are (belt ring, first
 // pixel) blocks of belt_mma_block() outputs; maps in groups of belt_mma_maps().
@@ -277,14 +300,13 @@ cudaError_t launch_conv_belt_mma(const ConvPlan &p, const int2 *d_items, int n_i
 // chunks of sym_chunk(nside) classes (the tile launch_conv_sym uses for that nside).
 int sym_chunk(int nside);
 int sym_classes(int len, int phase);  // reflection classes of a ring's first quarter
-// CTAs claim items in list order through per-call counters taken from the
-// stream-ordered allocator.  Items from n_first on are taken only where ring_flags
+// CTAs claim items in list order through a counter per map (d_counters, zero at
+// launch, or NULL: taken from the stream-ordered allocator).  Items from n_first on are taken only where ring_flags
 // ([map][nrings + 1], the last word: any) says so (n_first = n_items: no flags).
 cudaError_t launch_conv_sym(const ConvPlan &p, const WorkItem *d_items, int n_items,
-                            const float *d_in, float *d_out, int n_maps,
-                            long long map_stride, int belt_split, int band_lo,
-                            int band_hi, int n_first, const int *ring_flags, int *d_err,
-                            cudaStream_t st);
+                            const MapSet &maps, int n_maps, int belt_split, int band_lo,
+                            int band_hi, int n_first, const int *ring_flags, int *d_counters,
+                            int *d_err, cudaStream_t st);
 
 // ---------------------------------------------------------------------------
 // Batched persistent launches (csrc/batch.cpp).  An entry is one map convolved
@@ -295,12 +317,6 @@ cudaError_t launch_conv_sym(const ConvPlan &p, const WorkItem *d_items, int n_it
 // (sym_variant_chunk(v) reflection classes per item).  CTAs claim items from *d_counter,
 // which must be zero at launch.  per_sm_cap > 0 caps the resident CTAs per SM.
 // ---------------------------------------------------------------------------
-struct BatchEntry {
-    const float *in;
-    float *out;
-    int plan;        // index into the batch's ConvPlan array
-    int belt_split;  // 1: the belt kernel wrote this entry's belt-belt part
-};
 int belt_variant_chunk(int variant);  // variants 0, 1
 int sym_variants();                   // number of gather variants
 int sym_variant_chunk(int variant);
@@ -417,3 +433,25 @@ struct ksc_split {
     cudaStream_t own_stream = nullptr;
     float *d_io = nullptr;  // 2 * npix floats, allocated on first host call
 };
+
+namespace ksc {
+// A convolution's scratch: the maps' block maxima and ring ranges, the flags of the
+// tensor-core tiles and rings, the gather's claim counters.
+struct ConvScratch {
+    unsigned *bm = nullptr;
+    uint2 *ranges = nullptr;
+    int *cap_flags = nullptr;
+    int *counters = nullptr;
+    unsigned char *belt_flags = nullptr;
+};
+bool has_cap_tc(const ksc_split *s);
+size_t conv_scratch_bytes(const ksc_split *s, int n_maps);
+// Lays the scratch out in mem and starts the launches that fill it.
+cudaError_t start_conv_scratch(const ksc_split *s, const MapSet &maps, int n_maps, void *mem,
+                               ConvScratch *w, cudaStream_t st);
+cudaError_t launch_belt(const ksc_split *s, const MapSet &maps, int n_maps, int r0, int r1,
+                        const ConvScratch &w, int *d_err, cudaStream_t st);
+cudaError_t launch_caps(const ksc_split *s, const MapSet &maps, int n_maps, int lo, int hi,
+                        int r0, int r1, bool stack, const ConvScratch &w, int *d_err,
+                        cudaStream_t st);
+}  // namespace ksc
