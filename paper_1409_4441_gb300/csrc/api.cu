@@ -609,6 +609,13 @@ int finish_split(ksc_split *s, const ksc_split_opts &o) {
         return cuda_fail(e, "upload work list");
     if ((e = dev_upload(&s->d_items_mma, items_mma.data(), items_mma.size())) != cudaSuccess)
         return cuda_fail(e, "upload work list");
+    // the coefficients are the one large table: without room for them the gather sums the caps
+    if (s->n_cap_tiles && cudaMalloc(&s->d_coef, 16ull * cap.coef_off.back()) != cudaSuccess) {
+        cudaGetLastError();
+        s->d_coef = nullptr;
+        s->n_cap_tiles = 0;
+        s->ctc = ksc::CapTc();
+    }
     if (s->n_cap_tiles) {
         if ((e = dev_upload(&s->d_cap_tiles, cap.tiles.data(), cap.tiles.size())) != cudaSuccess ||
             (e = dev_upload(&s->d_cap_tiles_lpt, cap_tiles_lpt.data(), cap_tiles_lpt.size())) !=
@@ -617,9 +624,8 @@ int finish_split(ksc_split *s, const ksc_split_opts &o) {
             (e = dev_upload(&s->d_coef_off, cap.coef_off.data(), cap.coef_off.size())) != cudaSuccess ||
             (e = dev_upload(&s->d_irr_items, cap.irr_items.data(), cap.irr_items.size())) != cudaSuccess ||
             (e = dev_upload(&s->d_irr_first, cap.irr_first.data(), cap.irr_first.size())) != cudaSuccess ||
-            (e = dev_upload(&s->d_irr, cap.irr.data(), cap.irr.size())) != cudaSuccess ||
-            (e = dev_malloc((void **)&s->d_coef, 16ull * cap.coef_off.back())) != cudaSuccess)
-            return cuda_fail(e, "cap tiles and coefficients");
+            (e = dev_upload(&s->d_irr, cap.irr.data(), cap.irr.size())) != cudaSuccess)
+            return cuda_fail(e, "cap tiles");
     }
     if ((e = dev_malloc((void **)&s->d_err, sizeof(int))) != cudaSuccess)
         return cuda_fail(e, "error flag");
@@ -757,7 +763,8 @@ struct CallScratch : ksc::ConvScratch {
     }
 };
 
-// Takes the scratch and starts the launches that fill it.
+// Takes the scratch and starts the launches that fill it.  Without room for it (npix / 16
+// bytes a map) the FFMA kernels do it all.
 cudaError_t start_scratch(const ksc_split *s, const ksc::MapSet &maps, int n_maps,
                           cudaStream_t st, CallScratch *w) {
     const size_t bytes = ksc::conv_scratch_bytes(s, n_maps);
@@ -766,7 +773,9 @@ cudaError_t start_scratch(const ksc_split *s, const ksc::MapSet &maps, int n_map
     const cudaError_t e = cudaMallocAsync(&w->mem, bytes, st);
     if (e != cudaSuccess) {
         w->mem = nullptr;
-        return e;
+        if (e != cudaErrorMemoryAllocation) return e;
+        cudaGetLastError();
+        return cudaSuccess;
     }
     return ksc::start_conv_scratch(s, maps, n_maps, w->mem, w, st);
 }
@@ -882,7 +891,7 @@ cudaError_t launch_belt(const ksc_split *s, const MapSet &maps, int n_maps, int 
                         const ConvScratch &w, int *d_err, cudaStream_t st) {
     const int a = s->ring_first_belt[r0], b = s->ring_first_belt[r1 + 1];
     if (a == b || s->n_items_belt == 0) return cudaSuccess;
-    if (s->btc.n_cols == 0)
+    if (!w.belt_flags)
         return launch_conv_belt(s->plan, s->d_items_belt + a, b - a, s->seg_cap, maps, n_maps,
                                 nullptr, nullptr, d_err, st);
     const cudaError_t e = launch_conv_belt_tc(s->plan, s->btc, maps, n_maps, r0, r1, w.bm,
@@ -912,7 +921,7 @@ cudaError_t launch_caps(const ksc_split *s, const MapSet &maps, int n_maps, int 
     }
     const int c = s->ring_first_sym[lo], d = s->ring_first_sym[hi + 1];
     const WorkItem *its = whole ? s->d_items_sym_lpt : s->d_items_sym + c;
-    if (!has_cap_tc(s))
+    if (!w.cap_flags)
         return launch_conv_sym(s->plan, its, d - c, maps, n_maps, belt_split, r0, r1, d - c,
                                     nullptr, w.counters, d_err, st);
     // the tensor-core stage, the irregular ring pairs, then the gather for the rings that

@@ -786,15 +786,17 @@ cap_coef_kernel(const ConvPlan P, const CapTc C, const CapCoef K, int ring_lo, i
 }
 
 // The irregular ring pairs of output ring r (and its mirror), added to the output.  A block
-// takes 32 first-quarter positions of r, a lane each; its eight warps share the ring's list
-// of input rings.  For one input pixel all lanes read the same values, eight (four quarter
-// turns, two hemispheres) per weight.
-__global__ void __launch_bounds__(256)
+// takes 32 first-quarter positions of r, a lane each; its sixteen warps share the ring's list
+// of input rings (99 blocks for 152 SMs at nside 1024, 160': 330 us with eight warps, 281 us
+// with sixteen; 612 blocks at 2048, 240': 6.60 and 6.47 ms).  For one input pixel all lanes
+// read the same values, eight (four quarter turns, two hemispheres) per weight.
+constexpr int kDirect = 512;
+__global__ void __launch_bounds__(kDirect)
 cap_direct_kernel(const ConvPlan P, const int2 *__restrict__ items,
                   const int *__restrict__ list_first, const int *__restrict__ list,
-                  const MapSet maps,
-                  int band_lo, int band_hi, const int *__restrict__ flags) {
-    __shared__ float part[8][8][32];
+                  const MapSet maps, int band_lo, int band_hi, const int *__restrict__ flags) {
+    constexpr int kW = kDirect / 32;
+    __shared__ float part[kW][8][32];
     const int2 it = items[blockIdx.x];
     const int r = it.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (flags[(long long)blockIdx.y * (P.nrings + 1) + r]) return;
@@ -806,7 +808,7 @@ cap_direct_kernel(const ConvPlan P, const int2 *__restrict__ items,
     float sum[8], comp[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) sum[i] = comp[i] = 0.0f;
-    for (int e = list_first[r] + warp; e < list_first[r + 1]; e += 8) {
+    for (int e = list_first[r] + warp; e < list_first[r + 1]; e += kW) {
         const int q = list[e];
         const DevRing G = P.d_rings[q];
         const int Lq = G.len, Qq = Lq / 4;
@@ -850,13 +852,14 @@ cap_direct_kernel(const ConvPlan P, const int2 *__restrict__ items,
 #pragma unroll
     for (int i = 0; i < 8; ++i) part[warp][i][lane] = sum[i] - comp[i];
     __syncthreads();
+    if (warp >= 8) return;
     // image `warp` of every position: the warps' sums in order
     const int a = warp & 3, south = warp >> 2;
     const int rs = P.nrings - 1 - r, ring = south ? rs : r;
     if (it.y + lane < Q && ring >= band_lo && ring <= band_hi && !(south && rs == r)) {
         float s = 0.0f, c = 0.0f;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < kW; ++i) {
             const float y = part[i][warp][lane] - c, t = s + y;
             c = (t - s) - y;
             s = t;
@@ -968,7 +971,7 @@ cudaError_t launch_cap_direct(const ConvPlan &p, const int2 *d_items, int n_item
                               cudaStream_t st) {
     if (n_items <= 0) return cudaSuccess;
     dim3 grid(n_items, n_maps);
-    cap_direct_kernel<<<grid, 256, 0, st>>>(p, d_items, d_first, d_list, maps, band_lo, band_hi,
+    cap_direct_kernel<<<grid, kDirect, 0, st>>>(p, d_items, d_first, d_list, maps, band_lo, band_hi,
                                             flags);
     return cudaGetLastError();
 }

@@ -29,6 +29,7 @@
 // pi J / L with the exact integer J = m (2k + t) mod 2L; the twiddles advance by one complex
 // product per step and are re-anchored from the exact J every 8 steps (the products'
 // rounding drifts by about one FP32 ulp per step in between).
+#include <algorithm>
 #include <cstdint>
 
 #include "ksc_internal.h"
@@ -38,7 +39,6 @@ namespace {
 
 constexpr double kPi = 3.14159265358979323846;
 constexpr int kAnchor = 8;        // twiddle steps between exact re-anchors
-constexpr double kScale = 120.0;  // log2 of one scale step of the recurrence
 
 __host__ __device__ inline long long n_alm(int lmax) {
     return (long long)(lmax + 1) * (lmax + 2) / 2;
@@ -47,42 +47,16 @@ __host__ __device__ inline long long alm_base(int lmax, int m) {  // index(0, m)
     return (long long)m * (2 * lmax + 1 - m) / 2;
 }
 
-// Ring r (0-based) of nside n: z, sin theta (FP64, 1 - z kept exact near the
-// north pole), pixel count, first pixel, phase flag.
+// Ring r (0-based) of nside n: pixel count, first pixel, phase flag.
 struct ShtRing {
-    double z, s;
     int len, start, t;
 };
-__device__ inline ShtRing sht_ring(int n, int r) {
-    const long long i = r + 1;
-    const double nn = (double)n;
-    ShtRing g;
-    double omz, opz;
-    if (i < n) {
-        omz = (double)(i * i) / (3.0 * nn * nn);
-        g.z = 1.0 - omz;
-        opz = 1.0 + g.z;
-        g.len = (int)(4 * i);
-        g.start = (int)(2 * i * (i - 1));
-        g.t = 1;
-    } else if (i <= 3LL * n) {
-        g.z = (double)(4LL * n - 2 * i) / (3.0 * nn);
-        omz = 1.0 - g.z;
-        opz = 1.0 + g.z;
-        g.len = 4 * n;
-        g.start = (int)(2LL * n * (n - 1) + 4LL * n * (i - n));
-        g.t = ((i - n) % 2 == 0) ? 1 : 0;
-    } else {
-        const long long ip = 4LL * n - i;
-        opz = (double)(ip * ip) / (3.0 * nn * nn);
-        g.z = opz - 1.0;
-        omz = 1.0 - g.z;
-        g.len = (int)(4 * ip);
-        g.start = (int)(12LL * n * n - 2 * ip * (ip + 1));
-        g.t = 1;
-    }
-    g.s = sqrt(omz * opz);
-    return g;
+__device__ __forceinline__ ShtRing sht_ring(int n, int r) {
+    const int i = r + 1;
+    if (i < n) return {4 * i, 2 * i * (i - 1), 1};
+    if (i <= 3 * n) return {4 * n, 2 * n * (n - 1) + 4 * n * (i - n), (i - n) % 2 == 0 ? 1 : 0};
+    const int ip = 4 * n - i;
+    return {4 * ip, 12 * n * n - 2 * ip * (ip + 1), 1};
 }
 
 // ---- FP32 pairs (hi + lo) -----------------------------------------------------
@@ -112,35 +86,117 @@ __device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
     return f2_norm(s, ((a.h - (s - t)) + (b.h - t)) + (a.l + b.l));
 }
 
+__device__ __forceinline__ F2 f2_of(int v) {  // |v| below 2^30, exact
+    F2 r;
+    r.h = __int2float_rn(v);
+    r.l = (float)(v - __float2int_rn(r.h));
+    return r;
+}
+__device__ __forceinline__ F2 f2_div(F2 a, F2 b) {
+    const float q = a.h / b.h;
+    return f2_norm(q, (fmaf(-q, b.h, a.h) + fmaf(-q, b.l, a.l)) / b.h);
+}
+__device__ __forceinline__ F2 f2_sqrt(F2 a) {
+    const float q = sqrtf(a.h);
+    return q > 0.0f ? f2_norm(q, (fmaf(-q, q, a.h) + a.l) * (0.5f / q)) : F2{0.0f, 0.0f};
+}
+__device__ __forceinline__ F2 f2_sum(float a, float b) {  // a + b exactly
+    const float s = a + b, t = s - a;
+    return F2{s, (a - (s - t)) + (b - t)};
+}
+// s + p with s.l left to collect the rounding errors (folded in at the end): three operations
+// less than f2_add, and |s.l| stays far below |s.h| over the few thousand terms of a sum.
+__device__ __forceinline__ F2 f2_acc(F2 s, F2 p) {
+    const float t = s.h + p.h, u = t - s.h;
+    return F2{t, s.l + (((s.h - (t - u)) + (p.h - u)) + p.l)};
+}
+
+// z and sin(theta) of northern ring r (0-based) or the equator as pairs, from whole numbers
+// below 2^30: in the cap 1 - z = i^2 / 3n^2, in the belt z = (4n - 2i) / 3n = a / 3n and
+// sin^2 = (3n - a)(3n + a) / 9n^2.  (In FP64 the rings, powers and
+// coefficients of a block cost as much as its recurrences: 36 and 26 us for the two Legendre
+// kernels at nside 128, l_max 64, against 26 and 16 us.)
+__device__ __forceinline__ void ring_zs(int n, int r, F2 *z, F2 *s) {
+    const int i = r + 1;
+    if (i < n) {
+        const F2 w = f2_div(f2_of(i * i), f2_of(3 * n * n));
+        *z = f2_add(F2{1.0f, 0.0f}, F2{-w.h, -w.l});
+        *s = f2_sqrt(f2_mul(w, f2_add(F2{2.0f, 0.0f}, F2{-w.h, -w.l})));
+    } else {
+        const int a = 4 * n - 2 * i, d = 3 * n;
+        *z = f2_div(f2_of(a), f2_of(d));
+        *s = f2_sqrt(f2_div(f2_of((d - a) * (d + a)), f2_of(d * d)));
+    }
+}
+
 // Orders above this do not reach 2^-60 on a ring (see the top of the file).
-__device__ __forceinline__ int order_limit(int lmax, double s) {
-    const float lim = (float)lmax * (float)s + 16.0f + 9.0f * cbrtf((float)lmax);
-    return min(lmax, (int)lim);
+__device__ __forceinline__ int order_limit(int lmax, float s) {
+    return min(lmax, (int)((float)lmax * s + 16.0f + 9.0f * cbrtf((float)lmax)));
+}
+__device__ __forceinline__ int ring_limit(int nside, int r, int lmax) {
+    F2 z, s;
+    ring_zs(nside, r, &z, &s);
+    return order_limit(lmax, s.h);
 }
 
-// log2 lambda_mm - m log2 sin(theta)
-__device__ inline double log2_norm(int m) {
-    return 0.5 * log2((2.0 * m + 1.0) / (4.0 * kPi)) +
-           0.5 * (lgamma(2.0 * m + 1.0) - 2.0 * lgamma(m + 1.0)) / log(2.0) - m;
+// lambda_mm / sin^m theta = sqrt((2m + 1) / 4pi C), C = prod_{k<=m} (2k - 1) / 2k: the product
+// (a factor a lane, by all lanes of a warp), or the series of Gamma(m + 1/2) / Gamma(m + 1)
+// for large m (the next term is below 1e-11).
+__device__ inline F2 norm_mm(int m) {
+    double c;
+    if (m <= 32) {
+        const int k = (threadIdx.x & 31) + 1;
+        c = k <= m ? (2.0 * k - 1.0) / (2.0 * k) : 1.0;
+        for (int o = 16; o > 0; o >>= 1) c *= __shfl_xor_sync(~0u, c, o);
+        c *= c;
+    } else {
+        const double x = 1.0 / m;
+        const double p = 1.0 + x * (-1.0 / 8 + x * (1.0 / 128 + x * (5.0 / 1024 + x * (-21.0 / 32768 +
+                                                                  x * (-399.0 / 262144)))));
+        c = x / kPi * p * p;
+    }
+    return f2_of(sqrt(sqrt(c) * ((2.0 * m + 1.0) / (4.0 * kPi))));
 }
 
-// The recurrence of one (ring, order): v1 = lambda_{l}, v2 = lambda_{l-1}, both 2^(120 e)
+// x = mantissa 2^ex with the mantissa's high part in [1, 2)
+__device__ __forceinline__ F2 f2_mant(F2 x, int *ex) {
+    const int e = ((__float_as_int(x.h) >> 23) & 255) - 127;
+    const float q = __int_as_float((127 - e) << 23);  // |e| stays below 100 here
+    *ex += e;
+    return F2{x.h * q, x.l * q};
+}
+
+// The recurrence of one (ring, order): v1 = lambda_{l}, v2 = lambda_{l-1}, both 2^(-120 e)
 // times the true values.
 struct Rec {
     F2 z, v1, v2;
     int e;
-    __device__ __forceinline__ void start(int m, double lg0, const ShtRing &g) {
-        z = f2_of(g.z);
-        const double lg = lg0 + (m > 0 ? m * log2(g.s) : 0.0);
-        e = min(0, (int)floor((lg + 60.0) / kScale));
-        v1 = f2_of(exp2(lg - kScale * e));
+    // v1 = norm s^m by binary powers (relative error below m 2^-46)
+    __device__ __forceinline__ void start(int m, F2 norm, F2 zz, F2 s) {
+        z = zz;
+        int ex = 0, eb = 0;
+        F2 b = f2_mant(s, &eb), v = f2_mant(norm, &ex);
+        for (int k = m; k; k >>= 1) {
+            if (k & 1) {
+                v = f2_mul(v, b);
+                ex += eb;
+                v = f2_mant(f2_norm(v.h, v.l), &ex);
+            }
+            b = f2_mul(b, b);
+            eb *= 2;
+            b = f2_mant(f2_norm(b.h, b.l), &eb);
+        }
+        // e = min(0, floor((ex + 60) / 120)): below 2^60 in v1, above 2^-60 once e = 0
+        e = min(0, (ex + 60 - (ex + 60 < 0 ? 119 : 0)) / 120);
+        const float q = __int_as_float((127 + ex - 120 * e) << 23);
+        v1 = F2{v.h * q, v.l * q};
         v2 = F2{0.0f, 0.0f};
     }
     // lambda_{l+1} = A (z lambda_l - B lambda_{l-1}), c = A as a pair, B as a pair
     __device__ __forceinline__ void step(float4 c) {
         const F2 x = f2_mul(z, v1), y = f2_mul(F2{c.z, c.w}, v2);
         const float d = x.h - y.h, t = d - x.h;
-        const F2 w = f2_norm(d, ((x.h - (d - t)) - (y.h + t)) + (x.l - y.l));
+        const F2 w{d, ((x.h - (d - t)) - (y.h + t)) + (x.l - y.l)};
         const F2 r = f2_mul(F2{c.x, c.y}, w);
         v2 = v1;
         v1 = f2_norm(r.h, r.l);
@@ -154,11 +210,12 @@ struct Rec {
 
 constexpr int kTile = 128;  // degrees whose coefficients a block stages at a time
 
-// Coefficients of the step to degree l (l > m): A_l and B_l = 1 / A_{l-1} (0 at l = m + 1).
-__device__ inline float4 step_coeffs(int l, int m) {
-    const double ll = (double)l, mm = (double)m, l1 = ll - 1.0;
-    const F2 a = f2_of(sqrt((4.0 * ll * ll - 1.0) / ((ll - mm) * (ll + mm))));
-    const F2 b = l > m + 1 ? f2_of(sqrt((l1 - mm) * (l1 + mm) / (4.0 * l1 * l1 - 1.0))) : F2{0.0f, 0.0f};
+// Coefficients of the step to degree l (l > m): A_l and B_l = 1 / A_{l-1} (0 at l = m + 1),
+// A_l^2 = (4 l^2 - 1) / (l^2 - m^2), whole numbers below 2^28.
+__device__ __forceinline__ float4 step_coeffs(int l, int m) {
+    const F2 a = f2_sqrt(f2_div(f2_of(4 * l * l - 1), f2_of((l - m) * (l + m))));
+    const int k = l - 1;
+    const F2 b = f2_sqrt(f2_div(f2_of((k - m) * (k + m)), f2_of(4 * k * k - 1)));
     return make_float4(a.h, a.l, b.h, b.l);
 }
 
@@ -169,10 +226,13 @@ template <int R>
 __global__ void __launch_bounds__(256)
 sht_leg_synth(int nside, int lmax, const double2 *__restrict__ alm, float2 *__restrict__ G) {
     __shared__ float4 co[kTile], al[kTile];
-    __shared__ double s_lg;
+    __shared__ F2 s_norm;
     const int m = blockIdx.y, nnorth = 2 * nside, nr = 4 * nside - 1;
     const int r0 = blockIdx.x * 256 * R + threadIdx.x;
-    if (threadIdx.x == 0) s_lg = log2_norm(m);
+    if (threadIdx.x < 32) {
+        const F2 v = norm_mm(m);
+        if (threadIdx.x == 0) s_norm = v;
+    }
     __syncthreads();
     Rec rec[R];
     F2 er[R], ei[R], od[R], oi[R];  // even / odd (l - m) sums
@@ -183,9 +243,10 @@ sht_leg_synth(int nside, int lmax, const double2 *__restrict__ alm, float2 *__re
         er[j] = ei[j] = od[j] = oi[j] = F2{0.0f, 0.0f};
         live[j] = false;
         if (r < nnorth) {
-            const ShtRing g = sht_ring(nside, r);
-            live[j] = m <= order_limit(lmax, g.s);
-            if (live[j]) rec[j].start(m, s_lg, g);
+            F2 z, s;
+            ring_zs(nside, r, &z, &s);
+            live[j] = m <= order_limit(lmax, s.h);
+            if (live[j]) rec[j].start(m, s_norm, z, s);
         }
         any |= live[j];
     }
@@ -213,11 +274,11 @@ sht_leg_synth(int nside, int lmax, const double2 *__restrict__ alm, float2 *__re
                 if (rec[j].e < 0) continue;
                 const F2 pr = f2_mul(rec[j].v1, F2{x.x, x.y}), pi = f2_mul(rec[j].v1, F2{x.z, x.w});
                 if (odd) {
-                    od[j] = f2_add(od[j], pr);
-                    oi[j] = f2_add(oi[j], pi);
+                    od[j] = f2_acc(od[j], pr);
+                    oi[j] = f2_acc(oi[j], pi);
                 } else {
-                    er[j] = f2_add(er[j], pr);
-                    ei[j] = f2_add(ei[j], pi);
+                    er[j] = f2_acc(er[j], pr);
+                    ei[j] = f2_acc(ei[j], pi);
                 }
             }
         }
@@ -237,25 +298,30 @@ sht_leg_synth(int nside, int lmax, const double2 *__restrict__ alm, float2 *__re
     }
 }
 
+constexpr int kGroup = 32;  // degrees between the block's reductions
+
 // Analysis, Legendre part: alm[l, m] = c K_l sum_rings lambda_lm(z) F_m over all northern
 // rings and their mirrors for order m = lmax - blockIdx.x; c = 4 pi / Npix, K_l = kl[l] (kl
 // NULL: 1).  One block per order, R rings a thread, in passes over the rings.  The
 // threads' terms of eight degrees go through shared memory: within a warp 32 -> 4 partial
-// sums a degree, then over the warps, in a fixed order and on FP32 pairs throughout.  The
+// sums a degree, then every 32 degrees over the warps, in a fixed order and on FP32 pairs throughout.  The
 // F_m enter divided by the power of two that covers the number of rings (exact; c carries it
 // back), so that a sum over all rings stays in range wherever the F_m do.
 template <int R>
 __global__ void __launch_bounds__(256)
 sht_leg_anal(int nside, int lmax, const float2 *__restrict__ F, const double *__restrict__ kl,
-             double scale, double c, double2 *__restrict__ alm) {
+             float scale, double c, double2 *__restrict__ alm) {
     extern __shared__ float4 acc[];  // [lmax + 1 - m]: re, im pairs
-    __shared__ float4 co[kTile], term[8][8][33], part[8][8];
-    __shared__ double s_lg;
+    __shared__ float4 co[kTile], term[8][8][33], part[8][kGroup];
+    __shared__ F2 s_norm;
     const int m = lmax - blockIdx.x, nnorth = 2 * nside, nr = 4 * nside - 1;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long stride = lmax + 1;
     for (int i = threadIdx.x; i <= lmax - m; i += 256) acc[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    if (threadIdx.x == 0) s_lg = log2_norm(m);
+    if (threadIdx.x < 32) {
+        const F2 v = norm_mm(m);
+        if (threadIdx.x == 0) s_norm = v;
+    }
     __syncthreads();
     for (int base = 0; base < nnorth; base += 256 * R) {
         Rec rec[R];
@@ -266,17 +332,20 @@ sht_leg_anal(int nside, int lmax, const float2 *__restrict__ F, const double *__
             const int r = base + 256 * j + threadIdx.x;
             live[j] = false;
             if (r < nnorth) {
-                const ShtRing g = sht_ring(nside, r);
-                live[j] = m <= order_limit(lmax, g.s);
+                F2 z, s;
+                ring_zs(nside, r, &z, &s);
+                live[j] = m <= order_limit(lmax, s.h);
                 if (live[j]) {
-                    rec[j].start(m, s_lg, g);
+                    rec[j].start(m, s_norm, z, s);
                     const int rs = nr - 1 - r;
                     const float2 fn = F[(long long)r * stride + m];
                     const float2 fs = rs != r ? F[(long long)rs * stride + m] : make_float2(0.0f, 0.0f);
-                    sr[j] = f2_of(scale * ((double)fn.x + (double)fs.x));
-                    si[j] = f2_of(scale * ((double)fn.y + (double)fs.y));
-                    dr[j] = f2_of(scale * ((double)fn.x - (double)fs.x));
-                    di[j] = f2_of(scale * ((double)fn.y - (double)fs.y));
+                    const float nx = scale * fn.x, ny = scale * fn.y;
+                    const float sx = scale * fs.x, sy = scale * fs.y;
+                    sr[j] = f2_sum(nx, sx);
+                    si[j] = f2_sum(ny, sy);
+                    dr[j] = f2_sum(nx, -sx);
+                    di[j] = f2_sum(ny, -sy);
                 }
             }
             any |= live[j];
@@ -289,8 +358,9 @@ sht_leg_anal(int nside, int lmax, const float2 *__restrict__ F, const double *__
             for (int i = threadIdx.x; i < n; i += 256)
                 if (l0 + i > m) co[i] = step_coeffs(l0 + i, m);
             __syncthreads();
-            for (int i0 = 0; i0 < n; i0 += 8) {
-                if (warp_any) {
+            for (int g0 = 0; g0 < n; g0 += kGroup) {
+                if (!warp_any) part[warp][lane] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                for (int i0 = g0; warp_any && i0 < g0 + kGroup; i0 += 8) {
 #pragma unroll 2
                     for (int i = 0; i < 8; ++i) {
                         F2 tr{0.0f, 0.0f}, ti{0.0f, 0.0f};
@@ -302,8 +372,8 @@ sht_leg_anal(int nside, int lmax, const float2 *__restrict__ F, const double *__
                                 if (!live[j]) continue;
                                 if (l0 + i0 + i > m) rec[j].step(cc);
                                 if (rec[j].e < 0) continue;
-                                tr = f2_add(tr, f2_mul(rec[j].v1, odd ? dr[j] : sr[j]));
-                                ti = f2_add(ti, f2_mul(rec[j].v1, odd ? di[j] : si[j]));
+                                tr = f2_acc(tr, f2_mul(rec[j].v1, odd ? dr[j] : sr[j]));
+                                ti = f2_acc(ti, f2_mul(rec[j].v1, odd ? di[j] : si[j]));
                             }
                         }
                         term[warp][i][lane] = make_float4(tr.h, tr.l, ti.h, ti.l);
@@ -327,13 +397,12 @@ sht_leg_anal(int nside, int lmax, const float2 *__restrict__ F, const double *__
                         tr = f2_add(tr, x);
                         ti = f2_add(ti, y);
                     }
-                    if ((lane & 3) == 0) part[warp][lane >> 2] = make_float4(tr.h, tr.l, ti.h, ti.l);
-                } else if (lane < 8) {
-                    part[warp][lane] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                    if ((lane & 3) == 0) part[warp][i0 - g0 + (lane >> 2)] = make_float4(tr.h, tr.l, ti.h, ti.l);
+                    __syncwarp();
                 }
                 __syncthreads();
-                if (threadIdx.x < 8 && i0 + (int)threadIdx.x < n) {
-                    const float4 o = acc[l0 - m + i0 + threadIdx.x];
+                if (threadIdx.x < kGroup && g0 + (int)threadIdx.x < n) {
+                    const float4 o = acc[l0 - m + g0 + threadIdx.x];
                     F2 tr{o.x, o.y}, ti{o.z, o.w};
 #pragma unroll
                     for (int k = 0; k < 8; ++k) {
@@ -341,7 +410,7 @@ sht_leg_anal(int nside, int lmax, const float2 *__restrict__ F, const double *__
                         tr = f2_add(tr, F2{t.x, t.y});
                         ti = f2_add(ti, F2{t.z, t.w});
                     }
-                    acc[l0 - m + i0 + threadIdx.x] = make_float4(tr.h, tr.l, ti.h, ti.l);
+                    acc[l0 - m + g0 + threadIdx.x] = make_float4(tr.h, tr.l, ti.h, ti.l);
                 }
                 __syncthreads();
             }
@@ -395,7 +464,7 @@ sht_ring_synth(int nside, int lmax, int r_first, const float2 *__restrict__ G,
     const bool mirror = rs != r;
     const long long stride = lmax + 1;
     const ShtRing g = sht_ring(nside, r), h = sht_ring(nside, rs);
-    const int L = g.len, Q = L / 4, lim = order_limit(lmax, g.s);
+    const int L = g.len, Q = L / 4, lim = ring_limit(nside, r, lmax);
     const float fl = (float)L, inv_l = 1.0f / fl;
     for (int k0 = blockIdx.y * 256; k0 < Q; k0 += gridDim.y * 256) {
         const int k = k0 + threadIdx.x;
@@ -481,7 +550,7 @@ sht_ring_anal(int nside, int lmax, int r_first, const float *__restrict__ map,
     const bool mirror = rs != r;
     const long long stride = lmax + 1;
     const ShtRing g = sht_ring(nside, r), h = sht_ring(nside, rs);
-    const int L = g.len, Q = L / 4, lim = order_limit(lmax, g.s);
+    const int L = g.len, Q = L / 4, lim = ring_limit(nside, r, lmax);
     const float fl = (float)L, inv_l = 1.0f / fl;
     for (int m0 = blockIdx.y * 256; m0 <= lim; m0 += gridDim.y * 256) {
         const int m = m0 + threadIdx.x, c = m & 3, mr = m % (2 * L);
@@ -617,7 +686,7 @@ sht_fft_anal(int nside, int lmax, int lg, int r_first, const float *__restrict__
     __syncthreads();
     fft_shared(fx, tw, lg, -1.0f);
     const long long stride = lmax + 1;
-    const int lim = order_limit(lmax, g.s);
+    const int lim = ring_limit(nside, r, lmax);
     const float inv = 1.0f / (float)n;
     for (int m = threadIdx.x; m <= lim; m += blockDim.x) {
         const float2 a = fx[m & (n - 1)], b = fx[(n - m) & (n - 1)];
@@ -646,7 +715,7 @@ sht_fft_synth(int nside, int lmax, int lg, int r_first, const float2 *__restrict
     const bool mirror = rs != r;
     const ShtRing g = sht_ring(nside, r), h = sht_ring(nside, rs);
     const long long stride = lmax + 1;
-    const int lim = order_limit(lmax, g.s);
+    const int lim = ring_limit(nside, r, lmax);
     const float inv = 1.0f / (float)n;
     fft_table(tw, lg);
     for (int b = threadIdx.x; b < n; b += blockDim.x) {
@@ -695,6 +764,10 @@ int belt_fft(int nside) {
     return lg >= 4 && lg <= 14 ? lg : 0;
 }
 
+// One radix-4 butterfly a thread and pass in short rings, up to four in long ones (two CTAs
+// of 512 threads per SM at n = 8192).
+int fft_threads(int lg) { return std::max(32, std::min(1 << (lg - 2), std::max(512, 1 << (lg - 4)))); }
+
 // Rings first .. last (northern half) by direct quarter sums; the rest of [0, 2 nside) by FFT.
 cudaError_t ring_synth(int nside, int lmax, const float2 *G, float *map, int add, cudaStream_t st) {
     const int lg = belt_fft(nside), n_cap = lg ? nside - 1 : 2 * nside;
@@ -708,8 +781,7 @@ cudaError_t ring_synth(int nside, int lmax, const float2 *G, float *map, int add
     cudaError_t e = cudaFuncSetAttribute(sht_fft_synth, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
-    sht_fft_synth<<<nside + 1, 1 << (lg - 4 > 5 ? lg - 4 : 5), smem, st>>>(nside, lmax, lg, nside - 1,
-                                                                          G, map, add);
+    sht_fft_synth<<<nside + 1, fft_threads(lg), smem, st>>>(nside, lmax, lg, nside - 1, G, map, add);
     return cudaGetLastError();
 }
 
@@ -725,8 +797,7 @@ cudaError_t ring_anal(int nside, int lmax, const float *map, float2 *F, cudaStre
     cudaError_t e = cudaFuncSetAttribute(sht_fft_anal, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
-    sht_fft_anal<<<nside + 1, 1 << (lg - 4 > 5 ? lg - 4 : 5), smem, st>>>(nside, lmax, lg, nside - 1,
-                                                                         map, F);
+    sht_fft_anal<<<nside + 1, fft_threads(lg), smem, st>>>(nside, lmax, lg, nside - 1, map, F);
     return cudaGetLastError();
 }
 
@@ -769,7 +840,7 @@ cudaError_t sht_analysis(int nside, int lmax, const float *d_map, const double *
     if (e == cudaSuccess) {
         const double up = 4.0 * (double)nside;
         const double c = 4.0 * kPi / (12.0 * (double)nside * (double)nside) * up;
-        kernel<<<lmax + 1, 256, smem, st>>>(nside, lmax, F, d_kl, 1.0 / up, c, d_alm);
+        kernel<<<lmax + 1, 256, smem, st>>>(nside, lmax, F, d_kl, (float)(1.0 / up), c, d_alm);
         e = cudaGetLastError();
     }
     const cudaError_t f = cudaFreeAsync(F, st);
