@@ -497,7 +497,7 @@ int finish_split(ksc_split *s, const ksc_split_opts &o) {
     // (per northern output ring: reflection classes x window positions per input ring).
     {
         const int eqr = (nr - 1) / 2;
-        double all = 0.0, tab = 0.0;
+        double all = 0.0, tab = 0.0, small = 0.0;
         for (int r = 0; r <= eqr; ++r) {
             const bool belt_r = r >= belt_lo && r <= belt_hi;
             const double cls = (double)ksc::sym_classes(g.len[r], g.phase[r]);
@@ -509,9 +509,19 @@ int finish_split(ksc_split *s, const ksc_split_opts &o) {
                 const double n = cls * std::min(2.0 * pairs[ip].hw + 3.0, (double)g.len[q]);
                 all += n;
                 if (xodd[ip].nct > 0) tab += n;
+                if (xodd[ip].nct > 0 && xodd[ip].nct + 1 <= ksc::kXCapSmall) small += n;
             }
         }
         s->frac_tabulated = all > 0.0 ? tab / all : 0.0;
+        // 128-class items with small tables (three CTAs per SM) where nearly all pairs that
+        // have a table fit one (pairs that do not take their weights one by one) and a map has
+        // items for two waves of two CTAs per SM.  Full / small tables, us: nside 512, 60'
+        // (about 800 items): 240 / 202; nside 256, 640' (about 300): 850 / 1070.  A batch fills
+        // its waves with several maps (32 of nside 256: 23.9 / 19.0 ms; 16 of 512: 35.1 / 28.7).
+        s->sym_small_ok = tab - small <= 0.01 * all;
+        s->sym_variant = ksc::sym_chunk(nside) == ksc::sym_variant_chunk(0) ? 0
+                         : s->sym_small_ok && s->n_items_sym >= 4 * 152    ? 1
+                                                                           : 2;
     }
 
     CapPlan cap;
@@ -922,7 +932,7 @@ cudaError_t launch_caps(const ksc_split *s, const MapSet &maps, int n_maps, int 
     const int c = s->ring_first_sym[lo], d = s->ring_first_sym[hi + 1];
     const WorkItem *its = whole ? s->d_items_sym_lpt : s->d_items_sym + c;
     if (!w.cap_flags)
-        return launch_conv_sym(s->plan, its, d - c, maps, n_maps, belt_split, r0, r1, d - c,
+        return launch_conv_sym(s->plan, its, d - c, s->sym_variant, maps, n_maps, belt_split, r0, r1, d - c,
                                     nullptr, w.counters, d_err, st);
     // the tensor-core stage, the irregular ring pairs, then the gather for the rings that
     // the first flagged (none in an ordinary map: that launch reads a flag and ends)
@@ -937,7 +947,7 @@ cudaError_t launch_caps(const ksc_split *s, const MapSet &maps, int n_maps, int 
     e = launch_cap_direct(s->plan, s->d_irr_items + i0, i1 - i0, s->d_irr_first, s->d_irr,
                                maps, n_maps, r0, r1, w.cap_flags, st);
     if (e != cudaSuccess) return e;
-    return launch_conv_sym(s->plan, its, d - c, maps, n_maps, belt_split, r0, r1, 0,
+    return launch_conv_sym(s->plan, its, d - c, s->sym_variant, maps, n_maps, belt_split, r0, r1, 0,
                                 w.cap_flags, w.counters, d_err, st);
 }
 

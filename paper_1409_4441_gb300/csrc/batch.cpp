@@ -63,10 +63,11 @@ TuneKey tune_key(const ksc_split *s) {
 }
 
 // Untuned default: half blocks only where a belt ring is shorter than a full
-// item; the single-map gather tile of that nside.
-std::pair<int, int> default_variants(const ksc_split *s) {
+// item; the single-map gather tile of that nside, of the two 128-class ones the one with
+// small tables where they fit and there are several entries to fill its three CTAs per SM.
+std::pair<int, int> default_variants(const ksc_split *s, int n) {
     return {4 * s->nside <= ksc::belt_variant_chunk(1) ? 1 : 0,
-            ksc::sym_chunk(s->nside) == ksc::sym_variant_chunk(0) ? 0 : 2};
+            s->sym_variant == 2 && s->sym_small_ok && n > 1 ? 1 : s->sym_variant};
 }
 
 struct Launch {
@@ -434,7 +435,7 @@ int ksc_batch_create(const ksc_split *const *splits, int n, const ksc_batch_opts
         b->group_of[i] = (int)(g - b->nsides.begin());
         if (g == b->nsides.end()) {
             b->nsides.push_back(s->nside);
-            std::pair<int, int> v = default_variants(s);
+            std::pair<int, int> v = default_variants(s, n);
             {
                 std::lock_guard<std::mutex> lk(g_tune_mu);
                 auto c = g_tune_cache.find(tune_key(s));

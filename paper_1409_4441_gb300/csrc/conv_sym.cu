@@ -61,7 +61,7 @@ template <int T_, int C_, int SPAN_, int MINB_, int XCAP_> struct SymShape {
     static constexpr size_t kDynSmem = sizeof(float4) * (size_t)XCAP_;
 };
 using ShapeC3 = SymShape<128, 3, 640, 2, kXCap>;    // variant 0: 384 classes per item
-using ShapeSmall = SymShape<128, 1, 448, 3, 2048>;  // variant 1: 128 classes, 3 CTAs per SM
+using ShapeSmall = SymShape<128, 1, 448, 3, kXCapSmall>;  // variant 1: 128 classes, 3 CTAs per SM
 using ShapeWide = SymShape<128, 1, 448, 2, kXCap>;  // variant 2: 128 classes, full tables
 static_assert(ShapeC3::kSpan % 4 == 0 && ShapeSmall::kSpan % 4 == 0, "quad-aligned spans");
 
@@ -747,12 +747,13 @@ int sym_classes(int len, int phase) {
 int sym_chunk(int nside) { return nside >= 2048 ? ShapeC3::kClasses : ShapeWide::kClasses; }
 
 cudaError_t launch_conv_sym(const ConvPlan &p, const WorkItem *d_items, int n_items,
-                            const MapSet &maps, int n_maps, int belt_split, int band_lo,
-                            int band_hi, int n_first, const int *ring_flags, int *d_counters,
-                            int *d_err, cudaStream_t st) {
+                            int variant, const MapSet &maps, int n_maps, int belt_split,
+                            int band_lo, int band_hi, int n_first, const int *ring_flags,
+                            int *d_counters, int *d_err, cudaStream_t st) {
     if (n_items <= 0 || n_maps <= 0) return cudaSuccess;
-    const auto launch = sym_chunk(p.nside) == ShapeC3::kClasses ? sym_launch<ShapeC3>
-                                                                : sym_launch<ShapeWide>;
+    const auto launch = variant == 0   ? sym_launch<ShapeC3>
+                        : variant == 1 ? sym_launch<ShapeSmall>
+                                       : sym_launch<ShapeWide>;
     return launch(p, d_items, n_items, maps, n_maps, belt_split, band_lo, band_hi, n_first,
                   ring_flags, d_counters, d_err, st);
 }

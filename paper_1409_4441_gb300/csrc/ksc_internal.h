@@ -297,16 +297,18 @@ cudaError_t launch_conv_belt_mma(const ConvPlan &p, const int2 *d_items, int n_i
 // Symmetric gather over northern rings (and the equator): each thread owns
 // one first-quarter position and writes its eight images; only output rings
 // in [band_lo, band_hi] are written.  Items are (ring, first quarter position)
-// chunks of sym_chunk(nside) classes (the tile launch_conv_sym uses for that nside).
+// chunks of sym_chunk(nside) classes; variant (of sym_variant_chunk(variant) = sym_chunk
+// classes): the split's sym_variant.
 int sym_chunk(int nside);
+constexpr int kXCapSmall = 2048;  // cells of variant 1's tables
 int sym_classes(int len, int phase);  // reflection classes of a ring's first quarter
 // CTAs claim items in list order through a counter per map (d_counters, zero at
 // launch, or NULL: taken from the stream-ordered allocator).  Items from n_first on are taken only where ring_flags
 // ([map][nrings + 1], the last word: any) says so (n_first = n_items: no flags).
 cudaError_t launch_conv_sym(const ConvPlan &p, const WorkItem *d_items, int n_items,
-                            const MapSet &maps, int n_maps, int belt_split, int band_lo,
-                            int band_hi, int n_first, const int *ring_flags, int *d_counters,
-                            int *d_err, cudaStream_t st);
+                            int variant, const MapSet &maps, int n_maps, int belt_split,
+                            int band_lo, int band_hi, int n_first, const int *ring_flags,
+                            int *d_counters, int *d_err, cudaStream_t st);
 
 // ---------------------------------------------------------------------------
 // Batched persistent launches (csrc/batch.cpp).  An entry is one map convolved
@@ -399,6 +401,8 @@ struct ksc_split {
     int n_items_smma = 0;
     std::vector<int> ring_first_smma;
     int cap_kernel = 0;                    // ksc_split_opts.cap_kernel
+    int sym_variant = 0;                   // the gather's tile (sym_variant_chunk)
+    bool sym_small_ok = false;             // its tables fit the small tile
     std::vector<int> ring_first_sym;
     int path = 0;                          // 0: belt + symmetric, 1: general only
     int2 *d_items_belt = nullptr;          // belt chunks for the circulant kernel
