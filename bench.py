@@ -56,6 +56,20 @@ FP32_LANES_PER_SM = 128
 DRAM_TRAFFIC = {}
 
 
+def step_kernels(K, nside, theta_cut, opts):
+    """(belt kernel, cap kernel, launches per step): the library's rules for the
+    tensor-core stages by size.  Belt: block maxima, the stage and the FFMA kernel for the
+    tiles it left.  Caps: ring ranges, the stage, its irregular pairs and the gather for the
+    rings it left."""
+    pairs = K.cost_pairs(nside, theta_cut)
+    belt = nside >= 64 and 2.0 / 3.0 * pairs >= 8e8
+    cap = opts.get("cap_kernel", 0) == 0 and 64 <= nside <= 4096 and pairs / 3.0 >= 8e9
+    return ("conv_belt_tc_kernel" if belt else "conv_belt_kernel",
+            "conv_cap_tc_kernel" if cap else
+            "conv_sym_tc_kernel" if opts.get("cap_kernel", 0) == 1 else "conv_sym_kernel",
+            1 + (1 if belt or cap else 0) + (1 if belt else 0) + 1 + (3 if cap else 0))
+
+
 def workload_desc(extra=None):
     W = WORKLOAD
     npix = 12 * W["nside"] ** 2
@@ -456,9 +470,10 @@ def run_ours(args, world, rank, local):
     sm_max = (clocks or {}).get("sm_max_mhz") or pk.get("sm_max_mhz") or 2070.0
     peak_tflops = N_SM * FP32_LANES_PER_SM * 2 * sm_max * 1e6 / 1e12
     n_belt = info["n_pairs_belt"] if info["n_pairs_belt"] >= 0 else 0
+    belt_name, cap_name, launches = step_kernels(K, nside, tc, split_opts(args))
     stages = {
-        "conv_belt_kernel": {"pairs": n_belt, "ms": stage_ms[1]},
-        "conv_sym_kernel": {"pairs": n_pairs - n_belt, "ms": stage_ms[2]},
+        belt_name: {"pairs": n_belt, "ms": stage_ms[1]},
+        cap_name: {"pairs": n_pairs - n_belt, "ms": stage_ms[2]},
     }
     for v in stages.values():
         v["tflops"] = 2.0 * v["pairs"] / (v["ms"] / 1e3) / 1e12 if v["ms"] > 0 else 0.0
@@ -542,12 +557,13 @@ def run_ours(args, world, rank, local):
                      "traffic_unit": "bytes per launch (ncu dram__bytes_read.sum + "
                                      "dram__bytes_write.sum of one full-size launch)",
                      "note": "2 FLOP (one FMA) per in-disc pixel pair the kernel handles; "
-                             "peak = 152 SMs x 128 FP32 lanes x 2 x max SM clock; the cap "
-                             "gather is bound by instruction issue at 8 warps per SM "
-                             "(ncu smsp__issue_active ~53%, about a third of the issued "
-                             "instructions useful FFMAs: per 16 FFMAs a weight costs a "
-                             "table-cell load, an index and three FMAs; stalls on fixed "
-                             "latency, staging loads and barriers)"},
+                             "peak = 152 SMs x 128 FP32 lanes x 2 x max SM clock (the FP32 "
+                             "pipe that the paper's formulation uses; the belt and cap "
+                             "stages run on the tensor cores, two-part FP16 products with "
+                             "FP32 sums, so a stage may exceed it).  The cap stage is bound "
+                             "by shared-memory bandwidth: operand reads of N = 144 MMAs and "
+                             "the turning of their accumulators (ncu: tensor pipe 17%, issue "
+                             "52%)"},
         "target": {"roofline_frac": 0.5, "met": bool(achieved / peak_tflops >= 0.5),
                    "step_frac": 2.0 * n_pairs / statistics.mean(launch_ms) * 1e3 / 1e12
                    / peak_tflops},
@@ -556,7 +572,7 @@ def run_ours(args, world, rank, local):
         "step_tflops": 2.0 * n_pairs / statistics.mean(launch_ms) * 1e3 / 1e12,
         "e2e": {"value": total_pairs / e2e_t, "unit": UNIT, "h2d_bytes_per_step": 4 * npix,
                 "d2h_bytes_per_step": 4 * npix},
-        "gpu_launches": 2 * args.steps,
+        "gpu_launches": launches * args.steps,
         "clocks": clocks,
         "cpu_baseline": cpu,
         "multimap": multimap,
@@ -612,9 +628,9 @@ def _event_ms(fn, stream, torch, reps=3):
 
 def run_stack(K, torch, dev, stream, sp, make_tensor_split, n_pairs, n_maps, single_maps_per_s):
     """n_maps maps of the benchmark workload itself (nside 2048, the same split) as one
-    map-stack call: the default path (the single-map FFMA kernels, one launch per stage
+    map-stack call: the default path (the single-map kernels, one launch of each
     for the stack) and the opt-in tensor path (tensor=1: cap ring pairs on the tensor
-    cores, belt on the FFMA kernel), maps/s against the single-map step.  Maps: i.i.d.
+    cores, belt on the default stage), maps/s against the single-map step.  Maps: i.i.d.
     N(0,1) drawn on the device from a seeded generator (throughput does not depend on
     the values)."""
     npix = 12 * 2048 * 2048
@@ -634,16 +650,16 @@ def run_stack(K, torch, dev, stream, sp, make_tensor_split, n_pairs, n_maps, sin
             "pairs_per_s": n_maps * n_pairs / (ms / 1e3),
             "maps_per_s_tensor": n_maps / (ms_t / 1e3), "ms_per_call_tensor": ms_t,
             "tensor_note": "opts.tensor = 1 (TF32 x3 caps, C_l-level accuracy: per pixel "
-                           "within ~3e-5 of the output rms of the FFMA result)",
+                           "within ~3e-5 of the output rms of the default path's result)",
             "single_map_maps_per_s": single_maps_per_s}
 
 
 def run_multimap(K, torch, dev, stream, pk, nside=1024, n_maps=64):
     """n_maps maps sharing one split (at nside 1024: 15' beam, l_max 3071, l_cut 768,
     theta_cut 480'; other nside scale every angle by 1024/nside).  Default path: the
-    single-map FFMA kernels.  Opt-in tensor path (tensor=1): the cap ring pairs as a
+    single-map kernels.  Opt-in tensor path (tensor=1): the cap ring pairs as a
     tcgen05 contraction (each weight shared by 16 images x 8 maps, TF32 x3, FP32
-    accumulate), the belt ring pairs on the FFMA circulant kernel.  Reports maps/s of
+    accumulate), the belt ring pairs on the default belt stage.  Reports maps/s of
     both, the roofline of the tensor cap stage, and the tensor form of the belt stage
     (tensor=2) for comparison."""
     sc = 1024.0 / nside
@@ -681,7 +697,7 @@ def run_multimap(K, torch, dev, stream, pk, nside=1024, n_maps=64):
             "maps_per_s": n_maps / t_ffma, "ms_per_call": 1e3 * t_ffma,
             "maps_per_s_tensor": n_maps / t_all, "ms_per_call_tensor": 1e3 * t_all,
             "pairs_per_map": n_pairs, "belt_pairs_per_map": belt_pairs,
-            "stages_ms": {"belt_ffma": 1e3 * t_belt, "caps_tensor": 1e3 * t_caps},
+            "stages_ms": {"belt": 1e3 * t_belt, "caps_tensor": 1e3 * t_caps},
             "tensor_stage": {"kernel": "conv_sym_mma_kernel", "ms": 1e3 * t_caps,
                              "achieved": caps_tf, "unit": "TFLOP/s", "peak": tf32_peak,
                              "frac": caps_tf / tf32_peak,

@@ -79,7 +79,7 @@ typedef struct {
     int path;          /* 0 (default): circulant belt kernel + symmetric gather;
                           1: general ring-pair gather only (reference path)   */
     int tensor;        /* map stacks (ksc_conv_real_multimap, n_maps >= 16):
-                          0 (default): FP32 FFMA kernels for every ring pair
+                          0 (default): the single-map kernels for every map
                           (per pixel the single-map result, within 1e-6 of
                           the output rms of the FP64 sum);
                           1: the symmetric (cap) ring pairs on the tcgen05
@@ -87,10 +87,10 @@ typedef struct {
                           ring pair's window in tensor memory: per pixel
                           within ~3e-5 of the output rms, rms ~2e-6,
                           fractional rms C_l ~1e-6; faster for stacks), the
-                          belt ring pairs on the FFMA circulant kernel;
+                          belt ring pairs on the default belt stage;
                           2: both kinds of ring pair on the tensor cores
-                          (the belt's tensor form is slower than its
-                          circulant FFMA form on GB300)                     */
+                          (the belt's TF32 form is slower than the
+                          default belt stage on GB300)                      */
     int cut_continuity; /* LSQ mode: how the fitted real-space kernel meets the
                           cut.  KSC_CUT_FREE is the paper's fit as printed
                           (Sec. 2, Eq. 3-5: K_r truncated at theta_cut, free
@@ -112,16 +112,25 @@ typedef struct {
                           1: every weight from the double-float chord and
                           the K_r table                                      */
     int cap_kernel;    /* single maps and stacks of fewer than 16 maps: which
-                          kernel sums the cap ring pairs.  0 (default): FP32
-                          FFMAs, three reflection classes per thread sharing
-                          each staged image value; 1: the tcgen05 tensor
+                          kernel sums the cap ring pairs.  0 (default): from
+                          8e9 pairs with a cap ring on (5e10 where the gather
+                          keeps three CTAs per SM), nside 64..4096, unless
+                          exact_weights is set, the tcgen05 tensor cores on
+                          two-part FP16 values and per-cell polynomials of the
+                          weights (coefficients laid out with the split, 2.4
+                          GB at nside 2048 with a 240' cut, at most 8 GB;
+                          output rings whose input spans more than 2^14 in
+                          magnitude or is not finite go to the gather); else
+                          FP32 FFMAs, one or three reflection classes per
+                          thread sharing each staged image value; 1: the
+                          tcgen05 tensor
                           cores, each weight and map value split exactly into
                           three BF16 parts and six MMAs per 16 positions
                           (products to FP32 rounding), a fresh accumulator
                           drained every 16 positions into Kahan-folded FP32
                           sums (slower for one map: each weight serves only
                           the 16 symmetry images).  Both use the same
-                          weights; their outputs agree to FP32 rounding of
+                          kernel K_r; their outputs agree to FP32 rounding of
                           the sums                                          */
 } ksc_split_opts;
 
@@ -201,10 +210,12 @@ int ksc_split_table(const ksc_split *s, float *host_coeffs);
 /*
  * out = real-space convolution of `in` with the split's K_r (both device
  * arrays of 12 nside^2 floats, nside as given to the split; in != out).
- * Asynchronous on `stream`.  Each call takes a few bytes of work-claim
- * counters from the device's default stream-ordered memory pool
+ * Asynchronous on `stream`.  Each call takes its scratch (work-claim counters;
+ * with the tensor-core stages, from 8e8 belt pairs on, also npix / 16 bytes a map
+ * of block maxima, and flags; without room for these the FFMA kernels run) from
+ * the device's default stream-ordered memory pool
  * (cudaMallocAsync / cudaFreeAsync on `stream`), so calls on several streams
- * may overlap and a call captured into a CUDA graph holds its own counters.
+ * may overlap and a call captured into a CUDA graph holds its own scratch.
  * Errors: KSC_ERR_ARG, KSC_ERR_CUDA.
  */
 int ksc_conv_real(const ksc_split *s, const float *d_in, float *d_out,
@@ -226,7 +237,7 @@ int ksc_conv_real_rings(const ksc_split *s, const float *d_in, float *d_out,
  * single-map kernels (same results, one launch per stage for the stack).
  * With opts.tensor = 1 and n_maps >= 16 the cap ring pairs run on the tensor
  * cores (each kernel weight evaluated once for a group of 8 maps and their 16
- * symmetry images; per pixel within ~3e-5 of the output rms of the FFMA
+ * symmetry images; per pixel within ~3e-5 of the output rms of the default
  * result, see ksc_split_opts.tensor).  With opts.tensor = 2 the belt ring pairs
  * also run on the tensor cores, through a per-split workspace (the map stack
  * pre-split into TF32 tiles, about 2.6x the input size) allocated on the
@@ -255,7 +266,8 @@ int ksc_conv_real_batch(const ksc_split *const *splits,
  * are merged into one list per kernel and tile variant (entries in decreasing
  * order of work, each entry's items longest first) and each list runs as ONE
  * persistent launch whose CTAs claim items from a device counter (so short
- * maps fill the tail of long ones).  With use_graph the launch sequence is
+ * maps fill the tail of long ones).  Entries whose split has tensor-core stages
+ * run as one stack per split through them instead.  With use_graph the launch sequence is
  * captured once as a CUDA graph and replayed.  Results equal those of
  * ksc_conv_real on each entry to FP32 rounding (the batch kernels are separate
  * instantiations, free to contract multiply-adds differently, and the
@@ -312,7 +324,7 @@ int ksc_batch_autotune(ksc_batch *b, const float *const *d_in,
 
 typedef struct {
     int n_entries, n_splits, n_groups;
-    int n_items_belt, n_items_sym;  /* items over all persistent launches   */
+    int n_items_belt, n_items_sym;  /* items over the persistent launches   */
     int n_launches;                 /* kernel launches per run              */
     int use_graph;
     long long n_pairs;              /* in-disc pairs per run, or -1 when a
@@ -444,8 +456,8 @@ int ksc_build_table_noalloc(const double *d_c, int lmax, double theta_cut,
  * Legendre functions without the Condon-Shortley phase.  a_lm are complex
  * doubles (re, im interleaved) in m-major order: index(l, m) = m (2 lmax + 1 - m)
  * / 2 + l, m = 0..lmax, l = m..lmax; (lmax + 1)(lmax + 2) / 2 entries.
- * Legendre recurrences in FP64 (scaled against underflow near the poles), ring
- * sums in FP32.  Device pointers; asynchronous on `stream`; scratch from the
+ * Legendre recurrences and sums on FP32 pairs (48 bits, scaled against underflow
+ * near the poles), ring sums in FP32 (FFT on the belt, quarter sums in the caps).  Device pointers; asynchronous on `stream`; scratch from the
  * stream-ordered allocator.  nside a power of two <= 8192, 0 <= lmax <= 4 nside.
  * Errors: KSC_ERR_ARG, KSC_ERR_NOMEM, KSC_ERR_CUDA.
  */

@@ -162,11 +162,13 @@ void plan_cap_tc(ksc_split *s, const ksc_split_opts &o, const ksc::RingGeom &g,
     if (s->path != 0 || o.exact_weights || o.cap_kernel != 0 || nside < 64 || nside > 4096 ||
         s->theta_cut >= kPi || s->n_items_belt == 0)
         return;
-    // Below about 8e9 pairs with a cap ring the gather is the faster one: a tile spends about
-    // 5 us on an input ring, with few tiles on small maps (gather / tensor stage, ms: nside
-    // 256, 640' (1.8e9 pairs): 0.85 / 1.09; 512, 160': 0.84 / 1.00; 256, 30 deg (1.4e10): 8.7 /
-    // 7.4; 512, 640' (2.9e10): 9.0 / 7.1; 1024, 160': 7.5 / 6.6; 2048, 240' (1.0e12): 150 / 108).
-    if (ksc_cost_pairs(nside, s->theta_cut) / 3.0 < 8e9) return;
+    // Below about 8e9 pairs with a cap ring the gather is the faster one, and below 5e10 where
+    // its small-table tile serves: a tile of the stage spends about 5 us on an input ring, with
+    // few tiles on small maps (gather / tensor stage, ms: nside 256, 640' (1.8e9 pairs): 0.85 /
+    // 1.09; 512, 160': 0.84 / 1.00; 256, 30 deg (1.4e10): 8.7 / 7.4; 512, 640' (2.9e10): 9.0 /
+    // 7.1; 2048, 240' (1.0e12): 150 / 108; with the small tables 1024, 160' (2.9e10): 6.1 / 6.6,
+    // the whole call 6.95 / 7.35).
+    if (ksc_cost_pairs(nside, s->theta_cut) / 3.0 < (s->sym_variant == 1 ? 5e10 : 8e9)) return;
     // the cells' polynomials: Chebyshev interpolation of degree n leaves, of a term l of the
     // kernel, at most about 4 J_{n+1}(l h / 2) ~ 4 (l h / 4)^{n+1} / (n+1)!, h the largest
     // pixel step (1.2826 / nside at the poles)

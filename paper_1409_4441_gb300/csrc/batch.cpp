@@ -16,19 +16,8 @@
 // plans are made) leave those lists: the entries of one split run as one stack through the
 // single-map kernels' tensor-core stages, which read their maps through the same entry
 // table.  The belt stage or both stages go that way.  (8 maps of nside 256, 4 of 512 and 1 of
-// 1024, cuts of 16 beams: belt lists 10.8 ms, as stacks 5.0 ms; the nside-1024 caps 7.3 and
-// 6.6 ms; the run 33.2 and 26.7 ms.)
-//
-// The tile variants are the full and half block size of the belt kernel
-// (2080 or 1040 outputs per item) and three gather tiles: 256 reflection
-// classes per item with 4096-cell weight tables (two CTAs per SM), 128 classes
-// with 2048-cell tables (three CTAs per SM; ring pairs needing more cells take
-// per-pair weights), and 128 classes with 4096-cell tables (two CTAs per SM).
-// Smaller items suit short rings (a 1024-pixel belt ring fills only half of a
-// 2080-output item, a ring of 512 pixels has 64 reflection classes).  The autotuner times every
-// variant of both kernels on every nside group of the batch, with the caller's
-// maps, keeps the fastest of each, and caches the choice per (device, nside,
-// l_max, table size, theta_cut) for the rest of the process.
+// 1024, cuts of 16 beams: belt lists 10.8 ms, as stacks 5.0 ms; the run, with the gather's
+// small-table tile, 33.2 and 23.3 ms.)
 #include <algorithm>
 #include <cstdint>
 #include <cstring>

@@ -45,7 +45,7 @@ def _pixels(nside, tc, n, seed):
 # 256: one sector a ring, wide windows (polar rings mostly direct); 512: one to three
 # sectors; 1024: narrow windows
 @pytest.mark.parametrize("nside,theta", [(256, 1800.0), (256, 1920.0), (256, 2700.0), (512, 640.0),
-                                         (1024, 160.0)])
+                                         (1024, 160.0), (1024, 220.0)])
 def test_cap_parity(K, nside, theta):
     sp, tc, tab = _split(K, nside, theta)
     m = inputs.white_noise_map(nside, 91).astype(np.float32)
