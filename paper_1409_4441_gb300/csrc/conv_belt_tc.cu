@@ -575,7 +575,8 @@ cudaError_t launch_tc(const ConvPlan &p, const BeltTc &t, const MapSet &maps, in
     const int tk = p.nside / (2 * N);
     const size_t smem = tc_smem<N>(t.wpos, t.nq);
     cudaError_t e = cudaFuncSetAttribute(conv_belt_tc_kernel<N>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         kMaxDynSmem);  // (one value: calls may race)
     if (e != cudaSuccess) return e;
     dim3 grid((b1 - b0 + 1) * tk, n_maps);
     conv_belt_tc_kernel<N><<<grid, kThreads, smem, st>>>(
@@ -608,7 +609,7 @@ bool belt_tc_plan(int nside, int wpos, int nq, BeltTc *t) {
     for (int n = 32; n <= 256 && 2 * n <= nside; n *= 2) {
         const size_t smem = n == 256 ? tc_smem<256>(wpos, nq) : n == 128 ? tc_smem<128>(wpos, nq)
                             : n == 64 ? tc_smem<64>(wpos, nq) : tc_smem<32>(wpos, nq);
-        if (smem > 226u * 1024) continue;
+        if (smem > (size_t)kMaxDynSmem) continue;
         // waves of one CTA per SM x the larger of the MMAs' and the builders' cycles
         const double waves = std::ceil(n_blocks * (nside / (2.0 * n)) / 152.0);
         const double mma = wpos / 16.0 * 3.0 * std::max(n / 2.0, 48.0);

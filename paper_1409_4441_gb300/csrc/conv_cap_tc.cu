@@ -944,7 +944,7 @@ int cap_tc_positions(int w, int L) {
 }
 
 bool cap_tc_fits(const CapTc &c) {
-    return cap_smem(c) <= 226u * 1024 && c.span + c.wpos <= kXr * kBuild;
+    return cap_smem(c) <= (size_t)kMaxDynSmem && c.span + c.wpos <= kXr * kBuild;
 }
 
 int cap_tc_words(int jE) { return coef_words(jE); }
@@ -990,7 +990,8 @@ cudaError_t launch_conv_cap_tc(const ConvPlan &p, const CapTc &c, const int2 *d_
     if (n_tiles <= 0) return cudaSuccess;
     const size_t smem = cap_smem(c);
     cudaError_t e = cudaFuncSetAttribute(conv_cap_tc_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         kMaxDynSmem);  // (one value: calls may race)
     if (e != cudaSuccess) return e;
     dim3 grid(n_tiles, n_maps);
     conv_cap_tc_kernel<<<grid, kThreads, smem, st>>>(p, c, d_tiles, maps, belt_split, band_lo,

@@ -8,6 +8,7 @@
 #include "ksc_tc.cuh"
 
 namespace ksc {
+constexpr int kMaxDynSmem = 226 * 1024;  // of the split kernels, beside 1 kB of static
 namespace tc {
 
 constexpr int kXExp = 14;           // a tile's largest |m| is scaled into [2^14, 2^15)

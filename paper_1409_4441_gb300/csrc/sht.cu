@@ -757,6 +757,10 @@ sht_fft_synth(int nside, int lmax, int lg, int r_first, const float2 *__restrict
     }
 }
 
+// The longest FFT's shared memory.  The limits are set to the largest value whatever the
+// call needs: calls of several threads may race on them.
+constexpr int kFftSmem = 8 * 5 * 4096;
+
 // log2 of the belt rings' length where they go through the FFT (16 <= L <= 16384), else 0.
 int belt_fft(int nside) {
     int lg = 2;
@@ -779,7 +783,7 @@ cudaError_t ring_synth(int nside, int lmax, const float2 *G, float *map, int add
     }
     const size_t smem = sizeof(float2) * (5u << (lg - 2));
     cudaError_t e = cudaFuncSetAttribute(sht_fft_synth, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+                                         kFftSmem);
     if (e != cudaSuccess) return e;
     sht_fft_synth<<<nside + 1, fft_threads(lg), smem, st>>>(nside, lmax, lg, nside - 1, G, map, add);
     return cudaGetLastError();
@@ -795,7 +799,7 @@ cudaError_t ring_anal(int nside, int lmax, const float *map, float2 *F, cudaStre
     }
     const size_t smem = sizeof(float2) * (5u << (lg - 2));
     cudaError_t e = cudaFuncSetAttribute(sht_fft_anal, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+                                         kFftSmem);
     if (e != cudaSuccess) return e;
     sht_fft_anal<<<nside + 1, fft_threads(lg), smem, st>>>(nside, lmax, lg, nside - 1, map, F);
     return cudaGetLastError();
@@ -831,7 +835,8 @@ cudaError_t sht_analysis(int nside, int lmax, const float *d_map, const double *
     const int nr = 4 * nside - 1, nnorth = 2 * nside;
     const size_t smem = sizeof(float4) * (size_t)(lmax + 1);
     auto kernel = nnorth > 512 ? sht_leg_anal<4> : sht_leg_anal<1>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sizeof(float4) * 8192);  // (as kFftSmem)
     if (e != cudaSuccess) return e;
     float2 *F = nullptr;
     if ((e = cudaMallocAsync(&F, sizeof(float2) * (size_t)nr * (lmax + 1), st)) != cudaSuccess)
