@@ -457,7 +457,7 @@ int ksc_build_table_noalloc(const double *d_c, int lmax, double theta_cut,
  * doubles (re, im interleaved) in m-major order: index(l, m) = m (2 lmax + 1 - m)
  * / 2 + l, m = 0..lmax, l = m..lmax; (lmax + 1)(lmax + 2) / 2 entries.
  * Legendre recurrences and sums on FP32 pairs (48 bits, scaled against underflow
- * near the poles), ring sums in FP32 (FFT on the belt, quarter sums in the caps).  Device pointers; asynchronous on `stream`; scratch from the
+ * near the poles), ring sums in FP32 (FFT on the belt of larger maps, else quarter sums).  Device pointers; asynchronous on `stream`; scratch from the
  * stream-ordered allocator.  nside a power of two <= 8192, 0 <= lmax <= 4 nside.
  * Errors: KSC_ERR_ARG, KSC_ERR_NOMEM, KSC_ERR_CUDA.
  */

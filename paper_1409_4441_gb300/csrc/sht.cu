@@ -23,8 +23,8 @@
 // functions decay exponentially past their turning point): a ring leaves them out.
 //
 // Ring sums: pixel k of a ring of L pixels with phase flag t sits at phi_k = pi (2k + t) / L.
-// Belt rings (L = 4 nside, a power of two) go through an FP32 FFT in shared memory, north
-// and mirror ring as one complex sequence.  Cap rings (L = 4i) are summed directly over a
+// Belt rings (L = 4 nside, a power of two) of larger transforms go through an FP32 FFT in shared memory, north
+// and mirror ring as one complex sequence.  Other rings (L = 4i) are summed directly over a
 // quarter: the quarter turns of pixel k1 enter order m through m mod 4 alone.  m phi_k =
 // pi J / L with the exact integer J = m (2k + t) mod 2L; the twiddles advance by one complex
 // product per step and are re-anchored from the exact J every 8 steps (the products'
@@ -220,38 +220,32 @@ __device__ __forceinline__ float4 step_coeffs(int l, int m) {
 }
 
 // Synthesis, Legendre part: G[ring][m] = sum_l a_lm lambda_lm(z_ring) for the northern rings
-// (and their southern mirrors) of the block's range and order m = blockIdx.y, R rings a
-// thread.  Orders past a ring's limit are not written (nor read).
-template <int R>
+// (and their southern mirrors) of the block's range and order m = blockIdx.y, a ring a
+// thread.  Orders past a ring's limit are not written (nor read).  Bound by issue: 47 FP32
+// operations per ring pair, degree and order.  nside 2048, l_max 1024: 30.1 ms in FP64,
+// 3.77 ms (two rings a thread for the same staged coefficients: 3.77; nside 512: 1.01
+// against 1.04).
 __global__ void __launch_bounds__(256)
 sht_leg_synth(int nside, int lmax, const double2 *__restrict__ alm, float2 *__restrict__ G) {
     __shared__ float4 co[kTile], al[kTile];
     __shared__ F2 s_norm;
     const int m = blockIdx.y, nnorth = 2 * nside, nr = 4 * nside - 1;
-    const int r0 = blockIdx.x * 256 * R + threadIdx.x;
+    const int r = blockIdx.x * 256 + threadIdx.x, rs = nr - 1 - r;
     if (threadIdx.x < 32) {
         const F2 v = norm_mm(m);
         if (threadIdx.x == 0) s_norm = v;
     }
     __syncthreads();
-    Rec rec[R];
-    F2 er[R], ei[R], od[R], oi[R];  // even / odd (l - m) sums
-    bool live[R], any = false;
-#pragma unroll
-    for (int j = 0; j < R; ++j) {
-        const int r = r0 + 256 * j;
-        er[j] = ei[j] = od[j] = oi[j] = F2{0.0f, 0.0f};
-        live[j] = false;
-        if (r < nnorth) {
-            F2 z, s;
-            ring_zs(nside, r, &z, &s);
-            live[j] = m <= order_limit(lmax, s.h);
-            if (live[j]) rec[j].start(m, s_norm, z, s);
-        }
-        any |= live[j];
+    Rec rec;
+    F2 er{0.0f, 0.0f}, ei = er, od = er, oi = er;  // even / odd (l - m) sums
+    bool live = false;
+    if (r < nnorth) {
+        F2 z, s;
+        ring_zs(nside, r, &z, &s);
+        live = m <= order_limit(lmax, s.h);
+        if (live) rec.start(m, s_norm, z, s);
     }
-    if (!__syncthreads_or(any)) return;
-    const bool warp_any = __any_sync(~0u, any);
+    if (!__syncthreads_or(live)) return;
     const double2 *a = alm + alm_base(lmax, m);
     for (int l0 = m; l0 <= lmax; l0 += kTile) {
         const int n = min(kTile, lmax + 1 - l0);
@@ -263,39 +257,28 @@ sht_leg_synth(int nside, int lmax, const double2 *__restrict__ alm, float2 *__re
             al[i] = make_float4(x.h, x.l, y.h, y.l);
         }
         __syncthreads();
-        if (!warp_any) continue;
+        if (!live) continue;
         for (int i = 0; i < n; ++i) {
-            const float4 c = co[i], x = al[i];
-            const bool odd = (l0 + i - m) & 1;
-#pragma unroll
-            for (int j = 0; j < R; ++j) {
-                if (!live[j]) continue;
-                if (l0 + i > m) rec[j].step(c);
-                if (rec[j].e < 0) continue;
-                const F2 pr = f2_mul(rec[j].v1, F2{x.x, x.y}), pi = f2_mul(rec[j].v1, F2{x.z, x.w});
-                if (odd) {
-                    od[j] = f2_acc(od[j], pr);
-                    oi[j] = f2_acc(oi[j], pi);
-                } else {
-                    er[j] = f2_acc(er[j], pr);
-                    ei[j] = f2_acc(ei[j], pi);
-                }
+            const float4 x = al[i];
+            if (l0 + i > m) rec.step(co[i]);
+            if (rec.e < 0) continue;
+            const F2 pr = f2_mul(rec.v1, F2{x.x, x.y}), pi = f2_mul(rec.v1, F2{x.z, x.w});
+            if ((l0 + i - m) & 1) {
+                od = f2_acc(od, pr);
+                oi = f2_acc(oi, pi);
+            } else {
+                er = f2_acc(er, pr);
+                ei = f2_acc(ei, pi);
             }
         }
     }
+    if (!live) return;
     const long long stride = lmax + 1;
-#pragma unroll
-    for (int j = 0; j < R; ++j) {
-        const int r = r0 + 256 * j, rs = nr - 1 - r;
-        if (!live[j]) continue;
-        const F2 a0 = f2_add(er[j], od[j]), a1 = f2_add(ei[j], oi[j]);
-        G[(long long)r * stride + m] = make_float2(a0.h, a1.h);
-        if (rs == r) continue;
-        od[j].h = -od[j].h; od[j].l = -od[j].l;
-        oi[j].h = -oi[j].h; oi[j].l = -oi[j].l;
-        const F2 b0 = f2_add(er[j], od[j]), b1 = f2_add(ei[j], oi[j]);
-        G[(long long)rs * stride + m] = make_float2(b0.h, b1.h);
-    }
+    G[(long long)r * stride + m] = make_float2(f2_add(er, od).h, f2_add(ei, oi).h);
+    if (rs == r) return;
+    od = F2{-od.h, -od.l};
+    oi = F2{-oi.h, -oi.l};
+    G[(long long)rs * stride + m] = make_float2(f2_add(er, od).h, f2_add(ei, oi).h);
 }
 
 constexpr int kGroup = 32;  // degrees between the block's reductions
@@ -305,6 +288,9 @@ constexpr int kGroup = 32;  // degrees between the block's reductions
 // NULL: 1).  One block per order, R rings a thread, in passes over the rings.  The
 // threads' terms of eight degrees go through shared memory: within a warp 32 -> 4 partial
 // sums a degree, then every 32 degrees over the warps, in a fixed order and on FP32 pairs throughout.  The
+// Four rings a thread share the reduction: 5.76 ms at nside 2048, l_max 1024 (one ring 8.11;
+// 70.1 in FP64 with atomics); with one pass or two over the rings (nside <= 128) one ring is
+// the shorter chain (25.5 against 27.9 us at nside 128, l_max 64).  The
 // F_m enter divided by the power of two that covers the number of rings (exact; c carries it
 // back), so that a sum over all rings stays in range wherever the F_m do.
 template <int R>
@@ -761,11 +747,14 @@ sht_fft_synth(int nside, int lmax, int lg, int r_first, const float2 *__restrict
 // call needs: calls of several threads may race on them.
 constexpr int kFftSmem = 8 * 5 * 4096;
 
-// log2 of the belt rings' length where they go through the FFT (16 <= L <= 16384), else 0.
-int belt_fft(int nside) {
+// log2 of the belt rings' length where they go through the FFT (L <= 16384, and from 1e8
+// products of a direct sum on), else 0.  Direct for all rings / quarter sums and FFT, both
+// directions, us: nside 128, l_max 64 (8e6): 18.6 / 25.4; nside 512, l_max 1024 (2e9,
+// synthesis): 257 / 126; nside 2048, l_max 1024 (3e10): 7910 / 2480.
+int belt_fft(int nside, int lmax) {
     int lg = 2;
     while ((1 << (lg - 2)) < nside) ++lg;
-    return lg >= 4 && lg <= 14 ? lg : 0;
+    return 8.0 * nside * nside * (lmax + 1) >= 1e8 && lg <= 14 ? lg : 0;
 }
 
 // One radix-4 butterfly a thread and pass in short rings, up to four in long ones (two CTAs
@@ -774,7 +763,7 @@ int fft_threads(int lg) { return std::max(32, std::min(1 << (lg - 2), std::max(5
 
 // Rings first .. last (northern half) by direct quarter sums; the rest of [0, 2 nside) by FFT.
 cudaError_t ring_synth(int nside, int lmax, const float2 *G, float *map, int add, cudaStream_t st) {
-    const int lg = belt_fft(nside), n_cap = lg ? nside - 1 : 2 * nside;
+    const int lg = belt_fft(nside, lmax), n_cap = lg ? nside - 1 : 2 * nside;
     if (n_cap > 0) {
         dim3 grid(n_cap, nside > 512 ? 2 : 1);
         sht_ring_synth<<<grid, 256, 0, st>>>(nside, lmax, 0, G, map, add);
@@ -790,7 +779,7 @@ cudaError_t ring_synth(int nside, int lmax, const float2 *G, float *map, int add
 }
 
 cudaError_t ring_anal(int nside, int lmax, const float *map, float2 *F, cudaStream_t st) {
-    const int lg = belt_fft(nside), n_cap = lg ? nside - 1 : 2 * nside;
+    const int lg = belt_fft(nside, lmax), n_cap = lg ? nside - 1 : 2 * nside;
     if (n_cap > 0) {
         dim3 grid(n_cap, (lmax + 256) / 256);
         sht_ring_anal<<<grid, 256, 0, st>>>(nside, lmax, 0, map, F);
@@ -814,14 +803,8 @@ cudaError_t sht_synthesis(int nside, int lmax, const double2 *d_alm, float *d_ma
     float2 *G = nullptr;
     cudaError_t e = cudaMallocAsync(&G, sizeof(float2) * (size_t)nr * (lmax + 1), st);
     if (e != cudaSuccess) return e;
-    // two rings a thread share the staged coefficients; one where rings are few
-    if (nnorth > 512) {
-        dim3 grid((nnorth + 511) / 512, lmax + 1);
-        sht_leg_synth<2><<<grid, 256, 0, st>>>(nside, lmax, d_alm, G);
-    } else {
-        dim3 grid((nnorth + 255) / 256, lmax + 1);
-        sht_leg_synth<1><<<grid, 256, 0, st>>>(nside, lmax, d_alm, G);
-    }
+    dim3 grid((nnorth + 255) / 256, lmax + 1);
+    sht_leg_synth<<<grid, 256, 0, st>>>(nside, lmax, d_alm, G);
     e = cudaGetLastError();
     if (e == cudaSuccess) e = ring_synth(nside, lmax, G, d_map, add, st);
     const cudaError_t f = cudaFreeAsync(G, st);

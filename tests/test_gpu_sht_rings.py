@@ -1,5 +1,5 @@
 """The transforms' ring sums (FFT of the belt, quarter sums of the caps) and FP32-pair
-recurrences where their tiles and branches change: belts too short for the FFT, transforms
+recurrences where their tiles and branches change: belts too short for the FFT, FFTs
 with and without a radix-2 pass, orders at and past the ring length (l_max = 4 nside), one and
 several rings a thread, more orders than one staged block.
 
@@ -27,7 +27,8 @@ def K():
 
 
 @pytest.mark.parametrize("nside,lmax", [(2, 8), (4, 16), (16, 64), (32, 128), (256, 300),
-                                        (256, 1024), (512, 40)])
+                                        (256, 1024), (512, 40),
+                                        (512, 60)])
 def test_transforms_match_oracle(K, nside, lmax):
     alm = inputs.grf_alm(lmax, inputs.cl_grf(lmax), inputs.seed_for(7, nside + lmax))
     ref = O.alm2map(nside, alm, lmax)
