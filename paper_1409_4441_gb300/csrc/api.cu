@@ -92,6 +92,18 @@ void release(ksc_split *s) {
     delete s;
 }
 
+// Without the tensor-core cap stage: the gather sums the caps.
+void drop_cap_tc(ksc_split *s) {
+    for (void **p : {(void **)&s->d_cap_tiles, (void **)&s->d_cap_tiles_lpt, (void **)&s->d_ncut,
+                     (void **)&s->d_coef_off, (void **)&s->d_coef, (void **)&s->d_irr_items,
+                     (void **)&s->d_irr_first, (void **)&s->d_irr}) {
+        cudaFree(*p);
+        *p = nullptr;
+    }
+    s->n_cap_tiles = 0;
+    s->ctc = ksc::CapTc();
+}
+
 // Plan of the tensor-core belt stage: the widest window and the most input rings of a
 // 16-ring tile, and the power of two that scales the kernel's largest value (for the cap
 // stage too).
@@ -108,15 +120,12 @@ int plan_belt_tc(ksc_split *s, const ksc::RingGeom &g, const std::vector<int2> &
     // scaled weights and sums stay normal FP32 numbers; otherwise the FFMA kernels
     const int ex = std::isfinite(top) && top > 0.0 ? 13 - std::ilogb(top) : 1000;
     if (ex < -20 || ex > 40) {
-        s->ctc.ring_end = s->ctc.ring_first - 1;
+        drop_cap_tc(s);
         return KSC_OK;
     }
     s->btc.wscale = s->ctc.wscale = (float)std::ldexp(1.0, ex);
     s->ctc.wunscale = 1.0f / s->ctc.wscale;
     s->ctc.domega_lo = (float)(4.0 * kPi / s->plan.npix - (double)s->plan.domega);
-    s->ctc.d_ncut = s->d_ncut;
-    s->ctc.d_coef_off = s->d_coef_off;
-    s->ctc.d_coef = s->d_coef;
     // Below about 8e8 belt pairs the FFMA kernel is the faster one: a tile spends 0.7 to
     // 1.8 us on an input ring however short the window, small maps have few tiles, and the
     // block maxima (5 us) and their scratch come on top (FFMA / tensor stage, us: nside 64,
@@ -147,6 +156,7 @@ int plan_belt_tc(ksc_split *s, const ksc::RingGeom &g, const std::vector<int2> &
 // fewer than 32 pixels.
 struct CapPlan {
     std::vector<int2> tiles;         // {rings - 1 << 16 | first ring, sectors << 16 | sector}
+    std::vector<int2> tiles_lpt;     // the same, longest first
     std::vector<double> cost;        // of each tile
     std::vector<int> ncut;           // per ring pair: the largest |N| within the cut, -1: none
     std::vector<unsigned> coef_off;  // per ring pair, in units of four words; then their end
@@ -311,6 +321,42 @@ void plan_cap_tc(ksc_split *s, const ksc_split_opts &o, const ksc::RingGeom &g,
     c.ring_end = last;
     plan->n_ext = n_ext;
     s->ctc = c;
+}
+
+// Uploads the cap stage's tiles and lays out its coefficients.  The stage is left out (the
+// gather sums the caps) where there is no room for them, and where a coefficient does not fit
+// an FP16 number: the scale comes from the kernel inside the cut, the polynomials of the cells
+// that the cut divides from the kernel past it too, which may be larger.
+int build_cap_tc(ksc_split *s, const CapPlan &cap, ksc::CapCoef cc) {
+    if (s->n_cap_tiles == 0) return KSC_OK;
+    cudaError_t e = cudaMalloc(&s->d_coef, 16ull * cap.coef_off.back());
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        s->d_coef = nullptr;
+        drop_cap_tc(s);
+        return KSC_OK;
+    }
+    if ((e = dev_upload(&s->d_cap_tiles, cap.tiles.data(), cap.tiles.size())) != cudaSuccess ||
+        (e = dev_upload(&s->d_cap_tiles_lpt, cap.tiles_lpt.data(), cap.tiles_lpt.size())) !=
+            cudaSuccess ||
+        (e = dev_upload(&s->d_ncut, cap.ncut.data(), cap.ncut.size())) != cudaSuccess ||
+        (e = dev_upload(&s->d_coef_off, cap.coef_off.data(), cap.coef_off.size())) != cudaSuccess ||
+        (e = dev_upload(&s->d_irr_items, cap.irr_items.data(), cap.irr_items.size())) != cudaSuccess ||
+        (e = dev_upload(&s->d_irr_first, cap.irr_first.data(), cap.irr_first.size())) != cudaSuccess ||
+        (e = dev_upload(&s->d_irr, cap.irr.data(), cap.irr.size())) != cudaSuccess)
+        return cuda_fail(e, "cap tiles");
+    s->ctc.d_ncut = s->d_ncut;
+    s->ctc.d_coef_off = s->d_coef_off;
+    s->ctc.d_coef = cc.d_coef = s->d_coef;
+    int too_large = 0;
+    e = cudaMemsetAsync(cc.d_too_large, 0, sizeof(int), 0);
+    if (e == cudaSuccess) e = ksc::launch_cap_coef(s->plan, s->ctc, cc, 0);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(&too_large, cc.d_too_large, sizeof(int), cudaMemcpyDeviceToHost, 0);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(0);
+    if (e != cudaSuccess) return cuda_fail(e, "cap coefficients");
+    if (too_large) drop_cap_tc(s);
+    return KSC_OK;
 }
 
 // Geometry, work list and device table for the real-space part s->c_real.
@@ -563,13 +609,12 @@ int finish_split(ksc_split *s, const ksc_split_opts &o) {
         s->ring_first_smma[nr] = (int)items_smma.size();
     }
     std::vector<ksc::WorkItem> items_smma_lpt = lpt(items_smma, ksc::sym_mma_chunk());
-    std::vector<int2> cap_tiles_lpt;
     {
         std::vector<int> order(cap.tiles.size());
         for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
         std::stable_sort(order.begin(), order.end(),
                          [&](int a, int b) { return cap.cost[a] > cap.cost[b]; });
-        for (int i : order) cap_tiles_lpt.push_back(cap.tiles[i]);
+        for (int i : order) cap.tiles_lpt.push_back(cap.tiles[i]);
         s->n_cap_tiles = (int)cap.tiles.size();
         s->cap_tile_first.assign(nr + 1, 0);
         size_t i = 0;
@@ -584,7 +629,8 @@ int finish_split(ksc_split *s, const ksc_split_opts &o) {
             s->irr_item_first[r] = (int)i;
         }
     }
-    std::vector<float2> ringc(s->n_cap_tiles ? nr : 0);
+    const bool plan_cap = s->n_cap_tiles > 0;
+    std::vector<float2> ringc(plan_cap ? nr : 0);
     for (size_t r = 0; r < ringc.size(); ++r) {
         const ksc::DF c = ksc::df_from_double(kPi / (double)g.len[r]);
         ringc[r] = make_float2(c.h, c.l);
@@ -621,24 +667,6 @@ int finish_split(ksc_split *s, const ksc_split_opts &o) {
         return cuda_fail(e, "upload work list");
     if ((e = dev_upload(&s->d_items_mma, items_mma.data(), items_mma.size())) != cudaSuccess)
         return cuda_fail(e, "upload work list");
-    // the coefficients are the one large table: without room for them the gather sums the caps
-    if (s->n_cap_tiles && cudaMalloc(&s->d_coef, 16ull * cap.coef_off.back()) != cudaSuccess) {
-        cudaGetLastError();
-        s->d_coef = nullptr;
-        s->n_cap_tiles = 0;
-        s->ctc = ksc::CapTc();
-    }
-    if (s->n_cap_tiles) {
-        if ((e = dev_upload(&s->d_cap_tiles, cap.tiles.data(), cap.tiles.size())) != cudaSuccess ||
-            (e = dev_upload(&s->d_cap_tiles_lpt, cap_tiles_lpt.data(), cap_tiles_lpt.size())) !=
-                cudaSuccess ||
-            (e = dev_upload(&s->d_ncut, cap.ncut.data(), cap.ncut.size())) != cudaSuccess ||
-            (e = dev_upload(&s->d_coef_off, cap.coef_off.data(), cap.coef_off.size())) != cudaSuccess ||
-            (e = dev_upload(&s->d_irr_items, cap.irr_items.data(), cap.irr_items.size())) != cudaSuccess ||
-            (e = dev_upload(&s->d_irr_first, cap.irr_first.data(), cap.irr_first.size())) != cudaSuccess ||
-            (e = dev_upload(&s->d_irr, cap.irr.data(), cap.irr.size())) != cudaSuccess)
-            return cuda_fail(e, "cap tiles");
-    }
     if ((e = dev_malloc((void **)&s->d_err, sizeof(int))) != cudaSuccess)
         return cuda_fail(e, "error flag");
     if ((e = cudaMemset(s->d_err, 0, sizeof(int))) != cudaSuccess)
@@ -650,14 +678,14 @@ int finish_split(ksc_split *s, const ksc_split_opts &o) {
         return cuda_fail(e, "upload coefficients");
     // With a tensor-core cap stage the table runs past the cut; its intervals up to the
     // cut, and the entry at the cut with its higher terms dropped, are the table proper.
-    const int n_build = s->n_cap_tiles ? n_ext : n_int;
-    // nodes | the table run past the cut, its rounding errors, pi / L per ring
+    const int n_build = plan_cap ? n_ext : n_int;
+    // nodes | the table run past the cut, its rounding errors, pi / L per ring, a flag
     const size_t b_nodes = sizeof(double) * 2 * (size_t)(n_build + 1);
-    const size_t b_ext = s->n_cap_tiles ? sizeof(float4) * (size_t)(n_build + 1) : 0;
-    const size_t b_lo = s->n_cap_tiles ? (sizeof(float) * (size_t)n_build + 15) / 16 * 16 : 0;
+    const size_t b_ext = plan_cap ? sizeof(float4) * (size_t)(n_build + 1) : 0;
+    const size_t b_lo = plan_cap ? (sizeof(float) * (size_t)n_build + 15) / 16 * 16 : 0;
     unsigned char *d_scratch = nullptr;
     if ((e = dev_malloc((void **)&d_scratch,
-                        (b_nodes + 15) / 16 * 16 + b_ext + b_lo + sizeof(float2) * ringc.size())) !=
+                        (b_nodes + 15) / 16 * 16 + b_ext + b_lo + sizeof(float2) * ringc.size() + sizeof(int))) !=
         cudaSuccess) {
         cudaFree(d_c);
         return cuda_fail(e, "allocate table nodes");
@@ -670,11 +698,11 @@ int finish_split(ksc_split *s, const ksc_split_opts &o) {
     float4 *d_ext = reinterpret_cast<float4 *>(d_scratch + (b_nodes + 15) / 16 * 16);
     float *d_lo = reinterpret_cast<float *>(d_ext + b_ext / sizeof(float4));
     float2 *d_ringc = reinterpret_cast<float2 *>(reinterpret_cast<unsigned char *>(d_lo) + b_lo);
-    float4 *built = s->n_cap_tiles ? d_ext : s->d_tab;
+    float4 *built = plan_cap ? d_ext : s->d_tab;
     ksc::TableBuild tb{d_c, s->lmax, n_build, s->chord_cut / n_int, built, d_nodes, 1};
-    if (s->n_cap_tiles) tb.d_lo = d_lo;
+    if (plan_cap) tb.d_lo = d_lo;
     e = ksc::launch_table_build(tb, 0);
-    if (e == cudaSuccess && s->n_cap_tiles) {
+    if (e == cudaSuccess && plan_cap) {
         e = cudaMemcpyAsync(s->d_tab, built, sizeof(float4) * (n_int + 1),
                             cudaMemcpyDeviceToDevice, 0);
         if (e == cudaSuccess) e = cudaMemsetAsync(&s->d_tab[n_int].z, 0, 2 * sizeof(float), 0);
@@ -721,12 +749,10 @@ int finish_split(ksc_split *s, const ksc_split_opts &o) {
         p.belt_c1l = c1.l;
     }
     const int rc = plan_belt_tc(s, g, range, pairs, pair_base);
-    if (rc || s->ctc.ring_end < s->ctc.ring_first) return rc;
-    ksc::CapCoef cc{d_ext, d_lo, d_ringc, s->d_coef, n_ext, (float)((double)n_ext * n_ext), {}, {}};
-    e = ksc::launch_cap_coef(s->plan, s->ctc, cc, 0);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(0);
-    if (e != cudaSuccess) return cuda_fail(e, "cap coefficients");
-    return KSC_OK;
+    if (rc || !plan_cap) return rc;
+    ksc::CapCoef cc{d_ext, d_lo, d_ringc, nullptr, reinterpret_cast<int *>(d_ringc + ringc.size()),
+                    n_ext, (float)((double)n_ext * n_ext), {}, {}};
+    return build_cap_tc(s, cap, cc);
 }
 
 int check_common(int lmax, int nside, double theta_cut) {

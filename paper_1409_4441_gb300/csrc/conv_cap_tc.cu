@@ -785,6 +785,7 @@ cap_coef_kernel(const ConvPlan P, const CapTc C, const CapCoef K, int ring_lo, i
 #pragma unroll
             for (int p = 0; p < kP; ++p) {
                 const double v = c[p] * (double)C.wscale;
+                if (!(fabs(v) <= 65504.0)) *K.d_too_large = 1;
                 const __half h = __float2half_rn((float)v);
                 const __half l = __float2half_rn((float)(v - (double)__half2float(h)));
                 dst[j * kP + p] = (uint32_t)__half_as_ushort(l) << 16 | __half_as_ushort(h);

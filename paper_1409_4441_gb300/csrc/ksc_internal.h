@@ -257,6 +257,7 @@ struct CapCoef {                        // what building the coefficients needs
     const float *d_tab_lo;              // ... and the rounding errors of its node values
     const float2 *d_ringc;              // per ring: pi / L as a double-float pair
     unsigned *d_coef;
+    int *d_too_large;                   // set where a coefficient does not fit an FP16 number
     int n_ext;                          // intervals of d_tab
     float next2;                        // n_ext^2
     double me[16], mo[16];              // node values -> even, odd coefficients

@@ -1,0 +1,54 @@
+"""The tensor-core cap stage where a kernel or a map is outside what its FP16 operands carry.
+
+Tolerance: the per-pixel parity bound of the other kernels, 1e-6 of the output rms plus the
+oracle's bound on pairs whose chord lies within rounding of the cut.
+"""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_1409_4441_gb300 import inputs
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def K():
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_1409_4441_gb300 import ksconv
+    return ksconv
+
+
+def _legendre(lmax, z):
+    p = np.zeros(lmax + 1)
+    p[0], p[1] = 1.0, z
+    for l in range(2, lmax + 1):
+        p[l] = ((2 * l - 1) * z * p[l - 1] - (l - 1) * p[l - 2]) / l
+    return p
+
+
+def _cap_pixels(nside, n, seed):
+    cap, N = 2 * nside * (nside - 1), 12 * nside * nside
+    north = np.concatenate([np.arange(24), inputs.rng(seed).choice(cap, n, replace=False)])
+    return np.unique(np.concatenate([north, N - 1 - north]))
+
+
+# A ring of 2.5 pixels FWHM around the cut: the kernel rises past the cut, where the edge cells'
+# polynomials reach (up to 1.1e5 in units that put the largest value inside the cut at 2^13).
+def test_kernel_that_rises_past_the_cut(K):
+    nside, tc = 512, 640.0 * inputs.ARCMIN
+    pixel = 3518.0 / nside * inputs.ARCMIN
+    c = inputs.gaussian_beam(2 * nside, 2.5 * pixel) * _legendre(2 * nside, np.cos(tc + 3.5 * pixel))
+    with K.make_split_real(c, nside, tc) as sp:
+        m = inputs.white_noise_map(nside, 191).astype(np.float32)
+        x = torch.tensor(m, device="cuda")
+        y = torch.empty_like(x)
+        K.conv_real(sp, x, y)
+        K.device_status(sp)
+        tab = O.hermite_nodes(c, tc, K.split_info(sp)["n_intervals"])
+    pix = _cap_pixels(nside, 300, 5)
+    ref, amb = O.brute_conv(nside, m.astype(np.float64), tc, table=tab, out_pix=pix)
+    err = np.abs(y.cpu().numpy()[pix] - ref) - amb
+    assert err.max() <= 1e-6 * np.sqrt(np.mean(ref ** 2))
