@@ -840,8 +840,9 @@ cap_direct_kernel(const ConvPlan P, const int2 *__restrict__ items,
                 const float xh = nf * pi.ch, xl = fmaf(nf, pi.ch, -xh) + nf * pi.cl;
                 int ti;
                 float f;
-                const bool in_cut = chord_to_table_sel(A, B, sin_df(xh, xl), P.nint2, &ti, &f);
-                const float w = in_cut ? hermite(__ldg(&P.d_tab[min(ti, P.n_int)]), f) : 0.0f;
+                // (a pixel past the cut adds nothing, whatever its value)
+                if (!chord_to_table_sel(A, B, sin_df(xh, xl), P.nint2, &ti, &f)) continue;
+                const float w = hermite(__ldg(&P.d_tab[min(ti, P.n_int)]), f);
 #pragma unroll
                 for (int a = 0; a < 4; ++a) {
                     int i = j + a * Qq;

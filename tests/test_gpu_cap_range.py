@@ -52,3 +52,33 @@ def test_kernel_that_rises_past_the_cut(K):
     ref, amb = O.brute_conv(nside, m.astype(np.float64), tc, table=tab, out_pix=pix)
     err = np.abs(y.cpu().numpy()[pix] - ref) - amb
     assert err.max() <= 1e-6 * np.sqrt(np.mean(ref ** 2))
+
+
+def _far_from_ring_97(nside, tc):
+    """A pixel of ring 98 (from 1) of nside 256, whose windows there are wider than any tile's, and pixels
+    of the rings around it on the far side of the pole, beyond the cut."""
+    z, _, n, st, _ = O.ring_table(nside)
+    bad = int(st[97])
+    pix = np.concatenate([np.arange(st[r] + int(0.43 * n[r]), st[r] + int(0.57 * n[r])) for r in range(85, 125)])
+    vec = O.pix2vec(nside)
+    return bad, pix[np.arccos(np.clip(vec[pix] @ vec[bad], -1, 1)) > tc + np.radians(2.0)]
+
+
+@pytest.mark.parametrize("bad", [-1.6375e30, float("inf"), float("nan")])
+def test_polar_value_past_the_cut_stays_out(K, bad):
+    nside, tc = 256, 1800.0 * inputs.ARCMIN
+    c = inputs.gaussian_beam(2 * nside, 3.0 * 3518.0 / nside * inputs.ARCMIN)
+    p_bad, far = _far_from_ring_97(nside, tc)
+    assert far.size > 500
+    m = inputs.white_noise_map(nside, 193).astype(np.float32)
+    clean = m.astype(np.float64)
+    m[p_bad], clean[p_bad] = bad, 0.0
+    with K.make_split_real(c, nside, tc) as sp:
+        x = torch.tensor(m, device="cuda")
+        y = torch.empty_like(x)
+        K.conv_real(sp, x, y)
+        K.device_status(sp)
+        tab = O.hermite_nodes(c, tc, K.split_info(sp)["n_intervals"])
+    ref, amb = O.brute_conv(nside, clean, tc, table=tab, out_pix=far)
+    err = np.abs(y.cpu().numpy()[far] - ref) - amb
+    assert err.max() <= 1e-6 * np.sqrt(np.mean(ref ** 2))
