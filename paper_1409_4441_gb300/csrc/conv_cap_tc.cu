@@ -129,7 +129,8 @@ struct QInfo {      // an input ring as the tile sees it
     short n_e;      // elements staged
     short base;     // d0 + 16 s0: Delta of element 0 at offset i = 0
     short jE[2];    // edge cell of each ring (-1: no pixel within the cut)
-    short s0, s1, mid, pad;  // window steps and the chunk of the closest approach
+    short s0, s1, mid;  // window steps and the chunk of the closest approach
+    unsigned short c[2];  // constants taken off the ring and its mirror, BF16 numbers
 };
 
 // Words of a ring pair's coefficients, [cell][power], rounded up to 16 bytes.
@@ -170,8 +171,8 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
     __shared__ __align__(8) uint64_t b_full[kStages], b_free[kStages], d_done, d_free[2], e_ready[2],
         s_drain[4];
     __shared__ uint32_t tmem_base, s_max, s_min;
-    __shared__ int s_abort, s_lo, s_hi, s_bad;
-    __shared__ float s_mean[kT / 32], s_edge[2][2][kP + 3], s_sum[2][2][kP];
+    __shared__ int s_abort, s_lo, s_hi, s_bad, s_shift;
+    __shared__ float s_edge[2][2][kP + 3], s_sum[2][2][kP];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int2 tile = tiles[blockIdx.x];
@@ -190,7 +191,7 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
     if (tid == 0) {
         s_max = 0u;
         s_min = 0xffffffffu;
-        s_abort = s_bad = 0;
+        s_abort = s_bad = s_shift = 0;
         s_lo = min(P.d_range[r0].x, P.d_range[r0 + n_r - 1].x);
         s_hi = max(P.d_range[r0].y, P.d_range[r0 + n_r - 1].y);
         for (int b = 0; b < kStages; ++b) {
@@ -216,6 +217,7 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
         g.jE[0] = g.jE[1] = -1;
         g.eR[0] = g.eR[1] = 0;
         g.off[0] = g.off[1] = 0u;
+        g.c[0] = g.c[1] = 0;
         const bool skip = add && q >= P.belt_lo && q <= P.belt_hi;
         for (int R = 0; R < n_r && !skip; ++R) {
             const int2 rg = P.d_range[r0 + R];
@@ -270,12 +272,6 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
     }
     vmax = __reduce_max_sync(~0u, vmax);
     vmin = __reduce_min_sync(~0u, vmin);
-    if (warp < kT / 32) {  // mean of 512 pixels of the tile's first ring
-        float v = m[Ra.start + (int)((long long)tid * L0 / kT)];
-#pragma unroll
-        for (int s = 16; s > 0; s >>= 1) v += __shfl_xor_sync(~0u, v, s);
-        if (lane == 0) s_mean[warp] = v * (1.0f / 32.0f);
-    }
     if (lane == 0) {
         atomicMax(&s_max, vmax);
         atomicMin(&s_min, vmin);
@@ -305,19 +301,37 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
         }
         if (s_bad) atomicExch(err, KSC_ERR_DEVICE_BOUNDS);
     }
-    // a constant taken off where every block is within a factor of four of the largest: a
-    // multiple of 2^-3 of the largest value's power of two (none for maps about zero)
-    float mean = 0.0f;
-    if (!zero && !flag && emax - emin <= 1u) {
+    // A constant taken off an input ring whose blocks are all within a factor of four of its
+    // largest: near the mean of 32 of its pixels, a multiple of 2^-3 of the largest value's
+    // power of two (none for maps about zero).  The MMAs' cuts are toward zero and add up
+    // where all products have one sign; the sums of the weights put the constant back.
+    if (!zero && !flag && !s_bad) {
+        for (int i = warp; i < 2 * nq; i += kThreads / 32) {
+            QInfo &g = sQ[i >> 1];
+            const int h = i & 1;
+            if (max((int)g.jE[0], (int)g.jE[1]) < 0) continue;
+            const uint2 e = rr[h ? P.nrings - 1 - (q_lo + (i >> 1)) : q_lo + (i >> 1)];
+            if (e.x == 0u || (e.x >> 23) - (e.y >> 23) > 1u) continue;
+            int k = g.a + lane * g.n_e / 32;
+            while (k >= g.len) k -= g.len;
+            float v = __ldg(m + g.start[h] + k);
 #pragma unroll
-        for (int i = 0; i < kT / 32; ++i) mean += s_mean[i];
-        const float quantum = __uint_as_float((emax - 3u) << 23);
-        mean = rintf(mean * (1.0f / (kT / 32)) / quantum) * quantum;
+            for (int s = 16; s > 0; s >>= 1) v += __shfl_xor_sync(~0u, v, s);
+            const float quantum = __uint_as_float(((e.x >> 23) - 3u) << 23);
+            v = rintf(v * (1.0f / 32.0f) / quantum) * quantum;
+            if (lane == 0 && v != 0.0f) {
+                g.c[h] = (unsigned short)(__float_as_uint(v) >> 16);  // (five digits: exact)
+                s_shift = 1;
+            }
+        }
     }
-    const uint32_t ex = emax + (mean != 0.0f ? 1u : 0u);
+    __syncthreads();
+    const uint32_t ex = emax + (s_shift ? 1u : 0u);  // |m - c| may reach twice the largest |m|
     const float xscale = zero || flag ? 1.0f : __uint_as_float((127u + tc::kXExp + 127u - ex) << 23);
     const float xunscale = zero || flag ? 1.0f : __uint_as_float((ex - tc::kXExp) << 23);
-    const float ms = mean * xscale;
+    auto shift_of = [&](const QInfo &g, int h) {  // scaled
+        return __uint_as_float((uint32_t)g.c[h] << 16) * xscale;
+    };
     bool drained = true;
     // hemispheres with an output ring in the band; the other one's products are left out (its
     // accumulators hold anything, and nothing of them is written; the 1023 rings of the
@@ -430,6 +444,8 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
                 // the ring's other warps have added ring n - 1: outputs change hands
                 asm volatile("bar.sync %0, 128;" ::"r"(2 + R) : "memory");
                 const int jE = g.jE[R], Lq = g.len, step = 2 * Lq;
+                const bool shifted = g.c[0] | g.c[1];
+                const float ms_n = shift_of(g, 0), ms_s = shift_of(g, 1);
                 // outputs at positions n0 + 256 quarter .. + 255: k in [kA, kB]
                 auto first = [&](int pos) {  // ceil(num / step)
                     const int num = (2 * pos + g.phase - 1) * L - t * Lq;
@@ -493,8 +509,7 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
                         uint32_t a[8], b[8];
                         tc::tmem_ld8(c, a);
                         tc::tmem_ld8(c + kHemi, b);
-                        float off = 0.0f;
-                        if (mean != 0.0f && !(p & 1)) off = ms * s_sum[buf][R][p];
+                        const float ws = shifted && !(p & 1) ? s_sum[buf][R][p] : 0.0f;
                         uint64_t w[8];
                         if (p < kP3) {
                             uint32_t xa[8], xb[8];
@@ -509,9 +524,9 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
 #pragma unroll
                             for (int i = 0; i < 8; ++i) w[i] = (uint64_t)b[i] << 32 | a[i];
                         }
-                        if (mean != 0.0f)
+                        if (shifted)
 #pragma unroll
-                            for (int i = 0; i < 8; ++i) w[i] = add2(w[i], pack2(off, off));
+                            for (int i = 0; i < 8; ++i) w[i] = add2(w[i], pack2(ms_n * ws, ms_s * ws));
                         __syncwarp();
                         ulonglong2 *dst = reinterpret_cast<ulonglong2 *>(turn + 10 * lane);
 #pragma unroll
@@ -597,6 +612,7 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
                 const QInfo g = sQ[qi];
                 const uint32_t buf = n & 1u;
                 const int n_pos = 16 * (g.s1 - g.s0);
+                const float ms_n = shift_of(g, 0), ms_s = shift_of(g, 1);
                 // ring n - 2 has left these buffers
                 if (n >= 2) wait_all(&d_free[buf], ((n >> 1) - 1u) & 1u, &s_abort);
                 // ---- the segments, as they are and scaled and split
@@ -609,7 +625,7 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
                     for (int h = 0; h < 2; ++h) {
                         if (!(h ? band_s : band_n)) continue;
                         __half *xh = sX + (h * 2 + buf) * 2 * xc;
-                        const float y = fmaf(h ? xs[e] : xn[e], xscale, -ms);
+                        const float y = fmaf(h ? xs[e] : xn[e], xscale, h ? -ms_s : -ms_n);
                         const __half hh = __float2half_rn(y);
                         xh[i] = hh;
                         xh[xc + i] = __float2half_rn(y - __half2float(hh));
@@ -659,7 +675,7 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
                                                 __half2float(__ushort_as_half((unsigned short)(hl >> 16)));
                         }
                     }
-                    if (mean != 0.0f) {  // sums of the even coefficients over a window
+                    if (g.c[0] | g.c[1]) {  // sums of the even coefficients over a window
                         for (int task = bw; task < 10; task += kBuild / 32) {
                             const int R = task / 5, p = 2 * (task % 5);
                             const uint32_t *src = raw + (R ? raw1 : 0) + p;

@@ -82,3 +82,49 @@ def test_polar_value_past_the_cut_stays_out(K, bad):
     ref, amb = O.brute_conv(nside, clean, tc, table=tab, out_pix=far)
     err = np.abs(y.cpu().numpy()[far] - ref) - amb
     assert err.max() <= 1e-6 * np.sqrt(np.mean(ref ** 2))
+
+
+@pytest.mark.parametrize("bad", [1e8, float("nan")])
+def test_polar_value_does_not_set_the_constant(K, bad):
+    """A map about 50: what a tile takes off its input rings comes from those rings, not from one that
+    its products leave out."""
+    nside, tc = 256, 1800.0 * inputs.ARCMIN
+    c = inputs.gaussian_beam(2 * nside, 3.0 * 3518.0 / nside * inputs.ARCMIN)
+    p_bad, far = _far_from_ring_97(nside, tc)
+    m = (inputs.white_noise_map(nside, 194) + 50.0).astype(np.float32)
+    clean = m.astype(np.float64)
+    m[p_bad], clean[p_bad] = bad, 0.0
+    with K.make_split_real(c, nside, tc) as sp:
+        x = torch.tensor(m, device="cuda")
+        y = torch.empty_like(x)
+        K.conv_real(sp, x, y)
+        K.device_status(sp)
+        tab = O.hermite_nodes(c, tc, K.split_info(sp)["n_intervals"])
+    ref, amb = O.brute_conv(nside, clean, tc, table=tab, out_pix=far)
+    err = np.abs(y.cpu().numpy()[far] - ref) - amb
+    assert err.max() <= 1e-6 * np.sqrt(np.mean(ref ** 2))
+
+
+def test_positive_map_has_no_bias(K):
+    """Products of one sign and a kernel whose lobes cancel: the mean relative error of belt and of
+    cap outputs stays below the FP32 spacing of the result, 2^-23 (rounding to nearest leaves a
+    few tenths of it, the scale factors' own)."""
+    nside, tc = 1024, 400.0 * inputs.ARCMIN
+    ell = np.arange(2 * nside + 1)
+    b = inputs.gaussian_beam(2 * nside, 10.0 * inputs.ARCMIN)
+    z, _, n, _, _ = O.ring_table(nside)
+    g = inputs.rng(195).standard_normal(12 * nside * nside)
+    m = (np.exp(2.5 * np.repeat(z, n.astype(int)) + 0.3 * g) + 0.01).astype(np.float32)
+    with K.make_split(b, nside, 512, tc, cl_in=1.0 / (ell + 10.0) ** 2) as sp:
+        x = torch.tensor(m, device="cuda")
+        y = torch.empty_like(x)
+        K.conv_real(sp, x, y)
+        K.device_status(sp)
+        tab = O.hermite_nodes(K.split_real_coeffs(sp), tc, K.split_info(sp)["n_intervals"])
+    cap, N = 2 * nside * (nside - 1), 12 * nside * nside
+    for lo, hi in ((cap, N - cap), (0, cap)):
+        pix = np.sort(inputs.rng(196).choice(np.arange(lo, hi), 700, replace=False))
+        ref, amb = O.brute_conv(nside, m.astype(np.float64), tc, table=tab, out_pix=pix)
+        d = y.cpu().numpy()[pix] - ref
+        rel = np.sign(d) * np.maximum(np.abs(d) - amb, 0.0) / np.abs(ref)
+        assert abs(rel.mean()) <= 2.0 ** -23
