@@ -342,7 +342,7 @@ conv_belt_tc_kernel(const ConvPlan P, int block_lo, int n_tiles_k, int ring_lo, 
                 const uint32_t t = td + b * N + c;
                 __syncwarp();
                 if constexpr (kStep == 16) tc::tmem_ld16(t, v); else tmem_ld8(t, v);
-                tc::tmem_wait_ld();
+                tc::loaded(v);
 #pragma unroll
                 for (int e = 0; e < kStep; e += 2) {
                     const uint64_t y = pack2(v[e], v[e + 1]), t0 = tot[(c + e) / 2];
@@ -527,7 +527,8 @@ conv_belt_tc_kernel(const ConvPlan P, int block_lo, int n_tiles_k, int ring_lo, 
                 for (int e = 0; e < 8; ++e) v0[e] = v1[e] = 0u;
                 if (n_rings >= 1) tmem_ld8(td + c, v0);
                 if (n_rings >= 2) tmem_ld8(td + N + c, v1);
-                tc::tmem_wait_ld();
+                tc::loaded(v0);
+                tc::loaded(v1);
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
                     const uint64_t tt = tot[(c + e) / 2];

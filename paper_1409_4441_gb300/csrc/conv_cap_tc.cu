@@ -515,12 +515,16 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
                             uint32_t xa[8], xb[8];
                             tc::tmem_ld8(c + kN, xa);
                             tc::tmem_ld8(c + kN + kHemi, xb);
-                            tc::tmem_wait_ld();
+                            tc::loaded(a);
+                            tc::loaded(b);
+                            tc::loaded(xa);
+                            tc::loaded(xb);
 #pragma unroll
                             for (int i = 0; i < 8; ++i)
                                 w[i] = add2((uint64_t)b[i] << 32 | a[i], (uint64_t)xb[i] << 32 | xa[i]);
                         } else {
-                            tc::tmem_wait_ld();
+                            tc::loaded(a);
+                            tc::loaded(b);
 #pragma unroll
                             for (int i = 0; i < 8; ++i) w[i] = (uint64_t)b[i] << 32 | a[i];
                         }

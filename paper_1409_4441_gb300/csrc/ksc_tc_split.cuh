@@ -49,6 +49,15 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t *v) {
         : "memory");
 }
 
+// Waits for this thread's tensor-memory loads, the last of them into v: a use of v cannot be
+// moved before the wait (the load's asm statement alone would allow it).
+template <int N>
+__device__ __forceinline__ void loaded(uint32_t (&v)[N]) {
+    tmem_wait_ld();
+#pragma unroll
+    for (int i = 0; i < N; ++i) asm volatile("" : "+r"(v[i]));
+}
+
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(bar)) : "memory");
 }
