@@ -193,18 +193,22 @@ conv_belt_tc_kernel(const ConvPlan P, int block_lo, int n_tiles_k, int ring_lo, 
         vmax = max(vmax, qmax);
         vmin = min(vmin, qmin);
         // A constant taken off the ring where its blocks are all within a factor of four of the
-        // largest: near the mean of 32 of its pixels, a multiple of 2^-3 of the largest value's
-        // power of two (none for maps about zero).
+        // largest: near the mean of 128 of its pixels, a multiple of 2^-3 of the largest value's
+        // power of two, where it is at least two of them (not for maps about zero).
         unsigned short shift = 0;
         if (qmax != 0u && qmax < 0x7f800000u && qmax >= 0x02000000u && (qmax >> 23) - (qmin >> 23) <= 1u) {
-            int i = a + (int)((long long)lane * len / 32);
-            i -= i >= L ? L : 0;
-            float v = __ldg(m + start + i);
+            float v = 0.0f;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                int i = a + (int)((4u * lane + j) * (unsigned)len / 128u);
+                i -= i >= L ? L : 0;
+                v += __ldg(m + start + i);
+            }
 #pragma unroll
             for (int s = 16; s > 0; s >>= 1) v += __shfl_xor_sync(~0u, v, s);
             const float quantum = __uint_as_float(((qmax >> 23) - 3u) << 23);
-            v = rintf(v * (1.0f / 32.0f) / quantum) * quantum;
-            shift = (unsigned short)(__float_as_uint(v) >> 16);  // (five digits: exact)
+            v = rintf(v * (1.0f / 128.0f) / quantum) * quantum;
+            if (fabsf(v) >= 2.0f * quantum) shift = (unsigned short)(__float_as_uint(v) >> 16);  // (five digits: exact)
         }
         if (lane == 0 && q - q_lo < nq_cap) {
             sC[q - q_lo] = shift;

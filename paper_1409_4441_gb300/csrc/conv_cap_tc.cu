@@ -265,6 +265,8 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
                 const uint2 e = rr[h ? P.nrings - 1 - q : q];
                 vmax = max(vmax, e.x);
                 vmin = min(vmin, e.y);
+                // blocks all within a factor of four of the largest: a constant may be taken off
+                g.c[h] = e.x != 0u && (e.x >> 23) - (e.y >> 23) <= 1u;
             }
         }
         if (qi < C.nq) sQ[qi] = g;
@@ -302,26 +304,30 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
         if (s_bad) atomicExch(err, KSC_ERR_DEVICE_BOUNDS);
     }
     // A constant taken off an input ring whose blocks are all within a factor of four of its
-    // largest: near the mean of 32 of its pixels, a multiple of 2^-3 of the largest value's
-    // power of two (none for maps about zero).  The MMAs' cuts are toward zero and add up
+    // largest: near the mean of 128 of its pixels, a multiple of 2^-3 of the largest value's
+    // power of two, where it is at least two of them (not for maps about zero).  The MMAs' cuts are toward zero and add up
     // where all products have one sign; the sums of the weights put the constant back.
     if (!zero && !flag && !s_bad) {
         for (int i = warp; i < 2 * nq; i += kThreads / 32) {
             QInfo &g = sQ[i >> 1];
             const int h = i & 1;
-            if (max((int)g.jE[0], (int)g.jE[1]) < 0) continue;
-            const uint2 e = rr[h ? P.nrings - 1 - (q_lo + (i >> 1)) : q_lo + (i >> 1)];
-            if (e.x == 0u || (e.x >> 23) - (e.y >> 23) > 1u) continue;
-            int k = g.a + lane * g.n_e / 32;
-            while (k >= g.len) k -= g.len;
-            float v = __ldg(m + g.start[h] + k);
+            if (!g.c[h]) continue;
+            const uint32_t top = rr[h ? P.nrings - 1 - (q_lo + (i >> 1)) : q_lo + (i >> 1)].x;
+            float v = 0.0f;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                int k = g.a + (4 * lane + j) * g.n_e / 128;
+                while (k >= g.len) k -= g.len;
+                v += __ldg(m + g.start[h] + k);
+            }
 #pragma unroll
             for (int s = 16; s > 0; s >>= 1) v += __shfl_xor_sync(~0u, v, s);
-            const float quantum = __uint_as_float(((e.x >> 23) - 3u) << 23);
-            v = rintf(v * (1.0f / 32.0f) / quantum) * quantum;
-            if (lane == 0 && v != 0.0f) {
-                g.c[h] = (unsigned short)(__float_as_uint(v) >> 16);  // (five digits: exact)
-                s_shift = 1;
+            const float quantum = __uint_as_float(((top >> 23) - 3u) << 23);
+            v = rintf(v * (1.0f / 128.0f) / quantum) * quantum;
+            if (fabsf(v) < 2.0f * quantum) v = 0.0f;
+            if (lane == 0) {
+                g.c[h] = (unsigned short)(__float_as_uint(v + 0.0f) >> 16);  // (five digits: exact)
+                if (v != 0.0f) s_shift = 1;
             }
         }
     }
@@ -445,7 +451,6 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
                 asm volatile("bar.sync %0, 128;" ::"r"(2 + R) : "memory");
                 const int jE = g.jE[R], Lq = g.len, step = 2 * Lq;
                 const bool shifted = g.c[0] | g.c[1];
-                const float ms_n = shift_of(g, 0), ms_s = shift_of(g, 1);
                 // outputs at positions n0 + 256 quarter .. + 255: k in [kA, kB]
                 auto first = [&](int pos) {  // ceil(num / step)
                     const int num = (2 * pos + g.phase - 1) * L - t * Lq;
@@ -509,7 +514,6 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
                         uint32_t a[8], b[8];
                         tc::tmem_ld8(c, a);
                         tc::tmem_ld8(c + kHemi, b);
-                        const float ws = shifted && !(p & 1) ? s_sum[buf][R][p] : 0.0f;
                         uint64_t w[8];
                         if (p < kP3) {
                             uint32_t xa[8], xb[8];
@@ -528,9 +532,6 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
 #pragma unroll
                             for (int i = 0; i < 8; ++i) w[i] = (uint64_t)b[i] << 32 | a[i];
                         }
-                        if (shifted)
-#pragma unroll
-                            for (int i = 0; i < 8; ++i) w[i] = add2(w[i], pack2(ms_n * ws, ms_s * ws));
                         __syncwarp();
                         ulonglong2 *dst = reinterpret_cast<ulonglong2 *>(turn + 10 * lane);
 #pragma unroll
@@ -541,7 +542,8 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
                             v[o] = fma2(v[o], pack2(f[o], f[o]),
                                         *reinterpret_cast<const uint64_t *>(turn + at[o]));
                     }
-                    if (kb + 32 * kOut > kB) {  // the accumulators are no longer needed
+                    const bool last = kb + 32 * kOut > kB;
+                    if (last && !shifted) {  // the accumulators are no longer needed
                         tc::fence_before_sync();
                         __syncwarp();
                         if (lane == 0) tc::mbar_arrive(&d_free[buf]);
@@ -558,6 +560,28 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
                         s.y = fma2(z, cut, fma2(d, m1, fma2(s.x, m1, w)));
                         s.x = w;
                         *q = s;
+                    }
+                    if (shifted) {  // the constants' share
+                        const float *S = s_sum[buf][R];
+                        const float ms_n = shift_of(g, 0), ms_s = shift_of(g, 1);
+#pragma unroll 1
+                        for (int k = kb + lane; k <= min(kB, kb + 32 * kOut - 1); k += 32) {
+                            const int u = (2 * k + t) * Lq + (1 - g.phase) * L - two_l * p0;
+                            const float f = (float)(u % two_l - L) * inv2L, f2 = f * f;
+                            const float c = fmaf(f2, fmaf(f2, fmaf(f2, fmaf(f2, S[8], S[6]), S[4]), S[2]), S[0]);
+                            ulonglong2 *q = reinterpret_cast<ulonglong2 *>(tot + k - k_lo);
+                            ulonglong2 s = *q;
+                            const uint64_t z = pack2(ms_n * c, ms_s * c);
+                            const uint64_t d = fma2(s.y, m1, z), w = add2(s.x, d);
+                            s.y = fma2(d, m1, fma2(s.x, m1, w));
+                            s.x = w;
+                            *q = s;
+                        }
+                    }
+                    if (last && shifted) {  // (nor the sums of the weights)
+                        tc::fence_before_sync();
+                        __syncwarp();
+                        if (lane == 0) tc::mbar_arrive(&d_free[buf]);
                     }
                 }
                 if (!waited) {  // no outputs here: keep step
