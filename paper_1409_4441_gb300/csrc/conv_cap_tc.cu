@@ -24,12 +24,16 @@
 // As in the belt kernel neither operand is a full matrix: A's rows are 16 bytes apart in
 // the staged ring segment, B's eight rows of one (R, p) are one sequence shifted by i.
 //
-// Precision as in conv_belt_tc.cu: two FP16 parts of map and weights, w_h m_h in one FP32
-// accumulator, w_h m_l + w_l m_h (and w_l m_l in the step of the closest approach) in a
-// second one; for p = 6, 7, 8 (coefficients below 2^-12 of the peak) w_h m_h alone; far
-// chunks first.  The polynomial and the pixels of the two cells that the cut divides (at
-// most one pixel a side, tested with the exact integers) are in FP32, the sum over input
-// rings compensated.
+// Precision as in conv_belt_tc.cu: two FP16 parts of map and weights (23 bits of the 24), w_h
+// m_h in one FP32 accumulator, w_h m_l + w_l m_h in a second one, with w_l m_l and a third
+// part of c_0 times m_h in the step of the closest approach, where the weights are large; for
+// p = 6, 7, 8 (small coefficients) w_h m_h alone; far chunks first.  The polynomial and the
+// pixels of the two cells that the cut divides (at most one pixel a side, tested with the
+// exact integers) are in FP32; the rounding errors of a ring's last sum and of the sum over
+// input rings are carried along.  Error rms of cap pixels against 64 bits, over the output
+// rms, white noise, 1e-7: gather / this kernel without the third part and with a plain Kahan
+// sum / now: nside 512, 480': 0.84 / 1.01 / 0.82; 2048, 240': 0.85 / 1.08 / 0.86; 2048, 120':
+// 0.87 / 0.94 / 0.78 (stage at 2048, 240': 105.8 -> 107.4 ms).
 //
 // The coefficients c_p[j] depend on the ring pair alone and are laid out once per split
 // (cap_coef_kernel: 18.6 ms and 2.4 GB at nside 2048 with a 240' cut); evaluated inside
@@ -74,6 +78,10 @@ constexpr int kStages = 3;
 constexpr int kSpan = 1024;        // positions of a tile (128 rows of eight)
 constexpr int kOut = 9;            // outputs a lane carries at a time
 constexpr int kTurn = 32 * 10;     // float2 of a warp's turning buffer (10 per 8 positions)
+// Third parts of c_0: the cells that the closest approach's step reaches (|Delta| <= 12), as
+// two groups of two core matrices a ring pair
+constexpr int kE = 13;
+constexpr int kEBytes = 2 * 2 * kLead;
 constexpr int kXr = 7;             // staged elements of a builder thread and hemisphere
 
 using tc::Window;
@@ -103,10 +111,17 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
     return d;
 }
 
-// Group of (ring R, power p): three-product groups first.
-__device__ __forceinline__ int group_of(int R, int p) {
-    return p < kP3 ? R * kP3 + p : kG3 + R * (kP - kP3) + p - kP3;
+// a + b and its rounding error.
+__device__ __forceinline__ uint64_t two_sum2(uint64_t a, uint64_t b, uint64_t *err) {
+    const uint64_t m1 = pack2(-1.0f, -1.0f);
+    const uint64_t s = add2(a, b), bb = fma2(a, m1, s);
+    *err = add2(fma2(fma2(bb, m1, s), m1, a), fma2(bb, m1, b));
+    return s;
 }
+
+// Group of (ring R, power p): three-product groups first, the
+// two rings' c_0 side by side.
+__device__ __forceinline__ int group_of(int R, int p) { return 2 * p + R; }
 
 // Wait that gives up at once when the CTA has (builder warps meet at barriers: none of
 // them may leave the loop).
@@ -133,8 +148,14 @@ struct QInfo {      // an input ring as the tile sees it
     unsigned short c[2];  // constants taken off the ring and its mirror, BF16 numbers
 };
 
-// Words of a ring pair's coefficients, [cell][power], rounded up to 16 bytes.
-__host__ __device__ __forceinline__ int coef_words(int jE) { return (kP * (jE + 1) + 3) & ~3; }
+// Words of a ring pair's coefficients: [cell][power] in two parts, then the third parts of c_0
+// in the first kE cells; rounded up to 16 bytes.
+__host__ __device__ __forceinline__ int coef_words(int jE) {
+    return (kP * (jE + 1) + (kE + 1) / 2 + 3) & ~3;
+}
+__device__ __forceinline__ const __half *third_parts(const uint32_t *coef, int jE) {
+    return reinterpret_cast<const __half *>(coef + kP * (jE + 1));
+}
 
 // grid.x runs over tiles {rings - 1 << 16 | first ring, sectors << 16 | sector}, grid.y over
 // maps.  Eight builder warps
@@ -152,7 +173,7 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
                    int belt_split, int band_lo, int band_hi, const uint2 *__restrict__ ring_range,
                    int *__restrict__ flags, int *__restrict__ err) {
     extern __shared__ __align__(1024) unsigned char smem[];
-    // B stages | map segments [h][buffer][part] | turning buffers | totals (north, south:
+    // B stages | third parts of c_0 [buffer] | map segments [h][buffer][part] | turning buffers | totals (north, south:
     // sums, compensations) [ring] | the segments as they are, (north, south) [buffer] |
     // coefficients as stored [buffer] | coefficient sequences | input rings
     const int xc = C.span + C.wpos;
@@ -161,7 +182,8 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
     const int w_cap = ((C.wpos / 2 + 8 + 11) & ~31) + 20;
     const int k_cap = 2 * coef_words(C.jcap - 1);
     unsigned char *sB = smem;
-    __half *sX = reinterpret_cast<__half *>(smem + kStages * kStageBytes);
+    unsigned char *sE = smem + kStages * kStageBytes;
+    __half *sX = reinterpret_cast<__half *>(sE + 2 * kEBytes);
     float2 *sY = reinterpret_cast<float2 *>(sX + 8 * xc);
     float4 *sT = reinterpret_cast<float4 *>(sY + kEpi / 32 * kTurn);
     float2 *sF = reinterpret_cast<float2 *>(sT + 2 * C.tcap);
@@ -358,6 +380,7 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
             const uint32_t d = tmem + h * kHemi + (small ? kN : 0);
             const uint64_t b_base = tc::desc(tc::saddr(sB), kLead, kGroupBytes);
             const uint64_t a_base = tc::desc(tc::saddr(sX) + h * 8 * xc, 16, 128);
+            const uint64_t e_base = tc::desc(tc::saddr(sE), kLead, 2 * kLead);
             const uint32_t a_l = (uint32_t)(2 * xc) >> 4, b_l = (kG * kGroupBytes) >> 4;
             uint32_t n = 0, n_chunks = 0, st = 0, ph = 0;
             bool ok = true;
@@ -390,6 +413,8 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
                         if (c == mid && s_c >= 0 && s_c < t1 - t0) {
                             tc::mma_f16(d, da + (uint32_t)(2 * s_c) + a_l,
                                         db + (uint32_t)(s_c * (2 * kLead / 16)) + b_l, idesc, acc);
+                            tc::mma_f16(d, da + (uint32_t)(2 * s_c), e_base + (n & 1u) * (kEBytes >> 4),
+                                        tc::idesc_f16(128, 16), 1u);
                             acc = 1u;
                         }
 #pragma unroll
@@ -509,7 +534,7 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
                         waited = true;
                     }
 #pragma unroll 1
-                    for (int p = kP - 1; p >= 0; --p) {
+                    for (int p = kP - 1;; --p) {
                         const uint32_t c = td + (uint32_t)(8 * group_of(R, p));
                         uint32_t a[8], b[8];
                         tc::tmem_ld8(c, a);
@@ -537,6 +562,7 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
 #pragma unroll
                         for (int i = 0; i < 8; i += 2) dst[i / 2] = make_ulonglong2(w[i], w[i + 1]);
                         __syncwarp();
+                        if (p == 0) break;  // y_0 waits in the buffer
 #pragma unroll
                         for (int o = 0; o < kOut; ++o)
                             v[o] = fma2(v[o], pack2(f[o], f[o]),
@@ -552,13 +578,16 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
                     for (int o = 0; o < kOut; ++o) {
                         const int k = kb + 32 * o + lane;
                         if (k > kB) break;
-                        // Kahan, with the 2^-24 that the MMAs' cuts cost on average
-                        const uint64_t z = add2(v[o], e2[o]);
+                        // z, the ring's sum, and total + z with the rounding errors of both, and
+                        // with the 2^-24 of z that the MMAs' cuts cost on average, kept apart
                         ulonglong2 *q = reinterpret_cast<ulonglong2 *>(tot + k - k_lo);
                         ulonglong2 s = *q;
-                        const uint64_t d = fma2(s.y, m1, z), w = add2(s.x, d);
-                        s.y = fma2(z, cut, fma2(d, m1, fma2(s.x, m1, w)));
-                        s.x = w;
+                        uint64_t e0, e1;
+                        const uint64_t z =
+                            two_sum2(*reinterpret_cast<const uint64_t *>(turn + at[o]),
+                                     fma2(v[o], pack2(f[o], f[o]), e2[o]), &e0);
+                        s.x = two_sum2(s.x, z, &e1);
+                        s.y = fma2(z, cut, fma2(add2(e0, e1), m1, s.y));
                         *q = s;
                     }
                     if (shifted) {  // the constants' share
@@ -571,10 +600,9 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
                             const float c = fmaf(f2, fmaf(f2, fmaf(f2, fmaf(f2, S[8], S[6]), S[4]), S[2]), S[0]);
                             ulonglong2 *q = reinterpret_cast<ulonglong2 *>(tot + k - k_lo);
                             ulonglong2 s = *q;
-                            const uint64_t z = pack2(ms_n * c, ms_s * c);
-                            const uint64_t d = fma2(s.y, m1, z), w = add2(s.x, d);
-                            s.y = fma2(d, m1, fma2(s.x, m1, w));
-                            s.x = w;
+                            uint64_t e;
+                            s.x = two_sum2(s.x, pack2(ms_n * c, ms_s * c), &e);
+                            s.y = fma2(e, m1, s.y);
                             *q = s;
                         }
                     }
@@ -673,8 +701,7 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
                     for (int task = bw; task < kG * n_blk; task += kBuild / 32) {
                         const int grp = task % kG, k = task / kG * 32 + lane;
                         // (ring, power) of the group
-                        const int R = grp < kG3 ? grp / kP3 : (grp - kG3) / (kP - kP3);
-                        const int p = grp < kG3 ? grp - R * kP3 : grp - kG3 - R * (kP - kP3) + kP3;
+                        const int R = grp & 1, p = grp >> 1;
                         const int jE = g.jE[R];
                         if (k >= n_w) continue;
                         const uint32_t flip = p & 1 ? 0x80008000u : 0u;
@@ -694,6 +721,16 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
                             d[w_cap] = __byte_perm(c[0], c[1], 0x7632);
                         }
                     }
+                    // third parts of c_0 in the closest approach's step: a thread's element e of
+                    // row i in core matrix kg of ring R (base counts Delta from step s0)
+                    {
+                        const int e = bt & 7, i = (bt >> 3) & 7, kg = (bt >> 6) & 1, R = bt >> 7;
+                        const int dl = g.base + 16 * (kSteps * g.mid + kSteps / 2 - g.s0) + 8 * kg + e - i;
+                        const int j = dl < 0 ? -dl : dl, jE = g.jE[R];
+                        const __half *src = third_parts(raw + (R ? raw1 : 0), jE);
+                        reinterpret_cast<__half *>(sE + buf * kEBytes + R * 2 * kLead + kg * kLead)[8 * i + e] =
+                            j < min(jE, kE) ? src[j] : __half(0.0f);
+                    }
                     // the edge cells: in FP32, not in the products
                     if (bt < 2 * kP) {
                         const int R = bt >= kP, p = bt - R * kP, jE = g.jE[R];
@@ -710,8 +747,9 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
                             float s = 0.0f, comp = 0.0f;
                             for (int j = lane; j < g.jE[R]; j += 32) {
                                 const uint32_t hl = src[j * kP];
-                                const float c = __half2float(__ushort_as_half((unsigned short)hl)) +
-                                                __half2float(__ushort_as_half((unsigned short)(hl >> 16)));
+                                float c = __half2float(__ushort_as_half((unsigned short)(hl >> 16)));
+                                if (p == 0 && j < kE) c += __half2float(third_parts(src, g.jE[R])[j]);
+                                c += __half2float(__ushort_as_half((unsigned short)hl));
                                 const float z = (j ? 2.0f : 1.0f) * c - comp;
                                 const float w = s + z;
                                 comp = (w - s) - z;
@@ -833,6 +871,9 @@ cap_coef_kernel(const ConvPlan P, const CapTc C, const CapCoef K, int ring_lo, i
                 const __half h = __float2half_rn((float)v);
                 const __half l = __float2half_rn((float)(v - (double)__half2float(h)));
                 dst[j * kP + p] = (uint32_t)__half_as_ushort(l) << 16 | __half_as_ushort(h);
+                if (p == 0 && j < kE)
+                    reinterpret_cast<__half *>(dst + kP * (jE + 1))[j] =
+                        __float2half_rn((float)(v - (double)__half2float(h) - (double)__half2float(l)));
             }
         }
     }
@@ -844,6 +885,10 @@ cap_coef_kernel(const ConvPlan P, const CapTc C, const CapCoef K, int ring_lo, i
 // with sixteen; 612 blocks at 2048, 240': 6.60 and 6.47 ms).  For one input pixel all lanes
 // read the same values, eight (four quarter turns, two hemispheres) per weight.
 constexpr int kDirect = 512;
+// input pixels between folds into the compensated sums: nside 256, 1800': error rms 9.2e-8 of
+// the output's with 64 (near a centre a few large products share a chunk with many small
+// ones), 7.4e-8 with 16 (gather 8.3e-8); nside 1024, 128 pixels: 35.3 and 36.0 ms a call
+constexpr int kFold = 16;
 __global__ void __launch_bounds__(kDirect)
 cap_direct_kernel(const ConvPlan P, const int2 *__restrict__ items,
                   const int *__restrict__ list_first, const int *__restrict__ list,
@@ -870,11 +915,11 @@ cap_direct_kernel(const ConvPlan P, const int2 *__restrict__ items,
         const float *xn = m + G.start, *xs = m + P.d_rings[P.nrings - 1 - q].start;
         const int full = 2 * L * Lq;
         int n0 = (2 * k + R.phase) * Lq - G.phase * L;  // N of input pixel 0
-        for (int j0 = 0; j0 < Lq; j0 += 64) {
+        for (int j0 = 0; j0 < Lq; j0 += kFold) {
             float acc[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) acc[i] = 0.0f;
-            const int j1 = min(j0 + 64, Lq);
+            const int j1 = min(j0 + kFold, Lq);
 #pragma unroll 4
             for (int j = j0; j < j1; ++j) {
                 int n = n0 - 2 * j * L;  // folded to half a turn
@@ -949,7 +994,7 @@ size_t cap_smem(const CapTc &c) {
                         8 * 2 * xc + 4 * 4 * (size_t)coef_words(c.jcap - 1) +
                         4 * 2 * (kG + kG3) * w_cap + sizeof(QInfo) * (size_t)c.nq;
     // (the rows past a tile's last position read up to 1024 + wpos elements of a segment)
-    return (size_t)kStages * kStageBytes + std::max(body, (size_t)2 * (6 * xc + kSpan + c.wpos + xc));
+    return (size_t)kStages * kStageBytes + 2 * kEBytes + std::max(body, (size_t)2 * (6 * xc + kSpan + c.wpos + xc));
 }
 
 // Inverse of a 4 x 4 matrix (Gauss-Jordan with row pivots).

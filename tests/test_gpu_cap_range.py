@@ -128,3 +128,30 @@ def test_positive_map_has_no_bias(K):
         d = y.cpu().numpy()[pix] - ref
         rel = np.sign(d) * np.maximum(np.abs(d) - amb, 0.0) / np.abs(ref)
         assert abs(rel.mean()) <= 2.0 ** -23
+
+
+# wide windows that are mostly the stage's own, and wide ones that near the poles go the direct way
+@pytest.mark.parametrize("nside,lcut,theta", [(512, 384, 480.0), (256, -1, 1800.0)])
+def test_cap_pixels_are_as_accurate_as_the_gather(K, nside, lcut, theta):
+    """Error rms against 64 bits over 4000 pixels of the caps, the stage and the gather with every
+    weight from the chord on the same map: no larger but for the scatter of such an rms (1.1% each:
+    10% is six times the two together)."""
+    tc, lmax = theta * inputs.ARCMIN, (3 if lcut > 0 else 2) * nside - 1
+    b = inputs.gaussian_beam(lmax, (4.4 if lcut > 0 else 3.0) * 3518.0 / nside * inputs.ARCMIN)
+    ell = np.arange(lmax + 1)
+    m = inputs.white_noise_map(nside, 197).astype(np.float32)
+    x = torch.tensor(m, device="cuda")
+    pix = _cap_pixels(nside, 2000, 8)
+    rms = []
+    for exact in (0, 1):
+        with (K.make_split(b, nside, lcut, tc, cl_in=1.0 / (ell + 10.0) ** 2, exact_weights=exact) if lcut > 0
+              else K.make_split_real(b, nside, tc, exact_weights=exact)) as sp:
+            y = torch.empty_like(x)
+            K.conv_real(sp, x, y)
+            K.device_status(sp)
+            if not exact:
+                tab = O.hermite_nodes(K.split_real_coeffs(sp), tc, K.split_info(sp)["n_intervals"])
+                ref, amb = O.brute_conv(nside, m.astype(np.float64), tc, table=tab, out_pix=pix)
+        err = np.maximum(np.abs(y.cpu().numpy()[pix] - ref) - amb, 0.0)
+        rms.append(np.sqrt(np.mean(err ** 2)))
+    assert rms[0] <= 1.1 * rms[1]
