@@ -56,18 +56,14 @@ FP32_LANES_PER_SM = 128
 DRAM_TRAFFIC = {}
 
 
-def step_kernels(K, nside, theta_cut, opts):
-    """(belt kernel, cap kernel, launches per step): the library's rules for the
-    tensor-core stages by size.  Belt: block maxima, the stage and the FFMA kernel for the
-    tiles it left.  Caps: ring ranges, the stage, its irregular pairs and the gather for the
-    rings it left."""
-    pairs = K.cost_pairs(nside, theta_cut)
-    belt = nside >= 64 and 2.0 / 3.0 * pairs >= 8e8
-    cap = opts.get("cap_kernel", 0) == 0 and 64 <= nside <= 4096 and pairs / 3.0 >= 8e9
-    return ("conv_belt_tc_kernel" if belt else "conv_belt_kernel",
-            "conv_cap_tc_kernel" if cap else
+def step_kernels(K, sp, opts):
+    """(belt kernel, cap kernel, launches per step) of a split's single-map call, as the split
+    reports them."""
+    st = K.split_stages(sp)
+    return ("conv_belt_tc_kernel" if st["belt_columns"] else "conv_belt_kernel",
+            "conv_cap_tc_kernel" if st["cap_stage"] else
             "conv_sym_tc_kernel" if opts.get("cap_kernel", 0) == 1 else "conv_sym_kernel",
-            1 + (1 if belt or cap else 0) + (1 if belt else 0) + 1 + (3 if cap else 0))
+            st["n_launches"])
 
 
 def workload_desc(extra=None):
@@ -470,7 +466,7 @@ def run_ours(args, world, rank, local):
     sm_max = (clocks or {}).get("sm_max_mhz") or pk.get("sm_max_mhz") or 2070.0
     peak_tflops = N_SM * FP32_LANES_PER_SM * 2 * sm_max * 1e6 / 1e12
     n_belt = info["n_pairs_belt"] if info["n_pairs_belt"] >= 0 else 0
-    belt_name, cap_name, launches = step_kernels(K, nside, tc, split_opts(args))
+    belt_name, cap_name, launches = step_kernels(K, sp, split_opts(args))
     stages = {
         belt_name: {"pairs": n_belt, "ms": stage_ms[1]},
         cap_name: {"pairs": n_pairs - n_belt, "ms": stage_ms[2]},

@@ -196,6 +196,18 @@ typedef struct {
 
 /* Describe a split (host struct, filled synchronously). */
 int ksc_split_info(const ksc_split *s, ksc_split_desc *out);
+
+/* The kernels that a single-map call with this split runs. */
+typedef struct {
+    int belt_columns;   /* tensor-core belt stage: tile columns of 8 pixels;
+                           0: FFMA circulant kernel                           */
+    int cap_stage;      /* 1: tensor-core cap stage; 0: gather (or cap_kernel
+                           = 1's tensor form)                                 */
+    int gather_variant; /* tile of the gather: 0 three reflection classes a
+                           thread, 1 small tables, 2 full tables              */
+    int n_launches;     /* kernel launches of one ksc_conv_real               */
+} ksc_stage_desc;
+int ksc_split_stages(const ksc_split *s, ksc_stage_desc *out);
 /* Copy out the harmonic part Khat_l, l = 0..l_cut (host array). */
 int ksc_split_harmonic(const ksc_split *s, double *k_harm);
 /* Copy out the real-space Legendre coefficients c_l, l = 0..lmax (host). */

@@ -1207,6 +1207,21 @@ int ksc_split_info(const ksc_split *s, ksc_split_desc *d) {
     return KSC_OK;
 }
 
+int ksc_split_stages(const ksc_split *s, ksc_stage_desc *d) {
+    if (!s || !d) return fail(KSC_ERR_ARG, "null argument");
+    *d = ksc_stage_desc{};
+    d->gather_variant = s->sym_variant;
+    d->n_launches = 1;
+    if (s->path == 1) return KSC_OK;
+    const bool cap = ksc::has_cap_tc(s), belt = s->btc.n_cols > 0;
+    d->belt_columns = s->btc.n_cols;
+    d->cap_stage = cap;
+    // block maxima, ring ranges; the belt kernel, the stage's too; the gather, the stage's too
+    d->n_launches = (cap || belt) + cap + (s->n_items_belt > 0) + belt + 1 + cap;
+    if (cap && s->irr_item_first.back() > 0) ++d->n_launches;
+    return KSC_OK;
+}
+
 int ksc_split_harmonic(const ksc_split *s, double *k) {
     if (!s || !k) return fail(KSC_ERR_ARG, "null argument");
     std::copy(s->k_harm.begin(), s->k_harm.end(), k);

@@ -38,6 +38,7 @@ KSC_CUT_FREE = 2  # unconstrained fit (K_r may jump at the cut)
 # Every symbol include/ksconv.h declares.
 EXPORTS = [
     "ksc_default_opts", "ksc_make_split", "ksc_make_split_real", "ksc_split_info",
+    "ksc_split_stages",
     "ksc_split_harmonic", "ksc_split_real_coeffs", "ksc_split_model", "ksc_split_table",
     "ksc_conv_real", "ksc_conv_real_rings", "ksc_conv_real_multimap", "ksc_conv_real_batch",
     "ksc_conv_real_host", "ksc_conv_real_stage", "ksc_conv_real_multimap_stage",
@@ -93,6 +94,11 @@ class BatchDesc(ctypes.Structure):
                 ("group_sym_variant", ctypes.c_int * 8)]
 
 
+class StageDesc(ctypes.Structure):
+    _fields_ = [("belt_columns", ctypes.c_int), ("cap_stage", ctypes.c_int),
+                ("gather_variant", ctypes.c_int), ("n_launches", ctypes.c_int)]
+
+
 class CostModel(ctypes.Structure):
     _fields_ = [("gpu_ms0", ctypes.c_double), ("gpu_ms_per_tpair", ctypes.c_double),
                 ("host_ms0", ctypes.c_double), ("host_ms_eq8", ctypes.c_double),
@@ -117,6 +123,7 @@ _sig = {
     "ksc_make_split": [_vp, _i, _i, _i, _d, _vp, ctypes.POINTER(Opts), ctypes.POINTER(_vp)],
     "ksc_make_split_real": [_vp, _i, _i, _d, ctypes.POINTER(Opts), ctypes.POINTER(_vp)],
     "ksc_split_info": [_vp, ctypes.POINTER(Desc)],
+    "ksc_split_stages": [_vp, ctypes.POINTER(StageDesc)],
     "ksc_split_harmonic": [_vp, _vp],
     "ksc_split_real_coeffs": [_vp, _vp],
     "ksc_split_model": [_vp, _vp],
@@ -279,6 +286,13 @@ def split_info(s: Split) -> dict:
     d = Desc()
     _check(_lib.ksc_split_info(s.handle, ctypes.byref(d)), "ksc_split_info")
     return {f: getattr(d, f) for f, _ in Desc._fields_}
+
+
+def split_stages(s: Split) -> dict:
+    """The kernels that a single-map call with this split runs (ksc_split_stages)."""
+    d = StageDesc()
+    _check(_lib.ksc_split_stages(s.handle, ctypes.byref(d)), "ksc_split_stages")
+    return {f: getattr(d, f) for f, _ in StageDesc._fields_}
 
 
 def split_harmonic(s: Split) -> np.ndarray:

@@ -1,0 +1,50 @@
+"""Which kernels a split runs, and the tensor-core stages against the FP64 oracle at sizes that are
+known to be theirs: every tile width of the belt stage, ragged ring blocks, bands and stacks.
+
+Tolerance: the per-pixel parity bound of the other kernels, 1e-6 of the output rms plus the
+oracle's bound on pairs whose chord lies within rounding of the cut.
+"""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_1409_4441_gb300 import inputs
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def K():
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_1409_4441_gb300 import ksconv
+    return ksconv
+
+
+def _split(K, nside, theta_arcmin, **opts):
+    c = inputs.gaussian_beam(2 * nside, 3.0 * 3518.0 / nside * inputs.ARCMIN)
+    return K.make_split_real(c, nside, theta_arcmin * inputs.ARCMIN, **opts), c
+
+
+def _launched(K, sp, x, y):
+    """Kernels of one ksc_conv_real, by name."""
+    from torch.profiler import ProfilerActivity, profile
+    for _ in range(2):  # (the first profile of a process may record nothing)
+        with profile(activities=[ProfilerActivity.CUDA]) as p:
+            K.conv_real(sp, x, y)
+            torch.cuda.synchronize()
+    return [e.name for e in p.events() if "kernel" in e.name]
+
+
+# (nside, cut in arcmin): neither stage, the belt's, both
+@pytest.mark.parametrize("nside,theta", [(64, 360.0), (512, 240.0), (512, 640.0)])
+def test_reported_kernels_are_the_ones_that_run(K, nside, theta):
+    sp, _ = _split(K, nside, theta)
+    x = torch.tensor(inputs.white_noise_map(nside, 11).astype(np.float32), device="cuda")
+    with sp:
+        names = _launched(K, sp, x, torch.empty_like(x))
+        st = K.split_stages(sp)
+    assert len(names) == st["n_launches"], names
+    assert any("conv_belt_tc_kernel" in n for n in names) == (st["belt_columns"] > 0)
+    assert any("conv_cap_tc_kernel" in n for n in names) == (st["cap_stage"] == 1)
