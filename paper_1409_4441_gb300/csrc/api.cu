@@ -104,6 +104,28 @@ void drop_cap_tc(ksc_split *s) {
     s->ctc = ksc::CapTc();
 }
 
+// Whether the cell polynomials carry the kernel to the gather's accuracy; top = the largest |K_r|
+// within the cut, to which outputs compare (not the sum of the Legendre terms, which lies far
+// above it where K_r peaks past the cut or its terms cancel).
+bool cap_polynomials_ok(const ksc_split *s, double top) {
+    // Chebyshev interpolation of degree n leaves, of a term l of the kernel, at most about
+    // 4 J_{n+1}(l h / 2) ~ 4 (l h / 4)^{n+1} / (n+1)!, h the largest pixel step (1.2826 / nside
+    // at the poles).  The coefficients that are multiplied in one part, c_p f^p for p >= n1,
+    // |f| <= 1/2, amount to about (l h / 4)^p / (p/2)!^2 of a term (the p-th derivative of
+    // J_0): one FP16 part keeps them to 2^-12.
+    const int n = ksc::cap_tc_degree(), n1 = ksc::cap_tc_split_powers();
+    double err = 0.0, single = 0.0, fact = 1.0, half = 1.0;
+    for (int i = 2; i <= n + 1; ++i) fact *= i;
+    for (int i = 2; i <= n1 / 2; ++i) half *= i;
+    for (int l = 0; l <= s->lmax; ++l) {
+        const double a = (2.0 * l + 1.0) * std::fabs(s->c_real[l]), x = l * 1.2826 / s->nside / 4.0;
+        err += a * 4.0 * std::pow(x, n + 1) / fact;
+        single += a * std::pow(x, n1) / (half * half);
+    }
+    const double peak = 4.0 * kPi * top;
+    return err <= 5e-8 * peak && single <= std::ldexp(peak, -12);
+}
+
 // Plan of the tensor-core belt stage: the widest window and the most input rings of a
 // 16-ring tile, and the power of two that scales the kernel's largest value (for the cap
 // stage too).
@@ -123,6 +145,7 @@ int plan_belt_tc(ksc_split *s, const ksc::RingGeom &g, const std::vector<int2> &
         drop_cap_tc(s);
         return KSC_OK;
     }
+    if (s->n_cap_tiles && !cap_polynomials_ok(s, top)) drop_cap_tc(s);
     s->btc.wscale = s->ctc.wscale = (float)std::ldexp(1.0, ex);
     s->ctc.wunscale = 1.0f / s->ctc.wscale;
     s->ctc.domega_lo = (float)(4.0 * kPi / s->plan.npix - (double)s->plan.domega);
@@ -179,20 +202,6 @@ void plan_cap_tc(ksc_split *s, const ksc_split_opts &o, const ksc::RingGeom &g,
     // 7.1; 2048, 240' (1.0e12): 150 / 108; with the small tables 1024, 160' (2.9e10): 6.1 / 6.6,
     // the whole call 6.95 / 7.35).
     if (ksc_cost_pairs(nside, s->theta_cut) / 3.0 < (s->sym_variant == 1 ? 5e10 : 8e9)) return;
-    // the cells' polynomials: Chebyshev interpolation of degree n leaves, of a term l of the
-    // kernel, at most about 4 J_{n+1}(l h / 2) ~ 4 (l h / 4)^{n+1} / (n+1)!, h the largest
-    // pixel step (1.2826 / nside at the poles)
-    {
-        const int n = ksc::cap_tc_degree();
-        double err = 0.0, all = 0.0, fact = 1.0;
-        for (int i = 2; i <= n + 1; ++i) fact *= i;
-        for (int l = 0; l <= s->lmax; ++l) {
-            const double a = (2.0 * l + 1.0) * std::fabs(s->c_real[l]);
-            err += a * 4.0 * std::pow(l * 1.2826 / nside / 4.0, n + 1) / fact;
-            all += a;
-        }
-        if (!(err <= 5e-8 * all)) return;
-    }
     const double dc = s->chord_cut, n_int = s->n_int;
     const double scale2 = (n_int / dc) * (n_int / dc), nint2 = n_int * n_int;
     // room for the table past the cut (chords up to 2)

@@ -272,6 +272,7 @@ cudaError_t launch_cap_direct(const ConvPlan &p, const int2 *d_items, int n_item
                               cudaStream_t st);
 int cap_tc_span();                       // input positions of a tile
 int cap_tc_degree();                     // of the cells' polynomials
+int cap_tc_split_powers();               // powers below it are multiplied in two parts
 int cap_tc_positions(int w, int L);
 bool cap_tc_fits(const CapTc &c);
 cudaError_t launch_ring_range(const ConvPlan &p, const unsigned *bm, int n_maps, uint2 *rr,
