@@ -5,6 +5,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <new>
+#include <queue>
 #include <string>
 #include <vector>
 
@@ -173,6 +174,24 @@ int plan_belt_tc(ksc_split *s, const ksc::RingGeom &g, const std::vector<int2> &
     return KSC_OK;
 }
 
+constexpr int kSms = 152;
+
+// Time of independent pieces of work on so many slots, the longest first.
+double makespan(std::vector<double> t, int slots) {
+    std::sort(t.begin(), t.end(), std::greater<double>());
+    std::priority_queue<double, std::vector<double>, std::greater<double>> end;
+    double last = 0.0;
+    for (double x : t) {
+        if ((int)end.size() == slots) {
+            x += end.top();
+            end.pop();
+        }
+        end.push(x);
+        last = std::max(last, x);
+    }
+    return last;
+}
+
 // Plan of the tensor-core cap stage (host): the tiles of the northern rings that have a cap
 // input, the sizes of the kernel's buffers, and the ring pairs that go the direct way:
 // windows that are whole rings or wider than any farther from the poles, input rings of
@@ -189,18 +208,15 @@ struct CapPlan {
 };
 void plan_cap_tc(ksc_split *s, const ksc_split_opts &o, const ksc::RingGeom &g,
                  const std::vector<int2> &range, const std::vector<ksc::PairInfo> &pairs,
-                 const std::vector<int> &pair_base, CapPlan *plan) {
+                 const std::vector<int> &pair_base, double gather_us, CapPlan *plan) {
     const int nside = s->nside, nr = 4 * nside - 1, eq = (nr - 1) / 2;
     const int belt_lo = nside - 1, belt_hi = 3 * nside - 1;
     if (s->path != 0 || o.exact_weights || o.cap_kernel != 0 || nside < 64 || nside > 4096 ||
         s->theta_cut >= kPi || s->n_items_belt == 0)
         return;
-    // Below about 8e9 pairs with a cap ring the gather is the faster one, and below 5e10 where
-    // its small-table tile serves: a tile of the stage spends about 5 us on an input ring, with
-    // few tiles on small maps (gather / tensor stage, ms: nside 256, 640' (1.8e9 pairs): 0.85 /
-    // 1.09; 512, 160': 0.84 / 1.00; 256, 30 deg (1.4e10): 8.7 / 7.4; 512, 640' (2.9e10): 9.0 /
-    // 7.1; 2048, 240' (1.0e12): 150 / 108; with the small tables 1024, 160' (2.9e10): 6.1 / 6.6,
-    // the whole call 6.95 / 7.35).
+    // Not below 8e9 pairs with a cap ring, and below 5e10 where the gather's small-table tile
+    // serves (nside 256, 640' (1.8e9 pairs): gather 0.85, stage 1.09 ms); from there on by the
+    // estimates at the end.
     if (ksc_cost_pairs(nside, s->theta_cut) / 3.0 < (s->sym_variant == 1 ? 5e10 : 8e9)) return;
     const double dc = s->chord_cut, n_int = s->n_int;
     const double scale2 = (n_int / dc) * (n_int / dc), nint2 = n_int * n_int;
@@ -292,7 +308,8 @@ void plan_cap_tc(ksc_split *s, const ksc_split_opts &o, const ksc::RingGeom &g,
             jm = std::max(jm, w);
             const int np = ksc::cap_tc_positions(w, Lq);
             c.wpos = std::max(c.wpos, np);
-            work += np + 60.0;
+            // us on an SM: 5.7 for windows up to about 80 positions, then the products
+            work += 5.7 + 0.024 * std::max(np - 80, 0);
         }
         // (cap rings without a regular pair have a tile too: it writes what the direct ones add to)
         if (lq_max == 0 && r0 >= belt_lo) continue;
@@ -325,6 +342,23 @@ void plan_cap_tc(ksc_split *s, const ksc_split_opts &o, const ksc::RingGeom &g,
         }
     if (!ksc::cap_tc_fits(c) || n4 * 16 > 8ull << 30) plan->tiles.clear();
     if (plan->tiles.empty()) return;
+    // The stage has to be the faster one: its tiles, and the direct pairs (sixteen warps share
+    // a ring's list: 20 ns a pixel), against the gather.  Measured / estimated ratio to the
+    // gather, three-pixel beams: nside 256, 128 pixels 0.74 / 0.81; 512, 96 pixels 0.79 / 0.69; 1024,
+    // 64 pixels 0.98 / 0.98; 2048, 16, 32 and 64 pixels 1.33 / 1.33, 1.07 / 1.06 and 0.83 / 0.85;
+    // 4096, 16 pixels 1.45 / 1.49 (a tile spends 5 us on an input ring however short the window);
+    // 256, 512 pixels 1.40 / 1.77 (all direct).
+    std::vector<double> direct;
+    for (const int2 &it : plan->irr_items) {
+        double us = 0.0;
+        for (int e = plan->irr_first[it.x]; e < plan->irr_first[it.x + 1]; ++e)
+            us += 0.66 + 0.020 * g.len[plan->irr[e]];
+        direct.push_back(us);
+    }
+    if (makespan(plan->cost, kSms) + makespan(direct, kSms) > 0.95 * gather_us) {
+        plan->tiles.clear();
+        return;
+    }
     plan->coef_off.back() = (unsigned)n4;
     c.ring_first = 0;
     c.ring_end = last;
@@ -550,11 +584,14 @@ int finish_split(ksc_split *s, const ksc_split_opts &o) {
         }
     }
 
+    std::vector<double> gather_rings, gather_pos;  // of a northern ring's items
     // Share of the symmetric gather's weight evaluations that the dphi tables serve
     // (per northern output ring: reflection classes x window positions per input ring).
     {
         const int eqr = (nr - 1) / 2;
         double all = 0.0, tab = 0.0, small = 0.0;
+        gather_rings.assign(nr, 0.0);
+        gather_pos.assign(nr, 0.0);
         for (int r = 0; r <= eqr; ++r) {
             const bool belt_r = r >= belt_lo && r <= belt_hi;
             const double cls = (double)ksc::sym_classes(g.len[r], g.phase[r]);
@@ -563,7 +600,9 @@ int finish_split(ksc_split *s, const ksc_split_opts &o) {
                 if (pairs[ip].hw < 0.0f) continue;
                 const bool belt_q = q >= belt_lo && q <= belt_hi;
                 if (s->path == 0 && belt_r && belt_q && !items_belt.empty()) continue;
-                const double n = cls * std::min(2.0 * pairs[ip].hw + 3.0, (double)g.len[q]);
+                const double pos = std::min(2.0 * pairs[ip].hw + 3.0, (double)g.len[q]), n = cls * pos;
+                gather_rings[r] += 1.0;
+                gather_pos[r] += pos;
                 all += n;
                 if (xodd[ip].nct > 0) tab += n;
                 if (xodd[ip].nct > 0 && xodd[ip].nct + 1 <= ksc::kXCapSmall) small += n;
@@ -581,8 +620,21 @@ int finish_split(ksc_split *s, const ksc_split_opts &o) {
                                                                            : 2;
     }
 
+    // The gather's time, about: us per item, input ring and window position, by tile (measured
+    // over nside 512 to 4096, 4 to 64 pixels: within 10%; with the full tables of nside 64 to
+    // 256 about 30%, of which the two factors for maps of few items take half).
+    double gather_us;
+    {
+        const double us_ring[3] = {7.06, 3.41, 1.88}, us_pos[3] = {0.140, 0.091, 0.105};
+        const int v = s->sym_variant;
+        std::vector<double> t;
+        for (const ksc::WorkItem &it : items_sym)
+            t.push_back(us_ring[v] * gather_rings[it.ring] + us_pos[v] * gather_pos[it.ring]);
+        gather_us = makespan(t, (v == 1 ? 3 : 2) * kSms);
+        if (v == 2 && (int)t.size() <= 6 * kSms) gather_us *= (int)t.size() <= kSms ? 0.8 : 1.25;
+    }
     CapPlan cap;
-    plan_cap_tc(s, o, g, range, pairs, pair_base, &cap);
+    plan_cap_tc(s, o, g, range, pairs, pair_base, gather_us, &cap);
     const int n_ext = cap.n_ext;
 
     // The symmetric items longest first, for whole-map launches: CTAs claim items
