@@ -440,6 +440,7 @@ int finish_split(ksc_split *s, const ksc_split_opts &o) {
         int hi = (int)(std::upper_bound(th.begin(), th.end(), th[r] + tc) - th.begin()) - 1;
         range[r] = make_int2(std::max(lo, 0), std::min(hi, nr - 1));
     }
+    s->range = range;
     // Work lists (ring by ring, with per-ring prefixes for latitude bands):
     //  - all:  256-pixel chunks of every ring (pair counting, fallback);
     //  - belt: belt_chunk()-pixel chunks of belt rings (circulant kernel);
@@ -865,8 +866,8 @@ struct CallScratch : ksc::ConvScratch {
 // Takes the scratch and starts the launches that fill it.  Without room for it (npix / 16
 // bytes a map) the FFMA kernels do it all.
 cudaError_t start_scratch(const ksc_split *s, const ksc::MapSet &maps, int n_maps,
-                          cudaStream_t st, CallScratch *w) {
-    const size_t bytes = ksc::conv_scratch_bytes(s, n_maps);
+                          const ksc::ConvUse &use, cudaStream_t st, CallScratch *w) {
+    const size_t bytes = ksc::conv_scratch_bytes(s, n_maps, use);
     if (bytes == 0) return cudaSuccess;
     w->st = st;
     const cudaError_t e = cudaMallocAsync(&w->mem, bytes, st);
@@ -876,7 +877,7 @@ cudaError_t start_scratch(const ksc_split *s, const ksc::MapSet &maps, int n_map
         cudaGetLastError();
         return cudaSuccess;
     }
-    return ksc::start_conv_scratch(s, maps, n_maps, w->mem, w, st);
+    return ksc::start_conv_scratch(s, maps, n_maps, use, w->mem, w, st);
 }
 
 // Tensor-core belt stage for a stack of maps; grows the split's pre-tiled map
@@ -917,12 +918,14 @@ int launch_conv(const ksc_split *s, const float *d_in, float *d_out, int n_maps,
         return KSC_OK;
     }
     const ksc::MapSet maps{d_in, d_out, stride};
-    CallScratch w;
-    e = start_scratch(s, maps, n_maps, st, &w);
-    if (e != cudaSuccess) return cuda_fail(e, "call scratch");
     const bool whole = r0 == 0 && r1 == s->plan.nrings - 1;
     const bool stack = whole && n_maps >= 16;
-    if (stack && s->tensor == 2 && s->n_items_mma > 0) {
+    const bool belt_mma = stack && s->tensor == 2 && s->n_items_mma > 0;
+    CallScratch w;
+    e = start_scratch(s, maps, n_maps,
+                      ksc::conv_use(s, r0, r1, !belt_mma, !(stack && s->tensor >= 1)), st, &w);
+    if (e != cudaSuccess) return cuda_fail(e, "call scratch");
+    if (belt_mma) {
         int rc = launch_belt_tensor(s, d_in, d_out, n_maps, stride, st);
         if (rc) return rc;
     } else {
@@ -948,20 +951,72 @@ namespace ksc {
 
 bool has_cap_tc(const ksc_split *s) { return s->ctc.ring_end >= s->ctc.ring_first; }
 
-size_t conv_scratch_bytes(const ksc_split *s, int n_maps) {
-    const bool cap = has_cap_tc(s), belt = s->btc.n_cols > 0;
+ConvUse conv_use(const ksc_split *s, int r0, int r1, bool want_belt, bool want_cap) {
+    ConvUse u;
+    const int nr = s->plan.nrings, nside = s->nside, eq = (nr - 1) / 2;
+    const int belt_lo = s->plan.belt_lo, belt_hi = s->plan.belt_hi;
+    u.belt = want_belt && s->btc.n_cols > 0 && r0 <= belt_hi && r1 >= belt_lo;
+    // northern rings of the band and its mirror, with the other ring of a cap tile
+    const int lo = std::max(std::min(r0, nr - 1 - r1) - 1, 0);
+    const int hi = std::min((r1 <= eq ? r1 : r0 >= eq ? nr - 1 - r0 : eq) + 1, eq);
+    u.cap = want_cap && has_cap_tc(s) && lo <= s->ctc.ring_end;
+    if (!u.belt && !u.cap) return u;
+    InputReach &in = u.in;
+    if (u.cap) {
+        in.q0 = s->range[lo].x;
+        in.q1 = s->range[hi].y;
+        in.q2 = nr - 1 - in.q1;
+        in.q3 = nr - 1 - in.q0;
+    }
+    if (u.belt) {  // whole blocks of rings
+        const int nb = belt_tc_rings();
+        const int a = belt_lo + (std::max(r0, belt_lo) - belt_lo) / nb * nb;
+        const int b = std::min(belt_hi, belt_lo + (std::min(r1, belt_hi) - belt_lo) / nb * nb + nb - 1);
+        const int q0 = std::max(s->range[a].x, belt_lo), q1 = std::min(s->range[b].y, belt_hi);
+        if (!u.cap) {
+            in.q0 = q0;
+            in.q1 = q1;
+        } else if (q0 + q1 <= nr - 1) {
+            in.q0 = std::min(in.q0, q0);
+            in.q1 = std::max(in.q1, q1);
+        } else {
+            in.q2 = std::min(in.q2, q0);
+            in.q3 = std::max(in.q3, q1);
+        }
+    }
+    if (in.q2 <= in.q1 + 1 && in.q3 >= in.q2) {  // one interval
+        in.q0 = std::min(in.q0, in.q2);
+        in.q1 = std::max(in.q1, in.q3);
+        in.q2 = 0;
+        in.q3 = -1;
+    }
+    const auto start = [&](int r) -> long long {  // first pixel of a ring
+        const long long i = r + 1, n = nside, j = 4 * n - i;
+        return i <= n ? 2 * i * (i - 1)
+                      : i <= 3 * n ? 2 * n * (n - 1) + 4 * n * (i - n) : 12 * n * n - 2 * j * (j + 1);
+    };
+    const auto blocks = [&](int qa, int qb, int *b, int *n) {
+        *b = (int)(start(qa) >> 6);
+        *n = qb < qa ? 0 : (int)((start(qb + 1) - 1) >> 6) + 1 - *b;
+    };
+    blocks(in.q0, in.q1, &in.b0, &in.n0);
+    blocks(in.q2, in.q3, &in.b1, &in.n1);
+    return u;
+}
+
+size_t conv_scratch_bytes(const ksc_split *s, int n_maps, const ConvUse &use) {
     const size_t nr = (size_t)s->plan.nrings;
-    if (!cap && !belt) return 0;
+    if (!use.cap && !use.belt) return 0;
     size_t b = sizeof(int);  // the gather's claim counter
     b += sizeof(unsigned) * (size_t)map_blocks(s->plan);
-    if (cap) b += sizeof(uint2) * nr + sizeof(int) * (nr + 1);
-    if (belt) b += (size_t)belt_tc_tiles(s->plan, s->btc);
+    if (use.cap) b += sizeof(uint2) * nr + sizeof(int) * (nr + 1);
+    if (use.belt) b += (size_t)belt_tc_tiles(s->plan, s->btc);
     return b * (size_t)n_maps;
 }
 
-cudaError_t start_conv_scratch(const ksc_split *s, const MapSet &maps, int n_maps, void *mem,
-                               ConvScratch *w, cudaStream_t st) {
-    const bool cap = has_cap_tc(s), belt = s->btc.n_cols > 0;
+cudaError_t start_conv_scratch(const ksc_split *s, const MapSet &maps, int n_maps,
+                               const ConvUse &use, void *mem, ConvScratch *w, cudaStream_t st) {
+    const bool cap = use.cap, belt = use.belt;
     if (!cap && !belt) return cudaSuccess;
     const size_t nr = (size_t)s->plan.nrings, n = (size_t)n_maps;
     unsigned char *at = static_cast<unsigned char *>(mem);
@@ -977,9 +1032,10 @@ cudaError_t start_conv_scratch(const ksc_split *s, const MapSet &maps, int n_map
     w->bm = reinterpret_cast<unsigned *>(take(sizeof(unsigned) * (size_t)map_blocks(s->plan)));
     if (belt) w->belt_flags = at;
     const size_t n_zero = (size_t)(zero_end - (unsigned char *)w->counters);
-    cudaError_t e = launch_block_max(s->plan, maps, n_maps, w->bm, w->counters,
+    cudaError_t e = launch_block_max(s->plan, maps, n_maps, use.in, w->bm, w->counters,
                                      (long long)(n_zero / sizeof(int)), st);
-    if (e == cudaSuccess && cap) e = launch_ring_range(s->plan, w->bm, n_maps, w->ranges, st);
+    if (e == cudaSuccess && cap)
+        e = launch_ring_range(s->plan, w->bm, n_maps, use.in, w->ranges, st);
     return e;
 }
 
@@ -1447,11 +1503,16 @@ int ksc_conv_real_multimap_stage(const ksc_split *s, const float *d_in, float *d
     if (stage != 1 && stage != 2) return fail(KSC_ERR_ARG, "stage must be 1 or 2");
     const ksc::MapSet maps{d_in, d_out, stride};
     CallScratch w;
-    cudaError_t e = s->path == 1 ? cudaSuccess : start_scratch(s, maps, n_maps, st, &w);
+    const bool belt_mma = n_maps >= 16 && s->tensor == 2 && s->n_items_mma > 0;
+    cudaError_t e = cudaSuccess;
+    if (s->path != 1)
+        e = start_scratch(s, maps, n_maps,
+                          ksc::conv_use(s, 0, s->plan.nrings - 1, stage == 1 && !belt_mma,
+                                        stage == 2 && !(n_maps >= 16 && s->tensor >= 1)), st, &w);
     if (e != cudaSuccess) return cuda_fail(e, "call scratch");
     if (stage == 1) {
         if (s->path == 1) return KSC_OK;
-        if (n_maps >= 16 && s->tensor == 2 && s->n_items_mma > 0)
+        if (belt_mma)
             return launch_belt_tensor(s, d_in, d_out, n_maps, stride, st);
         else
             e = ksc::launch_belt(s, maps, n_maps, 0, s->plan.nrings - 1, w, s->d_err, st);
@@ -1475,7 +1536,10 @@ int ksc_conv_real_stage(const ksc_split *s, const float *d_in, float *d_out, int
     if (stage != 1 && stage != 2) return fail(KSC_ERR_ARG, "stage must be 1 or 2");
     const ksc::MapSet maps{d_in, d_out, 0};
     CallScratch w;
-    cudaError_t e = s->path == 1 ? cudaSuccess : start_scratch(s, maps, 1, st, &w);
+    cudaError_t e = cudaSuccess;
+    if (s->path != 1)
+        e = start_scratch(s, maps, 1,
+                          ksc::conv_use(s, 0, s->plan.nrings - 1, stage == 1, stage == 2), st, &w);
     if (e != cudaSuccess) return cuda_fail(e, "call scratch");
     if (stage == 1) {
         e = ksc::launch_belt(s, maps, 1, 0, s->plan.nrings - 1, w, s->d_err, st);

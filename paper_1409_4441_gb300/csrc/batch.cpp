@@ -231,6 +231,11 @@ int rebuild(ksc_batch *b) {
     return upload_items(b, items, launches);
 }
 
+// A whole map on the stages that its split has.
+ksc::ConvUse whole_use(const ksc_split *s) {
+    return ksc::conv_use(s, 0, s->plan.nrings - 1, true, true);
+}
+
 // Groups the entries on the tensor-core stages by split and takes their scratch.
 cudaError_t plan_tc(ksc_batch *b) {
     size_t bytes = 0;
@@ -247,7 +252,7 @@ cudaError_t plan_tc(ksc_batch *b) {
     }
     for (TcGroup &g : b->tc) {
         g.at = bytes;
-        bytes += (ksc::conv_scratch_bytes(g.split, g.count) + 255) & ~(size_t)255;
+        bytes += (ksc::conv_scratch_bytes(g.split, g.count, whole_use(g.split)) + 255) & ~(size_t)255;
     }
     return bytes ? cudaMalloc(&b->d_scratch, bytes) : cudaSuccess;
 }
@@ -259,7 +264,7 @@ int enqueue_tc(const ksc_batch *b, cudaStream_t st) {
         maps.table = b->d_entries + g.first;
         ksc::ConvScratch w;
         const int last = s->plan.nrings - 1;
-        cudaError_t e = ksc::start_conv_scratch(s, maps, g.count,
+        cudaError_t e = ksc::start_conv_scratch(s, maps, g.count, whole_use(s),
                                                 static_cast<char *>(b->d_scratch) + g.at, &w, st);
         if (e == cudaSuccess) e = ksc::launch_belt(s, maps, g.count, 0, last, w, b->d_err, st);
         if (e == cudaSuccess && ksc::has_cap_tc(s))

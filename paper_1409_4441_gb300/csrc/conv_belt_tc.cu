@@ -556,11 +556,12 @@ conv_belt_tc_kernel(const ConvPlan P, int block_lo, int n_tiles_k, int ring_lo, 
 }
 
 // blockmax[map][b] = the bits of the largest |m| over map pixels [64 b, 64 b + 64)
-// (infinities and NaNs compare above every number).  One read of the map.  Clears the
-// n_zero words that the call's later kernels count and flag in.
+// (infinities and NaNs compare above every number), for the blocks of the reach (a band reads
+// its own part of the map: nine belt rings of nside 2048, 4 pixels: 36 us for the whole map).
+// One read of them.  Clears the n_zero words that the call's later kernels count and flag in.
 __global__ void __launch_bounds__(256)
-block_max_kernel(const MapSet maps, int n_blocks, uint32_t *__restrict__ blockmax,
-                 long long block_stride, int *__restrict__ zero, long long n_zero) {
+block_max_kernel(const MapSet maps, int b0, int n0, int b1, int n1,
+                 uint32_t *__restrict__ blockmax, long long block_stride, int *__restrict__ zero, long long n_zero) {
     for (long long i = (blockIdx.y * (long long)gridDim.x + blockIdx.x) * 256 + threadIdx.x;
          i < n_zero; i += (long long)gridDim.x * gridDim.y * 256)
         zero[i] = 0;
@@ -568,7 +569,8 @@ block_max_kernel(const MapSet maps, int n_blocks, uint32_t *__restrict__ blockma
     uint32_t *bm = blockmax + (long long)blockIdx.y * block_stride;
     const int half = (blockIdx.x * 256 + threadIdx.x) >> 4, l16 = threadIdx.x & 15;
     const int n_half = gridDim.x * 16;
-    for (int b = half; b < n_blocks; b += n_half) {
+    for (int i = half; i < n0 + n1; i += n_half) {
+        const int b = i < n0 ? b0 + i : b1 + (i - n0);
         const float4 v = __ldg(m + (long long)b * 16 + l16);
         uint32_t x = max(max(__float_as_uint(v.x) & 0x7fffffffu, __float_as_uint(v.y) & 0x7fffffffu),
                          max(__float_as_uint(v.z) & 0x7fffffffu, __float_as_uint(v.w) & 0x7fffffffu));
@@ -643,11 +645,13 @@ bool belt_tc_plan(int nside, int wpos, int nq, BeltTc *t) {
 
 long long map_blocks(const ConvPlan &p) { return p.npix / 64; }
 
-cudaError_t launch_block_max(const ConvPlan &p, const MapSet &maps, int n_maps, uint32_t *bm,
-                             int *zero, long long n_zero, cudaStream_t st) {
-    const int n = (int)map_blocks(p);
-    dim3 grid(std::min((n + 15) / 16, 152 * 8), n_maps);
-    block_max_kernel<<<grid, 256, 0, st>>>(maps, n, bm, n, zero, n_zero);
+cudaError_t launch_block_max(const ConvPlan &p, const MapSet &maps, int n_maps,
+                             const InputReach &in, uint32_t *bm, int *zero, long long n_zero,
+                             cudaStream_t st) {
+    const int n = in.n0 + in.n1;
+    dim3 grid(std::max(1, std::min((n + 15) / 16, 152 * 8)), n_maps);
+    block_max_kernel<<<grid, 256, 0, st>>>(maps, in.b0, in.n0, in.b1, in.n1, bm, map_blocks(p), zero,
+                                           n_zero);
     return cudaGetLastError();
 }
 

@@ -971,13 +971,15 @@ cap_direct_kernel(const ConvPlan P, const int2 *__restrict__ items,
 }
 
 // ring_range[map][ring] = the largest and the smallest nonzero block maximum (bits) over
-// the 64-pixel blocks that the ring touches; one warp per ring.
+// the 64-pixel blocks that the ring touches; one warp per ring of the reach.
 __global__ void __launch_bounds__(256)
 ring_range_kernel(const ConvPlan P, const uint32_t *__restrict__ blockmax, long long block_stride,
-                  uint2 *__restrict__ ring_range) {
+                  const InputReach in, uint2 *__restrict__ ring_range) {
     const uint32_t *bm = blockmax + (long long)blockIdx.y * block_stride;
-    const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (r >= P.nrings) return;
+    const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int n0 = in.q1 - in.q0 + 1, n = n0 + max(in.q3 - in.q2 + 1, 0);
+    if (i >= n) return;
+    const int r = i < n0 ? in.q0 + i : in.q2 + (i - n0);
     const DevRing R = P.d_rings[r];
     uint32_t mx = 0u, mn = 0xffffffffu;
     for (int b = (R.start >> 6) + lane; b <= (R.start + R.len - 1) >> 6; b += 32) {
@@ -1060,10 +1062,11 @@ cudaError_t launch_cap_coef(const ConvPlan &p, const CapTc &c, const CapCoef &k,
     return cudaGetLastError();
 }
 
-cudaError_t launch_ring_range(const ConvPlan &p, const unsigned *bm, int n_maps, uint2 *rr,
-                              cudaStream_t st) {
-    dim3 grid((p.nrings + 7) / 8, n_maps);
-    ring_range_kernel<<<grid, 256, 0, st>>>(p, bm, map_blocks(p), rr);
+cudaError_t launch_ring_range(const ConvPlan &p, const unsigned *bm, int n_maps,
+                              const InputReach &in, uint2 *rr, cudaStream_t st) {
+    const int n = in.q1 - in.q0 + 1 + std::max(in.q3 - in.q2 + 1, 0);
+    dim3 grid((n + 7) / 8, n_maps);
+    ring_range_kernel<<<grid, 256, 0, st>>>(p, bm, map_blocks(p), in, rr);
     return cudaGetLastError();
 }
 

@@ -231,10 +231,16 @@ int belt_tc_positions(int w, int L);      // window positions for a half window 
 bool belt_tc_plan(int nside, int wpos, int nq, BeltTc *t);
 int belt_tc_tiles(const ConvPlan &p, const BeltTc &t);
 long long map_blocks(const ConvPlan &p);  // blocks of 64 pixels in a map
-// bm[map][block] = bits of the block's largest |m|; map_blocks() words per map; clears
-// zero[0 .. n_zero)
-cudaError_t launch_block_max(const ConvPlan &p, const MapSet &maps, int n_maps, unsigned *bm,
-                             int *zero, long long n_zero, cudaStream_t st);
+// The input that a call's tensor-core stages read: rings [q0, q1] and [q2, q3] (none: q3 < q2),
+// in 64-pixel blocks [b0, b0 + n0) and [b1, b1 + n1).
+struct InputReach {
+    int q0 = 0, q1 = -1, q2 = 0, q3 = -1, b0 = 0, n0 = 0, b1 = 0, n1 = 0;
+};
+// bm[map][block] = bits of the block's largest |m|, blocks of the reach; map_blocks() words per
+// map; clears zero[0 .. n_zero)
+cudaError_t launch_block_max(const ConvPlan &p, const MapSet &maps, int n_maps,
+                             const InputReach &in, unsigned *bm, int *zero, long long n_zero,
+                             cudaStream_t st);
 // Writes output rings [r0, r1] of the belt but for the tiles it flags (tiles whose values
 // span too wide a range, or are not finite), which launch_conv_belt then computes.
 cudaError_t launch_conv_belt_tc(const ConvPlan &p, const BeltTc &t, const MapSet &maps,
@@ -275,8 +281,8 @@ int cap_tc_degree();                     // of the cells' polynomials
 int cap_tc_split_powers();               // powers below it are multiplied in two parts
 int cap_tc_positions(int w, int L);
 bool cap_tc_fits(const CapTc &c);
-cudaError_t launch_ring_range(const ConvPlan &p, const unsigned *bm, int n_maps, uint2 *rr,
-                              cudaStream_t st);
+cudaError_t launch_ring_range(const ConvPlan &p, const unsigned *bm, int n_maps,
+                              const InputReach &in, uint2 *rr, cudaStream_t st);
 // Writes (adds, for belt rings with belt_split) the tiles' outputs in rings [band_lo,
 // band_hi] but for the ring pairs it flags (flags[map][ring], flags[map][nrings]: any),
 // which conv_sym_kernel then computes; flags must be zero at launch.
@@ -406,6 +412,7 @@ struct ksc_split {
     int sym_variant = 0;                   // the gather's tile (sym_variant_chunk)
     bool sym_small_ok = false;             // its tables fit the small tile
     std::vector<int> ring_first_sym;
+    std::vector<int2> range;               // input rings of each output ring
     int path = 0;                          // 0: belt + symmetric, 1: general only
     int2 *d_items_belt = nullptr;          // belt chunks for the circulant kernel
     int n_items_belt = 0;
@@ -451,10 +458,16 @@ struct ConvScratch {
     unsigned char *belt_flags = nullptr;
 };
 bool has_cap_tc(const ksc_split *s);
-size_t conv_scratch_bytes(const ksc_split *s, int n_maps);
+// The tensor-core stages of a call for output rings [r0, r1], and what they read of the map.
+struct ConvUse {
+    bool belt = false, cap = false;
+    InputReach in;
+};
+ConvUse conv_use(const ksc_split *s, int r0, int r1, bool want_belt, bool want_cap);
+size_t conv_scratch_bytes(const ksc_split *s, int n_maps, const ConvUse &use);
 // Lays the scratch out in mem and starts the launches that fill it.
-cudaError_t start_conv_scratch(const ksc_split *s, const MapSet &maps, int n_maps, void *mem,
-                               ConvScratch *w, cudaStream_t st);
+cudaError_t start_conv_scratch(const ksc_split *s, const MapSet &maps, int n_maps,
+                               const ConvUse &use, void *mem, ConvScratch *w, cudaStream_t st);
 cudaError_t launch_belt(const ksc_split *s, const MapSet &maps, int n_maps, int r0, int r1,
                         const ConvScratch &w, int *d_err, cudaStream_t st);
 cudaError_t launch_caps(const ksc_split *s, const MapSet &maps, int n_maps, int lo, int hi,

@@ -27,12 +27,12 @@ def _split(K, nside, theta_arcmin, **opts):
     return K.make_split_real(c, nside, theta_arcmin * inputs.ARCMIN, **opts), c
 
 
-def _launched(K, sp, x, y):
-    """Kernels of one ksc_conv_real, by name."""
+def _launched(call):
+    """Kernels of one call, by name."""
     from torch.profiler import ProfilerActivity, profile
     for _ in range(2):  # (the first profile of a process may record nothing)
         with profile(activities=[ProfilerActivity.CUDA]) as p:
-            K.conv_real(sp, x, y)
+            call()
             torch.cuda.synchronize()
     return [e.name for e in p.events() if "kernel" in e.name]
 
@@ -43,7 +43,8 @@ def test_reported_kernels_are_the_ones_that_run(K, nside, theta):
     sp, _ = _split(K, nside, theta)
     x = torch.tensor(inputs.white_noise_map(nside, 11).astype(np.float32), device="cuda")
     with sp:
-        names = _launched(K, sp, x, torch.empty_like(x))
+        y = torch.empty_like(x)
+        names = _launched(lambda: K.conv_real(sp, x, y))
         st = K.split_stages(sp)
     assert len(names) == st["n_launches"], names
     assert any("conv_belt_tc_kernel" in n for n in names) == (st["belt_columns"] > 0)
@@ -82,3 +83,48 @@ def test_cap_stage_is_taken_where_it_is_faster(K, nside, theta, want):
     sp, _ = _split(K, nside, theta)
     with sp:
         assert K.split_stages(sp)["cap_stage"] == want
+
+
+def test_calls_take_only_what_their_stages_need(K):
+    """A cap band of a split with a belt stage, and a stack whose stages are both the TF32 kernels: no
+    block maxima.  A belt band: one launch of them."""
+    nside = 256
+    sp, _ = _split(K, nside, 900.0)
+    x = torch.tensor(inputs.white_noise_map(nside, 12).astype(np.float32), device="cuda")
+    y = torch.empty_like(x)
+    with sp:
+        st = K.split_stages(sp)
+        assert st["belt_columns"] > 0 and not st["cap_stage"]
+        cap = _launched(lambda: K.conv_real_rings(sp, x, y, 100, 140))
+        belt = _launched(lambda: K.conv_real_rings(sp, x, y, 500, 540))
+    assert not any("block_max" in n for n in cap)
+    assert sum("block_max" in n for n in belt) == 1
+    sp, _ = _split(K, nside, 900.0, tensor=2)
+    xs = x.repeat(16, 1).contiguous()
+    ys = torch.empty_like(xs)
+    with sp:
+        names = _launched(lambda: K.conv_real_multimap(sp, xs, ys, 16))
+    assert any("conv_belt_mma" in n for n in names) and not any("block_max" in n for n in names)
+
+
+@pytest.mark.parametrize("nside,theta", [(256, 900.0), (512, 700.0)])
+def test_bands_of_the_stages_equal_the_whole_map(K, nside, theta):
+    """Bit for bit, for bands that start and end inside a block of 16 belt rings, of one ring, across
+    the equator and both cap boundaries, at both poles; the rest of the output untouched."""
+    sp, _ = _split(K, nside, theta)
+    m = inputs.white_noise_map(nside, 13).astype(np.float32)
+    m[: 6 * nside * nside] += np.float32(3.0)  # a constant is taken off northern rings
+    x = torch.tensor(m, device="cuda")
+    one = torch.empty_like(x)
+    _, _, n, st, _ = O.ring_table(nside)
+    with sp:
+        assert K.split_stages(sp)["belt_columns"] > 0
+        K.conv_real(sp, x, one)
+        for lo, hi in ((nside + 5, nside + 40), (2 * nside, 2 * nside), (2 * nside - 9, 2 * nside + 3),
+                       (nside - 7, nside + 1), (3 * nside - 3, 3 * nside + 9), (1, 9),
+                       (4 * nside - 30, 4 * nside - 1), (nside // 2, 3 * nside)):
+            part = torch.zeros_like(x)
+            K.conv_real_rings(sp, x, part, lo, hi)
+            a, b = int(st[lo - 1]), int(st[hi - 1] + n[hi - 1])
+            assert torch.equal(part[a:b], one[a:b]), (lo, hi)
+            assert not part[:a].any() and not part[b:].any()
