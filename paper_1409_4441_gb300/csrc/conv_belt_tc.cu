@@ -90,7 +90,9 @@ __host__ __device__ __forceinline__ Window tile_window(int w, int L) {
 }
 
 // N columns: 8 N pixels per ring.  grid.x runs over tiles (16-ring block, pixel tile),
-// grid.y over maps.  Sixteen builder warps stage the map, evaluate the weights, lay out A
+// grid.y over maps.  A tile belongs to one of the split's (of plan_cols >= N columns), from
+// which its scale, its constants and its flag come: a band of few rings takes narrower tiles, more
+// of them, for the same bits.  Sixteen builder warps stage the map, evaluate the weights, lay out A
 // and fold the accumulators; a seventeenth issues the MMAs (the
 // rest of its warpgroup only gives its registers to the builders).  A builder warp hands a stage
 // over by arriving on a_full; that arrival also says that its part of the ring's input
@@ -101,7 +103,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 conv_belt_tc_kernel(const ConvPlan P, int block_lo, int n_tiles_k, int ring_lo, int ring_hi,
                     const MapSet maps,
                     const uint32_t *__restrict__ blockmax, long long block_stride,
-                    unsigned char *__restrict__ flags, int n_tiles, int wpos_cap, int nq_cap,
+                    unsigned char *__restrict__ flags, int n_tiles, int plan_cols, int wpos_cap,
+                    int nq_cap,
                     float wscale, float wunscale, float domega_lo, int *__restrict__ err) {
     constexpr int kCols = N / 4;  // columns per thread (four warps share a lane quarter)
     constexpr int kStep = kCols < 16 ? 8 : 16;
@@ -127,6 +130,7 @@ conv_belt_tc_kernel(const ConvPlan P, int block_lo, int n_tiles_k, int ring_lo, 
     const int r_first = P.belt_lo + rb * kRings;
     const int n_rows = min(kRings, P.belt_hi - r_first + 1);
     const int L = 4 * P.nside, k0 = ct * 8 * N;
+    const int plan_tile = k0 / (8 * plan_cols), plan_k0 = plan_tile * 8 * plan_cols;
     const float *__restrict__ m = maps.input(blockIdx.y);
     float *__restrict__ o = maps.output(blockIdx.y);
     const uint32_t *bm = blockmax + (long long)blockIdx.y * block_stride;
@@ -174,8 +178,8 @@ conv_belt_tc_kernel(const ConvPlan P, int block_lo, int n_tiles_k, int ring_lo, 
         }
         const int start = P.d_rings[q].start;
         // pixels [a, a + len) of the ring, wrapped; every block of 64 map pixels in them
-        const int len = min(8 * N + 16 * (g.s1 - g.s0), L);
-        int a = (k0 + g.d0 + 16 * g.s0) % L;
+        const int len = min(8 * plan_cols + 16 * (g.s1 - g.s0), L);
+        int a = (plan_k0 + g.d0 + 16 * g.s0) % L;
         a += a < 0 ? L : 0;
         const int head = min(len, L - a);
         uint32_t qmax = 0u, qmin = 0xffffffffu;
@@ -237,7 +241,7 @@ conv_belt_tc_kernel(const ConvPlan P, int block_lo, int n_tiles_k, int ring_lo, 
     const bool flag = !zero && (emax >= 255u || emax < 48u || emax > 206u || emin == 0u ||
                                 emax - emin > kRangeExp);
     if (tid == 0) {
-        flags[(long long)blockIdx.y * n_tiles + rb * n_tiles_k + ct] = flag ? 1 : 0;
+        flags[(long long)blockIdx.y * n_tiles + rb * (L / (8 * plan_cols)) + plan_tile] = flag ? 1 : 0;
         if (s_bad) atomicExch(err, KSC_ERR_DEVICE_BOUNDS);
     }
     // |m - constant| may reach twice the largest |m|
@@ -320,7 +324,7 @@ conv_belt_tc_kernel(const ConvPlan P, int block_lo, int n_tiles_k, int ring_lo, 
         const int my_r = r_first + warp;  // the ring this warp builds weights for
         int2 rg = make_int2(P.belt_hi + 1, P.belt_lo - 1);
         int base = 0, my_phase = 0;
-        if (warp < n_rows) {
+        if (warp < n_rows && my_r >= ring_lo && my_r <= ring_hi) {  // (no weights for other rings)
             rg = P.d_range[my_r];
             base = P.d_pair_base[my_r] - rg.x;
             my_phase = P.d_rings[my_r].phase;
@@ -601,7 +605,7 @@ cudaError_t launch_tc(const ConvPlan &p, const BeltTc &t, const MapSet &maps, in
     dim3 grid((b1 - b0 + 1) * tk, n_maps);
     conv_belt_tc_kernel<N><<<grid, kThreads, smem, st>>>(
         p, b0, tk, r0, r1, maps, bm, bm_stride, flags, belt_tc_tiles(p, t),
-        t.wpos, t.nq, t.wscale, 1.0f / t.wscale,
+        t.n_cols, t.wpos, t.nq, t.wscale, 1.0f / t.wscale,
         (float)(4.0 * 3.14159265358979323846 / p.npix - (double)p.domega), d_err);
     return cudaGetLastError();
 }
@@ -660,7 +664,12 @@ cudaError_t launch_conv_belt_tc(const ConvPlan &p, const BeltTc &t, const MapSet
                                 int *d_err, cudaStream_t st) {
     if (r0 > p.belt_hi || r1 < p.belt_lo) return cudaSuccess;
     const long long bs = map_blocks(p);
-    switch (t.n_cols) {
+    // Narrower tiles while twice as many are still one wave (one CTA per SM): nine rings of
+    // nside 2048, 64 pixels: 0.92 -> 0.54 ms (FFMA 0.50), 16 pixels: 0.31 -> 0.17 (0.09).
+    const int nb = (std::min(r1, p.belt_hi) - p.belt_lo) / kRings - (std::max(r0, p.belt_lo) - p.belt_lo) / kRings + 1;
+    int n = t.n_cols;
+    while (n > 32 && 2ll * nb * (p.nside / (2 * n)) * n_maps <= 152) n /= 2;
+    switch (n) {
     case 256: return launch_tc<256>(p, t, maps, n_maps, r0, r1, bm, bs, flags, d_err, st);
     case 128: return launch_tc<128>(p, t, maps, n_maps, r0, r1, bm, bs, flags, d_err, st);
     case 64: return launch_tc<64>(p, t, maps, n_maps, r0, r1, bm, bs, flags, d_err, st);
