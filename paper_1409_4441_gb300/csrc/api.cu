@@ -93,6 +93,8 @@ void release(ksc_split *s) {
     delete s;
 }
 
+constexpr int kSms = 152;
+
 // Without the tensor-core cap stage: the gather sums the caps.
 void drop_cap_tc(ksc_split *s) {
     for (void **p : {(void **)&s->d_cap_tiles, (void **)&s->d_cap_tiles_lpt, (void **)&s->d_ncut,
@@ -150,11 +152,10 @@ int plan_belt_tc(ksc_split *s, const ksc::RingGeom &g, const std::vector<int2> &
     s->btc.wscale = s->ctc.wscale = (float)std::ldexp(1.0, ex);
     s->ctc.wunscale = 1.0f / s->ctc.wscale;
     s->ctc.domega_lo = (float)(4.0 * kPi / s->plan.npix - (double)s->plan.domega);
-    // Below about 8e8 belt pairs the FFMA kernel is the faster one: a tile spends 0.7 to
-    // 1.8 us on an input ring however short the window, small maps have few tiles, and the
-    // block maxima (5 us) and their scratch come on top (FFMA / tensor stage, us: nside 64,
-    // 360': 58 / 72; 256, 160' (2.2e8 pairs): 91 / 99; 512, 60' (5e8): 123 / 122, the call's
-    // first pass 483 / 580; 256, 640' (3.6e9): 542 / 371; 1024, 160': 3605 / 1177).
+    // Below about 8e8 belt pairs the FFMA kernel is the faster one: small maps have few tiles,
+    // and the block maxima (5 us) and their scratch come on top (FFMA / tensor stage, us: nside
+    // 64, 360': 58 / 72; 256, 160' (2.2e8 pairs): 91 / 99; 512, 60' (5e8): 123 / 122, the call's
+    // first pass 483 / 580).  From there on by the estimate at the end.
     if (2.0 / 3.0 * ksc_cost_pairs(s->nside, s->theta_cut) < 8e8) return KSC_OK;
     const int lo = s->plan.belt_lo, hi = s->plan.belt_hi, nb = ksc::belt_tc_rings();
     int wpos = 0, nq = 0;
@@ -170,11 +171,31 @@ int plan_belt_tc(ksc_split *s, const ksc::RingGeom &g, const std::vector<int2> &
         }
         nq = std::max(nq, q1 - q0 + 1);
     }
-    if (!ksc::belt_tc_plan(s->nside, wpos, nq, &s->btc)) s->btc.n_cols = 0;
+    if (!ksc::belt_tc_plan(s->nside, wpos, nq, &s->btc)) {
+        s->btc.n_cols = 0;
+        return KSC_OK;
+    }
+    // A tile spends 2.2 (32 columns) to 3.5 us (256) on an input ring whose window has up to 150
+    // positions, and a band of a few rings, which takes the same kernel for the same bits, pays
+    // that for sixteen rings.  So only where the whole map's stage takes at most 0.7 of the FFMA
+    // kernel's time; estimate and measured ratio: nside 256, 32 and 48 pixels 0.76 / 0.77 and 0.63 /
+    // 0.66; 512, 16 and 24: 0.77 / 0.77 and 0.61 / 0.62; 1024, 8 and 12: 0.74 / 0.71 and 0.65 / 0.64;
+    // 2048, 4 and 8: 0.89 / 0.78 and 0.67 / 0.66.
+    double ffma = 0.0;
+    for (int r = lo; r <= hi; ++r) {
+        int rings = 0;
+        for (int q = std::max(range[r].x, lo); q <= std::min(range[r].y, hi); ++q)
+            rings += pairs[(size_t)pair_base[r] + (q - range[r].x)].hw >= 0.0f;
+        const int items = (g.len[r] + ksc::belt_chunk() - 1) / ksc::belt_chunk();
+        ffma += items * (0.47 * rings + 0.0108 * s->cost_belt[r]);
+    }
+    ffma *= (s->n_items_belt <= 4 * kSms ? 1.3 : 1.0) / kSms;
+    const int n = s->btc.n_cols;
+    const double step = (n >= 256 ? 3.5 : n >= 128 ? 2.9 : n >= 64 ? 2.5 : 2.2) + 0.013 * std::max(wpos - 150, 0);
+    const double tensor = std::ceil(ksc::belt_tc_tiles(s->plan, s->btc) / (double)kSms) * nq * step;
+    if (tensor > 0.7 * ffma) s->btc.n_cols = 0;
     return KSC_OK;
 }
-
-constexpr int kSms = 152;
 
 // Time of independent pieces of work on so many slots, the longest first.
 double makespan(std::vector<double> t, int slots) {

@@ -128,3 +128,12 @@ def test_bands_of_the_stages_equal_the_whole_map(K, nside, theta):
             a, b = int(st[lo - 1]), int(st[hi - 1] + n[hi - 1])
             assert torch.equal(part[a:b], one[a:b]), (lo, hi)
             assert not part[:a].any() and not part[b:].any()
+
+
+# (nside, cut in arcmin, whether the belt stage takes at most 0.7 of the FFMA kernel's time)
+@pytest.mark.parametrize("nside,theta,want", [(256, 440.0, 0), (256, 660.0, 1), (512, 110.0, 0), (512, 165.0, 1),
+                                              (2048, 7.0, 0), (2048, 20.0, 1), (2048, 240.0, 1)])
+def test_belt_stage_is_taken_where_it_is_faster(K, nside, theta, want):
+    sp, _ = _split(K, nside, theta)
+    with sp:
+        assert (K.split_stages(sp)["belt_columns"] > 0) == want
