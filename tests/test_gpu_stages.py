@@ -4,6 +4,11 @@ known to be theirs: every tile width of the belt stage, ragged ring blocks, band
 Tolerance: the per-pixel parity bound of the other kernels, 1e-6 of the output rms plus the
 oracle's bound on pairs whose chord lies within rounding of the cut.
 """
+import json
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -12,6 +17,7 @@ from paper_1409_4441_gb300 import inputs
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 @pytest.fixture(scope="module")
@@ -27,28 +33,48 @@ def _split(K, nside, theta_arcmin, **opts):
     return K.make_split_real(c, nside, theta_arcmin * inputs.ARCMIN, **opts), c
 
 
-def _launched(call):
-    """Kernels of one call, by name."""
-    from torch.profiler import ProfilerActivity, profile
+# Kernels by name of calls on splits of this file's beam, from a process of its own (a profiler in
+# this one would stay under the graphs that other tests replay).
+PROBE = """
+import json, sys
+import torch
+from torch.profiler import ProfilerActivity, profile
+from paper_1409_4441_gb300 import inputs, ksconv as K
+out = []
+for nside, theta, tensor, n_maps, lo, hi in json.loads(sys.argv[1]):
+    c = inputs.gaussian_beam(2 * nside, 3.0 * 3518.0 / nside * inputs.ARCMIN)
+    sp = K.make_split_real(c, nside, theta * inputs.ARCMIN, tensor=tensor)
+    x = torch.randn((n_maps, 12 * nside * nside), device="cuda")
+    y = torch.empty_like(x)
     for _ in range(2):  # (the first profile of a process may record nothing)
         with profile(activities=[ProfilerActivity.CUDA]) as p:
-            call()
+            if hi:
+                K.conv_real_rings(sp, x[0], y[0], lo, hi)
+            elif n_maps > 1:
+                K.conv_real_multimap(sp, x, y, n_maps)
+            else:
+                K.conv_real(sp, x[0], y[0])
             torch.cuda.synchronize()
-    return [e.name for e in p.events() if "kernel" in e.name]
+    out.append({"names": [e.name for e in p.events() if "kernel" in e.name], "stages": K.split_stages(sp)})
+    sp.close()
+print(json.dumps(out))
+"""
 
 
-# (nside, cut in arcmin): neither stage, the belt's, both
-@pytest.mark.parametrize("nside,theta", [(64, 360.0), (512, 240.0), (512, 640.0)])
-def test_reported_kernels_are_the_ones_that_run(K, nside, theta):
-    sp, _ = _split(K, nside, theta)
-    x = torch.tensor(inputs.white_noise_map(nside, 11).astype(np.float32), device="cuda")
-    with sp:
-        y = torch.empty_like(x)
-        names = _launched(lambda: K.conv_real(sp, x, y))
-        st = K.split_stages(sp)
-    assert len(names) == st["n_launches"], names
-    assert any("conv_belt_tc_kernel" in n for n in names) == (st["belt_columns"] > 0)
-    assert any("conv_cap_tc_kernel" in n for n in names) == (st["cap_stage"] == 1)
+def _launched(cases):
+    run = subprocess.run([sys.executable, "-c", PROBE, json.dumps(cases)], capture_output=True, text=True,
+                         timeout=300, cwd=ROOT)
+    assert run.returncode == 0, run.stderr[-2000:]
+    return json.loads(run.stdout.splitlines()[-1])
+
+
+def test_reported_kernels_are_the_ones_that_run(K):
+    """Neither stage, the belt's, both."""
+    for r in _launched([(64, 360.0, 0, 1, 0, 0), (512, 240.0, 0, 1, 0, 0), (512, 640.0, 0, 1, 0, 0)]):
+        names, st = r["names"], r["stages"]
+        assert len(names) == st["n_launches"], names
+        assert any("conv_belt_tc_kernel" in n for n in names) == (st["belt_columns"] > 0)
+        assert any("conv_cap_tc_kernel" in n for n in names) == (st["cap_stage"] == 1)
 
 
 def _legendre(lmax, z):
@@ -88,23 +114,13 @@ def test_cap_stage_is_taken_where_it_is_faster(K, nside, theta, want):
 def test_calls_take_only_what_their_stages_need(K):
     """A cap band of a split with a belt stage, and a stack whose stages are both the TF32 kernels: no
     block maxima.  A belt band: one launch of them."""
-    nside = 256
-    sp, _ = _split(K, nside, 900.0)
-    x = torch.tensor(inputs.white_noise_map(nside, 12).astype(np.float32), device="cuda")
-    y = torch.empty_like(x)
-    with sp:
-        st = K.split_stages(sp)
-        assert st["belt_columns"] > 0 and not st["cap_stage"]
-        cap = _launched(lambda: K.conv_real_rings(sp, x, y, 100, 140))
-        belt = _launched(lambda: K.conv_real_rings(sp, x, y, 500, 540))
-    assert not any("block_max" in n for n in cap)
-    assert sum("block_max" in n for n in belt) == 1
-    sp, _ = _split(K, nside, 900.0, tensor=2)
-    xs = x.repeat(16, 1).contiguous()
-    ys = torch.empty_like(xs)
-    with sp:
-        names = _launched(lambda: K.conv_real_multimap(sp, xs, ys, 16))
-    assert any("conv_belt_mma" in n for n in names) and not any("block_max" in n for n in names)
+    cap, belt, stack = _launched([(256, 900.0, 0, 1, 100, 140), (256, 900.0, 0, 1, 500, 540),
+                                  (256, 900.0, 2, 16, 0, 0)])
+    assert cap["stages"]["belt_columns"] > 0 and not cap["stages"]["cap_stage"]
+    assert not any("block_max" in n for n in cap["names"])
+    assert sum("block_max" in n for n in belt["names"]) == 1
+    assert any("conv_belt_mma" in n for n in stack["names"])
+    assert not any("block_max" in n for n in stack["names"])
 
 
 @pytest.mark.parametrize("nside,theta", [(256, 900.0), (512, 700.0)])
@@ -137,3 +153,29 @@ def test_belt_stage_is_taken_where_it_is_faster(K, nside, theta, want):
     sp, _ = _split(K, nside, theta)
     with sp:
         assert (K.split_stages(sp)["belt_columns"] > 0) == want
+
+
+@pytest.mark.parametrize("nside,theta", [(256, 660.0), (512, 700.0)])
+def test_captured_calls_hold_their_scratch(K, nside, theta):
+    """A call captured into a graph, replayed on other values, and a call on another stream between."""
+    sp, _ = _split(K, nside, theta)
+    x = torch.tensor(inputs.white_noise_map(nside, 15).astype(np.float32), device="cuda")
+    y, z, one = torch.zeros_like(x), torch.zeros_like(x), torch.zeros_like(x)
+    with sp:
+        K.conv_real(sp, x, y)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            K.conv_real(sp, x, y, stream=torch.cuda.current_stream())
+        side = torch.cuda.Stream()
+        for k in range(3):
+            x.copy_(torch.tensor(inputs.white_noise_map(nside, 16 + k).astype(np.float32)))
+            torch.cuda.synchronize()
+            g.replay()
+            K.conv_real(sp, x, z, stream=side)
+            torch.cuda.synchronize()
+            K.conv_real(sp, x, one)
+            torch.cuda.synchronize()
+            assert torch.equal(y, one) and torch.equal(z, one)
+        K.device_status(sp)
+        del g
