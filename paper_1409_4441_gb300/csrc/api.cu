@@ -1107,7 +1107,7 @@ cudaError_t launch_caps(const ksc_split *s, const MapSet &maps, int n_maps, int 
     const int t1 = whole ? s->n_cap_tiles : s->cap_tile_first[hi + 1];
     cudaError_t e = launch_conv_cap_tc(
         s->plan, s->ctc, whole ? s->d_cap_tiles_lpt : s->d_cap_tiles + t0, t1 - t0, maps,
-        n_maps, belt_split, r0, r1, w.ranges, w.cap_flags, d_err, st);
+        n_maps, belt_split, r0, r1, w.ranges, w.cap_flags, !whole, d_err, st);
     if (e != cudaSuccess) return e;
     const int i0 = s->irr_item_first[lo], i1 = s->irr_item_first[hi + 1];
     e = launch_cap_direct(s->plan, s->d_irr_items + i0, i1 - i0, s->d_irr_first, s->d_irr,

@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ tiles,
                    const MapSet maps,
                    int belt_split, int band_lo, int band_hi, const uint2 *__restrict__ ring_range,
-                   int *__restrict__ flags, int *__restrict__ err) {
+                   int *__restrict__ flags, int ring_order, int *__restrict__ err) {
     extern __shared__ __align__(1024) unsigned char smem[];
     // B stages | third parts of c_0 [buffer] | map segments [h][buffer][part] | turning buffers | totals (north, south:
     // sums, compensations) [ring] | the segments as they are, (north, south) [buffer] |
@@ -199,7 +199,8 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
     __shared__ float s_edge[2][2][kP + 3], s_sum[2][2][kP];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int2 tile = tiles[blockIdx.x];
+    // (a band's tiles come in ring order: the longer rings, which take longer, first)
+    const int2 tile = tiles[ring_order ? gridDim.x - 1 - blockIdx.x : blockIdx.x];
     const int r0 = tile.x & 0xffff, n_r = (tile.x >> 16) + 1;
     const int sector = tile.y & 0xffff, n_sec = tile.y >> 16;
     const bool add = belt_split && r0 >= P.belt_lo;
@@ -1083,7 +1084,8 @@ cudaError_t launch_cap_direct(const ConvPlan &p, const int2 *d_items, int n_item
 
 cudaError_t launch_conv_cap_tc(const ConvPlan &p, const CapTc &c, const int2 *d_tiles, int n_tiles,
                                const MapSet &maps, int n_maps, int belt_split, int band_lo,
-                               int band_hi, const uint2 *rr, int *flags, int *d_err, cudaStream_t st) {
+                               int band_hi, const uint2 *rr, int *flags, bool ring_order,
+                               int *d_err, cudaStream_t st) {
     if (n_tiles <= 0) return cudaSuccess;
     const size_t smem = cap_smem(c);
     cudaError_t e = cudaFuncSetAttribute(conv_cap_tc_kernel,
@@ -1092,7 +1094,7 @@ cudaError_t launch_conv_cap_tc(const ConvPlan &p, const CapTc &c, const int2 *d_
     if (e != cudaSuccess) return e;
     dim3 grid(n_tiles, n_maps);
     conv_cap_tc_kernel<<<grid, kThreads, smem, st>>>(p, c, d_tiles, maps, belt_split, band_lo,
-                                                     band_hi, rr, flags, d_err);
+                                                     band_hi, rr, flags, ring_order, d_err);
     return cudaGetLastError();
 }
 

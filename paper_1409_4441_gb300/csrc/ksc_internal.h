@@ -288,8 +288,8 @@ cudaError_t launch_ring_range(const ConvPlan &p, const unsigned *bm, int n_maps,
 // which conv_sym_kernel then computes; flags must be zero at launch.
 cudaError_t launch_conv_cap_tc(const ConvPlan &p, const CapTc &c, const int2 *d_tiles, int n_tiles,
                                const MapSet &maps, int n_maps, int belt_split, int band_lo,
-                               int band_hi, const uint2 *rr, int *flags, int *d_err,
-                               cudaStream_t st);
+                               int band_hi, const uint2 *rr, int *flags, bool ring_order,
+                               int *d_err, cudaStream_t st);
 
 // tcgen05 multi-map kernel for belt ring pairs: items are (belt ring, first
 // pixel) blocks of belt_mma_block() outputs; maps in groups of belt_mma_maps().
