@@ -52,11 +52,20 @@ TuneKey tune_key(const ksc_split *s) {
 }
 
 // Untuned default: half blocks only where a belt ring is shorter than a full
-// item; the single-map gather tile of that nside, of the two 128-class ones the one with
-// small tables where they fit and there are several entries to fill its three CTAs per SM.
-std::pair<int, int> default_variants(const ksc_split *s, int n) {
-    return {4 * s->nside <= ksc::belt_variant_chunk(1) ? 1 : 0,
-            s->sym_variant == 2 && s->sym_small_ok && n > 1 ? 1 : s->sym_variant};
+// item; the gather tile of that nside, of the two 128-class ones the one with small tables
+// where those of all the group's entries fit and the entries together have items for two waves
+// of two CTAs per SM (the single map's rule).
+std::pair<int, int> default_variants(const std::vector<const ksc_split *> &group) {
+    const int nside = group.front()->nside;
+    bool small = true;
+    long long items = 0;
+    for (const ksc_split *s : group) {
+        if (s->path != 0) continue;
+        small &= s->sym_small_ok;
+        items += s->n_items_sym;
+    }
+    return {4 * nside <= ksc::belt_variant_chunk(1) ? 1 : 0,
+            ksc::sym_chunk(nside) == ksc::sym_variant_chunk(0) ? 0 : small && items >= 4 * 152 ? 1 : 2};
 }
 
 struct Launch {
@@ -419,6 +428,7 @@ int ksc_batch_create(const ksc_split *const *splits, int n, const ksc_batch_opts
     b->splits.assign(splits, splits + n);
     b->plan_of.resize(n);
     b->group_of.resize(n);
+    std::vector<std::vector<const ksc_split *>> groups;
     bool counted = true;
     for (int i = 0; i < n; ++i) {
         const ksc_split *s = splits[i];
@@ -429,19 +439,21 @@ int ksc_batch_create(const ksc_split *const *splits, int n, const ksc_batch_opts
         b->group_of[i] = (int)(g - b->nsides.begin());
         if (g == b->nsides.end()) {
             b->nsides.push_back(s->nside);
-            std::pair<int, int> v = default_variants(s, n);
-            {
-                std::lock_guard<std::mutex> lk(g_tune_mu);
-                auto c = g_tune_cache.find(tune_key(s));
-                if (c != g_tune_cache.end()) v = c->second;
-            }
-            b->variants.push_back(v);
+            groups.emplace_back();
         }
+        groups[b->group_of[i]].push_back(s);
         if (s->path != 0) b->general.push_back(i);
         if (s->n_pairs < 0) counted = false;
         else b->n_pairs += s->n_pairs;
     }
     if (!counted) b->n_pairs = -1;
+    for (const std::vector<const ksc_split *> &group : groups) {
+        std::pair<int, int> v = default_variants(group);
+        std::lock_guard<std::mutex> lk(g_tune_mu);
+        auto c = g_tune_cache.find(tune_key(group.front()));
+        if (c != g_tune_cache.end()) v = c->second;
+        b->variants.push_back(v);
+    }
     std::vector<ksc::ConvPlan> plans;
     for (const ksc_split *s : b->uniq) plans.push_back(s->plan);
     cudaError_t e = plan_tc(b);

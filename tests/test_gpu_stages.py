@@ -179,3 +179,15 @@ def test_captured_calls_hold_their_scratch(K, nside, theta):
             assert torch.equal(y, one) and torch.equal(z, one)
         K.device_status(sp)
         del g
+
+
+def test_batch_gather_tile_suits_all_entries(K):
+    """One tile a group of one nside: small tables where those of every split fit and there are
+    items enough, whichever entry comes first."""
+    fits, wide, tiny = _split(K, 512, 440.0)[0], _split(K, 512, 660.0)[0], _split(K, 64, 360.0)[0]
+    assert K.split_stages(fits)["gather_variant"] == 1 and K.split_stages(wide)["gather_variant"] == 2
+    for splits, want in (([fits, fits], [1]), ([fits, wide], [2]), ([wide, fits], [2]), ([tiny, fits], [2, 1])):
+        with K.Batch(splits) as b:
+            assert [g["sym_variant"] for g in b.info()["groups"]] == want
+    for sp in (fits, wide, tiny):
+        sp.close()
