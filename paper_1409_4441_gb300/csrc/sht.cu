@@ -30,6 +30,7 @@
 // product per step and are re-anchored from the exact J every 8 steps (the products'
 // rounding drifts by about one FP32 ulp per step in between).
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 
 #include "ksc_internal.h"
@@ -129,15 +130,21 @@ __device__ __forceinline__ void ring_zs(int n, int r, F2 *z, F2 *s) {
     }
 }
 
-// Orders above this do not reach 2^-60 on a ring (see the top of the file).
-__device__ __forceinline__ int order_limit(int lmax, float s) {
-    return min(lmax, (int)((float)lmax * s + 16.0f + 9.0f * cbrtf((float)lmax)));
+// Orders above this do not reach 2^-60 on northern ring r (see the top of the file).  Some kernels
+// write G or F up to it and others read up to it, so it has to come out the same in all of
+// them: every step is rounded on its own, whatever the compiler does around it.
+__device__ __forceinline__ int ring_limit(int nside, int r, int lmax, float extra) {
+    const int i = r + 1, n = nside, a = 4 * n - 2 * i, d = 3 * n;
+    float s;
+    if (i < n) {
+        const float w = __fdiv_rn(__int2float_rn(i * i), __int2float_rn(3 * n * n));
+        s = __fsqrt_rn(__fmul_rn(w, __fsub_rn(2.0f, w)));
+    } else {
+        s = __fsqrt_rn(__fdiv_rn(__int2float_rn((d - a) * (d + a)), __int2float_rn(d * d)));
+    }
+    return min(lmax, (int)__fmaf_rn(__int2float_rn(lmax), s, extra));
 }
-__device__ __forceinline__ int ring_limit(int nside, int r, int lmax) {
-    F2 z, s;
-    ring_zs(nside, r, &z, &s);
-    return order_limit(lmax, s.h);
-}
+float order_extra(int lmax) { return 16.0f + 9.0f * std::cbrt((float)lmax); }
 
 // lambda_mm / sin^m theta = sqrt((2m + 1) / 4pi C), C = prod_{k<=m} (2k - 1) / 2k: the product
 // (a factor a lane, by all lanes of a warp), or the series of Gamma(m + 1/2) / Gamma(m + 1)
@@ -226,7 +233,7 @@ __device__ __forceinline__ float4 step_coeffs(int l, int m) {
 // 3.77 ms (two rings a thread for the same staged coefficients: 3.77; nside 512: 1.01
 // against 1.04).
 __global__ void __launch_bounds__(256)
-sht_leg_synth(int nside, int lmax, const double2 *__restrict__ alm, float2 *__restrict__ G) {
+sht_leg_synth(int nside, int lmax, float extra, const double2 *__restrict__ alm, float2 *__restrict__ G) {
     __shared__ float4 co[kTile], al[kTile];
     __shared__ F2 s_norm;
     const int m = blockIdx.y, nnorth = 2 * nside, nr = 4 * nside - 1;
@@ -242,7 +249,7 @@ sht_leg_synth(int nside, int lmax, const double2 *__restrict__ alm, float2 *__re
     if (r < nnorth) {
         F2 z, s;
         ring_zs(nside, r, &z, &s);
-        live = m <= order_limit(lmax, s.h);
+        live = m <= ring_limit(nside, r, lmax, extra);
         if (live) rec.start(m, s_norm, z, s);
     }
     if (!__syncthreads_or(live)) return;
@@ -295,7 +302,7 @@ constexpr int kGroup = 32;  // degrees between the block's reductions
 // back), so that a sum over all rings stays in range wherever the F_m do.
 template <int R>
 __global__ void __launch_bounds__(256)
-sht_leg_anal(int nside, int lmax, const float2 *__restrict__ F, const double *__restrict__ kl,
+sht_leg_anal(int nside, int lmax, float extra, const float2 *__restrict__ F, const double *__restrict__ kl,
              float scale, double c, double2 *__restrict__ alm) {
     extern __shared__ float4 acc[];  // [lmax + 1 - m]: re, im pairs
     __shared__ float4 co[kTile], term[8][8][33], part[8][kGroup];
@@ -320,7 +327,7 @@ sht_leg_anal(int nside, int lmax, const float2 *__restrict__ F, const double *__
             if (r < nnorth) {
                 F2 z, s;
                 ring_zs(nside, r, &z, &s);
-                live[j] = m <= order_limit(lmax, s.h);
+                live[j] = m <= ring_limit(nside, r, lmax, extra);
                 if (live[j]) {
                     rec[j].start(m, s_norm, z, s);
                     const int rs = nr - 1 - r;
@@ -442,7 +449,7 @@ __device__ __forceinline__ void fold(float &sum, float &comp, float v) {  // Kah
 // map.  The orders are staged in shared memory 1024 at a time.
 constexpr int kOrders = 1024;
 __global__ void __launch_bounds__(256)
-sht_ring_synth(int nside, int lmax, int r_first, const float2 *__restrict__ G,
+sht_ring_synth(int nside, int lmax, float extra, int r_first, const float2 *__restrict__ G,
                float *__restrict__ map, int add) {
     __shared__ float4 gs[kOrders];  // north, south
     // the longest rings first
@@ -450,7 +457,7 @@ sht_ring_synth(int nside, int lmax, int r_first, const float2 *__restrict__ G,
     const bool mirror = rs != r;
     const long long stride = lmax + 1;
     const ShtRing g = sht_ring(nside, r), h = sht_ring(nside, rs);
-    const int L = g.len, Q = L / 4, lim = ring_limit(nside, r, lmax);
+    const int L = g.len, Q = L / 4, lim = ring_limit(nside, r, lmax, extra);
     const float fl = (float)L, inv_l = 1.0f / fl;
     for (int k0 = blockIdx.y * 256; k0 < Q; k0 += gridDim.y * 256) {
         const int k = k0 + threadIdx.x;
@@ -528,7 +535,7 @@ sht_ring_synth(int nside, int lmax, int r_first, const float2 *__restrict__ G,
 // shared memory 512 pixels at a time (classes 0 and 2 are real, 3 is conjugate to 1).
 constexpr int kPix = 512;
 __global__ void __launch_bounds__(256)
-sht_ring_anal(int nside, int lmax, int r_first, const float *__restrict__ map,
+sht_ring_anal(int nside, int lmax, float extra, int r_first, const float *__restrict__ map,
               float2 *__restrict__ F) {
     __shared__ float4 y[4][kPix + 1];  // [class]: north re, im, south re, im
     // the longest rings first
@@ -536,7 +543,7 @@ sht_ring_anal(int nside, int lmax, int r_first, const float *__restrict__ map,
     const bool mirror = rs != r;
     const long long stride = lmax + 1;
     const ShtRing g = sht_ring(nside, r), h = sht_ring(nside, rs);
-    const int L = g.len, Q = L / 4, lim = ring_limit(nside, r, lmax);
+    const int L = g.len, Q = L / 4, lim = ring_limit(nside, r, lmax, extra);
     const float fl = (float)L, inv_l = 1.0f / fl;
     for (int m0 = blockIdx.y * 256; m0 <= lim; m0 += gridDim.y * 256) {
         const int m = m0 + threadIdx.x, c = m & 3, mr = m % (2 * L);
@@ -658,7 +665,7 @@ __device__ __forceinline__ void fft_table(float2 *tw, int lg) {
 
 // Analysis of belt ring r = r_first + blockIdx.x and its mirror by one FFT of north + i south.
 __global__ void __launch_bounds__(1024)
-sht_fft_anal(int nside, int lmax, int lg, int r_first, const float *__restrict__ map,
+sht_fft_anal(int nside, int lmax, float extra, int lg, int r_first, const float *__restrict__ map,
              float2 *__restrict__ F) {
     extern __shared__ float2 fx[];
     const int n = 1 << lg;
@@ -672,7 +679,7 @@ sht_fft_anal(int nside, int lmax, int lg, int r_first, const float *__restrict__
     __syncthreads();
     fft_shared(fx, tw, lg, -1.0f);
     const long long stride = lmax + 1;
-    const int lim = ring_limit(nside, r, lmax);
+    const int lim = ring_limit(nside, r, lmax, extra);
     const float inv = 1.0f / (float)n;
     for (int m = threadIdx.x; m <= lim; m += blockDim.x) {
         const float2 a = fx[m & (n - 1)], b = fx[(n - m) & (n - 1)];
@@ -692,7 +699,7 @@ sht_fft_anal(int nside, int lmax, int lg, int r_first, const float *__restrict__
 // Synthesis of belt ring r and its mirror: bin b of the Hermitian spectra collects the orders
 // m = b and, conjugate, m = -b mod n (each w_m / 2 G_m e^{i pi m t / n}); north + i south.
 __global__ void __launch_bounds__(1024)
-sht_fft_synth(int nside, int lmax, int lg, int r_first, const float2 *__restrict__ G,
+sht_fft_synth(int nside, int lmax, float extra, int lg, int r_first, const float2 *__restrict__ G,
               float *__restrict__ map, int add) {
     extern __shared__ float2 fx[];
     const int n = 1 << lg;
@@ -701,7 +708,7 @@ sht_fft_synth(int nside, int lmax, int lg, int r_first, const float2 *__restrict
     const bool mirror = rs != r;
     const ShtRing g = sht_ring(nside, r), h = sht_ring(nside, rs);
     const long long stride = lmax + 1;
-    const int lim = ring_limit(nside, r, lmax);
+    const int lim = ring_limit(nside, r, lmax, extra);
     const float inv = 1.0f / (float)n;
     fft_table(tw, lg);
     for (int b = threadIdx.x; b < n; b += blockDim.x) {
@@ -764,9 +771,10 @@ int fft_threads(int lg) { return std::max(32, std::min(1 << (lg - 2), std::max(5
 // Rings first .. last (northern half) by direct quarter sums; the rest of [0, 2 nside) by FFT.
 cudaError_t ring_synth(int nside, int lmax, const float2 *G, float *map, int add, cudaStream_t st) {
     const int lg = belt_fft(nside, lmax), n_cap = lg ? nside - 1 : 2 * nside;
+    const float extra = order_extra(lmax);
     if (n_cap > 0) {
         dim3 grid(n_cap, nside > 512 ? 2 : 1);
-        sht_ring_synth<<<grid, 256, 0, st>>>(nside, lmax, 0, G, map, add);
+        sht_ring_synth<<<grid, 256, 0, st>>>(nside, lmax, extra, 0, G, map, add);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess || !lg) return e;
     }
@@ -774,15 +782,16 @@ cudaError_t ring_synth(int nside, int lmax, const float2 *G, float *map, int add
     cudaError_t e = cudaFuncSetAttribute(sht_fft_synth, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          kFftSmem);
     if (e != cudaSuccess) return e;
-    sht_fft_synth<<<nside + 1, fft_threads(lg), smem, st>>>(nside, lmax, lg, nside - 1, G, map, add);
+    sht_fft_synth<<<nside + 1, fft_threads(lg), smem, st>>>(nside, lmax, extra, lg, nside - 1, G, map, add);
     return cudaGetLastError();
 }
 
 cudaError_t ring_anal(int nside, int lmax, const float *map, float2 *F, cudaStream_t st) {
     const int lg = belt_fft(nside, lmax), n_cap = lg ? nside - 1 : 2 * nside;
+    const float extra = order_extra(lmax);
     if (n_cap > 0) {
         dim3 grid(n_cap, (lmax + 256) / 256);
-        sht_ring_anal<<<grid, 256, 0, st>>>(nside, lmax, 0, map, F);
+        sht_ring_anal<<<grid, 256, 0, st>>>(nside, lmax, extra, 0, map, F);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess || !lg) return e;
     }
@@ -790,7 +799,7 @@ cudaError_t ring_anal(int nside, int lmax, const float *map, float2 *F, cudaStre
     cudaError_t e = cudaFuncSetAttribute(sht_fft_anal, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          kFftSmem);
     if (e != cudaSuccess) return e;
-    sht_fft_anal<<<nside + 1, fft_threads(lg), smem, st>>>(nside, lmax, lg, nside - 1, map, F);
+    sht_fft_anal<<<nside + 1, fft_threads(lg), smem, st>>>(nside, lmax, extra, lg, nside - 1, map, F);
     return cudaGetLastError();
 }
 
@@ -804,7 +813,7 @@ cudaError_t sht_synthesis(int nside, int lmax, const double2 *d_alm, float *d_ma
     cudaError_t e = cudaMallocAsync(&G, sizeof(float2) * (size_t)nr * (lmax + 1), st);
     if (e != cudaSuccess) return e;
     dim3 grid((nnorth + 255) / 256, lmax + 1);
-    sht_leg_synth<<<grid, 256, 0, st>>>(nside, lmax, d_alm, G);
+    sht_leg_synth<<<grid, 256, 0, st>>>(nside, lmax, order_extra(lmax), d_alm, G);
     e = cudaGetLastError();
     if (e == cudaSuccess) e = ring_synth(nside, lmax, G, d_map, add, st);
     const cudaError_t f = cudaFreeAsync(G, st);
@@ -828,7 +837,7 @@ cudaError_t sht_analysis(int nside, int lmax, const float *d_map, const double *
     if (e == cudaSuccess) {
         const double up = 4.0 * (double)nside;
         const double c = 4.0 * kPi / (12.0 * (double)nside * (double)nside) * up;
-        kernel<<<lmax + 1, 256, smem, st>>>(nside, lmax, F, d_kl, (float)(1.0 / up), c, d_alm);
+        kernel<<<lmax + 1, 256, smem, st>>>(nside, lmax, order_extra(lmax), F, d_kl, (float)(1.0 / up), c, d_alm);
         e = cudaGetLastError();
     }
     const cudaError_t f = cudaFreeAsync(F, st);
