@@ -23,8 +23,8 @@
 // functions decay exponentially past their turning point): a ring leaves them out.
 //
 // Ring sums: pixel k of a ring of L pixels with phase flag t sits at phi_k = pi (2k + t) / L.
-// Belt rings (L = 4 nside, a power of two) of larger transforms go through an FP32 FFT in shared memory, north
-// and mirror ring as one complex sequence.  Other rings (L = 4i) are summed directly over a
+// Belt rings (L = 4 nside, a power of two) of larger transforms go through an FP32 FFT in shared
+// memory, a ring and its mirror a block.  Other rings (L = 4i) are summed directly over a
 // quarter: the quarter turns of pixel k1 enter order m through m mod 4 alone.  m phi_k =
 // pi J / L with the exact integer J = m (2k + t) mod 2L; the twiddles advance by one complex
 // product per step and are re-anchored from the exact J every 8 steps (the products'
@@ -603,10 +603,10 @@ sht_ring_anal(int nside, int lmax, float extra, int r_first, const float *__rest
     }
 }
 
-// In-place FFT of 2^lg complex values in shared memory, sign -1 forward, +1 inverse
-// (unnormalised): Stockham radix 4 with one radix-2 pass when lg is odd; a thread holds the
-// values of its four butterflies between the two barriers of a pass.  tw[k] = e^{-2 pi i k /
-// n} for k < n / 4; the other quadrants by exact rotations.
+// In-place FFTs of two sequences of 2^lg complex values in shared memory, x[0 ..] and x[ss ..], sign
+// -1 forward, +1 inverse (unnormalised): Stockham radix 4 with one radix-2 pass when lg is odd; a
+// thread holds the values of its four butterflies between the two barriers of a pass.  tw[k] =
+// e^{-2 pi i k / n}, n = 2^(lg + 1), for k < n / 4; the other quadrants by exact rotations.
 __device__ __forceinline__ float2 fft_twiddle(const float2 *tw, int k, int lgq, float sgn) {
     const float2 w = tw[k & ((1 << lgq) - 1)];
     const int quad = k >> lgq;  // times (-i)^quad
@@ -614,42 +614,45 @@ __device__ __forceinline__ float2 fft_twiddle(const float2 *tw, int k, int lgq, 
     if (quad & 2) v = make_float2(-v.x, -v.y);
     return make_float2(v.x, -sgn * v.y);
 }
-__device__ __forceinline__ void fft_shared(float2 *x, const float2 *tw, int lg, float sgn) {
-    const int n = 1 << lg, q = n >> 2, T = blockDim.x;
+__device__ __forceinline__ void fft_shared(float2 *x, int ss, const float2 *tw, int lg, float sgn) {
+    const int n = 1 << lg, q = n >> 2, T = blockDim.x, lgq = lg - 1;
     int ls = 0;  // log2 of the stride s
     for (; ls + 2 <= lg; ls += 2) {
         float2 y[4][4];
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
-            const int t = threadIdx.x + b * T;
-            if (t >= q) break;
-            const float2 a0 = x[t], a1 = x[t + q], a2 = x[t + 2 * q], a3 = x[t + 3 * q];
-            const int k = (t >> ls) << ls;  // p s
+            const int i = threadIdx.x + b * T, t = i & (q - 1);
+            if (i >= 2 * q) break;
+            const float2 *v = x + (i >> (lg - 2)) * ss + t;
+            const float2 a0 = v[0], a1 = v[q], a2 = v[2 * q], a3 = v[3 * q];
+            const int k = ((t >> ls) << ls) << 1;  // p s, in steps of the table
             const float2 s02 = make_float2(a0.x + a2.x, a0.y + a2.y), d02 = make_float2(a0.x - a2.x, a0.y - a2.y);
             const float2 s13 = make_float2(a1.x + a3.x, a1.y + a3.y), d13 = make_float2(a1.x - a3.x, a1.y - a3.y);
             const float2 jd = make_float2(-sgn * d13.y, sgn * d13.x);  // sgn i d13
             y[b][0] = make_float2(s02.x + s13.x, s02.y + s13.y);
-            y[b][1] = cmul(make_float2(d02.x + jd.x, d02.y + jd.y), fft_twiddle(tw, k, lg - 2, sgn));
-            y[b][2] = cmul(make_float2(s02.x - s13.x, s02.y - s13.y), fft_twiddle(tw, 2 * k, lg - 2, sgn));
-            y[b][3] = cmul(make_float2(d02.x - jd.x, d02.y - jd.y), fft_twiddle(tw, 3 * k, lg - 2, sgn));
+            y[b][1] = cmul(make_float2(d02.x + jd.x, d02.y + jd.y), fft_twiddle(tw, k, lgq, sgn));
+            y[b][2] = cmul(make_float2(s02.x - s13.x, s02.y - s13.y), fft_twiddle(tw, 2 * k, lgq, sgn));
+            y[b][3] = cmul(make_float2(d02.x - jd.x, d02.y - jd.y), fft_twiddle(tw, 3 * k, lgq, sgn));
         }
         __syncthreads();
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
-            const int t = threadIdx.x + b * T;
-            if (t >= q) break;
+            const int i = threadIdx.x + b * T, t = i & (q - 1);
+            if (i >= 2 * q) break;
             const int lo = t & ((1 << ls) - 1), o = ((t >> ls) << (ls + 2)) + lo;
+            float2 *v = x + (i >> (lg - 2)) * ss + o;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) x[o + (j << ls)] = y[b][j];
+            for (int j = 0; j < 4; ++j) v[j << ls] = y[b][j];
         }
         __syncthreads();
     }
     if (ls < lg) {  // one radix-2 pass, stride n / 2
         const int hN = n >> 1;
-        for (int t = threadIdx.x; t < hN; t += T) {
-            const float2 a = x[t], b = x[t + hN];
-            x[t] = make_float2(a.x + b.x, a.y + b.y);
-            x[t + hN] = make_float2(a.x - b.x, a.y - b.y);
+        for (int i = threadIdx.x; i < n; i += T) {
+            float2 *v = x + (i >> (lg - 1)) * ss + (i & (hN - 1));
+            const float2 a = v[0], b = v[hN];
+            v[0] = make_float2(a.x + b.x, a.y + b.y);
+            v[hN] = make_float2(a.x - b.x, a.y - b.y);
         }
         __syncthreads();
     }
@@ -663,28 +666,42 @@ __device__ __forceinline__ void fft_table(float2 *tw, int lg) {
     }
 }
 
-// Analysis of belt ring r = r_first + blockIdx.x and its mirror by one FFT of north + i south.
+// Analysis of belt ring r = r_first + blockIdx.x and its mirror, each by a complex FFT of half its
+// length, even pixels + i odd ones (both rings as one complex sequence would round the fainter
+// one to the brighter one's last bits).
 __global__ void __launch_bounds__(1024)
 sht_fft_anal(int nside, int lmax, float extra, int lg, int r_first, const float *__restrict__ map,
              float2 *__restrict__ F) {
     extern __shared__ float2 fx[];
-    const int n = 1 << lg;
-    float2 *tw = fx + n;
+    const int n = 1 << lg, half = n >> 1;
+    float2 *tw = fx + n + 2;
     const int r = r_first + blockIdx.x, rs = 4 * nside - 2 - r;
     const bool mirror = rs != r;
     const ShtRing g = sht_ring(nside, r), h = sht_ring(nside, rs);
     fft_table(tw, lg);
-    for (int k = threadIdx.x; k < n; k += blockDim.x)
-        fx[k] = make_float2(__ldg(map + g.start + k), mirror ? __ldg(map + h.start + k) : 0.0f);
+    for (int k = threadIdx.x; k < half; k += blockDim.x) {
+        const float *a = map + g.start + 2 * k, *b = map + h.start + 2 * k;
+        fx[k] = make_float2(__ldg(a), __ldg(a + 1));
+        fx[half + k] = mirror ? make_float2(__ldg(b), __ldg(b + 1)) : make_float2(0.0f, 0.0f);
+    }
     __syncthreads();
-    fft_shared(fx, tw, lg, -1.0f);
+    fft_shared(fx, half, tw, lg - 1, -1.0f);
     const long long stride = lmax + 1;
     const int lim = ring_limit(nside, r, lmax, extra);
     const float inv = 1.0f / (float)n;
     for (int m = threadIdx.x; m <= lim; m += blockDim.x) {
-        const float2 a = fx[m & (n - 1)], b = fx[(n - m) & (n - 1)];
-        float2 fn = make_float2(0.5f * (a.x + b.x), 0.5f * (a.y - b.y));
-        float2 fs = make_float2(0.5f * (a.y + b.y), 0.5f * (b.x - a.x));
+        // X_k = (Z_k + Z*_{h-k}) / 2 - i/2 e^{-2 pi i k / n} (Z_k - Z*_{h-k}), h = n / 2, k <= h;
+        // X_{n-k} = X*_k
+        const int mm = m & (n - 1), k = min(mm, n - mm);
+        const float2 w = fft_twiddle(tw, k, lg - 2, -1.0f);
+        auto order = [&](const float2 *z) {
+            const float2 a = z[k & (half - 1)], b = z[(half - k) & (half - 1)];
+            const float2 e = make_float2(0.5f * (a.x + b.x), 0.5f * (a.y - b.y));
+            const float2 o = make_float2(0.5f * (a.y + b.y), 0.5f * (b.x - a.x));
+            const float2 p = cmul(w, o);
+            return make_float2(e.x + p.x, mm > half ? -(e.y + p.y) : e.y + p.y);
+        };
+        float2 fn = order(fx), fs = order(fx + half);
         if (g.t) {  // e^{-i pi m / n}, the argument exact
             float sn, cs;
             sincospif(-(float)m * inv, &sn, &cs);
@@ -697,13 +714,15 @@ sht_fft_anal(int nside, int lmax, float extra, int lg, int r_first, const float 
 }
 
 // Synthesis of belt ring r and its mirror: bin b of the Hermitian spectra collects the orders
-// m = b and, conjugate, m = -b mod n (each w_m / 2 G_m e^{i pi m t / n}); north + i south.
+// m = b and, conjugate, m = -b mod n (each w_m / 2 G_m e^{i pi m t / n}); each ring by a complex FFT
+// of half its length (see above) whose bins are Z_k = (H_k + H*_{h-k}) + i e^{2 pi i k / n} (H_k -
+// H*_{h-k}), h = n / 2.
 __global__ void __launch_bounds__(1024)
 sht_fft_synth(int nside, int lmax, float extra, int lg, int r_first, const float2 *__restrict__ G,
               float *__restrict__ map, int add) {
     extern __shared__ float2 fx[];
-    const int n = 1 << lg;
-    float2 *tw = fx + n;
+    const int n = 1 << lg, half = n >> 1;
+    float2 *tw = fx + n + 2;
     const int r = r_first + blockIdx.x, rs = 4 * nside - 2 - r;
     const bool mirror = rs != r;
     const ShtRing g = sht_ring(nside, r), h = sht_ring(nside, rs);
@@ -711,7 +730,7 @@ sht_fft_synth(int nside, int lmax, float extra, int lg, int r_first, const float
     const int lim = ring_limit(nside, r, lmax, extra);
     const float inv = 1.0f / (float)n;
     fft_table(tw, lg);
-    for (int b = threadIdx.x; b < n; b += blockDim.x) {
+    for (int b = threadIdx.x; b <= half; b += blockDim.x) {
         float2 zn = make_float2(0.0f, 0.0f), zs = zn;
         auto take = [&](int m, float conj) {
             if (m > lim) return;
@@ -734,25 +753,39 @@ sht_fft_synth(int nside, int lmax, float extra, int lg, int r_first, const float
         take(b + n, 1.0f);
         take(nb, -1.0f);
         take(nb + n, -1.0f);
-        fx[b] = make_float2(zn.x - zs.y, zn.y + zs.x);
+        fx[b] = zn;
+        fx[half + 1 + b] = zs;
     }
     __syncthreads();
-    fft_shared(fx, tw, lg, 1.0f);
+    for (int i = threadIdx.x; i < half + 2; i += blockDim.x) {  // k <= h / 2 of both rings
+        const int ring = i > half / 2, k = i - ring * (half / 2 + 1);
+        float2 *z = fx + ring * (half + 1);
+        const float2 a = z[k], b = z[half - k], w = fft_twiddle(tw, k, lg - 2, 1.0f);
+        // i w (H_k - H*_{h-k}); bin h - k has the conjugates of its terms
+        const float2 p = make_float2(a.x + b.x, a.y - b.y), q = cmul(w, make_float2(a.x - b.x, a.y + b.y));
+        z[k] = make_float2(p.x - q.y, p.y + q.x);
+        if (k > 0) z[half - k] = make_float2(p.x + q.y, q.x - p.y);
+    }
+    __syncthreads();
+    fft_shared(fx, half + 1, tw, lg - 1, 1.0f);
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
-        const float2 v = fx[k];
-        float *on = map + g.start + k, *os = map + h.start + k;
-        if (add) *on += v.x;
-        else *on = v.x;
-        if (mirror) {
-            if (add) *os += v.y;
-            else *os = v.y;
+        const int ring = k >= half, j = k - ring * half;
+        if (ring && !mirror) break;
+        const float2 v = fx[ring * (half + 1) + j];
+        float *o = map + (ring ? h.start : g.start) + 2 * j;
+        if (add) {
+            o[0] += v.x;
+            o[1] += v.y;
+        } else {
+            o[0] = v.x;
+            o[1] = v.y;
         }
     }
 }
 
 // The longest FFT's shared memory.  The limits are set to the largest value whatever the
 // call needs: calls of several threads may race on them.
-constexpr int kFftSmem = 8 * 5 * 4096;
+constexpr int kFftSmem = 8 * (5 * 4096 + 2);
 
 // log2 of the belt rings' length where they go through the FFT (L <= 16384, and from 1e8
 // products of a direct sum on), else 0.  Direct for all rings / quarter sums and FFT, both
@@ -778,7 +811,7 @@ cudaError_t ring_synth(int nside, int lmax, const float2 *G, float *map, int add
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess || !lg) return e;
     }
-    const size_t smem = sizeof(float2) * (5u << (lg - 2));
+    const size_t smem = sizeof(float2) * ((5u << (lg - 2)) + 2);
     cudaError_t e = cudaFuncSetAttribute(sht_fft_synth, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          kFftSmem);
     if (e != cudaSuccess) return e;
@@ -795,7 +828,7 @@ cudaError_t ring_anal(int nside, int lmax, const float *map, float2 *F, cudaStre
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess || !lg) return e;
     }
-    const size_t smem = sizeof(float2) * (5u << (lg - 2));
+    const size_t smem = sizeof(float2) * ((5u << (lg - 2)) + 2);
     cudaError_t e = cudaFuncSetAttribute(sht_fft_anal, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          kFftSmem);
     if (e != cudaSuccess) return e;

@@ -41,3 +41,29 @@ def test_nothing_unwritten_is_read(K, nside, lmax):
     torch.cuda.synchronize()
     assert torch.equal(got, clean) and torch.equal(back, back2)
     assert torch.isfinite(clean).all()
+
+
+# belt rings through the FFT, with and without a radix-2 pass in the halves
+@pytest.mark.parametrize("nside,lmax", [(512, 60), (1024, 60)])
+def test_faint_rings_keep_their_digits(K, nside, lmax):
+    """A broad source in one hemisphere: the other hemisphere's rings, 1e-3 of their mirrors, to 3e-6 of
+    their own rms (a handful of FP32 roundings of their own values, not of their mirrors')."""
+    sigma, t0 = np.radians(16.0), np.radians(118.0)  # the source's width and colatitude
+    z, s, n, _, phase = O.ring_table(nside)
+    ring = np.repeat(np.arange(n.size), n.astype(int))
+    k = np.concatenate([np.arange(int(c)) for c in n])
+    phi = (2.0 * k + phase[ring]) * np.pi / n[ring]
+    cosd = z[ring] * np.cos(t0) + s[ring] * np.sin(t0) * np.cos(phi)
+    alm = O.map2alm(nside, np.exp((cosd - 1.0) / sigma ** 2), lmax)
+    ref = O.alm2map(nside, alm, lmax)
+    y = torch.empty(12 * nside * nside, device="cuda")
+    K.sht_alm2map(nside, lmax, torch.tensor(alm, device="cuda"), y)
+    err = y.cpu().numpy().astype(np.float64) - ref
+    r = np.flatnonzero((np.arange(n.size) > nside) & (np.arange(n.size) < 2 * nside - 1))  # northern belt
+    start = np.concatenate([[0], np.cumsum(n)]).astype(int)
+    rms = np.array([np.sqrt(np.mean(ref[start[i]:start[i + 1]] ** 2)) for i in r])
+    bright = np.array([np.sqrt(np.mean(ref[start[j]:start[j + 1]] ** 2)) for j in n.size - 1 - r])
+    worst = np.array([np.abs(err[start[i]:start[i + 1]]).max() for i in r])
+    faint = rms < 0.02 * bright
+    assert faint.sum() > 50
+    assert (worst[faint] <= 3e-6 * rms[faint]).all()
