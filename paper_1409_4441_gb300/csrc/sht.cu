@@ -215,6 +215,22 @@ struct Rec {
     }
 };
 
+// Powers of two that take values of largest magnitude `top` (the high word of a double, the bits of
+// a float) to [2^30, 2^31), where sums over degrees or rings and the low parts of the pairs stay in
+// FP32's range, and back; 1 for zeros, infinities and NaN.
+constexpr int kTopExp = 30;
+__device__ __forceinline__ double pow2(int e) {  // |e| <= 1022
+    return __hiloint2double((1023 + e) << 20, 0);
+}
+__device__ __forceinline__ int scale_exp_f64(int top_hi) {
+    const int e = (top_hi >> 20) - 1023;
+    return top_hi == 0 || e == 1024 ? 0 : max(min(kTopExp - e, 1022), -1022);
+}
+__device__ __forceinline__ int scale_exp_f32(unsigned top) {
+    const int e = (int)(top >> 23) - 127;
+    return top == 0u || e == 128 ? 0 : min(kTopExp - e, 126);
+}
+
 constexpr int kTile = 128;  // degrees whose coefficients a block stages at a time
 
 // Coefficients of the step to degree l (l > m): A_l and B_l = 1 / A_{l-1} (0 at l = m + 1),
@@ -236,8 +252,10 @@ __global__ void __launch_bounds__(256)
 sht_leg_synth(int nside, int lmax, float extra, const double2 *__restrict__ alm, float2 *__restrict__ G) {
     __shared__ float4 co[kTile], al[kTile];
     __shared__ F2 s_norm;
+    __shared__ int s_top;
     const int m = blockIdx.y, nnorth = 2 * nside, nr = 4 * nside - 1;
     const int r = blockIdx.x * 256 + threadIdx.x, rs = nr - 1 - r;
+    if (threadIdx.x == 0) s_top = 0;
     if (threadIdx.x < 32) {
         const F2 v = norm_mm(m);
         if (threadIdx.x == 0) s_norm = v;
@@ -254,13 +272,23 @@ sht_leg_synth(int nside, int lmax, float extra, const double2 *__restrict__ alm,
     }
     if (!__syncthreads_or(live)) return;
     const double2 *a = alm + alm_base(lmax, m);
+    int top = 0;  // largest |re|, |im| of the order's coefficients
+    for (int l = m + threadIdx.x; l <= lmax; l += 256) {
+        const double2 c = __ldg(a + l);
+        top = max(top, max(__double2hiint(fabs(c.x)), __double2hiint(fabs(c.y))));
+    }
+    top = __reduce_max_sync(~0u, top);
+    if ((threadIdx.x & 31) == 0) atomicMax(&s_top, top);
+    __syncthreads();
+    const int ex = scale_exp_f64(s_top);
+    const double up = pow2(ex);
     for (int l0 = m; l0 <= lmax; l0 += kTile) {
         const int n = min(kTile, lmax + 1 - l0);
         __syncthreads();
         for (int i = threadIdx.x; i < n; i += 256) {
             if (l0 + i > m) co[i] = step_coeffs(l0 + i, m);
             const double2 c = __ldg(a + l0 + i);
-            const F2 x = f2_of(c.x), y = f2_of(c.y);
+            const F2 x = f2_of(c.x * up), y = f2_of(c.y * up);
             al[i] = make_float4(x.h, x.l, y.h, y.l);
         }
         __syncthreads();
@@ -281,11 +309,16 @@ sht_leg_synth(int nside, int lmax, float extra, const double2 *__restrict__ alm,
     }
     if (!live) return;
     const long long stride = lmax + 1;
-    G[(long long)r * stride + m] = make_float2(f2_add(er, od).h, f2_add(ei, oi).h);
+    const double down = pow2(-ex);
+    auto store = [&](int ring) {
+        G[(long long)ring * stride + m] = make_float2((float)((double)f2_add(er, od).h * down),
+                                                      (float)((double)f2_add(ei, oi).h * down));
+    };
+    store(r);
     if (rs == r) return;
     od = F2{-od.h, -od.l};
     oi = F2{-oi.h, -oi.l};
-    G[(long long)rs * stride + m] = make_float2(f2_add(er, od).h, f2_add(ei, oi).h);
+    store(rs);
 }
 
 constexpr int kGroup = 32;  // degrees between the block's reductions
@@ -298,19 +331,19 @@ constexpr int kGroup = 32;  // degrees between the block's reductions
 // Four rings a thread share the reduction: 5.76 ms at nside 2048, l_max 1024 (one ring 8.11;
 // 70.1 in FP64 with atomics); with one pass or two over the rings (nside <= 128) one ring is
 // the shorter chain (25.5 against 27.9 us at nside 128, l_max 64).  The
-// F_m enter divided by the power of two that covers the number of rings (exact; c carries it
-// back), so that a sum over all rings stays in range wherever the F_m do.
+// F_m of a pass enter scaled by a power of two (exact), and the passes add up in FP64.
 template <int R>
 __global__ void __launch_bounds__(256)
 sht_leg_anal(int nside, int lmax, float extra, const float2 *__restrict__ F, const double *__restrict__ kl,
-             float scale, double c, double2 *__restrict__ alm) {
-    extern __shared__ float4 acc[];  // [lmax + 1 - m]: re, im pairs
+             double c, double2 *__restrict__ alm) {
+    extern __shared__ double2 acc[];  // [lmax + 1 - m]
     __shared__ float4 co[kTile], term[8][8][33], part[8][kGroup];
     __shared__ F2 s_norm;
+    __shared__ unsigned s_top;
     const int m = lmax - blockIdx.x, nnorth = 2 * nside, nr = 4 * nside - 1;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long stride = lmax + 1;
-    for (int i = threadIdx.x; i <= lmax - m; i += 256) acc[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    for (int i = threadIdx.x; i <= lmax - m; i += 256) acc[i] = make_double2(0.0, 0.0);
     if (threadIdx.x < 32) {
         const F2 v = norm_mm(m);
         if (threadIdx.x == 0) s_norm = v;
@@ -319,31 +352,45 @@ sht_leg_anal(int nside, int lmax, float extra, const float2 *__restrict__ F, con
     for (int base = 0; base < nnorth; base += 256 * R) {
         Rec rec[R];
         F2 sr[R], si[R], dr[R], di[R];  // F north + south (even l - m), north - south (odd)
+        float4 f[R];                    // north, south
         bool live[R], any = false;
+        unsigned top = 0u;
+        if (threadIdx.x == 0) s_top = 0u;
+        __syncthreads();
 #pragma unroll
         for (int j = 0; j < R; ++j) {
             const int r = base + 256 * j + threadIdx.x;
             live[j] = false;
             if (r < nnorth) {
-                F2 z, s;
-                ring_zs(nside, r, &z, &s);
                 live[j] = m <= ring_limit(nside, r, lmax, extra);
                 if (live[j]) {
+                    F2 z, s;
+                    ring_zs(nside, r, &z, &s);
                     rec[j].start(m, s_norm, z, s);
                     const int rs = nr - 1 - r;
                     const float2 fn = F[(long long)r * stride + m];
                     const float2 fs = rs != r ? F[(long long)rs * stride + m] : make_float2(0.0f, 0.0f);
-                    const float nx = scale * fn.x, ny = scale * fn.y;
-                    const float sx = scale * fs.x, sy = scale * fs.y;
-                    sr[j] = f2_sum(nx, sx);
-                    si[j] = f2_sum(ny, sy);
-                    dr[j] = f2_sum(nx, -sx);
-                    di[j] = f2_sum(ny, -sy);
+                    f[j] = make_float4(fn.x, fn.y, fs.x, fs.y);
+                    top = max(max(top, max(__float_as_uint(fn.x) & 0x7fffffffu, __float_as_uint(fn.y) & 0x7fffffffu)),
+                              max(__float_as_uint(fs.x) & 0x7fffffffu, __float_as_uint(fs.y) & 0x7fffffffu));
                 }
             }
             any |= live[j];
         }
+        top = __reduce_max_sync(~0u, top);
+        if (lane == 0) atomicMax(&s_top, top);
         if (!__syncthreads_or(any)) continue;
+        const int ex = scale_exp_f32(s_top);
+        const float scale = __int_as_float((127 + ex) << 23);
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+            if (!live[j]) continue;
+            const float nx = scale * f[j].x, ny = scale * f[j].y, sx = scale * f[j].z, sy = scale * f[j].w;
+            sr[j] = f2_sum(nx, sx);
+            si[j] = f2_sum(ny, sy);
+            dr[j] = f2_sum(nx, -sx);
+            di[j] = f2_sum(ny, -sy);
+        }
         const bool warp_any = __any_sync(~0u, any);
         for (int l0 = m; l0 <= lmax; l0 += kTile) {
             const int n = min(kTile, lmax + 1 - l0);
@@ -395,15 +442,17 @@ sht_leg_anal(int nside, int lmax, float extra, const float2 *__restrict__ F, con
                 }
                 __syncthreads();
                 if (threadIdx.x < kGroup && g0 + (int)threadIdx.x < n) {
-                    const float4 o = acc[l0 - m + g0 + threadIdx.x];
-                    F2 tr{o.x, o.y}, ti{o.z, o.w};
+                    F2 tr{0.0f, 0.0f}, ti = tr;
 #pragma unroll
                     for (int k = 0; k < 8; ++k) {
                         const float4 t = part[k][threadIdx.x];
                         tr = f2_add(tr, F2{t.x, t.y});
                         ti = f2_add(ti, F2{t.z, t.w});
                     }
-                    acc[l0 - m + g0 + threadIdx.x] = make_float4(tr.h, tr.l, ti.h, ti.l);
+                    double2 &o = acc[l0 - m + g0 + threadIdx.x];
+                    const double down = pow2(-ex);
+                    o.x = fma((double)tr.h + (double)tr.l, down, o.x);
+                    o.y = fma((double)ti.h + (double)ti.l, down, o.y);
                 }
                 __syncthreads();
             }
@@ -412,9 +461,9 @@ sht_leg_anal(int nside, int lmax, float extra, const float2 *__restrict__ F, con
     __syncthreads();
     double2 *a = alm + alm_base(lmax, m);
     for (int l = m + threadIdx.x; l <= lmax; l += 256) {
-        const float4 t = acc[l - m];
+        const double2 t = acc[l - m];
         const double w = c * (kl ? kl[l] : 1.0);
-        a[l] = make_double2(w * ((double)t.x + (double)t.y), w * ((double)t.z + (double)t.w));
+        a[l] = make_double2(w * t.x, w * t.y);
     }
 }
 
@@ -868,9 +917,8 @@ cudaError_t sht_analysis(int nside, int lmax, const float *d_map, const double *
         return e;
     e = ring_anal(nside, lmax, d_map, F, st);
     if (e == cudaSuccess) {
-        const double up = 4.0 * (double)nside;
-        const double c = 4.0 * kPi / (12.0 * (double)nside * (double)nside) * up;
-        kernel<<<lmax + 1, 256, smem, st>>>(nside, lmax, order_extra(lmax), F, d_kl, (float)(1.0 / up), c, d_alm);
+        const double c = 4.0 * kPi / (12.0 * (double)nside * (double)nside);
+        kernel<<<lmax + 1, 256, smem, st>>>(nside, lmax, order_extra(lmax), F, d_kl, c, d_alm);
         e = cudaGetLastError();
     }
     const cudaError_t f = cudaFreeAsync(F, st);

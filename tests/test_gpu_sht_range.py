@@ -67,3 +67,36 @@ def test_faint_rings_keep_their_digits(K, nside, lmax):
     faint = rms < 0.02 * bright
     assert faint.sum() > 50
     assert (worst[faint] <= 3e-6 * rms[faint]).all()
+
+
+@pytest.mark.parametrize("scale", [1e40, 1e44])
+def test_coefficients_keep_the_range_of_a_double(K, scale):
+    """One sectoral coefficient past FP32's range: rings where its function takes it back into that
+    range, to 2e-6 of the ring's largest pixel (functions below 2^-60 count as zero: not the rings
+    where less than 1e6 of that is left)."""
+    nside, lmax = 64, 128
+    alm = inputs.grf_alm(lmax, inputs.cl_grf(lmax), 7)
+    alm[lmax * (2 * lmax + 1 - lmax) // 2 + lmax] = scale  # l = m = l_max
+    ref = O.alm2map(nside, alm, lmax)
+    y = torch.empty(12 * nside * nside, device="cuda")
+    K.sht_alm2map(nside, lmax, torch.tensor(alm, device="cuda"), y)
+    got = y.cpu().numpy().astype(np.float64)
+    _, _, n, start, _ = O.ring_table(nside)
+    checked = 0
+    for st, c in zip(start.astype(int), n.astype(int)):
+        top = np.abs(ref[st:st + c]).max()
+        if 1e6 * 2.0 ** -60 * scale < top < 1e37:
+            checked += 1
+            assert np.abs(got[st:st + c] - ref[st:st + c]).max() <= 2e-6 * top
+    assert checked >= 4
+
+
+def test_analysis_of_a_map_near_the_smallest_floats(K):
+    """A map of values about 1e-36: the a_lm of the same map about one, scaled, to 1e-6 of the largest."""
+    nside, lmax = 64, 128
+    m = torch.tensor(inputs.white_noise_map(nside, 21).astype(np.float32), device="cuda")
+    one = torch.zeros(K.n_alm(lmax), dtype=torch.complex128, device="cuda")
+    low = torch.zeros_like(one)
+    K.sht_map2alm(nside, lmax, m, one)
+    K.sht_map2alm(nside, lmax, m * 2.0 ** -119, low)
+    assert (low * 2.0 ** 119 - one).abs().max() <= 1e-6 * one.abs().max()
