@@ -52,7 +52,7 @@ def test_faint_rings_keep_their_digits(K, nside, lmax):
     z, s, n, _, phase = O.ring_table(nside)
     ring = np.repeat(np.arange(n.size), n.astype(int))
     k = np.concatenate([np.arange(int(c)) for c in n])
-    phi = (2.0 * k + phase[ring]) * np.pi / n[ring]
+    phi = phase[ring] + 2.0 * np.pi * k / n[ring]
     cosd = z[ring] * np.cos(t0) + s[ring] * np.sin(t0) * np.cos(phi)
     alm = O.map2alm(nside, np.exp((cosd - 1.0) / sigma ** 2), lmax)
     ref = O.alm2map(nside, alm, lmax)
@@ -100,3 +100,54 @@ def test_analysis_of_a_map_near_the_smallest_floats(K):
     K.sht_map2alm(nside, lmax, m, one)
     K.sht_map2alm(nside, lmax, m * 2.0 ** -119, low)
     assert (low * 2.0 ** 119 - one).abs().max() <= 1e-6 * one.abs().max()
+
+
+def _lambda(lmax, z):
+    """lambda_lm(z) as [l, m], no Condon-Shortley phase."""
+    lam = np.zeros((lmax + 1, lmax + 1))
+    s = np.sqrt((1.0 - z) * (1.0 + z))
+    lam[0, 0] = np.sqrt(1.0 / (4.0 * np.pi))
+    for m in range(1, lmax + 1):
+        lam[m, m] = lam[m - 1, m - 1] * s * np.sqrt((2.0 * m + 1.0) / (2.0 * m))
+    for m in range(lmax + 1):
+        for l in range(m + 1, lmax + 1):
+            a = np.sqrt((4.0 * l * l - 1.0) / (l * l - m * m))
+            b = np.sqrt(((l - 1.0) ** 2 - m * m) / (4.0 * (l - 1.0) ** 2 - 1.0)) * lam[l - 2, m] if l > m + 1 else 0.0
+            lam[l, m] = a * (z * lam[l - 1, m] - b)
+    return lam
+
+
+# FFT lengths 8192 and 16384, then belt rings too long for it
+@pytest.mark.parametrize("nside", [2048, 4096, 8192])
+def test_longest_rings(K, nside):
+    """Synthesis on rings of every kind, and the analysis of single pixels (a_lm = 4 pi / N lambda_lm
+    e^{-i m phi}), each to 2e-6 of the largest."""
+    lmax, npix = 24, 12 * nside * nside
+    alm = _alm(lmax, 9)
+    flat = alm.cpu().numpy()
+    a = np.zeros((lmax + 1, lmax + 1), complex)
+    at = 0
+    for m in range(lmax + 1):
+        a[m:, m] = flat[at:at + lmax + 1 - m]
+        at += lmax + 1 - m
+    z, _, n, start, phase = O.ring_table(nside)
+    y = torch.zeros(npix, device="cuda")
+    K.sht_alm2map(nside, lmax, alm, y)
+    ms = np.arange(lmax + 1)
+    for r in (0, 5, nside // 2, nside - 2, nside - 1, nside, 2 * nside - 1, 2 * nside, 3 * nside, 4 * nside - 2):
+        c = int(n[r])
+        phi = phase[r] + 2.0 * np.pi * np.arange(c) / c
+        g = (_lambda(lmax, z[r]) * a).sum(0) * np.where(ms > 0, 2.0, 1.0)
+        want = (g[None, :] * np.exp(1j * np.outer(phi, ms))).real.sum(1)
+        got = y[int(start[r]):int(start[r]) + c].cpu().numpy()
+        assert np.abs(got - want).max() <= 2e-6 * np.abs(want).max()
+    back = torch.zeros_like(alm)
+    for r in (nside // 2, nside - 1, 2 * nside - 1, 2 * nside + 7):
+        k = int(n[r]) // 3
+        y.zero_()
+        y[int(start[r]) + k] = 1.0
+        K.sht_map2alm(nside, lmax, y, back)
+        phi = phase[r] + 2.0 * np.pi * k / int(n[r])
+        want = 4.0 * np.pi / npix * _lambda(lmax, z[r]) * np.exp(-1j * ms * phi)[None, :]
+        want = np.concatenate([want[m:, m] for m in range(lmax + 1)])
+        assert np.abs(back.cpu().numpy() - want).max() <= 2e-6 * np.abs(want).max()
