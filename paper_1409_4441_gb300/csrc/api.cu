@@ -300,18 +300,24 @@ void plan_cap_tc(ksc_split *s, const ksc_split_opts &o, const ksc::RingGeom &g,
     }
     // blocks of two rings: input rings, windows, sectors
     // (cap rings or belt rings, not both; an odd ring out alone)
-    ksc::CapTc c;
+    struct Block {
+        int r0, r1;
+        int lq_max = 0, jm = 0, wpos = 0, span = 0;  // over the input rings; span: the whole ring's
+        double work = 0.0;
+    };
+    std::vector<Block> blocks;
     for (int r0 = 0, r1; r0 <= last; r0 = r1 + 1) {
         r1 = r0 < belt_lo && ((belt_lo - r0) & 1) ? r0 : std::min(r0 + 1, r0 < belt_lo ? belt_lo - 1 : last);
-        const int q0 = std::min(range[r0].x, range[r1].x), q1 = std::max(range[r0].y, range[r1].y);
-        const int L0 = g.len[r0], L1 = g.len[r1];
-        int lq_max = 0, jm = 0;
-        double work = 0.0;
-        bool one = true;  // the whole ring as one sector
-        int span_one = 0;
-        for (int q = q0; q <= q1; ++q) {
+        blocks.push_back({r0, r1});
+    }
+#pragma omp parallel for schedule(dynamic, 8)
+    for (size_t i = 0; i < blocks.size(); ++i) {
+        Block &b = blocks[i];
+        const int L0 = g.len[b.r0], L1 = g.len[b.r1];
+        const int q1 = std::max(range[b.r0].y, range[b.r1].y);
+        for (int q = std::min(range[b.r0].x, range[b.r1].x); q <= q1; ++q) {
             int w = -1;
-            for (int r = r0; r <= r1; ++r) {
+            for (int r = b.r0; r <= b.r1; ++r) {
                 if (q < range[r].x || q > range[r].y) continue;
                 const int nc = plan->ncut[(size_t)pair_base[r] + (q - range[r].x)];
                 if (nc >= 0) w = std::max(w, cell(nc, g.len[r]));
@@ -321,46 +327,61 @@ void plan_cap_tc(ksc_split *s, const ksc_split_opts &o, const ksc::RingGeom &g,
             auto pos = [&](int k, int t, int L) {
                 return (int)(((long long)(2 * k + t) * Lq + (long long)(1 - tq) * L) / (2 * L));
             };
-            const int lo = std::min(pos(0, g.phase[r0], L0), pos(0, g.phase[r1], L1));
-            const int hi = std::max(pos(L0 - 1, g.phase[r0], L0), pos(L1 - 1, g.phase[r1], L1));
-            span_one = std::max(span_one, hi - lo + 1);
-            one = span_one <= ksc::cap_tc_span();
-            lq_max = std::max(lq_max, Lq);
-            jm = std::max(jm, w);
+            const int lo = std::min(pos(0, g.phase[b.r0], L0), pos(0, g.phase[b.r1], L1));
+            const int hi = std::max(pos(L0 - 1, g.phase[b.r0], L0), pos(L1 - 1, g.phase[b.r1], L1));
+            b.span = std::max(b.span, hi - lo + 1);
+            b.lq_max = std::max(b.lq_max, Lq);
+            b.jm = std::max(b.jm, w);
             const int np = ksc::cap_tc_positions(w, Lq);
-            c.wpos = std::max(c.wpos, np);
+            b.wpos = std::max(b.wpos, np);
             // us on an SM: 5.7 for windows up to about 80 positions, then the products
-            work += 5.7 + 0.024 * std::max(np - 80, 0);
+            b.work += 5.7 + 0.024 * std::max(np - 80, 0);
         }
+    }
+    ksc::CapTc c;
+    for (const Block &b : blocks) {
         // (cap rings without a regular pair have a tile too: it writes what the direct ones add to)
-        if (lq_max == 0 && r0 >= belt_lo) continue;
+        if (b.lq_max == 0 && b.r0 >= belt_lo) continue;
         // a sector's positions: L' / n, the rings' different first outputs, rounding
-        int n_sec = 1;
-        if (!one) {
-            const int slack = (lq_max + L0 - 1) / L0 + 4;
-            n_sec = (lq_max + ksc::cap_tc_span() - slack - 1) / (ksc::cap_tc_span() - slack);
-            n_sec = std::max(n_sec, 2);
+        const int L0 = g.len[b.r0], L1 = g.len[b.r1], span = ksc::cap_tc_span();
+        const int slack = (b.lq_max + L0 - 1) / L0 + 4;
+        const bool one = b.span <= span;
+        const int n_sec = one ? 1 : slack < span ? std::max((b.lq_max + span - slack - 1) / (span - slack), 2) : L0 + 1;
+        if (n_sec > L0) {  // (the shortest rings, cuts of most of the sphere)
+            plan->tiles.clear();
+            return;
         }
-        c.nq = std::max(c.nq, q1 - q0 + 1);
-        c.jcap = std::max(c.jcap, jm + 1);
+        c.wpos = std::max(c.wpos, b.wpos);
+        c.nq = std::max(c.nq, std::max(range[b.r0].y, range[b.r1].y) - std::min(range[b.r0].x, range[b.r1].x) + 1);
+        c.jcap = std::max(c.jcap, b.jm + 1);
         c.tcap = std::max(c.tcap, (std::max(L0, L1) + n_sec - 1) / n_sec + 1);
-        c.span = std::max(c.span, one ? span_one : (lq_max + n_sec - 1) / n_sec + (lq_max + L0 - 1) / L0 + 4);
+        c.span = std::max(c.span, one ? b.span : (b.lq_max + n_sec - 1) / n_sec + slack);
         for (int t = 0; t < n_sec; ++t) {
-            plan->tiles.push_back(make_int2((r1 - r0) << 16 | r0, n_sec << 16 | t));
-            plan->cost.push_back(work);
+            plan->tiles.push_back(make_int2((b.r1 - b.r0) << 16 | b.r0, n_sec << 16 | t));
+            plan->cost.push_back(b.work);
         }
     }
     c.span = std::min((c.span + 15) & ~15, ksc::cap_tc_span());
     // the coefficients: up to 8 GB (2.4 GB at nside 2048 with a 240' cut); beyond it the
     // gather, which keeps none
-    unsigned long long n4 = 0;
-    plan->coef_off.assign(pairs.size() + 1, 0u);
+    const auto words4 = [&](int r, size_t ip) {
+        return plan->ncut[ip] >= 0 ? ksc::cap_tc_words(cell(plan->ncut[ip], g.len[r])) / 4 : 0;
+    };
+    std::vector<unsigned long long> first(last + 2, 0ull);
+#pragma omp parallel for schedule(dynamic, 16)
     for (int r = 0; r <= last; ++r)
-        for (int q = range[r].x; q <= range[r].y; ++q) {
-            const size_t ip = (size_t)pair_base[r] + (q - range[r].x);
-            plan->coef_off[ip] = (unsigned)n4;
-            if (plan->ncut[ip] >= 0) n4 += ksc::cap_tc_words(cell(plan->ncut[ip], g.len[r])) / 4;
+        for (size_t ip = pair_base[r]; ip < (size_t)pair_base[r + 1]; ++ip) first[r + 1] += words4(r, ip);
+    for (int r = 0; r <= last; ++r) first[r + 1] += first[r];
+    const unsigned long long n4 = first[last + 1];
+    plan->coef_off.assign(pairs.size() + 1, 0u);
+#pragma omp parallel for schedule(dynamic, 16)
+    for (int r = 0; r <= last; ++r) {
+        unsigned long long at = first[r];
+        for (size_t ip = pair_base[r]; ip < (size_t)pair_base[r + 1]; ++ip) {
+            plan->coef_off[ip] = (unsigned)at;
+            at += words4(r, ip);
         }
+    }
     if (!ksc::cap_tc_fits(c) || n4 * 16 > 8ull << 30) plan->tiles.clear();
     if (plan->tiles.empty()) return;
     // The stage has to be the faster one: its tiles, and the direct pairs (sixteen warps share
@@ -388,13 +409,19 @@ void plan_cap_tc(ksc_split *s, const ksc_split_opts &o, const ksc::RingGeom &g,
 }
 
 // Uploads the cap stage's tiles and lays out its coefficients.  The stage is left out (the
-// gather sums the caps) where there is no room for them, and where a coefficient does not fit
+// gather sums the caps) where there is no ample room for them, and where a coefficient does not fit
 // an FP16 number: the scale comes from the kernel inside the cut, the polynomials of the cells
 // that the cut divides from the kernel past it too, which may be larger.
 int build_cap_tc(ksc_split *s, const CapPlan &cap, ksc::CapCoef cc) {
     if (s->n_cap_tiles == 0) return KSC_OK;
-    cudaError_t e = cudaMalloc(&s->d_coef, 16ull * cap.coef_off.back());
+    // (no more than an eighth of what is free: a program that keeps many splits, or maps of its
+    // own, can fill the device with them as it could before the stage)
+    const size_t bytes = 16ull * cap.coef_off.back();
+    size_t free_bytes = 0, total = 0;
+    cudaError_t e = cudaMemGetInfo(&free_bytes, &total);
+    if (e == cudaSuccess) e = bytes <= free_bytes / 8 ? dev_malloc((void **)&s->d_coef, bytes) : cudaErrorMemoryAllocation;
     if (e != cudaSuccess) {
+        if (e != cudaErrorMemoryAllocation) return cuda_fail(e, "cap coefficients");
         cudaGetLastError();
         s->d_coef = nullptr;
         drop_cap_tc(s);
