@@ -122,7 +122,7 @@ conv_belt_tc_kernel(const ConvPlan P, int block_lo, int n_tiles_k, int ring_lo, 
     __shared__ __align__(8) uint64_t a_full[kStages], a_free[kStages], d_done[2];
     __shared__ uint32_t tmem_base;
     __shared__ uint32_t s_max, s_min;
-    __shared__ int s_abort, s_lo, s_hi, s_bad, s_shift;
+    __shared__ int s_abort, s_lo, s_hi, s_bad, s_shift, s_band_lo, s_band_hi, s_tail;
     __shared__ float s_wsum[kRings];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -140,9 +140,11 @@ conv_belt_tc_kernel(const ConvPlan P, int block_lo, int n_tiles_k, int ring_lo, 
     if (tid == 0) {
         s_max = 0u;
         s_min = 0xffffffffu;
-        s_abort = s_bad = s_shift = 0;
+        s_abort = s_bad = s_shift = s_tail = 0;
         s_lo = P.belt_hi;
         s_hi = P.belt_lo;
+        s_band_lo = P.belt_hi;
+        s_band_hi = P.belt_lo;
         for (int b = 0; b < kStages; ++b) {
             tc::mbar_init(&a_full[b], kRings);
             tc::mbar_init(&a_free[b], 1);
@@ -155,9 +157,18 @@ conv_belt_tc_kernel(const ConvPlan P, int block_lo, int n_tiles_k, int ring_lo, 
         const int2 g = P.d_range[r_first + lane];
         atomicMin(&s_lo, max(g.x, P.belt_lo));
         atomicMax(&s_hi, min(g.y, P.belt_hi));
+        if (r_first + lane >= ring_lo && r_first + lane <= ring_hi) {
+            atomicMin(&s_band_lo, max(g.x, P.belt_lo));
+            atomicMax(&s_band_hi, min(g.y, P.belt_hi));
+        }
     }
     __syncthreads();
     const int q_lo = s_lo, nq = s_hi - s_lo + 1;
+    // Input rings [s_band_lo, s_band_hi] reach an output ring of the band.  Those before add
+    // nothing to its sums, whose folds are then all zero; of the s_tail rings after, only the folds
+    // are carried out.  (Narrow tiles, which bands of few rings take: nine rings of nside 2048, 16
+    // pixels: 0.165 -> 0.133 ms; wide ones have no registers for a second kind of fold.)
+    constexpr bool kTrim = N <= 64;
     uint32_t vmax = 0u, vmin = 0xffffffffu;
     for (int q = q_lo + warp; q < q_lo + nq; q += kThreads / 32) {
         int w = -1;
@@ -173,8 +184,10 @@ conv_belt_tc_kernel(const ConvPlan P, int block_lo, int n_tiles_k, int ring_lo, 
         }
         const Window g = tile_window(w, L);
         if (lane == 0) {  // the host sized both for every tile: never expected
-            if (q - q_lo < nq_cap && 16 * (g.s1 - g.s0) <= wpos_cap) sQ[q - q_lo] = (short)w;
+            if (q - q_lo < nq_cap && 16 * (g.s1 - g.s0) <= wpos_cap)
+                sQ[q - q_lo] = (short)(kTrim && (q < s_band_lo || q > s_band_hi) ? -1 : w);
             else s_bad = 1;
+            if (kTrim && q > s_band_hi) atomicAdd(&s_tail, 1);
         }
         const int start = P.d_rings[q].start;
         // pixels [a, a + len) of the ring, wrapped; every block of 64 map pixels in them
@@ -338,10 +351,12 @@ conv_belt_tc_kernel(const ConvPlan P, int block_lo, int n_tiles_k, int ring_lo, 
 
         // fold the accumulator of ring n into the totals, leaving in it the sums' rounding
         // errors and the 2^-24 that the MMAs' cuts cost on average
-        auto drain = [&](uint32_t n) {
+        auto drain = [&](uint32_t n, bool multiplied = true) {
             const uint32_t b = n & 1u;
-            if (!__all_sync(~0u, wait_or_abort(&d_done[b], (n >> 1) & 1u, &s_abort))) return false;
-            tc::fence_after_sync();
+            if (multiplied) {
+                if (!__all_sync(~0u, wait_or_abort(&d_done[b], (n >> 1) & 1u, &s_abort))) return false;
+                tc::fence_after_sync();
+            }
             const uint64_t m1 = pack2(0xbf800000u, 0xbf800000u);  // -1
             const uint64_t cut = pack2(0x33800000u, 0x33800000u);  // 2^-24
             uint32_t v[kStep];
@@ -513,7 +528,13 @@ conv_belt_tc_kernel(const ConvPlan P, int block_lo, int n_tiles_k, int ring_lo, 
             // the previous ring's accumulator while this ring's MMAs run
             if (n_rings >= 2 && !(ok = drain(n_rings - 2))) break;
         }
-        if (ok && n_rings >= 1) ok = drain(n_rings - 1);
+        // the last ring's accumulator, and the folds of the rings after (n_used accumulators are in
+        // use: two, or one after a single ring)
+        const uint32_t n_used = n_rings;
+        for (int i = 0; i <= (kTrim ? s_tail : 0) && n_used > 0 && ok; ++i) {
+            const uint32_t n = n_used - 1u + i;
+            if (i == 0 || (n & 1u) < n_used) ok = drain(n, i == 0);
+        }
         if (s_shift) {  // every builder warp comes here, after an abort too
             wsum -= wcomp;
 #pragma unroll
@@ -533,8 +554,8 @@ conv_belt_tc_kernel(const ConvPlan P, int block_lo, int n_tiles_k, int ring_lo, 
                 uint32_t v0[8], v1[8];
 #pragma unroll
                 for (int e = 0; e < 8; ++e) v0[e] = v1[e] = 0u;
-                if (n_rings >= 1) tmem_ld8(td + c, v0);
-                if (n_rings >= 2) tmem_ld8(td + N + c, v1);
+                if (n_used >= 1) tmem_ld8(td + c, v0);
+                if (n_used >= 2) tmem_ld8(td + N + c, v1);
                 tc::loaded(v0);
                 tc::loaded(v1);
 #pragma unroll
