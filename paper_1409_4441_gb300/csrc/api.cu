@@ -79,6 +79,10 @@ void release(ksc_split *s) {
     cudaFree(s->d_items_mma);
     cudaFree(s->d_ws);
     cudaFree(s->d_items_belt);
+    for (ksc_split::ScratchSlot &c : s->slots) {
+        cudaFree(c.mem);
+        if (c.done) cudaEventDestroy(c.done);
+    }
     cudaFree(s->d_cap_tiles);
     cudaFree(s->d_cap_tiles_lpt);
     cudaFree(s->d_ncut);
@@ -449,6 +453,8 @@ int build_cap_tc(ksc_split *s, const CapPlan &cap, ksc::CapCoef cc) {
     if (too_large) drop_cap_tc(s);
     return KSC_OK;
 }
+
+void make_slots(ksc_split *s);
 
 // Geometry, work list and device table for the real-space part s->c_real.
 int finish_split(ksc_split *s, const ksc_split_opts &o) {
@@ -858,11 +864,12 @@ int finish_split(ksc_split *s, const ksc_split_opts &o) {
         p.belt_c1h = c1.h;
         p.belt_c1l = c1.l;
     }
-    const int rc = plan_belt_tc(s, g, range, pairs, pair_base);
-    if (rc || !plan_cap) return rc;
+    int rc = plan_belt_tc(s, g, range, pairs, pair_base);
     ksc::CapCoef cc{d_ext, d_lo, d_ringc, nullptr, reinterpret_cast<int *>(d_ringc + ringc.size()),
                     n_ext, (float)((double)n_ext * n_ext), {}, {}};
-    return build_cap_tc(s, cap, cc);
+    if (!rc && plan_cap) rc = build_cap_tc(s, cap, cc);
+    if (!rc) make_slots(s);
+    return rc;
 }
 
 int check_common(int lmax, int nside, double theta_cut) {
@@ -899,15 +906,45 @@ int check_maps(const ksc_split *s, const void *a, const void *b) {
     return KSC_OK;
 }
 
-// One convolution call's scratch, from the stream-ordered allocator.
+// One convolution call's scratch: a slot of the split whose last call has ended (the
+// stream-ordered pool gives its memory back at every synchronisation, and a call that follows
+// one pays 0.1 ms for it: a band of nine belt rings runs 0.03 to 0.5 ms), else from the
+// stream-ordered allocator; a captured call's is the graph's own.
 struct CallScratch : ksc::ConvScratch {
     void *mem = nullptr;
     cudaStream_t st = nullptr;
+    const ksc_split *split = nullptr;
+    ksc_split::ScratchSlot *slot = nullptr;
     CallScratch() = default;
     CallScratch(const CallScratch &) = delete;
     CallScratch &operator=(const CallScratch &) = delete;
     ~CallScratch() {
-        if (mem) cudaFreeAsync(mem, st);
+        if (slot) {
+            const cudaError_t e = cudaEventRecord(slot->done, st);
+            std::lock_guard<std::mutex> lk(split->slot_mu);
+            slot->taken = e != cudaSuccess;  // (without its event the slot is not used again)
+        } else if (mem) {
+            cudaFreeAsync(mem, st);
+        }
+    }
+    bool take_slot(const ksc_split *s) {
+        // (another thread's capture in global mode forbids event queries to this one)
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        std::lock_guard<std::mutex> lk(s->slot_mu);
+        for (ksc_split::ScratchSlot &c : s->slots) {
+            if (!c.mem || c.taken) continue;
+            if (cudaEventQuery(c.done) == cudaSuccess) {
+                c.taken = true;
+                split = s;
+                slot = &c;
+                mem = c.mem;
+                break;
+            }
+            cudaGetLastError();  // not ready
+        }
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        return slot != nullptr;
     }
 };
 
@@ -918,14 +955,32 @@ cudaError_t start_scratch(const ksc_split *s, const ksc::MapSet &maps, int n_map
     const size_t bytes = ksc::conv_scratch_bytes(s, n_maps, use);
     if (bytes == 0) return cudaSuccess;
     w->st = st;
-    const cudaError_t e = cudaMallocAsync(&w->mem, bytes, st);
-    if (e != cudaSuccess) {
-        w->mem = nullptr;
-        if (e != cudaErrorMemoryAllocation) return e;
-        cudaGetLastError();
-        return cudaSuccess;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(st, &capture);
+    if (e != cudaSuccess) return e;
+    if (bytes > s->slot_bytes || capture != cudaStreamCaptureStatusNone || !w->take_slot(s)) {
+        e = cudaMallocAsync(&w->mem, bytes, st);
+        if (e != cudaSuccess) {
+            w->mem = nullptr;
+            if (e != cudaErrorMemoryAllocation) return e;
+            cudaGetLastError();
+            return cudaSuccess;
+        }
     }
     return ksc::start_conv_scratch(s, maps, n_maps, use, w->mem, w, st);
+}
+
+// The slots of a split with tensor-core stages (without room for them its calls allocate).
+void make_slots(ksc_split *s) {
+    s->slot_bytes = ksc::conv_scratch_bytes(s, 1, ksc::conv_use(s, 0, s->plan.nrings - 1, true, true));
+    if (s->slot_bytes == 0) return;
+    for (ksc_split::ScratchSlot &c : s->slots) {
+        if (cudaEventCreateWithFlags(&c.done, cudaEventDisableTiming) != cudaSuccess ||
+            dev_malloc(&c.mem, s->slot_bytes) != cudaSuccess) {
+            cudaGetLastError();
+            c.mem = nullptr;
+        }
+    }
 }
 
 // Tensor-core belt stage for a stack of maps; grows the split's pre-tiled map

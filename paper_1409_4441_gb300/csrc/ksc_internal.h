@@ -428,6 +428,15 @@ struct ksc_split {
     float *d_ws = nullptr;                 // pre-tiled map stack (tensor path workspace)
     size_t ws_floats = 0;
     int *d_err = nullptr;                  // device error flag (bounded waits)
+    // scratch of a single map's call with tensor-core stages, for calls that find one free
+    struct ScratchSlot {
+        void *mem = nullptr;
+        cudaEvent_t done = nullptr;        // after the last launch of the call that had it
+        bool taken = false;                // by a call that is launching
+    };
+    mutable ScratchSlot slots[2];
+    mutable std::mutex slot_mu;
+    size_t slot_bytes = 0;
     ksc::BeltTc btc;                       // tensor-core belt stage (n_cols 0: not used)
     ksc::CapTc ctc;                        // tensor-core cap stage (ring_end < ring_first: not used)
     int2 *d_cap_tiles = nullptr;           // its tiles in ring order ...
