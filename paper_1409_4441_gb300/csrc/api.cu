@@ -732,6 +732,7 @@ int finish_split(ksc_split *s, const ksc_split_opts &o) {
                          [&](int a, int b) { return cap.cost[a] > cap.cost[b]; });
         for (int i : order) cap.tiles_lpt.push_back(cap.tiles[i]);
         s->n_cap_tiles = (int)cap.tiles.size();
+        s->cap_tile_us = cap.cost;
         s->cap_tile_first.assign(nr + 1, 0);
         size_t i = 0;
         for (int r = 0; r <= nr; ++r) {
@@ -1187,9 +1188,11 @@ cudaError_t launch_caps(const ksc_split *s, const MapSet &maps, int n_maps, int 
     // (a tile holds rings r and r + 1: from the one that may start just before lo)
     const int t0 = whole ? 0 : s->cap_tile_first[std::max(lo - 1, 0)];
     const int t1 = whole ? s->n_cap_tiles : s->cap_tile_first[hi + 1];
+    // a band's tiles in ring order, from the end that takes longer
+    const bool back = !whole && t1 > t0 && s->cap_tile_us[t1 - 1] > s->cap_tile_us[t0];
     cudaError_t e = launch_conv_cap_tc(
         s->plan, s->ctc, whole ? s->d_cap_tiles_lpt : s->d_cap_tiles + t0, t1 - t0, maps,
-        n_maps, belt_split, r0, r1, w.ranges, w.cap_flags, !whole, d_err, st);
+        n_maps, belt_split, r0, r1, w.ranges, w.cap_flags, back, d_err, st);
     if (e != cudaSuccess) return e;
     const int i0 = s->irr_item_first[lo], i1 = s->irr_item_first[hi + 1];
     e = launch_cap_direct(s->plan, s->d_irr_items + i0, i1 - i0, s->d_irr_first, s->d_irr,

@@ -28,7 +28,7 @@
 //
 // Precision as in conv_belt_tc.cu: two FP16 parts of map and weights (23 bits of the 24), w_h
 // m_h in one FP32 accumulator, w_h m_l + w_l m_h in a second one, with w_l m_l and a third
-// part of c_0 times m_h in the step of the closest approach, where the weights are large; for
+// part of c_0 times m_h (near rings) in the step of the closest approach, where the weights are large; for
 // p = 6, 7, 8 (coefficients below 2^-12 of the peak, which the host checks) w_h m_h alone; far chunks first.  The polynomial and the
 // pixels of the two cells that the cut divides (at most one pixel a side, tested with the
 // exact integers) are in FP32; the rounding errors of a ring's last sum and of the sum over
@@ -84,6 +84,7 @@ constexpr int kTurn = 32 * 10;     // float2 of a warp's turning buffer (10 per 
 // two groups of two core matrices a ring pair
 constexpr int kE = 13;
 constexpr int kEBytes = 2 * 2 * kLead;
+constexpr int kNear = 12;  // input rings this near the output rings have them
 constexpr int kXr = 7;             // staged elements of a builder thread and hemisphere
 
 using tc::Window;
@@ -173,7 +174,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ tiles,
                    const MapSet maps,
                    int belt_split, int band_lo, int band_hi, const uint2 *__restrict__ ring_range,
-                   int *__restrict__ flags, int ring_order, int *__restrict__ err) {
+                   int *__restrict__ flags, int back, int *__restrict__ err) {
     extern __shared__ __align__(1024) unsigned char smem[];
     // B stages | third parts of c_0 [buffer] | map segments [h][buffer][part] | turning buffers | totals (north, south:
     // sums, compensations) [ring] | the segments as they are, (north, south) [buffer] |
@@ -199,8 +200,7 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
     __shared__ float s_edge[2][2][kP + 3], s_sum[2][2][kP];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // (a band's tiles come in ring order: the longer rings, which take longer, first)
-    const int2 tile = tiles[ring_order ? gridDim.x - 1 - blockIdx.x : blockIdx.x];
+    const int2 tile = tiles[back ? gridDim.x - 1 - blockIdx.x : blockIdx.x];
     const int r0 = tile.x & 0xffff, n_r = (tile.x >> 16) + 1;
     const int sector = tile.y & 0xffff, n_sec = tile.y >> 16;
     const bool add = belt_split && r0 >= P.belt_lo;
@@ -416,8 +416,9 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
                         if (c == mid && s_c >= 0 && s_c < t1 - t0) {
                             tc::mma_f16(d, da + (uint32_t)(2 * s_c) + a_l,
                                         db + (uint32_t)(s_c * (2 * kLead / 16)) + b_l, idesc, acc);
-                            tc::mma_f16(d, da + (uint32_t)(2 * s_c), e_base + (n & 1u) * (kEBytes >> 4),
-                                        tc::idesc_f16(128, 16), 1u);
+                            if (abs(q_lo + qi - r0) <= kNear)
+                                tc::mma_f16(d, da + (uint32_t)(2 * s_c), e_base + (n & 1u) * (kEBytes >> 4),
+                                            tc::idesc_f16(128, 16), 1u);
                             acc = 1u;
                         }
 #pragma unroll
@@ -726,7 +727,7 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
                     }
                     // third parts of c_0 in the closest approach's step: a thread's element e of
                     // row i in core matrix kg of ring R (base counts Delta from step s0)
-                    {
+                    if (abs(q_lo + qi - r0) <= kNear) {
                         const int e = bt & 7, i = (bt >> 3) & 7, kg = (bt >> 6) & 1, R = bt >> 7;
                         const int dl = g.base + 16 * (kSteps * g.mid + kSteps / 2 - g.s0) + 8 * kg + e - i;
                         const int j = dl < 0 ? -dl : dl, jE = g.jE[R];
@@ -1084,7 +1085,7 @@ cudaError_t launch_cap_direct(const ConvPlan &p, const int2 *d_items, int n_item
 
 cudaError_t launch_conv_cap_tc(const ConvPlan &p, const CapTc &c, const int2 *d_tiles, int n_tiles,
                                const MapSet &maps, int n_maps, int belt_split, int band_lo,
-                               int band_hi, const uint2 *rr, int *flags, bool ring_order,
+                               int band_hi, const uint2 *rr, int *flags, bool back,
                                int *d_err, cudaStream_t st) {
     if (n_tiles <= 0) return cudaSuccess;
     const size_t smem = cap_smem(c);
@@ -1094,7 +1095,7 @@ cudaError_t launch_conv_cap_tc(const ConvPlan &p, const CapTc &c, const int2 *d_
     if (e != cudaSuccess) return e;
     dim3 grid(n_tiles, n_maps);
     conv_cap_tc_kernel<<<grid, kThreads, smem, st>>>(p, c, d_tiles, maps, belt_split, band_lo,
-                                                     band_hi, rr, flags, ring_order, d_err);
+                                                     band_hi, rr, flags, back, d_err);
     return cudaGetLastError();
 }
 

@@ -285,10 +285,11 @@ cudaError_t launch_ring_range(const ConvPlan &p, const unsigned *bm, int n_maps,
                               const InputReach &in, uint2 *rr, cudaStream_t st);
 // Writes (adds, for belt rings with belt_split) the tiles' outputs in rings [band_lo,
 // band_hi] but for the ring pairs it flags (flags[map][ring], flags[map][nrings]: any),
-// which conv_sym_kernel then computes; flags must be zero at launch.
+// which conv_sym_kernel then computes; flags must be zero at launch.  back: the tiles from the
+// last one on.
 cudaError_t launch_conv_cap_tc(const ConvPlan &p, const CapTc &c, const int2 *d_tiles, int n_tiles,
                                const MapSet &maps, int n_maps, int belt_split, int band_lo,
-                               int band_hi, const uint2 *rr, int *flags, bool ring_order,
+                               int band_hi, const uint2 *rr, int *flags, bool back,
                                int *d_err, cudaStream_t st);
 
 // tcgen05 multi-map kernel for belt ring pairs: items are (belt ring, first
@@ -442,6 +443,7 @@ struct ksc_split {
     int2 *d_cap_tiles = nullptr;           // its tiles in ring order ...
     int2 *d_cap_tiles_lpt = nullptr;       // ... and longest first (whole map)
     int n_cap_tiles = 0;
+    std::vector<double> cap_tile_us;       // about its time on an SM, per tile in ring order
     std::vector<int> cap_tile_first;       // per ring: first tile of rings >= it (nrings + 1)
     int *d_ncut = nullptr;
     unsigned *d_coef_off = nullptr, *d_coef = nullptr;

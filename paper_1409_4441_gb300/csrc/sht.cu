@@ -252,10 +252,17 @@ __global__ void __launch_bounds__(256)
 sht_leg_synth(int nside, int lmax, float extra, const double2 *__restrict__ alm, float2 *__restrict__ G) {
     __shared__ float4 co[kTile], al[kTile];
     __shared__ F2 s_norm;
-    __shared__ int s_top;
+    __shared__ int s_top[8];
     const int m = blockIdx.y, nnorth = 2 * nside, nr = 4 * nside - 1;
     const int r = blockIdx.x * 256 + threadIdx.x, rs = nr - 1 - r;
-    if (threadIdx.x == 0) s_top = 0;
+    const double2 *a = alm + alm_base(lmax, m);
+    int top = 0;  // largest |re|, |im| of the order's coefficients
+    for (int l = m + threadIdx.x; l <= lmax; l += 256) {
+        const double2 c = __ldg(a + l);
+        top = max(top, max(__double2hiint(fabs(c.x)), __double2hiint(fabs(c.y))));
+    }
+    top = __reduce_max_sync(~0u, top);
+    if ((threadIdx.x & 31) == 0) s_top[threadIdx.x >> 5] = top;
     if (threadIdx.x < 32) {
         const F2 v = norm_mm(m);
         if (threadIdx.x == 0) s_norm = v;
@@ -271,16 +278,9 @@ sht_leg_synth(int nside, int lmax, float extra, const double2 *__restrict__ alm,
         if (live) rec.start(m, s_norm, z, s);
     }
     if (!__syncthreads_or(live)) return;
-    const double2 *a = alm + alm_base(lmax, m);
-    int top = 0;  // largest |re|, |im| of the order's coefficients
-    for (int l = m + threadIdx.x; l <= lmax; l += 256) {
-        const double2 c = __ldg(a + l);
-        top = max(top, max(__double2hiint(fabs(c.x)), __double2hiint(fabs(c.y))));
-    }
-    top = __reduce_max_sync(~0u, top);
-    if ((threadIdx.x & 31) == 0) atomicMax(&s_top, top);
-    __syncthreads();
-    const int ex = scale_exp_f64(s_top);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) top = max(top, s_top[i]);
+    const int ex = scale_exp_f64(top);
     const double up = pow2(ex);
     for (int l0 = m; l0 <= lmax; l0 += kTile) {
         const int n = min(kTile, lmax + 1 - l0);
@@ -339,7 +339,7 @@ sht_leg_anal(int nside, int lmax, float extra, const float2 *__restrict__ F, con
     extern __shared__ double2 acc[];  // [lmax + 1 - m]
     __shared__ float4 co[kTile], term[8][8][33], part[8][kGroup];
     __shared__ F2 s_norm;
-    __shared__ unsigned s_top;
+    __shared__ unsigned s_top[8];
     const int m = lmax - blockIdx.x, nnorth = 2 * nside, nr = 4 * nside - 1;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long stride = lmax + 1;
@@ -355,8 +355,6 @@ sht_leg_anal(int nside, int lmax, float extra, const float2 *__restrict__ F, con
         float4 f[R];                    // north, south
         bool live[R], any = false;
         unsigned top = 0u;
-        if (threadIdx.x == 0) s_top = 0u;
-        __syncthreads();
 #pragma unroll
         for (int j = 0; j < R; ++j) {
             const int r = base + 256 * j + threadIdx.x;
@@ -378,9 +376,11 @@ sht_leg_anal(int nside, int lmax, float extra, const float2 *__restrict__ F, con
             any |= live[j];
         }
         top = __reduce_max_sync(~0u, top);
-        if (lane == 0) atomicMax(&s_top, top);
-        if (!__syncthreads_or(any)) continue;
-        const int ex = scale_exp_f32(s_top);
+        if (lane == 0) s_top[warp] = top;
+        if (!__syncthreads_or(any)) continue;  // (else barriers follow before the next pass writes)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) top = max(top, s_top[i]);
+        const int ex = scale_exp_f32(top);
         const float scale = __int_as_float((127 + ex) << 23);
 #pragma unroll
         for (int j = 0; j < R; ++j) {
