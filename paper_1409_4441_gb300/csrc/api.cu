@@ -401,7 +401,7 @@ void plan_cap_tc(ksc_split *s, const ksc_split_opts &o, const ksc::RingGeom &g,
             us += 0.66 + 0.020 * g.len[plan->irr[e]];
         direct.push_back(us);
     }
-    if (makespan(plan->cost, kSms) + makespan(direct, kSms) > 0.95 * gather_us) {
+    if (makespan(plan->cost, kSms) + makespan(direct, kSms) > gather_us) {
         plan->tiles.clear();
         return;
     }
