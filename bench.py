@@ -50,10 +50,9 @@ UNIT = "pairs/s"
 N_SM = 152
 FP32_LANES_PER_SM = 128
 # DRAM bytes per launch of the dominant kernel at the nside-2048 workload, from one ncu
-# capture of the current kernel (dram__bytes_read.sum + dram__bytes_write.sum, full launch);
-# absent until the current kernel has been captured (the last capture, 291 MB, predates the
-# kernel's present accumulation scheme)
-DRAM_TRAFFIC = {}
+# capture (dram__bytes_read.sum + dram__bytes_write.sum, full launch): the stage's coefficients,
+# 2.4 GB, then the map in and out; the gather (option exact_weights) is not captured
+DRAM_TRAFFIC = {"conv_cap_tc_kernel": 2.68e9 + 0.202e9}
 
 
 def step_kernels(K, sp, opts):
@@ -556,10 +555,10 @@ def run_ours(args, world, rank, local):
                              "peak = 152 SMs x 128 FP32 lanes x 2 x max SM clock (the FP32 "
                              "pipe that the paper's formulation uses; the belt and cap "
                              "stages run on the tensor cores, two-part FP16 products with "
-                             "FP32 sums, so a stage may exceed it).  The cap stage is bound "
-                             "by shared-memory bandwidth: operand reads of N = 144 MMAs and "
-                             "the turning of their accumulators (ncu: tensor pipe 17%, issue "
-                             "52%)"},
+                             "FP32 sums, so a stage may exceed it).  In the cap stage operand "
+                             "reads of N = 144 MMAs and the turning of their accumulators "
+                             "share shared memory, and warps wait for tensor-memory loads "
+                             "(ncu: LSU wavefronts 58%, issue 49%, tensor pipe 23%)"},
         "target": {"roofline_frac": 0.5, "met": bool(achieved / peak_tflops >= 0.5),
                    "step_frac": 2.0 * n_pairs / statistics.mean(launch_ms) * 1e3 / 1e12
                    / peak_tflops},

@@ -112,17 +112,24 @@ typedef struct {
                           1: every weight from the double-float chord and
                           the K_r table                                      */
     int cap_kernel;    /* single maps and stacks of fewer than 16 maps: which
-                          kernel sums the cap ring pairs.  0 (default): from
-                          8e9 pairs with a cap ring on (5e10 where the gather
-                          keeps three CTAs per SM), nside 64..4096, unless
-                          exact_weights is set, the tcgen05 tensor cores on
-                          two-part FP16 values and per-cell polynomials of the
-                          weights (coefficients laid out with the split, 2.4
-                          GB at nside 2048 with a 240' cut, at most 8 GB;
-                          output rings whose input spans more than 2^14 in
-                          magnitude or is not finite go to the gather); else
-                          FP32 FFMAs, one or three reflection classes per
-                          thread sharing each staged image value; 1: the
+                          kernel sums the cap ring pairs.  0 (default): the
+                          tcgen05 tensor cores on two-part FP16 values and
+                          per-cell polynomials of the weights, where that is
+                          estimated to be faster (nside 64..4096, from 8e9
+                          pairs with a cap ring on, 5e10 where the gather
+                          keeps three CTAs per SM; not for windows of a few
+                          tens of pixels, nor where they need more shared
+                          memory than an SM has), the polynomials carry the
+                          kernel (beams of about three pixels up or l_max up
+                          to 2 nside; no kernel that peaks past its cut),
+                          exact_weights is not set and their coefficients,
+                          laid out with the split (2.4 GB at nside 2048 with
+                          a 240' cut), take at most 8 GB and an eighth of
+                          the free device memory; output rings whose input
+                          spans more than 2^14 in magnitude or is not finite
+                          go to the gather; else FP32 FFMAs, one or three
+                          reflection classes per thread sharing each staged
+                          image value.  ksc_split_stages says which; 1: the
                           tcgen05 tensor
                           cores, each weight and map value split exactly into
                           three BF16 parts and six MMAs per 16 positions
@@ -223,11 +230,13 @@ int ksc_split_table(const ksc_split *s, float *host_coeffs);
  * out = real-space convolution of `in` with the split's K_r (both device
  * arrays of 12 nside^2 floats, nside as given to the split; in != out).
  * Asynchronous on `stream`.  Each call takes its scratch (work-claim counters;
- * with the tensor-core stages, from 8e8 belt pairs on, also npix / 16 bytes a map
- * of block maxima, and flags; without room for these the FFMA kernels run) from
- * the device's default stream-ordered memory pool
- * (cudaMallocAsync / cudaFreeAsync on `stream`), so calls on several streams
- * may overlap and a call captured into a CUDA graph holds its own scratch.
+ * with the tensor-core stages, taken from 8e8 belt pairs on where they are
+ * estimated to be clearly faster, also npix / 16 bytes a map of block maxima, and
+ * flags; without room for these the FFMA kernels run) from the device's default
+ * stream-ordered memory pool (cudaMallocAsync / cudaFreeAsync on `stream`), or from
+ * one of two sets that the split keeps, if the call that had it last has ended; so
+ * calls on several streams may overlap and a call captured into a CUDA graph holds
+ * its own scratch.
  * Errors: KSC_ERR_ARG, KSC_ERR_CUDA.
  */
 int ksc_conv_real(const ksc_split *s, const float *d_in, float *d_out,
@@ -468,8 +477,8 @@ int ksc_build_table_noalloc(const double *d_c, int lmax, double theta_cut,
  * Legendre functions without the Condon-Shortley phase.  a_lm are complex
  * doubles (re, im interleaved) in m-major order: index(l, m) = m (2 lmax + 1 - m)
  * / 2 + l, m = 0..lmax, l = m..lmax; (lmax + 1)(lmax + 2) / 2 entries.
- * Legendre recurrences and sums on FP32 pairs (48 bits, scaled against underflow
- * near the poles), ring sums in FP32 (FFT on the belt of larger maps, else quarter sums).  Device pointers; asynchronous on `stream`; scratch from the
+ * Legendre recurrences and sums on FP32 pairs (48 bits; functions scaled against underflow
+ * near the poles, coefficients and ring sums against FP32's range), ring sums in FP32 (FFT on the belt of larger maps, each ring its own; else quarter sums).  Device pointers; asynchronous on `stream`; scratch from the
  * stream-ordered allocator.  nside a power of two <= 8192, 0 <= lmax <= 4 nside.
  * Errors: KSC_ERR_ARG, KSC_ERR_NOMEM, KSC_ERR_CUDA.
  */

@@ -38,7 +38,7 @@
 // 0.87 / 0.94 / 0.78 (stage at 2048, 240': 105.8 -> 107.4 ms).
 //
 // The coefficients c_p[j] depend on the ring pair alone and are laid out once per split
-// (cap_coef_kernel: 18.6 ms and 2.4 GB at nside 2048 with a 240' cut); evaluated inside
+// (cap_coef_kernel: 20 ms and 2.4 GB at nside 2048 with a 240' cut); evaluated inside
 // this kernel they took half of its instructions, for every sector again.
 //
 // Ring pairs near the poles whose window is the whole ring or close to it, and input rings of
@@ -88,6 +88,9 @@ constexpr int kNear = 12;  // input rings this near the output rings have them
 constexpr int kXr = 7;             // staged elements of a builder thread and hemisphere
 
 using tc::Window;
+using tc::add2;
+using tc::fma2;
+using tc::pack2;
 __host__ __device__ __forceinline__ Window window_of(int w, int L) {
     return tc::tile_window<kChunk>(w, L);
 }
@@ -99,20 +102,6 @@ __host__ __device__ constexpr float node(int s) {
            : s == 3 ? 443.0f / 1024 : 504.0f / 1024;
 }
 
-// Two FP32 values in one register pair.
-__device__ __forceinline__ uint64_t pack2(float a, float b) {
-    return (uint64_t)__float_as_uint(b) << 32 | __float_as_uint(a);
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-    uint64_t d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-    uint64_t d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
 
 // a + b and its rounding error.
 __device__ __forceinline__ uint64_t two_sum2(uint64_t a, uint64_t b, uint64_t *err) {
@@ -886,7 +875,8 @@ cap_coef_kernel(const ConvPlan P, const CapTc C, const CapCoef K, int ring_lo, i
 // The irregular ring pairs of output ring r (and its mirror), added to the output.  A block
 // takes 32 first-quarter positions of r, a lane each; its sixteen warps share the ring's list
 // of input rings (99 blocks for 152 SMs at nside 1024, 160': 330 us with eight warps, 281 us
-// with sixteen; 612 blocks at 2048, 240': 6.60 and 6.47 ms).  For one input pixel all lanes
+// with sixteen; 612 blocks at 2048, 240': 6.47 ms, and 5.0 with weights and products inside the
+// cut only; two blocks per SM, at 64 registers: slower).  For one input pixel all lanes
 // read the same values, eight (four quarter turns, two hemispheres) per weight.
 constexpr int kDirect = 512;
 // input pixels between folds into the compensated sums: nside 256, 1800': error rms 9.2e-8 of

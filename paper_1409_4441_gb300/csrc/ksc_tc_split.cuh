@@ -14,6 +14,24 @@ namespace tc {
 constexpr int kXExp = 14;           // a tile's largest |m| is scaled into [2^14, 2^15)
 constexpr uint32_t kRangeExp = 14;  // a block may lie this many powers of two below it
 
+// Two FP32 values in one register pair.
+__device__ __forceinline__ uint64_t pack2(uint32_t a, uint32_t b) {
+    return (uint64_t)b << 32 | a;
+}
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+    return pack2(__float_as_uint(a), __float_as_uint(b));
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
 // K-major, no swizzle: 8-row x 16-byte core matrices; lead = bytes between core matrices
 // adjacent in K, stride = bytes between groups of eight rows.
 __device__ __forceinline__ uint64_t desc(uint32_t addr, uint32_t lead, uint32_t stride) {

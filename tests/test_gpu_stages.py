@@ -224,3 +224,31 @@ def test_calls_share_the_scratch_of_a_split(K):
         torch.cuda.synchronize()
         K.device_status(sp)
         assert torch.equal(got, want) and torch.equal(stack, want)
+
+
+# (nside, cut in arcmin, columns of the belt tiles, cap stage): each width that a plan takes, short and
+# long windows
+@pytest.mark.parametrize("nside,theta,columns,cap", [(128, 2400.0, 32, 0), (256, 660.0, 32, 0), (256, 1800.0, 32, 1),
+                                                     (512, 240.0, 128, 0), (512, 640.0, 128, 1),
+                                                     (1024, 60.0, 256, 0), (1024, 400.0, 256, 1)])
+def test_stages_match_the_oracle(K, nside, theta, columns, cap):
+    """First and last pixels of the first, sixteenth, seventeenth and last belt rings, the poles, both
+    sides of the cap boundaries, and random pixels."""
+    sp, c = _split(K, nside, theta)
+    tc = theta * inputs.ARCMIN
+    m = inputs.white_noise_map(nside, 17).astype(np.float32)
+    x = torch.tensor(m, device="cuda")
+    y = torch.full_like(x, float("nan"))
+    with sp:
+        st = K.split_stages(sp)
+        assert (st["belt_columns"], st["cap_stage"]) == (columns, cap)
+        K.conv_real(sp, x, y)
+        K.device_status(sp)
+        tab = O.hermite_nodes(c, tc, K.split_info(sp)["n_intervals"])
+    first, L, N = 2 * nside * (nside - 1), 4 * nside, 12 * nside * nside
+    edge = [first + r * L + k for r in (0, 15, 16, nside, 2 * nside - 1, 2 * nside) for k in (0, 7, 8, L - 1)]
+    pix = np.unique(np.concatenate([edge, np.arange(24), N - 1 - np.arange(24), np.arange(40) + first - 20,
+                                    inputs.rng(18).choice(N, 500, replace=False)]))
+    ref, amb = O.brute_conv(nside, m.astype(np.float64), tc, table=tab, out_pix=pix)
+    err = np.abs(y.cpu().numpy()[pix] - ref) - amb
+    assert err.max() <= 1e-6 * np.sqrt(np.mean(ref ** 2))
