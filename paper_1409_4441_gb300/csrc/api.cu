@@ -119,7 +119,10 @@ bool cap_polynomials_ok(const ksc_split *s, double top) {
     // 4 J_{n+1}(l h / 2) ~ 4 (l h / 4)^{n+1} / (n+1)!, h the largest pixel step (1.2826 / nside
     // at the poles).  The coefficients that are multiplied in one part, c_p f^p for p >= n1,
     // |f| <= 1/2, amount to about (l h / 4)^p / (p/2)!^2 of a term (the p-th derivative of
-    // J_0): one FP16 part keeps them to 2^-12.
+    // J_0); one FP16 part keeps them to 2^-12 of themselves.  Error rms of cap pixels, 1e-7 of the
+    // output's, stage / gather, nside 512, 640': l_max 2 nside, 3 pixels (2^-12.9 of the peak): 0.71 /
+    // 1.01; 3 nside, 3 pixels (2^-11.8): 0.71 / 1.02; 2 nside, 2.5 pixels, upper half of the degrees
+    // only (2^-11.3): 1.09 / 0.99.
     const int n = ksc::cap_tc_degree(), n1 = ksc::cap_tc_split_powers();
     double err = 0.0, single = 0.0, fact = 1.0, half = 1.0;
     for (int i = 2; i <= n + 1; ++i) fact *= i;
@@ -130,7 +133,7 @@ bool cap_polynomials_ok(const ksc_split *s, double top) {
         single += a * std::pow(x, n1) / (half * half);
     }
     const double peak = 4.0 * kPi * top;
-    return err <= 5e-8 * peak && single <= std::ldexp(peak, -12);
+    return err <= 5e-8 * peak && single <= std::exp2(-11.5) * peak;
 }
 
 // Plan of the tensor-core belt stage: the widest window and the most input rings of a
@@ -182,9 +185,9 @@ int plan_belt_tc(ksc_split *s, const ksc::RingGeom &g, const std::vector<int2> &
     // A tile spends 2.2 (32 columns) to 3.5 us (256) on an input ring whose window has up to 150
     // positions, and a band of a few rings, which takes the same kernel for the same bits, pays
     // that for sixteen rings.  So only where the whole map's stage takes at most 0.7 of the FFMA
-    // kernel's time; estimate and measured ratio: nside 256, 32 and 48 pixels 0.76 / 0.77 and 0.63 /
-    // 0.66; 512, 16 and 24: 0.77 / 0.77 and 0.61 / 0.62; 1024, 8 and 12: 0.74 / 0.71 and 0.65 / 0.64;
-    // 2048, 4 and 8: 0.89 / 0.78 and 0.67 / 0.66.
+    // kernel's time; estimate and measured ratio: nside 128, 96 pixels 0.71 / 0.65; 256, 32 and 48
+    // pixels 0.79 / 0.77 and 0.66 / 0.66; 512, 16 and 24: 0.78 / 0.77 and 0.60 / 0.62; 1024, 8 and 16: 0.79 /
+    // 0.71 and 0.55 / 0.55; 2048, 8 and 16: 0.72 / 0.66 and 0.49 / 0.51.
     double ffma = 0.0;
     for (int r = lo; r <= hi; ++r) {
         int rings = 0;
@@ -193,7 +196,8 @@ int plan_belt_tc(ksc_split *s, const ksc::RingGeom &g, const std::vector<int2> &
         const int items = (g.len[r] + ksc::belt_chunk() - 1) / ksc::belt_chunk();
         ffma += items * (0.47 * rings + 0.0108 * s->cost_belt[r]);
     }
-    ffma *= (s->n_items_belt <= 4 * kSms ? 1.3 : 1.0) / kSms;
+    const int waves = (s->n_items_belt + kSms - 1) / kSms;  // fewer items leave SMs short of CTAs
+    ffma *= (waves <= 1 ? 3.0 : waves <= 2 ? 1.8 : waves <= 4 ? 1.25 : waves <= 8 ? 1.1 : 0.93) / kSms;
     const int n = s->btc.n_cols;
     const double step = (n >= 256 ? 3.5 : n >= 128 ? 2.9 : n >= 64 ? 2.5 : 2.2) + 0.013 * std::max(wpos - 150, 0);
     const double tensor = std::ceil(ksc::belt_tc_tiles(s->plan, s->btc) / (double)kSms) * nq * step;

@@ -14,7 +14,7 @@
 // the degree-8 interpolant is within 2e-9 of the kernel's peak (4e-9 at l_max = 3 nside); c_p
 // falls off as the derivatives do: for a beam of three pixels at l_max = 2 nside c_6 / 2^6 is
 // 2^-12.7 of the peak, c_8 / 2^8 about 2e-6.  The host bounds both, and a split beyond the
-// bounds (such a beam with l_max = 3 nside, a kernel that peaks past its cut) has no cap stage.
+// bounds (2.7 pixels with l_max = 3 nside, a kernel that peaks past its cut) has no cap stage.
 //
 // A CTA owns two adjacent rings and their southern mirrors (which share every weight) over
 // one sector of longitude.  Per input ring:
@@ -29,7 +29,7 @@
 // Precision as in conv_belt_tc.cu: two FP16 parts of map and weights (23 bits of the 24), w_h
 // m_h in one FP32 accumulator, w_h m_l + w_l m_h in a second one, with w_l m_l and a third
 // part of c_0 times m_h (near rings) in the step of the closest approach, where the weights are large; for
-// p = 6, 7, 8 (coefficients below 2^-12 of the peak, which the host checks) w_h m_h alone; far chunks first.  The polynomial and the
+// p = 6, 7, 8 (coefficients below 2^-11.5 of the peak, which the host checks) w_h m_h alone; far chunks first.  The polynomial and the
 // pixels of the two cells that the cut divides (at most one pixel a side, tested with the
 // exact integers) are in FP32; the rounding errors of a ring's last sum and of the sum over
 // input rings are carried along.  Error rms of cap pixels against 64 bits, over the output
@@ -126,12 +126,12 @@ __device__ __forceinline__ void copy16(void *dst, const void *src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tc::saddr(dst)), "l"(src) : "memory");
 }
 
-struct QInfo {      // an input ring as the tile sees it
-    int n0;         // first position (input pixel) of row 0
-    int eR[2];      // rem <= eR: the right edge cell's pixel lies within the cut
+struct QInfo {      // an input ring as the tile sees it (shorts: the cut's width is bound by their memory)
     uint32_t off[2];  // first coefficient word of each ring, in units of four
-    int start[2];   // first pixel of the ring and of its mirror
-    int a;          // ring pixel of element 0 of the staged segments
+    int start;      // first pixel of the ring
+    short n0;       // first position (input pixel) of row 0
+    short eR[2];    // rem <= eR: the right edge cell's pixel lies within the cut
+    short a;        // ring pixel of element 0 of the staged segments
     short len, phase;  // of the input ring
     short n_e;      // elements staged
     short base;     // d0 + 16 s0: Delta of element 0 at offset i = 0
@@ -240,7 +240,7 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
             const int ncut = C.d_ncut[ip], L = R ? L1 : L0;
             if (ncut < 0) continue;
             g.jE[R] = ncut >= L ? (short)((ncut - L) / (2 * L) + 1) : 0;
-            g.eR[R] = ncut - 2 * L * g.jE[R];
+            g.eR[R] = (short)(ncut - 2 * L * g.jE[R]);
             g.off[R] = C.d_coef_off[ip];
         }
         const int w = max((int)g.jE[0], (int)g.jE[1]);
@@ -257,11 +257,10 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
             lo = min(lo, pos(k_lo1, Rb.phase, L1));
             hi = max(hi, pos(k_hi1, Rb.phase, L1));
         }
-        g.n0 = lo;
+        g.n0 = (short)lo;
         g.len = (short)Q.len;
         g.phase = (short)Q.phase;
-        g.start[0] = Q.start;
-        g.start[1] = P.d_rings[P.nrings - 1 - q].start;
+        g.start = Q.start;
         if (w >= 0) {
             const Window v = window_of(w, Q.len);
             g.s0 = (short)v.s0;
@@ -269,8 +268,8 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
             g.mid = (short)v.mid;
             g.base = (short)(v.d0 + 16 * v.s0);
             g.n_e = (short)(((hi - lo + 8) & ~7) + 16 * (v.s1 - v.s0));
-            g.a = (lo + g.base) % Q.len;
-            g.a += g.a < 0 ? Q.len : 0;
+            const int a = (lo + g.base) % Q.len;
+            g.a = (short)(a < 0 ? a + Q.len : a);
             // sized by the host for every tile: never expected
             if (16 * (v.s1 - v.s0) > C.wpos || w + 1 > C.jcap || hi - lo + 1 > C.span ||
                 g.n_e > kXr * kBuild || hi < lo || 2 * w + 1 > Q.len)
@@ -332,7 +331,7 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
             for (int j = 0; j < 4; ++j) {
                 int k = g.a + (4 * lane + j) * g.n_e / 128;
                 while (k >= g.len) k -= g.len;
-                v += __ldg(m + g.start[h] + k);
+                v += __ldg(m + (h ? P.npix - g.start - g.len : g.start) + k);
             }
 #pragma unroll
             for (int s = 16; s > 0; s >>= 1) v += __shfl_xor_sync(~0u, v, s);
@@ -635,7 +634,7 @@ conv_cap_tc_kernel(const ConvPlan P, const CapTc C, const int2 *__restrict__ til
             // loads of an input ring: segments into registers, coefficients by async copies
             auto fetch = [&](int qi, uint32_t m_) {
                 const QInfo g = sQ[qi];
-                const float *rn = m + g.start[0], *rs = m + g.start[1];
+                const float *rn = m + g.start, *rs = m + (P.npix - g.start - g.len);
 #pragma unroll
                 for (int e = 0; e < kXr; ++e) {
                     if (bt + e * kBuild >= g.n_e) break;
