@@ -120,8 +120,9 @@ typedef struct {
                           keeps three CTAs per SM; not for windows of a few
                           tens of pixels, nor where they need more shared
                           memory than an SM has), the polynomials carry the
-                          kernel (beams of about three pixels up or l_max up
-                          to 2 nside; no kernel that peaks past its cut),
+                          kernel (beams from 2.5 pixels at l_max = 3 nside,
+                          from 2 at 2 nside, splits from somewhat more; no
+                          kernel that peaks past its cut),
                           exact_weights is not set and their coefficients,
                           laid out with the split (2.4 GB at nside 2048 with
                           a 240' cut), take at most 8 GB and an eighth of

@@ -14,7 +14,7 @@
 // the degree-8 interpolant is within 2e-9 of the kernel's peak (4e-9 at l_max = 3 nside); c_p
 // falls off as the derivatives do: for a beam of three pixels at l_max = 2 nside c_6 / 2^6 is
 // 2^-12.7 of the peak, c_8 / 2^8 about 2e-6.  The host bounds both, and a split beyond the
-// bounds (2.7 pixels with l_max = 3 nside, a kernel that peaks past its cut) has no cap stage.
+// bounds (2.4 pixels with l_max = 3 nside, a kernel that peaks past its cut) has no cap stage.
 //
 // A CTA owns two adjacent rings and their southern mirrors (which share every weight) over
 // one sector of longitude.  Per input ring:
@@ -29,7 +29,7 @@
 // Precision as in conv_belt_tc.cu: two FP16 parts of map and weights (23 bits of the 24), w_h
 // m_h in one FP32 accumulator, w_h m_l + w_l m_h in a second one, with w_l m_l and a third
 // part of c_0 times m_h (near rings) in the step of the closest approach, where the weights are large; for
-// p = 6, 7, 8 (coefficients below 2^-11.5 of the peak, which the host checks) w_h m_h alone; far chunks first.  The polynomial and the
+// p = 6, 7, 8 (coefficients below 2^-10.5 of the peak, which the host checks) w_h m_h alone; far chunks first.  The polynomial and the
 // pixels of the two cells that the cut divides (at most one pixel a side, tested with the
 // exact integers) are in FP32; the rounding errors of a ring's last sum and of the sum over
 // input rings are carried along.  Error rms of cap pixels against 64 bits, over the output

@@ -86,8 +86,8 @@ def _legendre(lmax, z):
 
 
 def test_cap_stage_takes_kernels_that_its_polynomials_carry(K):
-    """At one nside and cut: a beam of three pixels with l_max = 2 nside and 3 nside; one of 2.7
-    pixels with l_max = 3 nside, whose sixth-order coefficients are above the 2^-11.5 of the peak
+    """At one nside and cut: a beam of three pixels with l_max = 2 nside and 3 nside; one of 2.2
+    pixels with l_max = 3 nside, whose sixth-order coefficients are above the 2^-10.5 of the peak
     that one FP16 part may serve; a ring of 2.5 pixels FWHM five pixels past the cut, of which the interpolation keeps
     5e-6 of what lies within."""
     nside, tc = 512, 640.0 * inputs.ARCMIN
@@ -95,7 +95,7 @@ def test_cap_stage_takes_kernels_that_its_polynomials_carry(K):
     ring = inputs.gaussian_beam(2 * nside, 2.5 * pixel) * _legendre(2 * nside, np.cos(tc + 5.0 * pixel))
     for c, want in ((inputs.gaussian_beam(2 * nside, 3.0 * pixel), 1),
                     (inputs.gaussian_beam(3 * nside - 1, 3.0 * pixel), 1),
-                    (inputs.gaussian_beam(3 * nside - 1, 2.7 * pixel), 0), (ring, 0)):
+                    (inputs.gaussian_beam(3 * nside - 1, 2.2 * pixel), 0), (ring, 0)):
         with K.make_split_real(c, nside, tc) as sp:
             assert K.split_stages(sp)["cap_stage"] == want
 
