@@ -113,8 +113,8 @@ void drop_cap_tc(ksc_split *s) {
 
 // Whether the cell polynomials carry the kernel to the gather's accuracy; top = the largest |K_r|
 // within the cut, to which outputs compare (not the sum of the Legendre terms, which lies far
-// above it where K_r peaks past the cut or its terms cancel).
-bool cap_polynomials_ok(const ksc_split *s, double top) {
+// above it where K_r peaks past the cut or its terms cancel), cuts = ksc::belt_tc_cuts.
+bool cap_polynomials_ok(const ksc_split *s, double top, double cuts) {
     // Chebyshev interpolation of degree n leaves, of a term l of the kernel, at most about
     // 4 J_{n+1}(l h / 2) ~ 4 (l h / 4)^{n+1} / (n+1)!, h the largest pixel step (1.2826 / nside
     // at the poles).  The coefficients that are multiplied in one part, c_p f^p for p >= n1,
@@ -133,8 +133,13 @@ bool cap_polynomials_ok(const ksc_split *s, double top) {
         err += a * 4.0 * std::pow(x, n + 1) / fact;
         single += a * std::pow(x, n1) / (half * half);
     }
-    const double peak = 4.0 * kPi * top;
-    return err <= 1.25e-7 * peak && single <= std::exp2(-10.5) * peak;
+    // And where the MMAs' cuts add up (the belt's measure serves; a wide kernel that rings to its cut)
+    // the gather is the more accurate one.  Cuts, single, stage / gather: 2048, 240' 1.18, 2^-12.4: 0.82 /
+    // 0.83; 512, 480' 1.19, 2^-13.0: 0.81 / 0.86; 512, 3 pixels, l_cut 460 of 1535: 1.17, 2^-10.8: 0.91 /
+    // 0.88; 512, 3.6 pixels, l_cut 460 of 1535: 1.22, 2^-11.8: 0.90 / 0.84; 512, 5.4 pixels, 800':
+    // 1.36, 2^-16: 0.95 / 0.90; 512, 6.3 pixels, 1200': 3.1, 2^-12.3: 1.76 / 0.99.
+    const double peak = 4.0 * kPi * top, rel = single / (std::exp2(-10.5) * peak);
+    return err <= 1.25e-7 * peak && rel <= 1.0 && cuts + 0.07 * rel <= 1.22;
 }
 
 // Plan of the tensor-core belt stage: the widest window and the most input rings of a
@@ -156,7 +161,8 @@ int plan_belt_tc(ksc_split *s, const ksc::RingGeom &g, const std::vector<int2> &
         drop_cap_tc(s);
         return KSC_OK;
     }
-    if (s->n_cap_tiles && !cap_polynomials_ok(s, top)) drop_cap_tc(s);
+    const double cuts = ksc::belt_tc_cuts(g, s->nside, s->chord_cut, tab.data(), s->n_int);
+    if (s->n_cap_tiles && !cap_polynomials_ok(s, top, cuts)) drop_cap_tc(s);
     s->btc.wscale = s->ctc.wscale = (float)std::ldexp(1.0, ex);
     s->ctc.wunscale = 1.0f / s->ctc.wscale;
     s->ctc.domega_lo = (float)(4.0 * kPi / s->plan.npix - (double)s->plan.domega);
@@ -165,6 +171,12 @@ int plan_belt_tc(ksc_split *s, const ksc::RingGeom &g, const std::vector<int2> &
     // 64, 360': 58 / 72; 256, 160' (2.2e8 pairs): 91 / 99; 512, 60' (5e8): 123 / 122, the call's
     // first pass 483 / 580).  From there on by the estimate at the end.
     if (2.0 / 3.0 * ksc_cost_pairs(s->nside, s->theta_cut) < 8e8) return KSC_OK;
+    // The MMAs' cuts cost an error of about 0.58 cuts in 1e-7 of the output, beside 0.62 of all else;
+    // the FFMA kernel's is 1.0 to 1.16.  Cuts, stage / FFMA: 1.0 to 1.35, 0.76 to 0.98 / 0.91 to 1.10;
+    // 1.42, 1.20 / 1.14 (where the table and the split of the weights err the same way at distance
+    // zero); 1.58, 1.11 / 1.03; 1.8, 1.22 / 1.04; 2.1, 1.36 / 1.14; 4.3 (nside 1024, 7 pixels, l_cut 1100 of
+    // 3016, 860'), 2.56 / 1.16.
+    if (cuts > 1.4) return KSC_OK;
     const int lo = s->plan.belt_lo, hi = s->plan.belt_hi, nb = ksc::belt_tc_rings();
     int wpos = 0, nq = 0;
     for (int r0 = lo; r0 <= hi; r0 += nb) {

@@ -657,6 +657,56 @@ bool belt_tc_plan(int nside, int wpos, int nq, BeltTc *t) {
     return t->n_cols > 0;
 }
 
+double belt_tc_cuts(const RingGeom &g, int nside, double chord_cut, const float4 *tab, int n_int) {
+    // For uncorrelated input a partial sum's variance is that of its weights, and the MMAs run in
+    // the order of the issuing warp; the eight offsets of a core matrix by their middle, the
+    // rings past 24 by one in `step`.
+    const int L = 4 * nside, r = 2 * nside - 1;
+    const double pi = 3.14159265358979323846;
+    const int reach = std::min((int)std::ceil(asin(std::min(1.0, chord_cut / 2.0)) * 3.0 * nside) + 1, nside);
+    const int step = std::max(1, reach / 96);
+    double sum = 0.0, sum2 = 0.0;
+    for (int dq = 0; dq <= reach; dq += dq < 24 ? 1 : step) {
+        const int q = r + dq;
+        const double dz = g.z[q] - g.z[r], ds = g.s[q] - g.s[r], a = dz * dz + ds * ds, b = 4.0 * g.s[q] * g.s[r];
+        const double left = chord_cut * chord_cut - a;
+        if (left <= 0.0) break;
+        const double half = left >= b ? 0.5 * pi : asin(sqrt(left / b));
+        const Window win = tile_window(std::min((int)std::ceil(half * L / pi) + 1, L / 2), L);
+        const double shift = 0.5 * (g.phase[q] - g.phase[r]) - 3.5 + win.d0;
+        auto energy = [&](int s) {
+            double e = 0.0;
+            for (int j = 0; j < 16; ++j) {
+                const double h = sin(pi * (shift + 16 * s + j) / L), d2 = a + b * h * h;
+                if (d2 > chord_cut * chord_cut) continue;
+                const double u = sqrt(d2) * (n_int / chord_cut);
+                const int i = std::min((int)u, n_int - 1);
+                const double f = u - i, v = tab[i].x + f * (tab[i].y + f * (tab[i].z + f * (double)tab[i].w));
+                e += v * v;
+            }
+            return e;
+        };
+        const int c_lo = win.s0 / kSteps, c_hi = (win.s1 - 1) / kSteps;
+        double var = 0.0, cuts = 0.0;  // of the sum so far; over the MMAs
+        for (int cc = c_lo; cc <= c_hi; ++cc) {
+            const int c = chunk_of(cc, c_hi, win.mid);
+            const int t0 = std::max(win.s0, kSteps * c), t1 = std::min(win.s1, kSteps * c + kSteps);
+            cuts += var * (2 * (t1 - t0) + (c == win.mid ? 1 : 0));  // the small products
+            for (int e = 0; e < kSteps; ++e) {
+                const int s = kSteps * c + (c == win.mid ? ((e & 1) ? kSteps - 1 - (e >> 1) : e >> 1) : e);
+                if (s < t0 || s >= t1) continue;
+                var += energy(s);
+                cuts += var;
+            }
+        }
+        if (!(var > 0.0)) continue;
+        const double w = (dq == 0 ? 1.0 : 2.0) * (dq > 24 ? step : 1);
+        sum += w * var;
+        sum2 += w * cuts * (cuts / var);
+    }
+    return sum > 0.0 ? sqrt(sum2 / sum) : 1.0;
+}
+
 long long map_blocks(const ConvPlan &p) { return p.npix / 64; }
 
 cudaError_t launch_block_max(const ConvPlan &p, const MapSet &maps, int n_maps,

@@ -111,7 +111,7 @@ __host__ __device__ __forceinline__ Window tile_window(int w, int L) {
     return g;
 }
 // The chunks of a window in order of work: the closest approach's last.
-__device__ __forceinline__ int chunk_of(int cc, int c_hi, int mid) {
+__host__ __device__ __forceinline__ int chunk_of(int cc, int c_hi, int mid) {
     return cc == c_hi ? mid : (cc >= mid ? cc + 1 : cc);
 }
 
