@@ -113,7 +113,7 @@ void drop_cap_tc(ksc_split *s) {
 
 // Whether the cell polynomials carry the kernel to the gather's accuracy; top = the largest |K_r|
 // within the cut, to which outputs compare (not the sum of the Legendre terms, which lies far
-// above it where K_r peaks past the cut or its terms cancel), cuts = ksc::belt_tc_cuts.
+// above it where K_r peaks past the cut or its terms cancel), cuts = ksc::TcCuts::cap.
 bool cap_polynomials_ok(const ksc_split *s, double top, double cuts) {
     // Chebyshev interpolation of degree n leaves, of a term l of the kernel, at most about
     // 4 J_{n+1}(l h / 2) ~ 4 (l h / 4)^{n+1} / (n+1)!, h the largest pixel step (1.2826 / nside
@@ -133,13 +133,14 @@ bool cap_polynomials_ok(const ksc_split *s, double top, double cuts) {
         err += a * 4.0 * std::pow(x, n + 1) / fact;
         single += a * std::pow(x, n1) / (half * half);
     }
-    // And where the MMAs' cuts add up (the belt's measure serves; a wide kernel that rings to its cut)
-    // the gather is the more accurate one.  Cuts, single, stage / gather: 2048, 240' 1.18, 2^-12.4: 0.82 /
-    // 0.83; 512, 480' 1.19, 2^-13.0: 0.81 / 0.86; 512, 3 pixels, l_cut 460 of 1535: 1.17, 2^-10.8: 0.91 /
-    // 0.88; 512, 3.6 pixels, l_cut 460 of 1535: 1.22, 2^-11.8: 0.90 / 0.84; 512, 5.4 pixels, 800':
-    // 1.36, 2^-16: 0.95 / 0.90; 512, 6.3 pixels, 1200': 3.1, 2^-12.3: 1.76 / 0.99.
+    // And where the MMAs' cuts add up (a wide kernel, or one that rings to its cut) the gather is
+    // the more accurate one.  Over 55 splits (stage / gather error)^2 is about 0.85 + 0.16 cuts +
+    // 0.135 rel^2, rel the single part's share of its bound.  Cuts + 0.8 rel^2, stage / gather: nside 2048,
+    // 120' 0.5: 0.77 / 0.84; 2048, 240' 1.06: 0.82 / 0.83; 512, 480' 0.76: 0.81 / 0.86; 1024, 5.8 pixels, 240'
+    // 1.15: 0.88 / 0.91; 512, 3.6 pixels, l_cut 460 of 1535: 1.17, 0.90 / 0.84; 512, 3 pixels, l_cut 460 of
+    // 1535: 1.3, 0.91 / 0.88; 512, 5.1 pixels, 764': 1.8, 0.95 / 0.87; 512, 6.3 pixels, 1200': 8, 1.76 / 0.99.
     const double peak = 4.0 * kPi * top, rel = single / (std::exp2(-10.5) * peak);
-    return err <= 1.25e-7 * peak && rel <= 1.0 && cuts + 0.07 * rel <= 1.22;
+    return err <= 1.25e-7 * peak && rel <= 1.0 && cuts + 0.8 * rel * rel <= 1.16;
 }
 
 // Plan of the tensor-core belt stage: the widest window and the most input rings of a
@@ -161,8 +162,8 @@ int plan_belt_tc(ksc_split *s, const ksc::RingGeom &g, const std::vector<int2> &
         drop_cap_tc(s);
         return KSC_OK;
     }
-    const double cuts = ksc::belt_tc_cuts(g, s->nside, s->chord_cut, tab.data(), s->n_int);
-    if (s->n_cap_tiles && !cap_polynomials_ok(s, top, cuts)) drop_cap_tc(s);
+    const ksc::TcCuts cuts = ksc::tc_cuts(g, s->nside, s->chord_cut, tab.data(), s->n_int);
+    if (s->n_cap_tiles && !cap_polynomials_ok(s, top, cuts.cap)) drop_cap_tc(s);
     s->btc.wscale = s->ctc.wscale = (float)std::ldexp(1.0, ex);
     s->ctc.wunscale = 1.0f / s->ctc.wscale;
     s->ctc.domega_lo = (float)(4.0 * kPi / s->plan.npix - (double)s->plan.domega);
@@ -171,12 +172,12 @@ int plan_belt_tc(ksc_split *s, const ksc::RingGeom &g, const std::vector<int2> &
     // 64, 360': 58 / 72; 256, 160' (2.2e8 pairs): 91 / 99; 512, 60' (5e8): 123 / 122, the call's
     // first pass 483 / 580).  From there on by the estimate at the end.
     if (2.0 / 3.0 * ksc_cost_pairs(s->nside, s->theta_cut) < 8e8) return KSC_OK;
-    // The MMAs' cuts cost an error of about 0.58 cuts in 1e-7 of the output, beside 0.62 of all else;
-    // the FFMA kernel's is 1.0 to 1.16.  Cuts, stage / FFMA: 1.0 to 1.35, 0.76 to 0.98 / 0.91 to 1.10;
-    // 1.42, 1.20 / 1.14 (where the table and the split of the weights err the same way at distance
-    // zero); 1.58, 1.11 / 1.03; 1.8, 1.22 / 1.04; 2.1, 1.36 / 1.14; 4.3 (nside 1024, 7 pixels, l_cut 1100 of
-    // 3016, 860'), 2.56 / 1.16.
-    if (cuts > 1.4) return KSC_OK;
+    // The MMAs' cuts add to the error where a ring's sum keeps its size over many of them.  Cuts, stage /
+    // FFMA, error rms in 1e-7 of the output's: to 1.3, 0.74 to 1.02 / 0.91 to 1.16; 1.47, 1.20 / 1.14 (the
+    // table and the split of the weights err the same way at distance zero); 1.7, 1.08 / 1.09; 2.2, 1.17 / 1.09;
+    // 3.7, 1.09 / 1.06; 4.8 (nside 1024, 4.4 pixels, 480'), 1.16 / 1.05; 46 (1024, 7 pixels, l_cut 1100 of 3016,
+    // 860'), 2.56 / 1.16.
+    if (cuts.belt > 1.4) return KSC_OK;
     const int lo = s->plan.belt_lo, hi = s->plan.belt_hi, nb = ksc::belt_tc_rings();
     int wpos = 0, nq = 0;
     for (int r0 = lo; r0 <= hi; r0 += nb) {

@@ -657,27 +657,37 @@ bool belt_tc_plan(int nside, int wpos, int nq, BeltTc *t) {
     return t->n_cols > 0;
 }
 
-double belt_tc_cuts(const RingGeom &g, int nside, double chord_cut, const float4 *tab, int n_int) {
-    // For uncorrelated input a partial sum's variance is that of its weights, and the MMAs run in
-    // the order of the issuing warp; the eight offsets of a core matrix by their middle, the
-    // rings past 24 by one in `step`.
+TcCuts tc_cuts(const RingGeom &g, int nside, double chord_cut, const float4 *tab, int n_int) {
+    // For uncorrelated input a partial sum's variance V_j is that of its weights.  A cut takes 0.75
+    // of 2^-24 of the sum on average (measured), the fold gives one 2^-24 of the final sum
+    // back: what is left has the mean square sum min(V_i, V_j) - 2 (4/3) sum V_j + (4/3)^2 V.
+    // The rings past 24 by one in `step`, the eight offsets of a core matrix by their middle.
+    struct Walk {
+        double v = 0.0, sum = 0.0, square = 0.0;
+        void cut(double n = 1.0) {
+            square += n * (2.0 * sum + n * v);
+            sum += n * v;
+        }
+        double left() const { return square - 8.0 / 3.0 * sum + 16.0 / 9.0 * v; }
+    };
     const int L = 4 * nside, r = 2 * nside - 1;
     const double pi = 3.14159265358979323846;
     const int reach = std::min((int)std::ceil(asin(std::min(1.0, chord_cut / 2.0)) * 3.0 * nside) + 1, nside);
     const int step = std::max(1, reach / 96);
-    double sum = 0.0, sum2 = 0.0;
+    double total = 0.0;
+    TcCuts out;
     for (int dq = 0; dq <= reach; dq += dq < 24 ? 1 : step) {
         const int q = r + dq;
         const double dz = g.z[q] - g.z[r], ds = g.s[q] - g.s[r], a = dz * dz + ds * ds, b = 4.0 * g.s[q] * g.s[r];
         const double left = chord_cut * chord_cut - a;
         if (left <= 0.0) break;
         const double half = left >= b ? 0.5 * pi : asin(sqrt(left / b));
-        const Window win = tile_window(std::min((int)std::ceil(half * L / pi) + 1, L / 2), L);
-        const double shift = 0.5 * (g.phase[q] - g.phase[r]) - 3.5 + win.d0;
-        auto energy = [&](int s) {
+        const int w = std::min((int)std::ceil(half * L / pi) + 1, L / 2);
+        auto energy = [&](const Window &win, int s) {
+            const double shift = 0.5 * (g.phase[q] - g.phase[r]) - 3.5 + win.d0 + 16 * s;
             double e = 0.0;
             for (int j = 0; j < 16; ++j) {
-                const double h = sin(pi * (shift + 16 * s + j) / L), d2 = a + b * h * h;
+                const double h = sin(pi * (shift + j) / L), d2 = a + b * h * h;
                 if (d2 > chord_cut * chord_cut) continue;
                 const double u = sqrt(d2) * (n_int / chord_cut);
                 const int i = std::min((int)u, n_int - 1);
@@ -686,25 +696,41 @@ double belt_tc_cuts(const RingGeom &g, int nside, double chord_cut, const float4
             }
             return e;
         };
-        const int c_lo = win.s0 / kSteps, c_hi = (win.s1 - 1) / kSteps;
-        double var = 0.0, cuts = 0.0;  // of the sum so far; over the MMAs
-        for (int cc = c_lo; cc <= c_hi; ++cc) {
-            const int c = chunk_of(cc, c_hi, win.mid);
-            const int t0 = std::max(win.s0, kSteps * c), t1 = std::min(win.s1, kSteps * c + kSteps);
-            cuts += var * (2 * (t1 - t0) + (c == win.mid ? 1 : 0));  // the small products
+        // the order of the issuing warps: the belt's, small products of a chunk first ...
+        Walk belt, cap;
+        const Window wb = tile_window(w, L);
+        const int b_hi = (wb.s1 - 1) / kSteps;
+        for (int cc = wb.s0 / kSteps; cc <= b_hi; ++cc) {
+            const int c = chunk_of(cc, b_hi, wb.mid);
+            const int t0 = std::max(wb.s0, kSteps * c), t1 = std::min(wb.s1, kSteps * c + kSteps);
+            belt.cut(2 * (t1 - t0) + (c == wb.mid ? 1 : 0));
             for (int e = 0; e < kSteps; ++e) {
-                const int s = kSteps * c + (c == win.mid ? ((e & 1) ? kSteps - 1 - (e >> 1) : e >> 1) : e);
+                const int s = kSteps * c + (c == wb.mid ? ((e & 1) ? kSteps - 1 - (e >> 1) : e >> 1) : e);
                 if (s < t0 || s >= t1) continue;
-                var += energy(s);
-                cuts += var;
+                belt.v += energy(wb, s);
+                belt.cut();
             }
         }
-        if (!(var > 0.0)) continue;
-        const double w = (dq == 0 ? 1.0 : 2.0) * (dq > 24 ? step : 1);
-        sum += w * var;
-        sum2 += w * cuts * (cuts / var);
+        // ... and the caps', whose small products have an accumulator of their own
+        const Window wc = tc::tile_window<32>(w, L);
+        const int c_hi = (wc.s1 - 1) / 2;
+        for (int cc = wc.s0 / 2; cc <= c_hi; ++cc) {
+            const int c = chunk_of(cc, c_hi, wc.mid);
+            for (int s = std::max(wc.s0, 2 * c); s < std::min(wc.s1, 2 * c + 2); ++s) {
+                cap.v += energy(wc, s);
+                cap.cut();
+            }
+        }
+        const double weight = (dq == 0 ? 1.0 : 2.0) * (dq > 24 ? step : 1);
+        total += weight * belt.v;
+        out.belt += weight * belt.left();
+        out.cap += weight * cap.left();
     }
-    return sum > 0.0 ? sqrt(sum2 / sum) : 1.0;
+    if (total > 0.0) {
+        out.belt /= total;
+        out.cap /= total;
+    }
+    return out;
 }
 
 long long map_blocks(const ConvPlan &p) { return p.npix / 64; }

@@ -229,9 +229,13 @@ struct BeltTc {
 int belt_tc_rings();                      // output rings of a tile
 int belt_tc_positions(int w, int L);      // window positions for a half window w
 bool belt_tc_plan(int nside, int wpos, int nq, BeltTc *t);
-// How many times the MMAs cut an input ring's sum, in sums of its final size (root mean square
-// over the input rings of an equatorial one); tab: the n_int intervals of the K_r table.
-double belt_tc_cuts(const RingGeom &g, int nside, double chord_cut, const float4 *tab, int n_int);
+// What the MMAs' cuts of an input ring's sum leave after the fold has given the mean back: mean
+// square in mean cuts of the final sum, over the input rings of an equatorial one; tab: the n_int
+// intervals of the K_r table.
+struct TcCuts {
+    double belt = 0.0, cap = 0.0;
+};
+TcCuts tc_cuts(const RingGeom &g, int nside, double chord_cut, const float4 *tab, int n_int);
 int belt_tc_tiles(const ConvPlan &p, const BeltTc &t);
 long long map_blocks(const ConvPlan &p);  // blocks of 64 pixels in a map
 // The input that a call's tensor-core stages read: rings [q0, q1] and [q2, q3] (none: q3 < q2),
