@@ -232,7 +232,7 @@ int ksc_split_table(const ksc_split *s, float *host_coeffs);
  * arrays of 12 nside^2 floats, nside as given to the split; in != out).
  * Asynchronous on `stream`.  Each call takes its scratch (work-claim counters;
  * with the tensor-core stages, taken from 8e8 belt pairs on where they are
- * estimated to be clearly faster, also npix / 16 bytes a map of block maxima, and
+ * estimated to be clearly faster and no less accurate, also npix / 16 bytes a map of block maxima, and
  * flags; without room for these the FFMA kernels run) from the device's default
  * stream-ordered memory pool (cudaMallocAsync / cudaFreeAsync on `stream`), or from
  * one of two sets that the split keeps, if the call that had it last has ended; so
